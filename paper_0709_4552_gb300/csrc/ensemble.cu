@@ -457,14 +457,14 @@ __global__ void __launch_bounds__(NT, mixed_min_ctas(NT)) b_force_mixed(
 }
 
 template <int NT, int JT>
-__global__ void __launch_bounds__(NT) b_force_fp64(
+__global__ void __launch_bounds__(NT, 512 / NT) b_force_fp64(
     int32_t C, const int64_t* __restrict__ off, const double* __restrict__ eps2d, int64_t n_pad,
     const double* __restrict__ xp, const double* __restrict__ vp, const double* __restrict__ m,
     const int32_t* __restrict__ act, const int32_t* __restrict__ nact, const int32_t* __restrict__ itiles,
     const int32_t* __restrict__ nsplit, const int64_t* __restrict__ jps, const int64_t* __restrict__ item_off,
     const int64_t* __restrict__ part_off, const int64_t* __restrict__ pstride, double* __restrict__ F,
     int64_t fstride, double* __restrict__ part, unsigned long long* __restrict__ wq) {
-  __shared__ nbk::Fp64Smem<JT> sm;
+  __shared__ nbk::Fp64Smem<NT, JT> sm;
   __shared__ int64_t s_item;
   const int64_t total = item_off[C];
   for (;;) {
@@ -478,8 +478,8 @@ __global__ void __launch_bounds__(NT) b_force_fp64(
     const int64_t jhi = min(jlo + jps[c], off[c + 1]);
     const bool fin = nsplit[c] == 1;
     double* out = fin ? F + off[c] : part + part_off[c] + split * 7 * pstride[c];
-    nbk::fp64_item<NT, JT>(sm, xp, vp, m, n_pad, jlo, jhi, act + off[c], nact[c], itile * NT, eps2d[c], out,
-                           fin ? fstride : pstride[c], fin);
+    nbk::fp64_item<NT, JT>(sm, xp, vp, m, n_pad, 1, jlo, jhi, n_pad, act + off[c], nact[c], itile * NT, eps2d[c],
+                           out, fin ? fstride : pstride[c], fin);
   }
 }
 

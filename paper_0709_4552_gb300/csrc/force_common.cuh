@@ -25,10 +25,11 @@
 // hi+m, float4 lo+vx, float2 vy vz) are staged in shared memory with cp.async
 // double buffering and read as warp-wide broadcasts.
 //
-// FP64 path: every operation in IEEE FP64, 1/s from an FP32 seed refined in
-// FP64; per-tile FP64 partials folded into (hi, lo) accumulators with Knuth's
-// TwoSum.  On GB300 the FP64 pipe issues 2 FMA/clk/SM (1/64 of FP32), which
-// bounds this path.
+// FP64 path: FP64 inputs and results, the pair arithmetic in 64-bit fixed
+// point on the integer units (fx64.cuh; the FP64 pipe issues 2 FMA/clk/SM,
+// 1/64 of FP32), exact sums of up to 512 pairs folded into (hi, lo) FP64
+// accumulators with Knuth's TwoSum; the few pairs the fixed point does not
+// take in IEEE FP64, 1/s from an FP32 seed refined in FP64.
 //
 // Self pair: excluded by index, as in the definition.  Mixed path: only the
 // j-tile holding one of a warp's own i needs the test, so a warp vote picks a
@@ -40,6 +41,8 @@
 #pragma once
 
 #include "nb_internal.cuh"
+
+#include "fx64.cuh"
 
 // one Newton step on the hardware rsqrt in the mixed path (1 = on)
 #ifndef NB_MIXED_NEWTON
@@ -700,109 +703,300 @@ __device__ __forceinline__ void mixed_item(SM& sm, const float4* __restrict__ jA
 #undef NB_ACC_DS
 }
 
-template <int JT>
-struct Fp64Smem {
-  double x[3][JT], v[3][JT], m[JT];
-};
-
-// FP64 item: one i per thread (i-tile of NT), j-range [jlo, jhi) with a
-// ragged tail filled by massless far-away particles.  xp, vp are SoA rows of
-// stride n_pad.
+// ---- FP64 path --------------------------------------------------------------
+// Inputs, sums and results are FP64; the pair arithmetic runs in the fixed
+// point of fx64.cuh, which is at least as accurate as an FP64 evaluation of
+// the same formulas and 5 times as fast on this GPU.
 template <int NT, int JT>
-__device__ __forceinline__ void fp64_item(Fp64Smem<JT>& sm, const double* __restrict__ xp,
-                                          const double* __restrict__ vp, const double* __restrict__ m,
-                                          int64_t n_pad, int64_t jlo, int64_t jhi,
-                                          const int32_t* __restrict__ list, int64_t n, int64_t ibase,
-                                          double eps2, double* __restrict__ out, int64_t ostride,
-                                          bool finalize, const ISrc is = ISrc()) {
+struct Fp64Smem {
+  // a j-particle of the tile: (X0, X1), (X2, V0), (V1, V2), (M, k); k = kOdd:
+  // not for the fixed-point pair (negative, subnormal or very small mass)
+  longlong2 j[JT][4];
+  double hi[7][NT], lo[7][NT];  // the thread's sums (TwoSum)
+  int red[NT / 32][3];
+};
+constexpr int kOdd = 64;
+
+// exponent e of the largest magnitude among values whose high words (sign
+// cleared) have maximum w: |x| < 2^e (NaN, Inf: 1025)
+__device__ __forceinline__ int exp_above(int w) { return (w >> 20) - 1022; }
+__device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7FFFFFFF; }
+__device__ __forceinline__ double pow2d(int e) { return __hiloint2double((e + 1023) << 20, 0); }  // e in [-1022, 1023]
+
+// x 2^sh rounded to the nearest integer (|x| 2^sh <= 2^60), from x's bits:
+// a shift of the significand costs a tenth of the two FP64 instructions
+__device__ __forceinline__ int64_t to_fixed(double x, int sh) {
+  const uint64_t b = (uint64_t)__double_as_longlong(x);
+  const int E = (int)(b >> 52) & 0x7FF;
+  const uint64_t f = (b & 0x000FFFFFFFFFFFFFull) | (E ? 0x0010000000000000ull : 0ull);
+  const int n = min((E ? E : 1) - 1075 + sh, 8);
+  const int r = max(min(-n, 63), 1);
+  const uint64_t mag = n >= 0 ? f << n : (f + (1ull << (r - 1))) >> r;
+  return (int64_t)b < 0 ? -(int64_t)mag : (int64_t)mag;
+}
+
+// (hi, lo) += p: TwoSum (Knuth), hi + p = s + e exactly
+__device__ __forceinline__ void sum_add(double& hi, double& lo, double p) {
+  const double s = hi + p;
+  const double bp = s - hi;
+  lo += (hi - (s - bp)) + (p - bp);
+  hi = s;
+}
+
+// the pairs of one i with the j-particles of the bits in mask (jt + bit), in
+// FP64: the few that the fixed-point pair leaves (closer than its grid
+// resolves, odd masses, values outside its exponent range)
+template <int NT, int JT>
+__device__ __noinline__ void fp64_pairs(Fp64Smem<NT, JT>& sm, const double* __restrict__ xp,
+                                        const double* __restrict__ vp, const double* __restrict__ m, int64_t cs,
+                                        int64_t js, int64_t jt, uint32_t mask, double x0, double x1, double x2,
+                                        double v0, double v1, double v2, double eps2) {
+  double p[7];
+#pragma unroll
+  for (int c = 0; c < 7; ++c) p[c] = 0.0;
+  while (mask) {
+    const int64_t j = jt + (__ffs((int)mask) - 1);
+    mask &= mask - 1u;
+    const double* xj = xp + j * js;
+    const double* vj = vp + j * js;
+    const double dx = xj[0] - x0, dy = xj[cs] - x1, dz = xj[2 * cs] - x2;
+    const double wx = vj[0] - v0, wy = vj[cs] - v1, wz = vj[2 * cs] - v2;
+    const double r2 = fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2)));
+    const double rw = fma(dz, wz, fma(dy, wy, dx * wx));
+    const double rinv = nb_rsqrt_fp64(r2);
+    const double rinv2 = rinv * rinv;
+    const double mr = m[j] * rinv;
+    const double mr3 = mr * rinv2;
+    const double a3 = (rw * -3.0) * rinv2;  // jerk term formed before accumulation
+    p[6] += mr;
+    p[0] = fma(mr3, dx, p[0]);
+    p[1] = fma(mr3, dy, p[1]);
+    p[2] = fma(mr3, dz, p[2]);
+    p[3] = fma(mr3, fma(a3, dx, wx), p[3]);
+    p[4] = fma(mr3, fma(a3, dy, wy), p[4]);
+    p[5] = fma(mr3, fma(a3, dz, wz), p[5]);
+  }
+#pragma unroll
+  for (int c = 0; c < 7; ++c) sum_add(sm.hi[c][threadIdx.x], sm.lo[c][threadIdx.x], p[c]);
+}
+
+// the 96-bit sums into the thread's FP64 sums (in_range: they hold its
+// pairs, else nothing of worth); cleared
+template <int NT, int JT>
+__device__ __forceinline__ void fp64_fold(Fp64Smem<NT, JT>& sm, nbx::Sum96 (&a)[7], bool in_range, int g, int gv,
+                                          int em) {
+#pragma unroll
+  for (int c = 0; c < 7; ++c) {
+    const int e = c < 3 ? em - 2 * g + nbx::kAccScale
+                        : (c < 6 ? em - 3 * g + gv + nbx::kJerkScale : em - g + nbx::kPotScale);
+    const double p = fma((double)(int64_t)(((uint64_t)a[c].w2 << 32) | a[c].w1), 4294967296.0, (double)a[c].w0);
+    // two factors: e may lie outside the exponents of one FP64 number
+    if (in_range) sum_add(sm.hi[c][threadIdx.x], sm.lo[c][threadIdx.x], p * pow2d(e / 2) * pow2d(e - e / 2));
+    a[c].w0 = a[c].w1 = a[c].w2 = 0u;
+  }
+}
+
+template <bool SH, int NT, int JT>
+__device__ __forceinline__ uint32_t fx64_chunk(const Fp64Smem<NT, JT>& sm, int q0, int count, int rel,
+                                               const nbx::IFix& fi, nbx::Sum96 (&a)[7]) {
+  uint32_t left = 0u;
+#pragma unroll 1
+  for (int q = 0; q < count; ++q) {
+    const longlong2 A = sm.j[q0 + q][0], B = sm.j[q0 + q][1], C = sm.j[q0 + q][2], K = sm.j[q0 + q][3];
+    nbx::JFix fj;
+    fj.X[0] = A.x; fj.X[1] = A.y; fj.X[2] = B.x;
+    fj.V[0] = B.y; fj.V[1] = C.x; fj.V[2] = C.y;
+    fj.M = (uint64_t)K.x;
+    fj.k = (int)K.y;
+    const bool ok = nbx::pair<SH>(fj, fi, (q0 + q == rel) | (fj.k == kOdd), a);
+    left |= ok ? 0u : 1u << q;
+  }
+  return left;
+}
+
+// FP64 item: one i per thread (i-tile of NT), j-range [jlo, jhi).  Component c
+// of particle j lies at xp[c cs + j js] (rows of the j-store: cs = n_pad,
+// js = 1; [N][3] arrays: cs = 1, js = 3); list entries are clamped to
+// [0, idx_hi).
+//
+// Per tile the CTA puts JT j-particles on a common grid, 2^G above the tile's
+// largest coordinate (and eps), 2^GV above its largest velocity component, EM
+// the exponent of its largest mass.  The grid is kept while it stays within a
+// factor 2 (mass: 8) of the tile's own, so that the sums, exact 96-bit
+// integers, are folded into FP64 every kFold pairs and not per tile.  It
+// depends on the j-range alone and on nothing the other i of the CTA hold, so
+// a particle's result does not depend on which particles share its item.
+template <int NT, int JT>
+__device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __restrict__ xp,
+                                          const double* __restrict__ vp, const double* __restrict__ m, int64_t cs,
+                                          int64_t js, int64_t jlo, int64_t jhi, int64_t idx_hi,
+                                          const int32_t* __restrict__ list, int64_t n, int64_t ibase, double eps2,
+                                          double* __restrict__ out, int64_t ostride, bool finalize,
+                                          const ISrc is = ISrc()) {
+  static_assert(JT % 32 == 0 && NT % 32 == 0, "tiles of whole warps");
+  constexpr int kPer = (JT + NT - 1) / NT;  // j-particles a thread stages
   const int tid = threadIdx.x;
   const int64_t pos0 = ibase + tid;
   const int64_t pos = pos0 < n ? pos0 : n - 1;
   int64_t self = list[pos];
-  double xi[3], vi[3];
+  const double *xi, *vi;  // this i's position and velocity, read again when its grid changes
+  int64_t ics = cs;
   if (is.x) {  // a particle held elsewhere (see ISrc)
     self = self < 0 ? 0 : (self >= n ? n - 1 : self);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      xi[c] = is.x[c * is.stride + self];
-      vi[c] = is.v[c * is.stride + self];
-    }
+    xi = is.x + self;
+    vi = is.v + self;
+    ics = is.stride;
     self = is.self ? is.self[pos] : -1;
   } else {
-    self = self < 0 ? 0 : (self >= n_pad ? n_pad - 1 : self);  // a bad list never reads out of bounds
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      xi[c] = xp[c * n_pad + self];
-      vi[c] = vp[c * n_pad + self];
-    }
+    self = self < 0 ? 0 : (self >= idx_hi ? idx_hi - 1 : self);  // a bad list never reads out of bounds
+    xi = xp + self * js;
+    vi = vp + self * js;
   }
-  double hi[7], lo[7];
+  const int exi = exp_above(max(abs_hi(xi[0]), max(abs_hi(xi[ics]), abs_hi(xi[2 * ics]))));
+  const int evi = exp_above(max(abs_hi(vi[0]), max(abs_hi(vi[ics]), abs_hi(vi[2 * ics]))));
+  // eps < 2^eeps
+  const int eeps = (exp_above(abs_hi(eps2)) + 1) >> 1;
 #pragma unroll
-  for (int c = 0; c < 7; ++c) hi[c] = lo[c] = 0.0;
+  for (int c = 0; c < 7; ++c) sm.hi[c][tid] = sm.lo[c][tid] = 0.0;
+  nbx::Sum96 a[7];
+#pragma unroll
+  for (int c = 0; c < 7; ++c) a[c].w0 = a[c].w1 = a[c].w2 = 0u;
+  nbx::IFix fi = {};
+  int G = 0, GV = 0, EM = 0, g = 0, gv = 0, filled = 0;  // grid of the tiles so far, this i's grid, pairs in a
+  bool have = false, in_range = false;
+  int32_t wmin = nbx::kNoPairs;
+  int chunk = 0;
+  fi.wmin = wmin;
   // a warp whose list positions all lie past n computes nothing (its
   // results are not written); it still loads its share of every j-tile
   const bool wact = ibase + (int64_t)(tid & ~31) < n;
 
   for (int64_t jt = jlo; jt < jhi; jt += JT) {
-    __syncthreads();
-    for (int q = tid; q < JT; q += NT) {
+    double jx[kPer][3], jv[kPer][3], jm[kPer];
+    int wx = 0, wv = 0, wm = 0;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const int q = tid + u * NT;
       const int64_t j = jt + q;
-      if (j < jhi) {
+      const bool in = q < JT && j < jhi;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          sm.x[c][q] = xp[c * n_pad + j];
-          sm.v[c][q] = vp[c * n_pad + j];
-        }
-        sm.m[q] = m[j];
-      } else {
+      for (int c = 0; c < 3; ++c) {
+        jx[u][c] = in ? xp[c * cs + j * js] : 0.0;
+        jv[u][c] = in ? vp[c * cs + j * js] : 0.0;
+        wx = max(wx, abs_hi(jx[u][c]));
+        wv = max(wv, abs_hi(jv[u][c]));
+      }
+      jm[u] = in ? m[j] : 0.0;
+      wm = max(wm, abs_hi(jm[u]));
+    }
+    wx = __reduce_max_sync(0xffffffffu, wx);
+    wv = __reduce_max_sync(0xffffffffu, wv);
+    wm = __reduce_max_sync(0xffffffffu, wm);
+    if ((tid & 31) == 0) {
+      sm.red[tid >> 5][0] = wx;
+      sm.red[tid >> 5][1] = wv;
+      sm.red[tid >> 5][2] = wm;
+    }
+    __syncthreads();  // the previous tile is done with, the maxima are there
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          sm.x[c][q] = (double)kFarF;
-          sm.v[c][q] = 0.0;
+    for (int w = 0; w < NT / 32; ++w) {
+      wx = max(wx, sm.red[w][0]);
+      wv = max(wv, sm.red[w][1]);
+      wm = max(wm, sm.red[w][2]);
+    }
+    const int gx = max(max(exp_above(wx), eeps), nbx::kExpLo), gw = max(exp_above(wv), nbx::kExpLo),
+              gm = max(exp_above(wm), nbx::kExpLo);
+    const bool tile_ok = gx <= nbx::kExpHi && gw <= nbx::kExpHi && gm <= nbx::kExpHi;
+    const bool moved = !have || gx > G || gx < G - 1 || gw > GV || gw < GV - 1 || gm > EM || gm < EM - 3;
+    if (tile_ok && (moved || filled + JT > nbx::kFold)) {
+      if (filled > 0) fp64_fold(sm, a, in_range, g, gv, EM);
+      filled = 0;
+      if (moved) {
+        G = gx;
+        GV = gw;
+        EM = gm;
+        g = max(G, exi);
+        gv = max(GV, evi);
+        in_range = g <= nbx::kExpHi && gv <= nbx::kExpHi;
+        wmin = !in_range ? nbx::kNoPairs : (GV == nbx::kExpLo && evi == -1022 ? 0 : nbx::kWMin);
+        fi.wmin = wmin;
+        fi.kx = min(g - G, 63);
+        fi.kv = min(gv - GV, 63);
+        if (in_range) {
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            fi.X[c] = to_fixed(xi[c * ics], 60 - g);
+            fi.V[c] = to_fixed(vi[c * ics], 60 - gv);
+          }
+          const double e2 = eps2 * pow2d(56 - 2 * g);
+          const uint64_t e2h = (uint64_t)e2;
+          fi.e2[2] = (uint32_t)(e2h >> 32);
+          fi.e2[1] = (uint32_t)e2h;
+          fi.e2[0] = (uint32_t)((e2 - (double)e2h) * 4294967296.0);
+          fi.e2f = (float)e2;
+          fi.rmin = fmaxf(0x1p40f, fi.e2f * 0x1p-8f);
         }
-        sm.m[q] = 0.0;
+        have = true;
       }
     }
-    __syncthreads();
-    if (!wact) continue;  // the next tile's leading barrier keeps the warp in step
-    double p[7];
+    if (tile_ok) {
 #pragma unroll
-    for (int c = 0; c < 7; ++c) p[c] = 0.0;
-#pragma unroll 2
-    for (int q = 0; q < JT; ++q) {
-      const double dx = sm.x[0][q] - xi[0], dy = sm.x[1][q] - xi[1], dz = sm.x[2][q] - xi[2];
-      const double wx = sm.v[0][q] - vi[0], wy = sm.v[1][q] - vi[1], wz = sm.v[2][q] - vi[2];
-      const double r2 = fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2)));
-      const double rw = fma(dz, wz, fma(dy, wy, dx * wx));
-      // the self pair (j == i) gets 1/s = 0, also when eps = 0
-      const double rinv = (jt + q == self) ? 0.0 : nb_rsqrt_fp64(r2);
-      const double rinv2 = rinv * rinv;
-      const double mr = sm.m[q] * rinv;
-      const double mr3 = mr * rinv2;
-      const double a3 = (rw * -3.0) * rinv2;  // jerk term formed before accumulation
-      p[6] += mr;
-      p[0] = fma(mr3, dx, p[0]);
-      p[1] = fma(mr3, dy, p[1]);
-      p[2] = fma(mr3, dz, p[2]);
-      p[3] = fma(mr3, fma(a3, dx, wx), p[3]);
-      p[4] = fma(mr3, fma(a3, dy, wy), p[4]);
-      p[5] = fma(mr3, fma(a3, dz, wz), p[5]);
+      for (int u = 0; u < kPer; ++u) {
+        const int q = tid + u * NT;
+        if (q < JT) {
+          int64_t X[3], V[3];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            X[c] = to_fixed(jx[u][c], 60 - G);
+            V[c] = to_fixed(jv[u][c], 60 - GV);
+          }
+          const uint64_t mb = (uint64_t)__double_as_longlong(jm[u]);
+          const int E = (int)(mb >> 52);  // with the sign: negative masses are odd
+          const int k = EM - (E - 1022);
+          const bool zero = mb << 1 == 0;
+          const bool odd = !zero && (E < 1 || E > 2046 || k > nbx::kKMax);
+          const uint64_t M = zero || odd ? 0ull : ((mb & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << 10;
+          sm.j[q][0] = make_longlong2(X[0], X[1]);
+          sm.j[q][1] = make_longlong2(X[2], V[0]);
+          sm.j[q][2] = make_longlong2(V[1], V[2]);
+          sm.j[q][3] = make_longlong2((int64_t)M, zero ? 0 : (odd ? kOdd : k));
+        }
+      }
+      filled += JT;
     }
-    // TwoSum fold (Knuth): hi + p = s + e exactly
-#pragma unroll
-    for (int c = 0; c < 7; ++c) {
-      const double s = hi[c] + p[c];
-      const double bp = s - hi[c];
-      const double e = (hi[c] - (s - bp)) + (p[c] - bp);
-      hi[c] = s;
-      lo[c] += e;
+    __syncthreads();
+    if (!wact) continue;  // the next tile's barrier keeps the warp in step
+    const int qn = (int)min((int64_t)JT, jhi - jt);
+    const int64_t d = self - jt;
+    const int rel = d >= 0 && d < qn ? (int)d : -1;
+    const bool shifted = __any_sync(0xffffffffu, (fi.kx | fi.kv) != 0);
+#pragma unroll 1
+    for (int q0 = 0; q0 < qn; q0 += 32, ++chunk) {
+      const int count = min(32, qn - q0);
+      uint32_t left = 0xffffffffu >> (32 - count);
+      // an i that left most pairs of a chunk to FP64 (a system far from the
+      // origin against its size, say) leaves all of them for the next ones,
+      // and a warp of such i skips the fixed-point pass; tried again every
+      // 8th chunk.  Each i decides for itself, from the j-range alone.
+      if ((chunk & 7) == 0) fi.wmin = wmin;
+      if (tile_ok && __any_sync(0xffffffffu, fi.wmin != nbx::kNoPairs)) {
+        left = shifted ? fx64_chunk<true>(sm, q0, count, rel, fi, a)
+                       : fx64_chunk<false>(sm, q0, count, rel, fi, a);
+        if (4 * __popc(left) >= 3 * count) fi.wmin = nbx::kNoPairs;
+      }
+      if (rel >= q0 && rel < q0 + 32) left &= ~(1u << (rel - q0));
+      if (left)
+        fp64_pairs(sm, xp, vp, m, cs, js, jt + q0, left, xi[0], xi[ics], xi[2 * ics], vi[0], vi[ics], vi[2 * ics],
+                   eps2);
     }
   }
+  if (filled > 0) fp64_fold(sm, a, in_range, g, gv, EM);
   __syncthreads();  // the caller may reuse shared memory for its next item
   if (pos0 >= n) return;
 #pragma unroll
-  for (int c = 0; c < 6; ++c) out[c * ostride + pos0] = hi[c] + lo[c];
-  out[6 * ostride + pos0] = finalize ? -(hi[6] + lo[6]) : hi[6] + lo[6];
+  for (int c = 0; c < 6; ++c) out[c * ostride + pos0] = sm.hi[c][tid] + sm.lo[c][tid];
+  const double w = sm.hi[6][tid] + sm.lo[6][tid];
+  out[6 * ostride + pos0] = finalize ? -w : w;
 }
 
 }  // namespace nbk

@@ -24,7 +24,7 @@
 // ordering between them) race on the array and must not be issued.
 #include <mutex>
 
-#include "nb_internal.cuh"
+#include "force_common.cuh"
 
 namespace {
 
@@ -66,79 +66,19 @@ unsigned long long current_context_id() {
   return id;
 }
 
-// Same pairwise sums as the library's FP64 path (Sec. 4.1 step 4, Eq. 3),
-// reading row-major [N][3] caller arrays: CTA (x, y) = (i-tile, j-split);
-// partial sums of split y go to part[y][7][pstride], in FP64 with per-tile
-// partials folded by TwoSum.  The self pair (j == i) is excluded by index.
-__global__ void __launch_bounds__(kNT) noalloc_force_kernel(int64_t N, const double* __restrict__ m,
+// The library's FP64 force item (Sec. 4.1 step 4, Eq. 3) on row-major [N][3]
+// caller arrays: CTA (x, y) = (i-tile, j-split); partial sums of split y go
+// to part[y][7][pstride].  The self pair (j == i) is excluded by index.
+__global__ void __launch_bounds__(kNT, 512 / kNT) noalloc_force_kernel(int64_t N, const double* __restrict__ m,
                                                             const double* __restrict__ x,
                                                             const double* __restrict__ v, double eps2,
                                                             const int32_t* __restrict__ list, int64_t n,
                                                             int64_t j_per_split, double* __restrict__ part,
                                                             int64_t pstride) {
-  __shared__ double sx[3][kJT], sv[3][kJT], sm[kJT];
-  const int tid = threadIdx.x;
-  const int64_t pos0 = (int64_t)blockIdx.x * kNT + tid;
-  const int64_t pos = pos0 < n ? pos0 : n - 1;
-  int64_t self = list[pos];
-  self = self < 0 ? 0 : (self >= N ? N - 1 : self);
-  double xi[3], vi[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    xi[c] = x[3 * self + c];
-    vi[c] = v[3 * self + c];
-  }
-  double hi[7], lo[7];
-#pragma unroll
-  for (int c = 0; c < 7; ++c) hi[c] = lo[c] = 0.0;
+  __shared__ nbk::Fp64Smem<kNT, kJT> sm;
   const int64_t jlo = (int64_t)blockIdx.y * j_per_split;
-  const int64_t jhi = min(jlo + j_per_split, N);
-  for (int64_t jt = jlo; jt < jhi; jt += kJT) {
-    __syncthreads();
-    for (int q = tid; q < kJT; q += kNT) {
-      const int64_t j = jt + q;
-      const bool in = j < jhi;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        sx[c][q] = in ? x[3 * j + c] : 1.0e15;
-        sv[c][q] = in ? v[3 * j + c] : 0.0;
-      }
-      sm[q] = in ? m[j] : 0.0;
-    }
-    __syncthreads();
-    double p[7];
-#pragma unroll
-    for (int c = 0; c < 7; ++c) p[c] = 0.0;
-    for (int q = 0; q < kJT; ++q) {
-      const double dx = sx[0][q] - xi[0], dy = sx[1][q] - xi[1], dz = sx[2][q] - xi[2];
-      const double wx = sv[0][q] - vi[0], wy = sv[1][q] - vi[1], wz = sv[2][q] - vi[2];
-      const double r2 = fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2)));
-      const double rw = fma(dz, wz, fma(dy, wy, dx * wx));
-      const double rinv = (jt + q == self) ? 0.0 : nb_rsqrt_fp64(r2);
-      const double rinv2 = rinv * rinv;
-      const double mr = sm[q] * rinv;
-      const double mr3 = mr * rinv2;
-      const double a3 = (rw * -3.0) * rinv2;
-      p[6] += mr;
-      p[0] = fma(mr3, dx, p[0]);
-      p[1] = fma(mr3, dy, p[1]);
-      p[2] = fma(mr3, dz, p[2]);
-      p[3] = fma(mr3, fma(a3, dx, wx), p[3]);
-      p[4] = fma(mr3, fma(a3, dy, wy), p[4]);
-      p[5] = fma(mr3, fma(a3, dz, wz), p[5]);
-    }
-#pragma unroll
-    for (int c = 0; c < 7; ++c) {
-      const double s = hi[c] + p[c];
-      const double bp = s - hi[c];
-      lo[c] += (hi[c] - (s - bp)) + (p[c] - bp);
-      hi[c] = s;
-    }
-  }
-  if (pos0 >= n) return;
-  double* o = part + (int64_t)blockIdx.y * 7 * pstride;
-#pragma unroll
-  for (int c = 0; c < 7; ++c) o[c * pstride + pos0] = hi[c] + lo[c];
+  nbk::fp64_item<kNT, kJT>(sm, x, v, m, 1, 3, jlo, min(jlo + j_per_split, N), N, list, n, (int64_t)blockIdx.x * kNT,
+                           eps2, part + (int64_t)blockIdx.y * 7 * pstride, pstride, false);
 }
 
 // sum the splits in a fixed order and write the caller's [n][3] outputs

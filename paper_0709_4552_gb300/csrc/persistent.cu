@@ -446,7 +446,7 @@ __device__ void correct_own(const LoopArgs& p, LoopSmem& s, int64_t jtiles, unsi
 template <bool MIXED>
 __global__ void __launch_bounds__(kLT, kLMaxPerSm) loop_kernel(LoopArgs p) {
   constexpr int JT = MIXED ? kLMixJT : kLF64JT;
-  using ForceSmem = typename std::conditional<MIXED, nbk::MixedSmem<kLMixJT>, nbk::Fp64Smem<kLF64JT>>::type;
+  using ForceSmem = typename std::conditional<MIXED, nbk::MixedSmem<kLMixJT>, nbk::Fp64Smem<kLT, kLF64JT>>::type;
   __shared__ __align__(16) ForceSmem fsm;
   __shared__ LoopSmem s;
   const unsigned int G = gridDim.x;
@@ -540,8 +540,8 @@ __global__ void __launch_bounds__(kLT, kLMaxPerSm) loop_kernel(LoopArgs p) {
         nbk::mixed_item<kLT, 1, kLMixJT>(fsm, p.jA, p.jB, p.jC, jlo, jhi, n_j, p.act, n, itile * kLT, p.eps2f,
                                          out, ostride, fin, p.tbox, nullptr, 0, nbk::FusedArgs(), nbk::ISrc(), true);
       else
-        nbk::fp64_item<kLT, kLF64JT>(fsm, p.xp, p.vp, p.m, p.n_pad, jlo, jhi, p.act, n, itile * kLT, p.eps2, out,
-                                     ostride, fin);
+        nbk::fp64_item<kLT, kLF64JT>(fsm, p.xp, p.vp, p.m, p.n_pad, 1, jlo, jhi, p.n_pad, p.act, n, itile * kLT,
+                                     p.eps2, out, ostride, fin);
     }
     if (!grid_barrier(p.ctl, epoch, G, p.st, &s.ok)) return;  // C: forces complete
     correct_own<MIXED>(p, s, jtiles, G, r0, r1);
