@@ -999,4 +999,89 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
   out[6 * ostride + pos0] = finalize ? -w : w;
 }
 
+// ---- split-j reduction --------------------------------------------------------
+// Sums the partials part[split][7][stride] of n list positions into F (the
+// sign of the potential applied here) and the caller's row-major outputs
+// (each may be null).  T = float2: double-single partials of the mixed item,
+// summed in FP32 and converted once per result; T = double: FP64 partials.
+//
+// CTA (32 x QL threads) = 32 consecutive positions of one row c; lane y sums
+// splits y, y + QL, ... in order, loaded kB at a time (one round trip per
+// batch), then a fixed pairwise tree over the lanes: the result depends only
+// on the number of splits, which alone chooses QL (launch_split_reduce).
+// What bounds it is the latency of the partials, in L2, and for large n the
+// bookkeeping of the tree: with 32 lanes for every split count 20 splits of
+// n = 32768 took 46 us, with 4 lanes 12 us (the tree of 32 lanes is five
+// barriers for less than one load per lane); 760 splits of n = 256 want the 32
+// (13 us), and 235 of n = 1001, summed by one thread per position, took 359 us
+// against 12.
+__device__ __forceinline__ void part_add(float2& a, float2 b) { ds_add(a.x, a.y, b.x, b.y); }
+__device__ __forceinline__ void part_add(double& a, double b) { a += b; }
+__device__ __forceinline__ double part_value(float2 a) { return (double)a.x + (double)a.y; }
+__device__ __forceinline__ double part_value(double a) { return a; }
+
+template <typename T, int QL>
+__global__ void __launch_bounds__(32 * QL) split_reduce_kernel(const T* __restrict__ part, int64_t stride, int nsplit,
+                                                               int64_t n, double* __restrict__ F, int64_t fstride,
+                                                               double* __restrict__ acc, double* __restrict__ jerk,
+                                                               double* __restrict__ pot) {
+  constexpr int kB = 8;
+  __shared__ T sm[QL][33];
+  const int tx = threadIdx.x, ty = threadIdx.y, c = blockIdx.y;
+  for (int64_t k0 = (int64_t)blockIdx.x * 32; k0 < n; k0 += (int64_t)gridDim.x * 32) {
+    const int64_t k = k0 + tx;
+    T s = T();
+    if (k < n) {
+      const T* src = part + (int64_t)c * stride + k;
+      const int64_t step = (int64_t)QL * 7 * stride;  // QL splits further on
+      int q = ty;
+      for (; q + (kB - 1) * QL < nsplit; q += kB * QL) {
+        T v[kB];
+#pragma unroll
+        for (int b = 0; b < kB; ++b) v[b] = src[(int64_t)q * 7 * stride + b * step];
+#pragma unroll
+        for (int b = 0; b < kB; ++b) part_add(s, v[b]);
+      }
+#pragma unroll 4
+      for (; q < nsplit; q += QL) part_add(s, src[(int64_t)q * 7 * stride]);
+    }
+    sm[ty][tx] = s;
+    __syncthreads();
+#pragma unroll
+    for (int h = QL / 2; h > 0; h >>= 1) {
+      if (ty < h) {
+        T a = sm[ty][tx];
+        part_add(a, sm[ty + h][tx]);
+        sm[ty][tx] = a;
+      }
+      __syncthreads();
+    }
+    if (ty == 0 && k < n) {
+      const double w = part_value(sm[0][tx]);
+      const double val = c == 6 ? -w : w;
+      if (F) F[c * fstride + k] = val;
+      if (c < 3) {
+        if (acc) acc[3 * k + c] = val;
+      } else if (c < 6) {
+        if (jerk) jerk[3 * k + (c - 3)] = val;
+      } else if (pot) {
+        pot[k] = val;
+      }
+    }
+    __syncthreads();
+  }
+}
+
+template <typename T>
+cudaError_t launch_split_reduce(const T* part, int64_t stride, int nsplit, int64_t n, double* F, int64_t fstride,
+                                double* acc, double* jerk, double* pot, int sm_count, cudaStream_t stream) {
+  const int64_t cols = (n + 31) / 32;
+  const dim3 grid((unsigned)(cols < (int64_t)sm_count * 16 ? cols : (int64_t)sm_count * 16), 7);
+  if (nsplit >= 32)
+    split_reduce_kernel<T, 32><<<grid, dim3(32, 32), 0, stream>>>(part, stride, nsplit, n, F, fstride, acc, jerk, pot);
+  else
+    split_reduce_kernel<T, 4><<<grid, dim3(32, 4), 0, stream>>>(part, stride, nsplit, n, F, fstride, acc, jerk, pot);
+  return cudaGetLastError();
+}
+
 }  // namespace nbk

@@ -25,47 +25,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) force_fp64_kernel(
                          ostride, finalize != 0, is);
 }
 
-// split-j reduction: F[c][k] = sum over s = 0..S-1 (in this order) of
-// part[s][c][k]; the potential is negated (kernels sum +m/s).
-// Split-j reduction of part[S][7][stride] into F (the sign of the potential
-// applied here).  Block = 32 list positions x QL split lanes for one row c:
-// lane y sums splits y, y + QL, y + 2 QL, ... in order, then a fixed binary
-// tree combines the lanes, so the result depends only on S and QL (one
-// launch configuration = one summation order), and a long split list is
-// read by QL warps at once instead of one dependent chain per position.
-template <int QL>
-__global__ void split_reduce_kernel(const double* __restrict__ part, int64_t stride, int nsplit,
-                                    int64_t n, double* __restrict__ F, int64_t fstride) {
-  __shared__ double sm[QL][33];
-  const int tx = threadIdx.x, ty = threadIdx.y, c = blockIdx.y;
-  for (int64_t k0 = (int64_t)blockIdx.x * 32; k0 < n; k0 += (int64_t)gridDim.x * 32) {
-    const int64_t k = k0 + tx;
-    double s = 0.0;
-    if (k < n) {
-      // splits ty, ty + QL, ... added in order, loaded 8 at a time (one
-      // round trip per batch instead of per split)
-      int q = ty;
-      for (; q + 7 * QL < nsplit; q += 8 * QL) {
-        double v[8];
-#pragma unroll
-        for (int b = 0; b < 8; ++b) v[b] = part[((int64_t)(q + b * QL) * 7 + c) * stride + k];
-#pragma unroll
-        for (int b = 0; b < 8; ++b) s += v[b];
-      }
-      for (; q < nsplit; q += QL) s += part[((int64_t)q * 7 + c) * stride + k];
-    }
-    sm[ty][tx] = s;
-    __syncthreads();
-#pragma unroll
-    for (int h = QL / 2; h > 0; h >>= 1) {
-      if (ty < h) sm[ty][tx] += sm[ty + h][tx];
-      __syncthreads();
-    }
-    if (ty == 0 && k < n) F[c * fstride + k] = c == 6 ? -sm[0][tx] : sm[0][tx];
-    __syncthreads();
-  }
-}
-
 template <int NT, int JT>
 cudaError_t launch(nb_ctx* c, const int32_t* d_list, int64_t n, const nb_tuning& cfg, const nbk::ISrc& is) {
   static int per_sm = 0;  // resident CTAs per SM of this instantiation
@@ -88,23 +47,16 @@ cudaError_t launch(nb_ctx* c, const int32_t* d_list, int64_t n, const nb_tuning&
                                                         tiles, c->eps * c->eps, out, ostride, fin ? 1 : 0, is);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || fin) return e;
-  return nb_launch_split_reduce(c, d_list, n, nsplit, ostride);
+  return nb_launch_split_reduce(c, n, nsplit, ostride);
 }
 
 }  // namespace
 
-cudaError_t nb_launch_split_reduce(nb_ctx* c, const int32_t* d_list, int64_t n, int nsplit,
-                                   int64_t stride) {
-  (void)d_list;
-  int64_t g = (n + 31) / 32;
-  if (g > (int64_t)c->sm_count * 16) g = (int64_t)c->sm_count * 16;
-  if (g < 1) g = 1;
-  const dim3 grid((unsigned)g, 7);
-  if (nsplit >= 32)
-    split_reduce_kernel<32><<<grid, dim3(32, 32), 0, c->stream>>>(c->part, stride, nsplit, n, c->F, c->n_pad);
-  else
-    split_reduce_kernel<4><<<grid, dim3(32, 4), 0, c->stream>>>(c->part, stride, nsplit, n, c->F, c->n_pad);
-  return cudaGetLastError();
+cudaError_t nb_launch_split_reduce(nb_ctx* c, int64_t n, int nsplit, int64_t stride) {
+  const cudaError_t e = nbk::launch_split_reduce((const double*)c->part, stride, nsplit, n, c->F, c->n_pad, c->fo_acc,
+                                                 c->fo_jerk, c->fo_pot, c->sm_count, c->stream);
+  if (c->fo_acc || c->fo_jerk || c->fo_pot) c->fo_done = true;
+  return e;
 }
 
 bool nb_fp64_supported(const nb_tuning& t) {

@@ -59,67 +59,6 @@ __global__ void __launch_bounds__(NT) force_mixed_fused_kernel(
                              finalize != 0, tbox, ord, 0, fa, nbk::ISrc(), true);
 }
 
-// Split-j reduction of double-single partials: CTA (32 x kQL threads) =
-// 32 consecutive list positions (coalesced rows) x kQL lanes over the
-// splits; lane ty sums splits ty, ty + kQL, ... in order (loads in batches of
-// kB, so that a thread waits for one round trip per batch), then a fixed
-// pairwise tree over ty; one FP64 conversion per result.  Also writes the
-// caller's AoS outputs when given.
-constexpr int kQL = 32, kB = 8;
-__global__ void __launch_bounds__(32 * kQL) split_reduce_ds_kernel(const float2* __restrict__ part, int64_t stride,
-                                                                  int nsplit, int64_t n, double* __restrict__ F,
-                                                                  int64_t fstride, double* __restrict__ acc,
-                                                                  double* __restrict__ jerk,
-                                                                  double* __restrict__ pot) {
-  __shared__ float2 sm[kQL][33];
-  const int tx = threadIdx.x, ty = threadIdx.y, c = blockIdx.y;
-  for (int64_t k0 = (int64_t)blockIdx.x * 32; k0 < n; k0 += (int64_t)gridDim.x * 32) {
-    const int64_t k = k0 + tx;
-    float hi = 0.0f, lo = 0.0f;
-    if (k < n) {
-      const float2* src = part + (int64_t)c * stride + k;
-      const int64_t step = (int64_t)kQL * 7 * stride;  // kQL splits further on
-      int q = ty;
-      for (; q + (kB - 1) * kQL < nsplit; q += kB * kQL) {
-        float2 v[kB];
-#pragma unroll
-        for (int b = 0; b < kB; ++b) v[b] = src[(int64_t)q * 7 * stride + b * step];
-#pragma unroll
-        for (int b = 0; b < kB; ++b) nbk::ds_add(hi, lo, v[b].x, v[b].y);
-      }
-      for (; q < nsplit; q += kQL) {
-        const float2 v = src[(int64_t)q * 7 * stride];
-        nbk::ds_add(hi, lo, v.x, v.y);
-      }
-    }
-    sm[ty][tx] = make_float2(hi, lo);
-    __syncthreads();
-#pragma unroll
-    for (int h = kQL / 2; h > 0; h >>= 1) {
-      if (ty < h) {
-        float2 a = sm[ty][tx];
-        const float2 b = sm[ty + h][tx];
-        nbk::ds_add(a.x, a.y, b.x, b.y);
-        sm[ty][tx] = a;
-      }
-      __syncthreads();
-    }
-    if (ty == 0 && k < n) {
-      const double s = (double)sm[0][tx].x + (double)sm[0][tx].y;
-      const double val = c == 6 ? -s : s;
-      F[c * fstride + k] = val;
-      if (c < 3) {
-        if (acc) acc[3 * k + c] = val;
-      } else if (c < 6) {
-        if (jerk) jerk[3 * k + (c - 3)] = val;
-      } else if (pot) {
-        pot[k] = val;
-      }
-    }
-    __syncthreads();
-  }
-}
-
 // resident CTAs per SM of an instantiation (0 when the query fails)
 template <int NT, int IPT, int JT>
 int per_sm_of() {
@@ -195,13 +134,11 @@ cudaError_t nb_forces_mixed_fused(nb_ctx* c, const int32_t* d_list, int64_t n, c
 }
 
 cudaError_t nb_launch_split_reduce_ds(nb_ctx* c, int64_t n, int nsplit, int64_t stride) {
-  int64_t g = (n + 31) / 32;
-  if (g > (int64_t)c->sm_count * 4) g = (int64_t)c->sm_count * 4;
-  if (g < 1) g = 1;
-  split_reduce_ds_kernel<<<dim3((unsigned)g, 7), dim3(32, kQL), 0, c->stream>>>(
-      reinterpret_cast<const float2*>(c->part), stride, nsplit, n, c->F, c->n_pad, c->fo_acc, c->fo_jerk, c->fo_pot);
+  const cudaError_t e =
+      nbk::launch_split_reduce(reinterpret_cast<const float2*>(c->part), stride, nsplit, n, c->F, c->n_pad, c->fo_acc,
+                               c->fo_jerk, c->fo_pot, c->sm_count, c->stream);
   if (c->fo_acc || c->fo_jerk || c->fo_pot) c->fo_done = true;
-  return cudaGetLastError();
+  return e;
 }
 
 int nb_mixed_ctas_per_sm(const nb_tuning& cfg) {

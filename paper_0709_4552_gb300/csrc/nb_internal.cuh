@@ -219,11 +219,10 @@ cudaError_t nb_forces_mixed(nb_ctx* c, const int32_t* d_list, int64_t n, const n
 // the mixed item with the j-tiles predicted to T from the j-memory
 cudaError_t nb_forces_mixed_fused(nb_ctx* c, const int32_t* d_list, int64_t n, const nb_tuning& cfg,
                                   const int32_t* ord, double T, const float4* boxes);
-// split-j reduction (force_fp64.cu): part[S][7][n] -> F in fixed order, potential sign
-cudaError_t nb_launch_split_reduce(nb_ctx* c, const int32_t* d_list, int64_t n, int nsplit,
-                                   int64_t stride);
-// the same for double-single partials (float2 in each 8-byte slot, force_mixed.cu),
-// summed in FP32; also writes the caller's device outputs c->fo_* when set
+// split-j reduction (force_common.cuh): part[S][7][n] -> F in fixed order,
+// potential sign; also writes the caller's device outputs c->fo_* when set
+cudaError_t nb_launch_split_reduce(nb_ctx* c, int64_t n, int nsplit, int64_t stride);
+// the same for double-single partials (float2 in each 8-byte slot), summed in FP32
 cudaError_t nb_launch_split_reduce_ds(nb_ctx* c, int64_t n, int nsplit, int64_t stride);
 bool nb_tuning_supported(int precision, const nb_tuning& cfg);
 nb_tuning nb_default_tuning(int precision);

@@ -81,26 +81,6 @@ __global__ void __launch_bounds__(kNT, 512 / kNT) noalloc_force_kernel(int64_t N
                            eps2, part + (int64_t)blockIdx.y * 7 * pstride, pstride, false);
 }
 
-// sum the splits in a fixed order and write the caller's [n][3] outputs
-__global__ void noalloc_reduce_kernel(const double* __restrict__ part, int64_t pstride, int nsplit, int64_t n,
-                                      double* __restrict__ acc, double* __restrict__ jerk,
-                                      double* __restrict__ pot) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-    double s[7];
-#pragma unroll
-    for (int c = 0; c < 7; ++c) {
-      double t = 0.0;
-      for (int q = 0; q < nsplit; ++q) t += part[((int64_t)q * 7 + c) * pstride + k];
-      s[c] = t;
-    }
-    if (acc)
-      for (int c = 0; c < 3; ++c) acc[3 * k + c] = s[c];
-    if (jerk)
-      for (int c = 0; c < 3; ++c) jerk[3 * k + c] = s[3 + c];
-    if (pot) pot[k] = -s[6];
-  }
-}
-
 // device address of the scratch array for the current device (set up once)
 int scratch_for_current_device(double** out) {
   int dev = -1;
@@ -152,9 +132,8 @@ extern "C" int nb_forces_fp64_noalloc(int64_t N, const double* m, const double* 
   noalloc_force_kernel<<<dim3((unsigned)itiles, (unsigned)nsplit), kNT, 0, s>>>(N, m, x, v, eps * eps, i_idx, n,
                                                                                 tps * kJT, scratch, pstride);
   if (cudaGetLastError() != cudaSuccess) return NB_ECUDA;
-  int g = (int)((n + 255) / 256);
-  if (g > 8 * sms) g = 8 * sms;
-  noalloc_reduce_kernel<<<g, 256, 0, s>>>(scratch, pstride, (int)nsplit, n, acc, jerk, pot);
-  if (cudaGetLastError() != cudaSuccess) return NB_ECUDA;
+  if (nbk::launch_split_reduce((const double*)scratch, pstride, (int)nsplit, n, (double*)nullptr, 0, acc, jerk, pot,
+                               sms, s) != cudaSuccess)
+    return NB_ECUDA;
   return NB_OK;
 }
