@@ -113,6 +113,18 @@ nb_tuning pick_tuning(const nb_ctx* c, int64_t n) {
   return nb_default_tuning(c->precision);
 }
 
+// Whether a caller's list is visited in spatial order.  The order of a list of
+// every particle is there already.  Any other costs two kernels and two
+// memsets over N (14 us at N = 20000, 28 us at 2^20) and takes about 3% off
+// the force launch from n = 1024 on, 5% from 4096, nothing below (ordered /
+// unordered: N = 2^20 n = 512 535 / 518 us, n = 1024 994 / 995, n = 4096
+// 3747 / 3915; N = 131072 n = 2048 286 / 287, n = 4096 522 / 545; N = 20000
+// n = 4096 123 / 112), so the line lies where the force launch takes about
+// half a millisecond.
+bool order_pays(const nb_ctx* c, int64_t n) {
+  return n == c->n || (n >= 1024 && n * c->n >= (int64_t)1 << 29);
+}
+
 // device view of a caller's list (copied to ulist for host lists)
 int stage_list(nb_ctx* c, const int32_t* list, int64_t n, int ptr_kind, const int32_t** d_list) {
   if (ptr_kind == NB_PTR_HOST) {
@@ -399,7 +411,7 @@ cudaError_t nb_forces(nb_ctx* c, const int32_t* d_list, int64_t n) {
   // caller's list (mapped to slots) is visited sorted by slot.
   const int32_t* ord = nullptr;
   if (c->perm_valid && c->n_clusters == 0 && d_list != c->act && d_list != c->ident &&
-      n >= 2048) {  // below that the sort costs more than the far tiles it finds
+      order_pays(c, n)) {
     cudaError_t e = nb_list_order(c, d_list, n, &ord);
     if (e != cudaSuccess) return e;
   }
@@ -689,7 +701,7 @@ int nb_compute_forces_at(nb_ctx* c, double t, const int32_t* i_idx, int64_t n, d
     const float4* boxes = nullptr;
     if ((r = jm_host_side(c, d_list, n, t, &boxes))) return r;
     const int32_t* ord = nullptr;
-    if (c->perm_valid && n >= 2048) NB_CUDA(c, nb_list_order(c, d_list, n, &ord));
+    if (c->perm_valid && order_pays(c, n)) NB_CUDA(c, nb_list_order(c, d_list, n, &ord));
     NB_CUDA(c, nb_forces_mixed_fused(c, d_list, n, pick_tuning(c, n), ord, t, boxes));
   } else {
     // the FP64 path predicts every particle (it has no on-the-fly prediction)
