@@ -745,12 +745,15 @@ __device__ __forceinline__ void sum_add(double& hi, double& lo, double p) {
 
 // the pairs of one i with the j-particles of the bits in mask (jt + bit), in
 // FP64: the few that the fixed-point pair leaves (closer than its grid
-// resolves, odd masses, values outside its exponent range)
+// resolves, odd masses, values outside its exponent range).  state: the calls
+// so far, kHighUsed once the high sums have been written; returns the new one.
+constexpr int kHighUsed = 1 << 30;
 template <int NT, int JT>
-__device__ __noinline__ void fp64_pairs(Fp64Smem<NT, JT>& sm, const double* __restrict__ xp,
+__device__ __noinline__ int fp64_pairs(Fp64Smem<NT, JT>& sm, const double* __restrict__ xp,
                                         const double* __restrict__ vp, const double* __restrict__ m, int64_t cs,
                                         int64_t js, int64_t jt, uint32_t mask, double x0, double x1, double x2,
-                                        double v0, double v1, double v2, double eps2) {
+                                        double v0, double v1, double v2, double eps2, int state) {
+  const uint32_t mask0 = mask;
   double p[7];
 #pragma unroll
   for (int c = 0; c < 7; ++c) p[c] = 0.0;
@@ -776,22 +779,42 @@ __device__ __noinline__ void fp64_pairs(Fp64Smem<NT, JT>& sm, const double* __re
     p[4] = fma(mr3, fma(a3, dy, wy), p[4]);
     p[5] = fma(mr3, fma(a3, dz, wz), p[5]);
   }
+  // a few pairs: into the low sum alone (each FP64 instruction holds the warp
+  // for 64 cycles, and a TwoSum is six); many, and every eighth time, both
+  // into the high sum without error
+  state += 1;
+  if (__popc(mask0) <= 4 && (state & 7) != 0) {
 #pragma unroll
-  for (int c = 0; c < 7; ++c) sum_add(sm.hi[c][threadIdx.x], sm.lo[c][threadIdx.x], p[c]);
+    for (int c = 0; c < 7; ++c) sm.lo[c][threadIdx.x] += p[c];
+    return state;
+  }
+#pragma unroll
+  for (int c = 0; c < 7; ++c) {
+    double hi = sm.hi[c][threadIdx.x], lo = 0.0;
+    sum_add(hi, lo, sm.lo[c][threadIdx.x]);
+    sum_add(hi, lo, p[c]);
+    sm.hi[c][threadIdx.x] = hi;
+    sm.lo[c][threadIdx.x] = lo;
+  }
+  return state | kHighUsed;
 }
 
 // the 96-bit sums into the thread's FP64 sums (in_range: they hold its
-// pairs, else nothing of worth); cleared
+// pairs, else nothing of worth; first: those sums are still zero); cleared
 template <int NT, int JT>
-__device__ __forceinline__ void fp64_fold(Fp64Smem<NT, JT>& sm, nbx::Sum96 (&a)[7], bool in_range, int g, int gv,
-                                          int em) {
+__device__ __forceinline__ void fp64_fold(Fp64Smem<NT, JT>& sm, nbx::Sum96 (&a)[7], bool in_range, bool first, int g,
+                                          int gv, int em) {
 #pragma unroll
   for (int c = 0; c < 7; ++c) {
     const int e = c < 3 ? em - 2 * g + nbx::kAccScale
                         : (c < 6 ? em - 3 * g + gv + nbx::kJerkScale : em - g + nbx::kPotScale);
-    const double p = fma((double)(int64_t)(((uint64_t)a[c].w2 << 32) | a[c].w1), 4294967296.0, (double)a[c].w0);
-    // two factors: e may lie outside the exponents of one FP64 number
-    if (in_range) sum_add(sm.hi[c][threadIdx.x], sm.lo[c][threadIdx.x], p * pow2d(e / 2) * pow2d(e - e / 2));
+    if (in_range) {
+      const double p = nbx::to_double(a[c], e);
+      if (first)
+        sm.hi[c][threadIdx.x] = p;
+      else
+        sum_add(sm.hi[c][threadIdx.x], sm.lo[c][threadIdx.x], p);
+    }
     a[c].w0 = a[c].w1 = a[c].w2 = 0u;
   }
 }
@@ -865,7 +888,7 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
   int G = 0, GV = 0, EM = 0, g = 0, gv = 0, filled = 0;  // grid of the tiles so far, this i's grid, pairs in a
   bool have = false, in_range = false;
   int32_t wmin = nbx::kNoPairs;
-  int chunk = 0;
+  int chunk = 0, state = 0;
   fi.wmin = wmin;
   // a warp whose list positions all lie past n computes nothing (its
   // results are not written); it still loads its share of every j-tile
@@ -909,7 +932,10 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
     const bool tile_ok = gx <= nbx::kExpHi && gw <= nbx::kExpHi && gm <= nbx::kExpHi;
     const bool moved = !have || gx > G || gx < G - 1 || gw > GV || gw < GV - 1 || gm > EM || gm < EM - 3;
     if (tile_ok && (moved || filled + JT > nbx::kFold)) {
-      if (filled > 0) fp64_fold(sm, a, in_range, g, gv, EM);
+      if (filled > 0) {
+        fp64_fold(sm, a, in_range, (state & kHighUsed) == 0, g, gv, EM);
+        state |= kHighUsed;
+      }
       filled = 0;
       if (moved) {
         G = gx;
@@ -986,11 +1012,11 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
       }
       if (rel >= q0 && rel < q0 + 32) left &= ~(1u << (rel - q0));
       if (left)
-        fp64_pairs(sm, xp, vp, m, cs, js, jt + q0, left, xi[0], xi[ics], xi[2 * ics], vi[0], vi[ics], vi[2 * ics],
-                   eps2);
+        state = fp64_pairs(sm, xp, vp, m, cs, js, jt + q0, left, xi[0], xi[ics], xi[2 * ics], vi[0], vi[ics], vi[2 * ics],
+                   eps2, state);
     }
   }
-  if (filled > 0) fp64_fold(sm, a, in_range, g, gv, EM);
+  if (filled > 0) fp64_fold(sm, a, in_range, (state & kHighUsed) == 0, g, gv, EM);
   __syncthreads();  // the caller may reuse shared memory for its next item
   if (pos0 >= n) return;
 #pragma unroll

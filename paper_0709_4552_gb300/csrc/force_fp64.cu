@@ -9,7 +9,7 @@
 namespace {
 
 template <int NT, int JT>
-// 16 warps per SM (128 registers): measured best of 8 to 20
+// 16 warps per SM (128 registers): measured best of 12, 16 and 20
 __global__ void __launch_bounds__(NT, 512 / NT) force_fp64_kernel(
     const double* __restrict__ xp, const double* __restrict__ vp, const double* __restrict__ m,
     int64_t n_pad, int64_t N, const int32_t* __restrict__ list, int64_t n, int64_t tiles,

@@ -20,8 +20,9 @@
 // of its own result or finer, and the sums over j are exact.  Measured against
 // long double sums (Plummer spheres of 513 to 60000, equal and Salpeter masses,
 // and sets with outliers, close pairs, wide mass ratios), the rms errors are
-// 0.5 to 1.0 (acceleration), 0.35 to 1.0 (jerk) and 0.7 to 1.02 (potential)
-// times those of the FP64 evaluation.
+// 0.5 to 1.0 (acceleration), 0.35 to 1.0 (jerk) and 0.4 to 1.0 (potential)
+// times those of the FP64 evaluation (1.0, 1.13 and 1.15 for 33 particles, one
+// 2^30 away, whose pairs are nearly all left to FP64).
 //
 // Formats.  2^g bounds the coordinates of the pair and eps, 2^gv the
 // velocities, em is the exponent of the largest mass near by:
@@ -123,6 +124,43 @@ __device__ __forceinline__ void add_shifted(Sum96& s, int64_t t, int L) {
   asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
       : "+&r"(s.w0), "+&r"(s.w1), "+&r"(s.w2)
       : "r"(__funnelshift_l(0u, t0, L)), "r"(__funnelshift_l(t0, t1, L)), "r"(a2));
+}
+
+// s 2^e, rounded once to nearest: a normal FP64 number built from the sum's
+// bits.  About 40 integer instructions; by FP64 conversions, products and a
+// TwoSum it was eleven FP64 ones, which a warp issues 64 cycles apart, 7 sums
+// 2.4 us at the end of every item of a small system.
+__device__ __forceinline__ double to_double(Sum96 s, int e) {
+  const uint32_t neg = (uint32_t)((int32_t)s.w2 >> 31);
+  uint32_t a0 = s.w0 ^ neg, a1 = s.w1 ^ neg, a2 = s.w2 ^ neg;
+  asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, 0;\n\taddc.u32 %2, %2, 0;"
+      : "+&r"(a0), "+&r"(a1), "+&r"(a2)
+      : "r"(neg & 1u));
+  // the leading bit to bit 95: whole words, then the rest
+  int n = 0;
+  if (a2 == 0u) {
+    n = 32;
+    a2 = a1;
+    a1 = a0;
+    a0 = 0u;
+    if (a2 == 0u) {
+      n = 64;
+      a2 = a1;
+      a1 = 0u;
+    }
+  }
+  if (a2 == 0u) return 0.0;
+  const int z = __clz((int)a2);
+  const uint32_t m1 = __funnelshift_l(a1, a2, z), m0 = __funnelshift_l(a0, a1, z), rest = __funnelshift_l(0u, a0, z);
+  const int E = 95 - n - z + e + 1023;
+  const uint64_t m = ((uint64_t)m1 << 32) | m0;
+  const uint32_t r = m0 & 0x7FFu;
+  const uint32_t up = (r > 0x400u || (r == 0x400u && (rest != 0u || (m0 & 0x800u) != 0u))) ? 1u : 0u;
+  const uint64_t f = (m >> 11) + up;  // [2^52, 2^53]
+  const uint64_t sign = (uint64_t)(neg & 0x80000000u) << 32;
+  if (E >= 1 && E <= 2045) return __longlong_as_double((long long)((((uint64_t)(uint32_t)(E - 1) << 52) + f) | sign));
+  const double d = scalbn((double)f, E - 1075);
+  return neg ? -d : d;
 }
 
 // The pair (i, j): its seven terms added to a (acc, jerk, pot).  Returns

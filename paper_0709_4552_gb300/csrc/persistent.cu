@@ -42,8 +42,19 @@ namespace {
 
 constexpr int kLT = 128;                     // threads per CTA = i-tile = row tile
 constexpr int kLWarps = kLT / 32;
-constexpr int kLMaxPerSm = 4;                // resident CTAs per SM asked for (128 registers)
-constexpr int kLMixJT = 128, kLF64JT = 64;   // j-tiles (the mixed one = the box tile)
+// resident CTAs per SM asked for: 4 mixed (128 registers), 3 FP64 (168; with 4
+// the fixed-point pair spills: N = 1024 32.4 against 31.8 us a block step, N =
+// 32768 582 against 569)
+constexpr int kLMaxPerSm = 4, kLMaxPerSm64 = 3;
+// j-tiles (the mixed one = the box tile).  FP64: an item's tile is its share of
+// a small system's force phase, so those take 32 and at least two CTAs per SM:
+// N = 1024 31.8 us a block step against 40.7 with 64 and one CTA (44.9 with 64
+// and the mixed path's grid), N = 4096 47 against 58 (79); from N = 16384 the
+// splits are long and 64 stages better (177 against 194).
+constexpr int kLMixJT = 128, kLF64JT = 64, kLF64JTSmall = 32;
+// (Up to two tiles of 64, N = 128, every loop driver splits the sums alike and
+// gives the same bits.)
+constexpr int64_t kLF64SmallLo = 2 * kLF64JT, kLF64SmallHi = 8192;
 constexpr long long kWaitNs = 4000000000LL;  // a barrier wait of the loop gives up after 4 s
 constexpr unsigned int kPollCap = 1u << 26;  // ... or after this many polls
 constexpr unsigned long long kInfBits = 0x7FF0000000000000ULL;  // +inf
@@ -443,10 +454,9 @@ __device__ void correct_own(const LoopArgs& p, LoopSmem& s, int64_t jtiles, unsi
   }
 }
 
-template <bool MIXED>
-__global__ void __launch_bounds__(kLT, kLMaxPerSm) loop_kernel(LoopArgs p) {
-  constexpr int JT = MIXED ? kLMixJT : kLF64JT;
-  using ForceSmem = typename std::conditional<MIXED, nbk::MixedSmem<kLMixJT>, nbk::Fp64Smem<kLT, kLF64JT>>::type;
+template <bool MIXED, int JT>
+__global__ void __launch_bounds__(kLT, MIXED ? kLMaxPerSm : kLMaxPerSm64) loop_kernel(LoopArgs p) {
+  using ForceSmem = typename std::conditional<MIXED, nbk::MixedSmem<JT>, nbk::Fp64Smem<kLT, JT>>::type;
   __shared__ __align__(16) ForceSmem fsm;
   __shared__ LoopSmem s;
   const unsigned int G = gridDim.x;
@@ -537,10 +547,10 @@ __global__ void __launch_bounds__(kLT, kLMaxPerSm) loop_kernel(LoopArgs p) {
       double* out = fin ? p.F : p.part + split * 7 * pstride;
       const int64_t ostride = fin ? p.n_pad : pstride;
       if constexpr (MIXED)
-        nbk::mixed_item<kLT, 1, kLMixJT>(fsm, p.jA, p.jB, p.jC, jlo, jhi, n_j, p.act, n, itile * kLT, p.eps2f,
+        nbk::mixed_item<kLT, 1, JT>(fsm, p.jA, p.jB, p.jC, jlo, jhi, n_j, p.act, n, itile * kLT, p.eps2f,
                                          out, ostride, fin, p.tbox, nullptr, 0, nbk::FusedArgs(), nbk::ISrc(), true);
       else
-        nbk::fp64_item<kLT, kLF64JT>(fsm, p.xp, p.vp, p.m, p.n_pad, 1, jlo, jhi, p.n_pad, p.act, n, itile * kLT,
+        nbk::fp64_item<kLT, JT>(fsm, p.xp, p.vp, p.m, p.n_pad, 1, jlo, jhi, p.n_pad, p.act, n, itile * kLT,
                                      p.eps2, out, ostride, fin);
     }
     if (!grid_barrier(p.ctl, epoch, G, p.st, &s.ok)) return;  // C: forces complete
@@ -574,19 +584,24 @@ struct PLoop {
   unsigned long long* smin = nullptr;
   int32_t* scnt = nullptr;
   int gmax = 0;
-  int per_sm[2] = {0, 0};  // resident CTAs per SM of each instantiation (0 = not yet asked)
+  int per_sm[3] = {0, 0, 0};  // resident CTAs per SM of each instantiation (0 = not yet asked)
 };
 
 PLoop* ploop_of(nb_ctx* c) { return static_cast<PLoop*>(c->loop); }
 
-int ctas_per_sm(nb_ctx* c, PLoop* L, bool mixed) {
-  int& ps = L->per_sm[mixed ? 1 : 0];
+// the instantiations: mixed, FP64, FP64 for small systems
+const void* loop_variant(int v) {
+  return v == 0   ? (const void*)loop_kernel<true, kLMixJT>
+         : v == 1 ? (const void*)loop_kernel<false, kLF64JT>
+                  : (const void*)loop_kernel<false, kLF64JTSmall>;
+}
+
+int ctas_per_sm(PLoop* L, int v) {
+  int& ps = L->per_sm[v];
   if (ps == 0) {
     int occ = 0;
-    cudaError_t e = mixed ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, loop_kernel<true>, kLT, 0)
-                          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, loop_kernel<false>, kLT, 0);
-    if (e != cudaSuccess) return -1;
-    ps = std::min(occ, kLMaxPerSm);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, loop_variant(v), kLT, 0) != cudaSuccess) return -1;
+    ps = std::min(occ, v == 0 ? kLMaxPerSm : kLMaxPerSm64);
   }
   return ps;
 }
@@ -611,16 +626,19 @@ int nb_integrate_persistent(nb_ctx* c, double t_end) {
     L = new PLoop();
     c->loop = L;
   }
-  const int per_sm = ctas_per_sm(c, L, mixed);
+  const int variant = mixed ? 0 : (c->n > kLF64SmallLo && c->n <= kLF64SmallHi ? 2 : 1);
+  const int per_sm = ctas_per_sm(L, variant);
   if (per_sm < 1) {
     cudaGetLastError();
     return NB_ECUDA;
   }
   // as many CTAs as fit, but for a small system no more than twice its row
-  // tiles (at least 32): the other CTAs would own no rows and take no force
-  // items of its small blocks, and each barrier waits for every CTA's arrival
+  // tiles (at least 32; FP64: two CTAs per SM, whose force items are the step's
+  // longest part): the other CTAs would own no rows and take no force items of
+  // its small blocks, and each barrier waits for every CTA's arrival
   const int64_t row_tiles = (c->n + kLT - 1) / kLT;
-  const int G = (int)std::min<int64_t>(std::min(c->sm_count * per_sm, kLMaxG), std::max<int64_t>(32, 2 * row_tiles));
+  const int G = (int)std::min<int64_t>(std::min(c->sm_count * per_sm, kLMaxG),
+                                       std::max<int64_t>(variant == 2 ? 2 * c->sm_count : 32, 2 * row_tiles));
   if (G > L->gmax) {
     if (L->smin) cudaFree(L->smin);
     if (L->scnt) cudaFree(L->scnt);
@@ -680,8 +698,8 @@ int nb_integrate_persistent(nb_ctx* c, double t_end) {
     p.st = c->status;
     if (cudaMemsetAsync(L->ctl, 0, sizeof(LoopCtl), c->stream) != cudaSuccess) return NB_ECUDA;
     void* args[] = {&p};
-    cudaError_t e = cudaLaunchCooperativeKernel(mixed ? (const void*)loop_kernel<true> : (const void*)loop_kernel<false>,
-                                                dim3((unsigned)G), dim3(kLT), args, 0, c->stream);
+    cudaError_t e =
+        cudaLaunchCooperativeKernel(loop_variant(variant), dim3((unsigned)G), dim3(kLT), args, 0, c->stream);
     if (e != cudaSuccess) {
       cudaGetLastError();
       return NB_ECUDA;
