@@ -169,11 +169,6 @@ __device__ void list_rows(CSmem& s, int me, int C, int nr, unsigned long long tn
   __syncthreads();
 }
 
-__device__ __forceinline__ void split_ds(double x, float& hi, float& lo) {
-  hi = __double2float_rn(x);
-  lo = __double2float_rn(x - (double)hi);
-}
-
 __global__ void __launch_bounds__(kCT, 1) cluster_loop_kernel(ClusterArgs p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CSmem& s = *reinterpret_cast<CSmem*>(smem_raw);
@@ -274,17 +269,17 @@ __global__ void __launch_bounds__(kCT, 1) cluster_loop_kernel(ClusterArgs p) {
       }
       float xh[3], xl[3];
 #pragma unroll
-      for (int d = 0; d < 3; ++d) split_ds(px[d], xh[d], xl[d]);
-      s.iA[k] = make_float4(xh[0], xh[1], xh[2], __double2float_rn(pv[0]));
-      s.iB[k] = make_float4(xl[0], xl[1], xl[2], __double2float_rn(pv[1]));
-      s.iC[k] = make_float2(__double2float_rn(pv[2]), __int_as_float((int)row));
+      for (int d = 0; d < 3; ++d) nb_split(px[d], xh[d], xl[d]);
+      s.iA[k] = make_float4(xh[0], xh[1], xh[2], nb_f32(pv[0]));
+      s.iB[k] = make_float4(xl[0], xl[1], xl[2], nb_f32(pv[1]));
+      s.iC[k] = make_float2(nb_f32(pv[2]), __int_as_float((int)row));
     }
     // own j rows predicted on the fly from the j-memory (Sec. 4.4 step 4)
     for (int q = (tid - iw + kCT) % kCT; q < nr; q += kCT) {
       const int64_t row = own_row(q, me, C);
       const float4 R0 = p.jm[row], R1 = p.jm[p.n_pad + row], R2 = p.jm[2 * p.n_pad + row],
                    R3 = p.jm[3 * p.n_pad + row], R4 = p.jm[4 * p.n_pad + row];
-      const float h = __double2float_rn(tn - p.t[row]);
+      const float h = nb_f32(tn - p.t[row]);
       const float h2 = 2.0f * h, h15 = 1.5f * h;
       float hi, lo, vv;
       nbk::ds_predict(R0.x, R1.x, R2.x, R3.x, R4.x, R2.w, h, h2, h15, hi, lo, vv);
@@ -430,7 +425,7 @@ __global__ void __launch_bounds__(kCT, 1) cluster_loop_kernel(ClusterArgs p) {
 #pragma unroll
         for (int cc = 0; cc < kMaxC; ++cc)
           if (cc < C) nbk::ds_add(h, l, pv[cc].x, pv[cc].y);
-        const double acc = (double)h + (double)l;
+        const double acc = nb_f64(h) + nb_f64(l);
         s.fsum[c][k] = c == 6 ? -acc : acc;
       }
       __syncthreads();
@@ -438,9 +433,9 @@ __global__ void __launch_bounds__(kCT, 1) cluster_loop_kernel(ClusterArgs p) {
         const int sub = tid & 3, cs = sub < 3 ? sub : 0;
         const int pos = lo_pos + k0 + (tid >> 2);
         const bool have = pos < hi_pos;
-        double fo[7];
-#pragma unroll
-        for (int c = 0; c < 7; ++c) fo[c] = have ? s.fsum[c][pos - (int)g0] : 0.0;
+        const int fk = have ? pos - (int)g0 : 0;
+        const double a1 = have ? s.fsum[cs][fk] : 0.0, j1 = have ? s.fsum[3 + cs][fk] : 0.0;
+        const double p1 = have ? s.fsum[6][fk] : 0.0;
         const int kk = have ? pos - before : lo_pos - before;  // own active index
         const int64_t row = s.irow[kk];
         nbh::CorrIn in;
@@ -450,7 +445,7 @@ __global__ void __launch_bounds__(kCT, 1) cluster_loop_kernel(ClusterArgs p) {
           const int64_t q = cs * p.n_pad + row;
           in = nbh::CorrIn{p.t[row], p.dt[row], p.a[q], p.jk[q], p.xp[q], p.vp[q]};
         }
-        const double nd = nbh::correct_lanes4(row, p.n_pad, tn, fo, in, p.eta, p.dt_min, p.dt_max, p.x, p.v, p.a,
+        const double nd = nbh::correct_lanes4(row, p.n_pad, tn, a1, j1, p1, in, p.eta, p.dt_min, p.dt_max, p.x, p.v, p.a,
                                               p.jk, p.pot, p.t, p.dt, p.st, sub, (tid & 31) - sub, have, p.jm);
         if (have && sub == 0) s.due[own_index(row, me, C)] = (unsigned long long)__double_as_longlong(nd);
       }

@@ -391,8 +391,36 @@ __global__ void b_predict(int64_t N, int64_t n_pad, const int32_t* __restrict__ 
     if (nact[c] == 0) continue;
     double px[3], pv[3];
     nbh::taylor(i, n_pad, own_time ? 0.0 : tnext[c] - ti[i], x, v, a, jk, px, pv);
-    nbh::store_predicted(i, n_pad, px, pv, m[i], xp, vp, jA, jB, jC, write_fp64 != 0, write_mixed != 0);
+    float hi[3];
+    nbh::store_predicted(i, n_pad, px, pv, m[i], xp, vp, jA, jB, jC, write_fp64 != 0, write_mixed != 0, hi);
   }
+}
+
+// the same by tiles of 128 rows counted from each cluster's first row (one CTA
+// per tile), with the tiles' boxes for the far test; tile_cl null: one cluster
+__global__ void __launch_bounds__(NB_BOX_TILE) b_predict_tiles(
+    int64_t n_pad, const int32_t* __restrict__ tile_cl, const int64_t* __restrict__ tile_off,
+    const int64_t* __restrict__ off, const int32_t* __restrict__ nact, const double* __restrict__ tnext, int own_time,
+    const double* __restrict__ m, const double* __restrict__ x, const double* __restrict__ v,
+    const double* __restrict__ a, const double* __restrict__ jk, const double* __restrict__ ti,
+    double* __restrict__ xp, double* __restrict__ vp, float4* __restrict__ jA, float4* __restrict__ jB,
+    float2* __restrict__ jC, float4* __restrict__ box) {
+  __shared__ nb_box wbox[NB_BOX_TILE / 32];
+  const int64_t g = blockIdx.x;
+  const int c = tile_cl ? tile_cl[g] : 0;
+  if (nact[c] == 0) return;  // (its rows keep the last prediction, and nobody reads it)
+  const int64_t i = off[c] + (g - (tile_cl ? tile_off[c] : 0)) * NB_BOX_TILE + threadIdx.x;
+  const bool in = i < off[c + 1];
+  float hi[3] = {0.0f, 0.0f, 0.0f};
+  if (in) {
+    double px[3], pv[3];
+    nbh::taylor(i, n_pad, own_time ? 0.0 : tnext[c] - ti[i], x, v, a, jk, px, pv);
+    nbh::store_predicted(i, n_pad, px, pv, m[i], xp, vp, jA, jB, jC, true, true, hi);
+  }
+  const nb_box b = nb_warp_box(in, hi);
+  if ((threadIdx.x & 31) == 0) wbox[threadIdx.x >> 5] = b;
+  __syncthreads();
+  if (threadIdx.x == 0) nb_write_box(wbox, NB_BOX_TILE / 32, box + 2 * g);
 }
 
 // ---------------------------------------------------------------------------
@@ -575,38 +603,6 @@ __global__ void b_cluster_keys(int64_t N, int64_t n_pad, const int32_t* __restri
   }
 }
 
-// one warp per box tile: box of the predicted FP32 hi positions, (lo, rmax), (hi, 0)
-__global__ void b_tile_boxes(int64_t ntiles, const int32_t* __restrict__ tile_cl,
-                             const int64_t* __restrict__ tile_off, const int64_t* __restrict__ off,
-                             const float4* __restrict__ jA, float4* __restrict__ box) {
-  const int64_t g = blockIdx.x * (int64_t)(blockDim.x / 32) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (g >= ntiles) return;
-  const int c = tile_cl[g];
-  const int64_t s0 = off[c] + (g - tile_off[c]) * NB_BOX_TILE;
-  const int64_t s1 = min(s0 + NB_BOX_TILE, off[c + 1]);
-  float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX}, r = 0.0f;
-  for (int64_t s = s0 + lane; s < s1; s += 32) {
-    const float4 a = jA[s];
-    const float p[3] = {a.x, a.y, a.z};
-    for (int d = 0; d < 3; ++d) {
-      lo[d] = fminf(lo[d], p[d]);
-      hi[d] = fmaxf(hi[d], p[d]);
-      r = fmaxf(r, fabsf(p[d]));
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    for (int d = 0; d < 3; ++d) {
-      lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
-      hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
-    }
-    r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, o));
-  }
-  if (lane == 0) {
-    box[2 * g] = make_float4(lo[0], lo[1], lo[2], r);
-    box[2 * g + 1] = make_float4(hi[0], hi[1], hi[2], 0.0f);
-  }
-}
 
 // corrector + block-step rule (Sec. 4.1 step 5), per slot of active clusters
 __global__ void b_correct(int32_t C, int64_t n_pad, const int64_t* __restrict__ citem_off,
@@ -899,16 +895,16 @@ void launch_force(nb_ctx* c, Batch* b, bool mixed) {
 
 cudaError_t body_after_plan(nb_ctx* c, Batch* b, bool own_time) {
   const bool mixed = c->precision == NB_MIXED;
-  const int g = grid_for(b->N, 256, c->sm_count * 16);
-  b_predict<<<g, 256, 0, c->stream>>>(b->N, c->n_pad, b->cid, b->nact, b->tnext, own_time ? 1 : 0, c->m, c->x,
-                                      c->v, c->a, c->jk, c->t, c->xp, c->vp, c->jA, c->jB, c->jC, 1, mixed ? 1 : 0);
-  if (single_boxes(c, b)) {
-    cudaError_t e = nb_launch_tile_boxes(c);  // boxes of the predicted tiles for the far test
-    if (e != cudaSuccess) return e;
-  } else if (cluster_boxes(c, b)) {
-    b_tile_boxes<<<(unsigned)((b->ntiles + 7) / 8), 256, 0, c->stream>>>(b->ntiles, b->tile_cl, b->tile_off, b->off,
-                                                                        c->jA, b->tbox);
-    c->launches += 1;
+  if (single_boxes(c, b) || cluster_boxes(c, b)) {
+    const bool cl = cluster_boxes(c, b);
+    const int64_t tiles = cl ? b->ntiles : (b->N + NB_BOX_TILE - 1) / NB_BOX_TILE;
+    b_predict_tiles<<<(unsigned)tiles, NB_BOX_TILE, 0, c->stream>>>(
+        c->n_pad, cl ? b->tile_cl : nullptr, cl ? b->tile_off : nullptr, b->off, b->nact, b->tnext, own_time ? 1 : 0,
+        c->m, c->x, c->v, c->a, c->jk, c->t, c->xp, c->vp, c->jA, c->jB, c->jC, cl ? b->tbox : c->tbox);
+  } else {
+    b_predict<<<grid_for(b->N, 256, c->sm_count * 16), 256, 0, c->stream>>>(
+        b->N, c->n_pad, b->cid, b->nact, b->tnext, own_time ? 1 : 0, c->m, c->x, c->v, c->a, c->jk, c->t, c->xp, c->vp,
+        c->jA, c->jB, c->jC, 1, mixed ? 1 : 0);
   }
   if (b->nt == 32)
     launch_force<32>(c, b, mixed);
@@ -1047,7 +1043,7 @@ int run_graph(nb_ctx* c, Batch* b, double t_end) {
     c->steps += steps;
     c->perm_age += (int)steps;
     c->interactions += (double)inter;
-    c->launches += iters * (seg ? 9 : 8);
+    c->launches += iters * 8;
     total += iters;
     if (!more) break;
     if (total > cap) return NB_ETIMEOUT;  // cannot happen for valid block steps

@@ -53,9 +53,8 @@ __global__ void ext_prepare_kernel(int64_t n, int64_t cap, const double* __restr
       const double x = xi[3 * k + c], v = vi[3 * k + c];
       ex[c * cap + k] = x;
       ev[c * cap + k] = v;
-      hi[c] = __double2float_rn(x);
-      lo[c] = __double2float_rn(x - (double)hi[c]);
-      vf[c] = __double2float_rn(v);
+      nb_split(x, hi[c], lo[c]);
+      vf[c] = nb_f32(v);
     }
     eA[k] = make_float4(hi[0], hi[1], hi[2], 0.0f);
     eB[k] = make_float4(lo[0], lo[1], lo[2], vf[0]);

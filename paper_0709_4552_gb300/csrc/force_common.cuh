@@ -268,7 +268,7 @@ __device__ __forceinline__ void jm_predict_tile(FusedSmem<JT>& sm, int buf, doub
     if (jt + q < jhi) {
       const float4 r0 = sm.R[buf][0][q], r1 = sm.R[buf][1][q], r2 = sm.R[buf][2][q], r3 = sm.R[buf][3][q],
                    r4 = sm.R[buf][4][q];
-      const float h = __double2float_rn(T - sm.T[buf][q]);
+      const float h = nb_f32(T - sm.T[buf][q]);
       const float h2 = 2.0f * h, h15 = 1.5f * h;  // exact scalings of an exact h
       float2 hi2, lo2, vp2;
       ds_predict(make_float2(r0.x, r0.y), make_float2(r1.x, r1.y), make_float2(r2.x, r2.y),
@@ -1043,7 +1043,7 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
 // against 12.
 __device__ __forceinline__ void part_add(float2& a, float2 b) { ds_add(a.x, a.y, b.x, b.y); }
 __device__ __forceinline__ void part_add(double& a, double b) { a += b; }
-__device__ __forceinline__ double part_value(float2 a) { return (double)a.x + (double)a.y; }
+__device__ __forceinline__ double part_value(float2 a) { return nb_f64(a.x) + nb_f64(a.y); }
 __device__ __forceinline__ double part_value(double a) { return a; }
 
 template <typename T, int QL>

@@ -231,11 +231,12 @@ __device__ __forceinline__ void taylor(int64_t i, int64_t n_pad, double h, const
 
 // the predicted row in the FP64 j-store and/or the mixed one; the
 // double-single split of a position is exact: hi = fl32(xp), lo = fl32(xp - hi)
+// (hi also to the caller, for the tile's box; mixed store only)
 __device__ __forceinline__ void store_predicted(int64_t i, int64_t n_pad, const double (&px)[3],
                                                 const double (&pv)[3], double mi, double* __restrict__ xp,
                                                 double* __restrict__ vp, float4* __restrict__ jA,
                                                 float4* __restrict__ jB, float2* __restrict__ jC,
-                                                bool write_fp64, bool write_mixed) {
+                                                bool write_fp64, bool write_mixed, float (&hi)[3]) {
   if (write_fp64) {
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -244,16 +245,23 @@ __device__ __forceinline__ void store_predicted(int64_t i, int64_t n_pad, const 
     }
   }
   if (write_mixed) {
-    float hi[3], lo[3];
+    float lo[3];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      hi[d] = __double2float_rn(px[d]);
-      lo[d] = __double2float_rn(px[d] - (double)hi[d]);
-    }
-    jA[i] = make_float4(hi[0], hi[1], hi[2], __double2float_rn(mi));
-    jB[i] = make_float4(lo[0], lo[1], lo[2], __double2float_rn(pv[0]));
-    jC[i] = make_float2(__double2float_rn(pv[1]), __double2float_rn(pv[2]));
+    for (int d = 0; d < 3; ++d) nb_split(px[d], hi[d], lo[d]);
+    jA[i] = make_float4(hi[0], hi[1], hi[2], nb_f32(mi));
+    jB[i] = make_float4(lo[0], lo[1], lo[2], nb_f32(pv[0]));
+    jC[i] = make_float2(nb_f32(pv[1]), nb_f32(pv[2]));
   }
+}
+
+// The reach of a j-memory record: a bound on every coordinate's move within a
+// step d, |v_c| d + |a_c| d^2/2 + |j_c| d^3/6 summed over components, from the
+// FP32 sums of the magnitudes (each rounding 2^-24, eight of them, under the
+// factor 1 + 2^-20: as a bound FP32 serves, and FP64 would be 13 instructions
+// of 64 cycles at the end of a correction)
+__device__ __forceinline__ float reach_of(float sv, float sa, float sj, double d) {
+  const float df = nb_f32(d);
+  return df * (sv + df * (0.5f * sa + df * (sj * (1.0f / 6.0f)))) * (1.0f + 0x1p-20f);
 }
 
 // Corrector (Sec. 4.1 step 5) of row i at block time t from its new force
@@ -323,6 +331,9 @@ struct CorrIn {
 // the dependent FP64 chain is about a third as long, which matters where one
 // particle's correction is the critical path of a block step.
 //
+// a1, j1: component `sub` (lane 3 and up: component 0) of the new acceleration
+// and jerk; p1: the new potential (used by lane 0).
+//
 // Every lane of the warp must call this with the same control flow: the
 // shuffles use the full mask and are taken unconditionally.  `base` is the
 // warp lane of the group's lane 0; `write` says whether this group's row is
@@ -332,8 +343,8 @@ struct CorrIn {
 // is): each lane its component, lane 0 the reach once the new step is known.
 // Returns, on the group's lane 0 of a real row, the row's next due time
 // t + dt_new (0 elsewhere).
-__device__ __forceinline__ double correct_lanes4(int64_t i, int64_t n_pad, double t, const double (&f)[7],
-                                                 const CorrIn& in, double eta, double dt_min, double dt_max,
+__device__ __forceinline__ double correct_lanes4(int64_t i, int64_t n_pad, double t, double a1, double j1,
+                                                 double p1, const CorrIn& in, double eta, double dt_min, double dt_max,
                                                  double* __restrict__ x, double* __restrict__ v,
                                                  double* __restrict__ a, double* __restrict__ jk,
                                                  double* __restrict__ pot, double* __restrict__ ti,
@@ -342,15 +353,12 @@ __device__ __forceinline__ double correct_lanes4(int64_t i, int64_t n_pad, doubl
   const double h = t - in.t0;
   const HPow hp = h_powers(h);
   double sq[4] = {0.0, 0.0, 0.0, 0.0};  // a1^2, j1^2, a2e^2, a3^2 of this lane's component
-  double ab[3];                         // |v1|, |a1|, |j1| of this lane's component (the record's reach)
+  float ab[3];                          // |v1|, |a1|, |j1| of this lane's component (the record's reach)
   int fin = 1;
   const int c = sub < 3 ? sub : 0;
   {
     const int64_t q = c * n_pad + i;
     const double a0 = in.a0, j0 = in.j0;
-    // (selects, not an index: f stays in registers)
-    const double a1 = c == 0 ? f[0] : (c == 1 ? f[1] : f[2]);
-    const double j1 = c == 0 ? f[3] : (c == 1 ? f[4] : f[5]);
     const double da = a0 - a1;
     const double a2 = div_h2(hp, -6.0 * da - h * (4.0 * j0 + 2.0 * j1));
     const double a3 = div_h3(hp, 12.0 * da + hp.h6 * (j0 + j1));
@@ -364,22 +372,24 @@ __device__ __forceinline__ double correct_lanes4(int64_t i, int64_t n_pad, doubl
       jk[q] = j1;
       if (jm) {
         float* r = reinterpret_cast<float*>(jm + i);
-        const float xh = __double2float_rn(x1), vh = __double2float_rn(v1);
+        float xh, xl, vh, vl;
+        nb_split(x1, xh, xl);
+        nb_split(v1, vh, vl);
         r[c] = xh;
-        r[4 * n_pad + c] = __double2float_rn(x1 - (double)xh);
+        r[4 * n_pad + c] = xl;
         r[8 * n_pad + c] = vh;
-        r[12 * n_pad + c] = __double2float_rn(v1 - (double)vh);
-        r[16 * n_pad + c] = __double2float_rn(0.5 * a1);
-        r[4 * n_pad * (2 + c) + 3] = __double2float_rn(j1 * (1.0 / 6.0));
+        r[12 * n_pad + c] = vl;
+        r[16 * n_pad + c] = 0.5f * nb_f32(a1);
+        r[4 * n_pad * (2 + c) + 3] = nb_f32(j1 * (1.0 / 6.0));
       }
     }
     sq[0] = a1 * a1;
     sq[1] = j1 * j1;
     sq[2] = a2e * a2e;
     sq[3] = a3 * a3;
-    ab[0] = fabs(v1);
-    ab[1] = fabs(a1);
-    ab[2] = fabs(j1);
+    ab[0] = jm ? fabsf(nb_f32(v1)) : 0.0f;
+    ab[1] = jm ? fabsf(nb_f32(a1)) : 0.0f;
+    ab[2] = jm ? fabsf(nb_f32(j1)) : 0.0f;
     fin = (isfinite(x1) && isfinite(v1) && isfinite(a1) && isfinite(j1)) ? 1 : 0;
   }
   // lane sub (< 4) sums squared norm `sub` in component order (0 + x^2 +
@@ -395,14 +405,14 @@ __device__ __forceinline__ double correct_lanes4(int64_t i, int64_t n_pad, doubl
     own[k] = sub == 1 ? t1 : (sub == 2 ? t2 : (sub == 3 ? t3 : t0));
   }
   const double mine = ((0.0 + own[0]) + own[1]) + own[2];
-  double sum_ab[3] = {0.0, 0.0, 0.0};  // write_jm_record's sums of |v|, |a|, |j| in component order
+  float sum_ab[3] = {0.0f, 0.0f, 0.0f};  // write_jm_record's sums of |v|, |a|, |j| in component order
   if (jm) {
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
-      const double s0 = __shfl_sync(0xffffffffu, ab[r], base);
-      const double s1 = __shfl_sync(0xffffffffu, ab[r], base + 1);
-      const double s2 = __shfl_sync(0xffffffffu, ab[r], base + 2);
-      sum_ab[r] = ((0.0 + s0) + s1) + s2;
+      const float s0 = __shfl_sync(0xffffffffu, ab[r], base);
+      const float s1 = __shfl_sync(0xffffffffu, ab[r], base + 1);
+      const float s2 = __shfl_sync(0xffffffffu, ab[r], base + 2);
+      sum_ab[r] = (s0 + s1) + s2;
     }
   }
   const int f0 = __shfl_sync(0xffffffffu, fin, base);
@@ -415,7 +425,6 @@ __device__ __forceinline__ double correct_lanes4(int64_t i, int64_t n_pad, doubl
   const double n2 = __shfl_sync(0xffffffffu, root, base + 2);
   const double n3 = __shfl_sync(0xffffffffu, root, base + 3);
   if (!write || sub != 0) return 0.0;
-  const double p1 = f[6];
   pot[i] = p1;
   bool crit_nan;
   const double dnew = new_step(t, in.dt0, na, nj, n2, n3, eta, dt_min, dt_max, st, crit_nan);
@@ -423,17 +432,13 @@ __device__ __forceinline__ double correct_lanes4(int64_t i, int64_t n_pad, doubl
   if (!finite || !isfinite(p1) || crit_nan) atomicOr(&st->flags, NB_ST_NUMERIC);
   ti[i] = t;
   dt[i] = dnew;
-  if (jm) {
-    const double d = dnew;
-    const double rr = d * (sum_ab[0] + d * (0.5 * sum_ab[1] + d * (sum_ab[2] * (1.0 / 6.0))));
-    reinterpret_cast<float*>(jm + n_pad + i)[3] = __double2float_ru(rr * (1.0 + 0x1p-20));
-  }
+  if (jm) reinterpret_cast<float*>(jm + n_pad + i)[3] = reach_of(sum_ab[0], sum_ab[1], sum_ab[2], dnew);
   return t + dnew;
 }
 
 // correct_lanes4 with its inputs read from the state and the predicted rows
-__device__ __forceinline__ double correct_row_lanes4(int64_t i, int64_t n_pad, double t, const double (&f)[7],
-                                                   double eta, double dt_min, double dt_max, double* __restrict__ x,
+__device__ __forceinline__ double correct_row_lanes4(int64_t i, int64_t n_pad, double t, double a1, double j1,
+                                                   double p1, double eta, double dt_min, double dt_max, double* __restrict__ x,
                                                    double* __restrict__ v, double* __restrict__ a,
                                                    double* __restrict__ jk, double* __restrict__ pot,
                                                    double* __restrict__ ti, double* __restrict__ dt,
@@ -441,7 +446,7 @@ __device__ __forceinline__ double correct_row_lanes4(int64_t i, int64_t n_pad, d
                                                    nb_dev_status* __restrict__ st, int sub, int base, bool write) {
   const int64_t q = (sub < 3 ? sub : 0) * n_pad + i;
   const CorrIn in{ti[i], dt[i], a[q], jk[q], xp[q], vp[q]};
-  return correct_lanes4(i, n_pad, t, f, in, eta, dt_min, dt_max, x, v, a, jk, pot, ti, dt, st, sub, base, write);
+  return correct_lanes4(i, n_pad, t, a1, j1, p1, in, eta, dt_min, dt_max, x, v, a, jk, pot, ti, dt, st, sub, base, write);
 }
 
 // j-memory record of row i (the on-the-fly j prediction's input, Sec. 4.4
@@ -455,25 +460,22 @@ __device__ __forceinline__ void write_jm_record(int64_t i, int64_t N, int64_t n_
                                                 const double* __restrict__ dt, float4* __restrict__ jm) {
   float xh[3], xl[3], vh[3], vl[3], a2[3], j6[3], mf = 0.0f, reach = 0.0f;
   if (i < N) {
-    double sv = 0.0, sa = 0.0, sj = 0.0;
+    float sv = 0.0f, sa = 0.0f, sj = 0.0f;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const int64_t q = c * n_pad + i;
       const double xv = x[q], vv = v[q], av = a[q], jv = jk[q];
-      xh[c] = __double2float_rn(xv);
-      xl[c] = __double2float_rn(xv - (double)xh[c]);
-      vh[c] = __double2float_rn(vv);
-      vl[c] = __double2float_rn(vv - (double)vh[c]);
-      a2[c] = __double2float_rn(0.5 * av);
-      j6[c] = __double2float_rn(jv * (1.0 / 6.0));
-      sv += fabs(vv);
-      sa += fabs(av);
-      sj += fabs(jv);
+      nb_split(xv, xh[c], xl[c]);
+      nb_split(vv, vh[c], vl[c]);
+      const float af = nb_f32(av);
+      a2[c] = 0.5f * af;
+      j6[c] = nb_f32(jv * (1.0 / 6.0));
+      sv += fabsf(vh[c]);
+      sa += fabsf(af);
+      sj += fabsf(nb_f32(jv));
     }
-    const double d = dt[i];
-    const double r = d * (sv + d * (0.5 * sa + d * (sj * (1.0 / 6.0))));
-    reach = __double2float_ru(r * (1.0 + 0x1p-20));
-    mf = __double2float_rn(m[i]);
+    reach = reach_of(sv, sa, sj, dt[i]);
+    mf = nb_f32(m[i]);
   } else {  // padding row: massless and far away
 #pragma unroll
     for (int c = 0; c < 3; ++c) {

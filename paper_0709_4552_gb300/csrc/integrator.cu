@@ -21,18 +21,26 @@ inline int grid_for(int64_t n, int threads, int cap = 1 << 20) {
 // ---------------------------------------------------------------------------
 // Predictor (Sec. 4.1 step 3) to time t (own_time: h = 0, i.e. t = t_i), for
 // i < N; padding particles [N, n_pad) get m = 0 far away.  Arithmetic in
-// hermite.cuh.
+// hermite.cuh.  With box, also the boxes of the 128-row tiles (the mixed path's
+// far test) from the FP32 high words the rows have in hand: a kernel of its own
+// read them back for it.
+//
+// Bound by the FP64 unit: 26 FP64 instructions a row, 19 cycles each per warp
+// and SM (52 us of 68 at N = 2^20; 95 with the conversions by the FP64 unit,
+// and the boxes' own kernel besides).
 // ---------------------------------------------------------------------------
-__global__ void predict_kernel(int64_t N, int64_t n_pad, const double* __restrict__ m,
-                               const double* __restrict__ x, const double* __restrict__ v,
-                               const double* __restrict__ a, const double* __restrict__ jk,
-                               const double* __restrict__ ti, double t, int own_time,
-                               double* __restrict__ xp, double* __restrict__ vp,
-                               float4* __restrict__ jA, float4* __restrict__ jB,
-                               float2* __restrict__ jC, int write_fp64, int write_mixed) {
+__global__ void __launch_bounds__(kThreads) predict_kernel(
+    int64_t N, int64_t n_pad, const double* __restrict__ m, const double* __restrict__ x,
+    const double* __restrict__ v, const double* __restrict__ a, const double* __restrict__ jk,
+    const double* __restrict__ ti, double t, int own_time, double* __restrict__ xp, double* __restrict__ vp,
+    float4* __restrict__ jA, float4* __restrict__ jB, float2* __restrict__ jC, int write_fp64, int write_mixed,
+    float4* __restrict__ box) {
+  constexpr int kTileWarps = NB_BOX_TILE / 32;
+  static_assert(kThreads % NB_BOX_TILE == 0 && NB_JPAD % kThreads == 0, "whole tiles per CTA, full CTAs of rows");
+  __shared__ nb_box wbox[kThreads / 32];
   // rows in the resident order: row i of every array is one particle
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_pad;
-       i += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t i0 = blockIdx.x * (int64_t)kThreads; i0 < n_pad; i0 += (int64_t)gridDim.x * kThreads) {
+    const int64_t i = i0 + threadIdx.x;
     double px[3], pv[3], mi;
     if (i < N) {
       mi = m[i];
@@ -42,7 +50,16 @@ __global__ void predict_kernel(int64_t N, int64_t n_pad, const double* __restric
 #pragma unroll
       for (int d = 0; d < 3; ++d) { px[d] = NB_PAD_POS; pv[d] = 0.0; }
     }
-    nbh::store_predicted(i, n_pad, px, pv, mi, xp, vp, jA, jB, jC, write_fp64 != 0, write_mixed != 0);
+    float hi[3] = {0.0f, 0.0f, 0.0f};
+    nbh::store_predicted(i, n_pad, px, pv, mi, xp, vp, jA, jB, jC, write_fp64 != 0, write_mixed != 0, hi);
+    if (box) {
+      const nb_box b = nb_warp_box(i < N, hi);
+      __syncthreads();  // the previous tiles' boxes have been read
+      if ((threadIdx.x & 31) == 0) wbox[threadIdx.x >> 5] = b;
+      __syncthreads();
+      if (threadIdx.x < kThreads / NB_BOX_TILE)
+        nb_write_box(&wbox[threadIdx.x * kTileWarps], kTileWarps, box + 2 * (i0 / NB_BOX_TILE + threadIdx.x));
+    }
   }
 }
 
@@ -312,12 +329,7 @@ cudaError_t nb_launch_predict(nb_ctx* c, double t, bool own_time) {
   c->launches += 1;
   predict_kernel<<<grid_for(c->n_pad, kThreads, c->sm_count * 16), kThreads, 0, c->stream>>>(
       c->n, c->n_pad, c->m, c->x, c->v, c->a, c->jk, c->t, t, own_time ? 1 : 0, c->xp, c->vp, c->jA,
-      c->jB, c->jC, 1, mixed ? 1 : 0);
-  if (mixed && c->perm_valid) {
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return nb_launch_tile_boxes(c);
-  }
+      c->jB, c->jC, 1, mixed ? 1 : 0, mixed && c->perm_valid ? c->tbox : nullptr);
   return cudaGetLastError();
 }
 

@@ -166,6 +166,7 @@ struct nb_ctx {
 };
 
 // ---- launchers (integrator.cu) -------------------------------------------
+// all rows to time t, and (mixed path in spatial order) the boxes of the tiles
 cudaError_t nb_launch_predict(nb_ctx* c, double t, bool own_time);
 cudaError_t nb_launch_select(nb_ctx* c);    // writes act, sel_cnt[total], sel_min[result]
 // write_jm: also write the corrected rows' j-memory records (c->jm)
@@ -248,7 +249,6 @@ cudaError_t nb_check_map_to_slots(nb_ctx* c, const int32_t* d_list, int64_t n, c
 cudaError_t nb_map_to_particles(nb_ctx* c, const int32_t* in, int64_t n, int32_t* out);
 // rows of particles [first, first + count) of a state array (rows x n_pad) to AoS dst
 cudaError_t nb_gather_rows(nb_ctx* c, const double* src, int rows, int64_t first, int64_t count, double* dst);
-cudaError_t nb_launch_tile_boxes(nb_ctx* c);  // tbox from the predicted (permuted) j-store
 // processing order of a list of slots: positions sorted by slot (device array of n positions)
 cudaError_t nb_list_order(nb_ctx* c, const int32_t* d_list, int64_t n, const int32_t** ord);
 
@@ -300,6 +300,97 @@ __device__ __forceinline__ float nb_rsqrt_approx(float x) {
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+
+// ---- FP64 <-> FP32 by bits --------------------------------------------------
+// A conversion between FP64 and FP32 goes through the FP64 unit: 16 cycles per
+// warp and SM, and like every FP64 instruction 64 cycles of the warp itself
+// (measured).  The predictor's and corrector's conversions are therefore made
+// of the operands' bits, 5 to 8 integer instructions each: the same values bit
+// for bit, with the conversion instruction for operands outside the range
+// stated (zero, subnormal, huge, non-finite).
+
+// fl32(x), |x| in [2^-126, 2^127)
+__device__ __forceinline__ float nb_f32(double x) {
+  const uint32_t lo = (uint32_t)__double2loint(x), hi = (uint32_t)__double2hiint(x);
+  if (((hi >> 20) & 0x7FFu) - 897u > 252u) return __double2float_rn(x);
+  // round to nearest even at bit 29, then rebias the exponent modulo 2^9
+  const uint64_t b = (((uint64_t)hi << 32) | lo) + (0x0FFFFFFFu + ((lo >> 29) & 1u));
+  const uint32_t q = __funnelshift_r((uint32_t)b, (uint32_t)(b >> 32), 29) + 0x40000000u;
+  return __uint_as_float((q & 0x7FFFFFFFu) | (hi & 0x80000000u));
+}
+
+// hi = fl32(x), lo = fl32(x - hi), |x| in [2^-74, 2^127)
+__device__ __forceinline__ void nb_split(double x, float& hi, float& lo) {
+  const uint32_t xl = (uint32_t)__double2loint(x), xh = (uint32_t)__double2hiint(x);
+  const uint32_t e = (xh >> 20) & 0x7FFu;
+  if (e - 949u > 200u) {
+    hi = __double2float_rn(x);
+    lo = __double2float_rn(x - (double)hi);
+    return;
+  }
+  const uint64_t b = (((uint64_t)xh << 32) | xl) + (0x0FFFFFFFu + ((xl >> 29) & 1u));
+  const uint32_t q = __funnelshift_r((uint32_t)b, (uint32_t)(b >> 32), 29) + 0x40000000u;
+  hi = __uint_as_float((q & 0x7FFFFFFFu) | (xh & 0x80000000u));
+  // what the rounding took off, in units of x's last place: |rest| <= 2^28
+  const int32_t rest = (int32_t)(xl - ((uint32_t)b & 0xE0000000u));
+  const float unit = __uint_as_float(((e - 948u) << 23) | (xh & 0x80000000u));
+  lo = fmaf((float)rest, unit, 0.0f);  // (+ 0: no negative zero)
+}
+
+// x as an FP64 number
+__device__ __forceinline__ double nb_f64(float x) {
+  const uint32_t u = __float_as_uint(x);
+  const uint32_t e = (u >> 23) & 0xFFu;
+  if (e - 1u > 253u && (u << 1) != 0u) return (double)x;  // subnormal, Inf, NaN
+  const uint32_t hi = (((uint32_t)((int32_t)u >> 3)) & 0x8FFFFFFFu) + (e ? 0x38000000u : 0u);
+  return __hiloint2double((int)hi, (int)(u << 29));
+}
+
+// ---- boxes of NB_BOX_TILE rows -----------------------------------------------
+// the box of a warp's points (empty: lo > hi), one reduction instruction per
+// bound: FP32 numbers order like these keys
+__device__ __forceinline__ int nb_fkey(float f) {
+  const int b = __float_as_int(f);
+  return b ^ ((b >> 31) & 0x7FFFFFFF);
+}
+__device__ __forceinline__ float nb_unkey(int k) { return __int_as_float(k ^ ((k >> 31) & 0x7FFFFFFF)); }
+
+struct nb_box {
+  int lo[3], hi[3];  // keys
+};
+
+__device__ __forceinline__ nb_box nb_warp_box(bool in, const float (&p)[3]) {
+  nb_box b;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int k = nb_fkey(p[c]);
+    b.lo[c] = __reduce_min_sync(0xffffffffu, in ? k : 0x7F7FFFFF);          // FLT_MAX
+    b.hi[c] = __reduce_max_sync(0xffffffffu, in ? k : ~0x7F7FFFFF);         // -FLT_MAX
+  }
+  return b;
+}
+
+// boxes of warps w0 .. w0 + count - 1 joined and written as (min corner, max
+// |coordinate|), (max corner, 0); a tile without rows: rmax = 0
+__device__ __forceinline__ void nb_write_box(const nb_box* w, int count, float4* __restrict__ out) {
+  nb_box b = w[0];
+  for (int q = 1; q < count; ++q)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      b.lo[c] = min(b.lo[c], w[q].lo[c]);
+      b.hi[c] = max(b.hi[c], w[q].hi[c]);
+    }
+  float lo[3], hi[3], r = 0.0f;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    lo[c] = nb_unkey(b.lo[c]);
+    hi[c] = nb_unkey(b.hi[c]);
+    r = fmaxf(r, fmaxf(fabsf(lo[c]), fabsf(hi[c])));
+  }
+  if (b.lo[0] > b.hi[0]) r = 0.0f;
+  out[0] = make_float4(lo[0], lo[1], lo[2], r);
+  out[1] = make_float4(hi[0], hi[1], hi[2], 0.0f);
 }
 
 // 1/sqrt(x) in FP64 for any x >= 0.  For x in the FP32 normal range

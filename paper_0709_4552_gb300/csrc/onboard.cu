@@ -71,7 +71,8 @@ __global__ void jm_host_side_kernel(int64_t box_blocks, int64_t N, int64_t ntile
       i = i < 0 ? 0 : (i >= n_pad ? n_pad - 1 : i);
       double px[3], pv[3];
       nbh::taylor(i, n_pad, t - ti[i], x, v, a, jk, px, pv);
-      nbh::store_predicted(i, n_pad, px, pv, m[i], xp, vp, jA, jB, jC, true, true);
+      float hi[3];
+      nbh::store_predicted(i, n_pad, px, pv, m[i], xp, vp, jA, jB, jC, true, true, hi);
     }
     return;
   }

@@ -42,10 +42,13 @@ namespace {
 
 constexpr int kLT = 128;                     // threads per CTA = i-tile = row tile
 constexpr int kLWarps = kLT / 32;
-// resident CTAs per SM asked for: 4 mixed (128 registers), 3 FP64 (168; with 4
-// the fixed-point pair spills: N = 1024 32.4 against 31.8 us a block step, N =
-// 32768 582 against 569)
-constexpr int kLMaxPerSm = 4, kLMaxPerSm64 = 3;
+// resident CTAs per SM asked for.  Mixed: 4 (128 registers, a few spilled) where
+// the force phase is the longest part of a step, 2 (no spills) where its
+// latencies are (us a block step, 4 / 2: N = 512 19.1 / 17.9, N = 12000 34.3 /
+// 31.5, N = 32768 67.5 / 64.4, N = 40000 84.4 / 88.0, N = 65536 169 / 184).  FP64: 3 (168; with 4 the fixed-point pair spills: N =
+// 1024 32.4 against 31.8 us a block step, N = 32768 582 against 569)
+constexpr int kLPerSmMixed = 4, kLPerSmMixedSmall = 2, kLPerSm64 = 3;
+constexpr int64_t kLMixedSmallHi = 32768;
 // j-tiles (the mixed one = the box tile).  FP64: an item's tile is its share of
 // a small system's force phase, so those take 32 and at least two CTAs per SM:
 // N = 1024 31.8 us a block step against 40.7 with 64 and one CTA (44.9 with 64
@@ -169,7 +172,7 @@ struct LoopSmem {
   unsigned long long wv[kLWarps];
   int wc[kLWarps];
   long long ws[2][kLWarps];
-  float wbox[kLWarps][7];
+  nb_box wbox[kLWarps];
   unsigned long long tnb;  // block time (bit pattern)
   long long before, total;
   int mine;                // this CTA has active rows this step
@@ -294,53 +297,23 @@ __device__ void write_active(const LoopArgs& p, int64_t r0, int64_t r1, unsigned
 }
 
 // predictor of this CTA's rows to tn; on the mixed path in spatial order the
-// box of each 128-row tile (thread q holds row q of every tile it visits):
-// (min corner, max |coordinate|), (max corner, 0) of the FP32 high words
+// box of each 128-row tile (thread q holds row q of every tile it visits)
 template <bool MIXED>
 __device__ void predict_rows(const LoopArgs& p, int64_t r0, int64_t r1, double tn, LoopSmem& s) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  static_assert(kLT == NB_BOX_TILE, "a tile of rows per pass");
   for (int64_t r = r0; r < r1; r += kLT) {
     const int64_t i = r + threadIdx.x;
-    float bx[7] = {FLT_MAX, FLT_MAX, FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX, 0.0f};
+    float hi[3] = {0.0f, 0.0f, 0.0f};
     if (i < r1) {
       double px[3], pv[3];
       nbh::taylor(i, p.n_pad, tn - p.t[i], p.x, p.v, p.a, p.jk, px, pv);
-      nbh::store_predicted(i, p.n_pad, px, pv, p.m[i], p.xp, p.vp, p.jA, p.jB, p.jC, true, MIXED);
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const float h = __double2float_rn(px[d]);
-        bx[d] = h;
-        bx[3 + d] = h;
-        bx[6] = fmaxf(bx[6], fabsf(h));
-      }
+      nbh::store_predicted(i, p.n_pad, px, pv, p.m[i], p.xp, p.vp, p.jA, p.jB, p.jC, true, MIXED, hi);
     }
     if (MIXED && p.tbox) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          bx[d] = fminf(bx[d], __shfl_xor_sync(0xffffffffu, bx[d], o));
-          bx[3 + d] = fmaxf(bx[3 + d], __shfl_xor_sync(0xffffffffu, bx[3 + d], o));
-        }
-        bx[6] = fmaxf(bx[6], __shfl_xor_sync(0xffffffffu, bx[6], o));
-      }
-      if (lane == 0)
-#pragma unroll
-        for (int d = 0; d < 7; ++d) s.wbox[warp][d] = bx[d];
+      const nb_box b = nb_warp_box(i < r1, hi);
+      if ((threadIdx.x & 31) == 0) s.wbox[threadIdx.x >> 5] = b;
       __syncthreads();
-      if (threadIdx.x == 0) {
-        for (int w = 1; w < kLWarps; ++w) {
-#pragma unroll
-          for (int d = 0; d < 3; ++d) {
-            bx[d] = fminf(bx[d], s.wbox[w][d]);
-            bx[3 + d] = fmaxf(bx[3 + d], s.wbox[w][3 + d]);
-          }
-          bx[6] = fmaxf(bx[6], s.wbox[w][6]);
-        }
-        const int64_t tile = r / kLT;
-        p.tbox[2 * tile] = make_float4(bx[0], bx[1], bx[2], bx[6]);
-        p.tbox[2 * tile + 1] = make_float4(bx[3], bx[4], bx[5], 0.0f);
-      }
+      if (threadIdx.x == 0) nb_write_box(s.wbox, kLWarps, p.tbox + 2 * (r / kLT));
       __syncthreads();
     }
   }
@@ -390,16 +363,14 @@ __device__ void correct_own(const LoopArgs& p, LoopSmem& s, int64_t jtiles, unsi
     const int q = threadIdx.x / L, l = threadIdx.x % L;
     const bool have = q < P;
     const int64_t k = before + k0 + (have ? q : 0);
+    // the row's sums: final FP64 rows, double-single partials (the mixed item's
+    // split output, summed and exchanged in FP32), or FP64 partials
+    float hi[7], lo[7];
     double f[7];
     if (fin) {
-      if (have && l < 4)
 #pragma unroll
-        for (int r = 0; r < 7; ++r) f[r] = p.F[r * p.n_pad + k];
+      for (int r = 0; r < 7; ++r) f[r] = have && l < 4 ? p.F[r * p.n_pad + k] : 0.0;
     } else if (MIXED) {
-      // double-single partials (the mixed item's split output): summed and
-      // exchanged in FP32 (a warp's FP64 instruction costs it 64 cycles
-      // here), converted to FP64 once
-      float hi[7], lo[7];
 #pragma unroll
       for (int r = 0; r < 7; ++r) hi[r] = lo[r] = 0.0f;
       const float2* part2 = reinterpret_cast<const float2*>(p.part);
@@ -417,9 +388,6 @@ __device__ void correct_own(const LoopArgs& p, LoopSmem& s, int64_t jtiles, unsi
           const float ol = __shfl_xor_sync(0xffffffffu, lo[r], o);
           nbk::ds_add(hi[r], lo[r], oh, ol);
         }
-#pragma unroll
-      for (int r = 0; r < 7; ++r) f[r] = (double)hi[r] + (double)lo[r];
-      f[6] = -f[6];
     } else {
 #pragma unroll
       for (int r = 0; r < 7; ++r) f[r] = 0.0;
@@ -435,16 +403,35 @@ __device__ void correct_own(const LoopArgs& p, LoopSmem& s, int64_t jtiles, unsi
     const bool cached = r1 - r0 <= kLDue;
     if (L >= 4) {
       // every lane of the CTA takes this branch (L is uniform) and every
-      // shuffle inside; lanes without a row read a valid own row, write nothing
+      // shuffle inside; lanes without a row read a valid own row, write
+      // nothing.  Each lane forms the FP64 values of its own component only (an
+      // FP64 addition holds the warp for 64 cycles: 3 of them instead of 7, and
+      // none of the 14 conversions)
       int64_t i = p.act[k];
       i = i < r0 ? r0 : (i >= r1 ? r1 - 1 : i);  // own rows only
-      if (!(have && l < 4))
-#pragma unroll
-        for (int r = 0; r < 7; ++r) f[r] = 0.0;
-      const double nd = nbh::correct_row_lanes4(i, p.n_pad, tn, f, p.eta, p.dt_min, p.dt_max, p.x, p.v, p.a, p.jk,
-                                                p.pot, p.t, p.dt, p.xp, p.vp, p.st, l, (int)(threadIdx.x & 31) - l, have);
+      double a1, j1, p1;
+      if (MIXED && !fin) {
+        const float ah = l == 1 ? hi[1] : (l == 2 ? hi[2] : hi[0]), al = l == 1 ? lo[1] : (l == 2 ? lo[2] : lo[0]);
+        const float jh = l == 1 ? hi[4] : (l == 2 ? hi[5] : hi[3]), jl = l == 1 ? lo[4] : (l == 2 ? lo[5] : lo[3]);
+        a1 = nb_f64(ah) + nb_f64(al);
+        j1 = nb_f64(jh) + nb_f64(jl);
+        p1 = -(nb_f64(hi[6]) + nb_f64(lo[6]));
+      } else {
+        a1 = l == 1 ? f[1] : (l == 2 ? f[2] : f[0]);
+        j1 = l == 1 ? f[4] : (l == 2 ? f[5] : f[3]);
+        p1 = f[6];
+      }
+      if (!(have && l < 4)) a1 = j1 = p1 = 0.0;
+      const double nd =
+          nbh::correct_row_lanes4(i, p.n_pad, tn, a1, j1, p1, p.eta, p.dt_min, p.dt_max, p.x, p.v, p.a, p.jk, p.pot,
+                                  p.t, p.dt, p.xp, p.vp, p.st, l, (int)(threadIdx.x & 31) - l, have);
       if (have && l == 0 && cached) s.due[i - r0] = (unsigned long long)__double_as_longlong(nd);
     } else if (have && l == 0) {
+      if (MIXED && !fin) {
+#pragma unroll
+        for (int r = 0; r < 7; ++r) f[r] = nb_f64(hi[r]) + nb_f64(lo[r]);
+        f[6] = -f[6];
+      }
       int64_t i = p.act[k];
       i = i < r0 ? r0 : (i >= r1 ? r1 - 1 : i);  // own rows only
       const double nd = nbh::correct_row(i, p.n_pad, tn, f, p.eta, p.dt_min, p.dt_max, p.x, p.v, p.a, p.jk, p.pot,
@@ -454,8 +441,8 @@ __device__ void correct_own(const LoopArgs& p, LoopSmem& s, int64_t jtiles, unsi
   }
 }
 
-template <bool MIXED, int JT>
-__global__ void __launch_bounds__(kLT, MIXED ? kLMaxPerSm : kLMaxPerSm64) loop_kernel(LoopArgs p) {
+template <bool MIXED, int JT, int PER_SM>
+__global__ void __launch_bounds__(kLT, PER_SM) loop_kernel(LoopArgs p) {
   using ForceSmem = typename std::conditional<MIXED, nbk::MixedSmem<JT>, nbk::Fp64Smem<kLT, JT>>::type;
   __shared__ __align__(16) ForceSmem fsm;
   __shared__ LoopSmem s;
@@ -485,7 +472,8 @@ __global__ void __launch_bounds__(kLT, MIXED ? kLMaxPerSm : kLMaxPerSm64) loop_k
   if (blockIdx.x == G - 1)
     for (int64_t i = N + threadIdx.x; i < min(T * kLT, p.n_pad); i += kLT) {
       const double px[3] = {NB_PAD_POS, NB_PAD_POS, NB_PAD_POS}, pv[3] = {0.0, 0.0, 0.0};
-      nbh::store_predicted(i, p.n_pad, px, pv, 0.0, p.xp, p.vp, p.jA, p.jB, p.jC, true, MIXED);
+      float hi[3];
+      nbh::store_predicted(i, p.n_pad, px, pv, 0.0, p.xp, p.vp, p.jA, p.jB, p.jC, true, MIXED, hi);
     }
   if (r1 - r0 <= kLDue)
     for (int64_t i = r0 + threadIdx.x; i < r1; i += kLT)
@@ -584,24 +572,30 @@ struct PLoop {
   unsigned long long* smin = nullptr;
   int32_t* scnt = nullptr;
   int gmax = 0;
-  int per_sm[3] = {0, 0, 0};  // resident CTAs per SM of each instantiation (0 = not yet asked)
+  int per_sm[4] = {0, 0, 0, 0};  // resident CTAs per SM of each instantiation (0 = not yet asked)
 };
 
 PLoop* ploop_of(nb_ctx* c) { return static_cast<PLoop*>(c->loop); }
 
-// the instantiations: mixed, FP64, FP64 for small systems
+// the instantiations: mixed, FP64 and each for small systems
 const void* loop_variant(int v) {
-  return v == 0   ? (const void*)loop_kernel<true, kLMixJT>
-         : v == 1 ? (const void*)loop_kernel<false, kLF64JT>
-                  : (const void*)loop_kernel<false, kLF64JTSmall>;
+  return v == 0   ? (const void*)loop_kernel<true, kLMixJT, kLPerSmMixed>
+         : v == 1 ? (const void*)loop_kernel<true, kLMixJT, kLPerSmMixedSmall>
+         : v == 2 ? (const void*)loop_kernel<false, kLF64JT, kLPerSm64>
+                  : (const void*)loop_kernel<false, kLF64JTSmall, kLPerSm64>;
+}
+int variant_of(bool mixed, int64_t n) {
+  if (mixed) return n <= kLMixedSmallHi ? 1 : 0;
+  return n > kLF64SmallLo && n <= kLF64SmallHi ? 3 : 2;
 }
 
 int ctas_per_sm(PLoop* L, int v) {
+  static const int most[4] = {kLPerSmMixed, kLPerSmMixedSmall, kLPerSm64, kLPerSm64};
   int& ps = L->per_sm[v];
   if (ps == 0) {
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, loop_variant(v), kLT, 0) != cudaSuccess) return -1;
-    ps = std::min(occ, v == 0 ? kLMaxPerSm : kLMaxPerSm64);
+    ps = std::min(occ, most[v]);
   }
   return ps;
 }
@@ -626,7 +620,7 @@ int nb_integrate_persistent(nb_ctx* c, double t_end) {
     L = new PLoop();
     c->loop = L;
   }
-  const int variant = mixed ? 0 : (c->n > kLF64SmallLo && c->n <= kLF64SmallHi ? 2 : 1);
+  const int variant = variant_of(mixed, c->n);
   const int per_sm = ctas_per_sm(L, variant);
   if (per_sm < 1) {
     cudaGetLastError();
@@ -638,7 +632,7 @@ int nb_integrate_persistent(nb_ctx* c, double t_end) {
   // its small blocks, and each barrier waits for every CTA's arrival
   const int64_t row_tiles = (c->n + kLT - 1) / kLT;
   const int G = (int)std::min<int64_t>(std::min(c->sm_count * per_sm, kLMaxG),
-                                       std::max<int64_t>(variant == 2 ? 2 * c->sm_count : 32, 2 * row_tiles));
+                                       std::max<int64_t>(variant == 3 ? 2 * c->sm_count : 32, 2 * row_tiles));
   if (G > L->gmax) {
     if (L->smin) cudaFree(L->smin);
     if (L->scnt) cudaFree(L->scnt);

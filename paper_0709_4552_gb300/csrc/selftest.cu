@@ -1,7 +1,8 @@
 // selftest.cu -- device self-check of the corrector's exponent forms
 // (hermite.cuh: h_powers, mul_pow2, new_step_nd) against their FP64
-// expressions (h_powers_fp64, the product by 2^k, new_step_fp64) on seeded
-// random operands, bit for bit.
+// expressions (h_powers_fp64, the product by 2^k, new_step_fp64) and of the
+// FP64 <-> FP32 conversions by bits (nb_internal.cuh: nb_f32, nb_split, nb_f64)
+// against the conversion instructions, on seeded random operands, bit for bit.
 // The operands cover the block-step regime and its edges: powers of two and
 // other steps, significands of N = eta num and den equal or one unit apart
 // (quotients at a power-of-two boundary), zero, subnormal, infinite and NaN
@@ -66,6 +67,26 @@ __global__ void selftest_kernel(int64_t samples, uint64_t seed, unsigned long lo
       const double y = (r3 & 3) == 0 ? random_norm(r4, r5) : make_pos(1 + (int)((r4 >> 8) % 2046), r5);
       const double ys = (r1 >> 63) ? -y : y;
       if (nbh::dbits(nbh::mul_pow2(ys, k, nbh::pow2i(k))) != nbh::dbits(ys * nbh::pow2i(k))) atomicAdd(bad, 1ULL);
+    }
+    // conversions by bits against the conversion instructions: magnitudes over
+    // and beyond FP32's range, ties of the rounding, zeros, Inf and NaN
+    {
+      uint64_t f = r5 & 0x000FFFFFFFFFFFFFULL;
+      if ((r4 & 7) == 0) f = (f & ~0x1FFFFFFFULL) | 0x10000000ULL;             // half way
+      if ((r4 & 7) == 1) f |= 0x000FFFFFE0000000ULL;                           // carries into the exponent
+      if ((r4 & 7) == 2) f &= ~0x1FFFFFFFULL;                                  // an FP32 value
+      const int E = (r3 & 3) == 0 ? (int)((r3 >> 8) % 2048) : 1023 - 160 + (int)((r3 >> 8) % 320);
+      double y = (r4 >> 59) == 0 ? random_norm(r1, r2) : from_bits(((uint64_t)E << 52) | f);
+      if (r1 >> 63) y = -y;
+      const float f0 = __double2float_rn(y), l0 = __double2float_rn(y - (double)f0);
+      float f1, l1;
+      nb_split(y, f1, l1);
+      const bool nan = isnan(y) || isinf(y);
+      if (__float_as_uint(nb_f32(y)) != __float_as_uint(f0) || __float_as_uint(f1) != __float_as_uint(f0) ||
+          (!nan && __float_as_uint(l1) != __float_as_uint(l0)))
+        atomicAdd(bad, 1ULL);
+      const float g = (r2 & 15) == 0 ? __uint_as_float((uint32_t)r5 & 0x807FFFFFu) : __uint_as_float((uint32_t)r5);
+      if (!isnan(g) && nbh::dbits(nb_f64(g)) != nbh::dbits((double)g)) atomicAdd(bad, 1ULL);
     }
     // the step rule
     const int emin = -30 + (int)(r0 >> 40) % 12;           // dt_min = 2^emin

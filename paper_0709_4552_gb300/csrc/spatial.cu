@@ -16,8 +16,6 @@
 // digit histograms, one scan, stable scatter ranked with warp match) -> the
 // rows gathered into a scratch block and copied back, perm composed and
 // inverted.  Deterministic.
-// nb_launch_tile_boxes: per j-tile of 128 slots, the box of the FP32 hi
-// positions of its real particles and their largest |coordinate|.
 #include <float.h>
 
 #include "nb_internal.cuh"
@@ -172,38 +170,6 @@ __global__ void radix_scatter(const uint32_t* __restrict__ kin, const int32_t* _
 __global__ void invert_perm(int64_t N, const int32_t* __restrict__ perm, int32_t* __restrict__ iperm) {
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x)
     iperm[perm[k]] = (int32_t)k;
-}
-
-// box of tile t (slots [t*JT, t*JT+JT) intersected with [0, N)): (lo, rmax), (hi, 0);
-// an empty intersection gives lo = +FLT_MAX, hi = -FLT_MAX, rmax = 0
-template <int JT>
-__global__ void tile_boxes(int64_t N, int64_t ntiles, const float4* __restrict__ jA, float4* __restrict__ box) {
-  const int64_t t = blockIdx.x * (int64_t)(blockDim.x / 32) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (t >= ntiles) return;
-  float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX}, r = 0.0f;
-  for (int q = lane; q < JT; q += 32) {
-    const int64_t s = t * JT + q;
-    if (s >= N) break;
-    const float4 a = jA[s];
-    const float p[3] = {a.x, a.y, a.z};
-    for (int c = 0; c < 3; ++c) {
-      lo[c] = fminf(lo[c], p[c]);
-      hi[c] = fmaxf(hi[c], p[c]);
-      r = fmaxf(r, fabsf(p[c]));
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    for (int c = 0; c < 3; ++c) {
-      lo[c] = fminf(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
-      hi[c] = fmaxf(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
-    }
-    r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, o));
-  }
-  if (lane == 0) {
-    box[2 * t] = make_float4(lo[0], lo[1], lo[2], r);
-    box[2 * t + 1] = make_float4(hi[0], hi[1], hi[2], 0.0f);
-  }
 }
 
 int grid_for(int64_t n, int threads, int cap) {
@@ -486,16 +452,5 @@ cudaError_t nb_list_order(nb_ctx* c, const int32_t* d_list, int64_t n, const int
   order_write<<<chunks, kOrderChunk, 0, c->stream>>>(pos, c->shist, chunks, n, c->n, c->sval[0]);
   c->launches += 2;
   *ord = c->sval[0];
-  return cudaGetLastError();
-}
-
-cudaError_t nb_launch_tile_boxes(nb_ctx* c) {
-  // every tile up to n_pad (tiles of padding alone get an empty box: always far)
-  const int64_t ntiles = c->n > 0 ? c->n_pad / NB_BOX_TILE : 0;
-  if (ntiles <= 0) return cudaSuccess;
-  const int warps = 8;
-  tile_boxes<NB_BOX_TILE><<<(unsigned)((ntiles + warps - 1) / warps), warps * 32, 0, c->stream>>>(c->n, ntiles, c->jA,
-                                                                                                    c->tbox);
-  c->launches += 1;
   return cudaGetLastError();
 }
