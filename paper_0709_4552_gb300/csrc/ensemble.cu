@@ -32,8 +32,9 @@ namespace {
 #define NB_ENS_ITEM_WAVES 4
 #endif
 constexpr int kItemWaves = NB_ENS_ITEM_WAVES;  // force items planned per resident CTA
-constexpr int kCorrItem = 128;    // active particles per corrector item (= its threads per CTA)
+constexpr int kCorrItem = 32;     // active particles per corrector item (four threads of its CTA each)
 constexpr int kSelChunk = 512;    // particles per selection chunk (chunks never straddle clusters)
+constexpr int kSelThreads = 256;
 // batched item shapes: i-tile = threads per CTA, one i per thread.  An
 // ensemble of small clusters has small active blocks (n = 0.20 N^0.81 is 18
 // at N = 256 and 169 at N = 4096), so it takes 32-particle i-tiles that
@@ -102,28 +103,46 @@ cudaError_t dalloc(T** p, size_t count) {
 
 // ---------------------------------------------------------------------------
 // selection (Sec. 4.1 step 2) per cluster: t_next[c] = min (t_i + dt_i) over
-// the cluster; active slots off[c] + k, k < n_c, ascending index.
+// the cluster; active slots off[c] + k, k < n_c, ascending index.  Two small
+// kernels of a few us each, bound by their launch and one round of loads: each
+// chunk's minimum with the number of rows at it, then the cluster's from its
+// chunks' (9 us a step at 240k rows in 96 clusters; as minimum, count over all
+// rows and write 14).
 // ---------------------------------------------------------------------------
-__global__ void b_sel_min(const int64_t* __restrict__ lo, const int64_t* __restrict__ hi,
-                          const double* __restrict__ ti, const double* __restrict__ dt,
-                          unsigned long long* __restrict__ ch_min) {
-  const int j = blockIdx.x;
-  unsigned long long best = 0x7FF0000000000000ULL;
-  for (int64_t i = lo[j] + threadIdx.x; i < hi[j]; i += blockDim.x) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(ti[i] + dt[i]);
-    best = b < best ? b : best;
+__global__ void __launch_bounds__(kSelThreads) b_sel_min(
+    const int64_t* __restrict__ lo, const int64_t* __restrict__ hi, const double* __restrict__ ti,
+    const double* __restrict__ dt, unsigned long long* __restrict__ ch_min, int32_t* __restrict__ ch_cnt) {
+  constexpr int kPer = kSelChunk / kSelThreads, kWarps = kSelThreads / 32;
+  const int j = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  unsigned long long v[kPer], best = 0x7FF0000000000000ULL;  // +inf
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const int64_t i = lo[j] + threadIdx.x + u * kSelThreads;
+    v[u] = i < hi[j] ? (unsigned long long)__double_as_longlong(ti[i] + dt[i]) : 0x7FF0000000000000ULL;
+    best = v[u] < best ? v[u] : best;
   }
   for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long w = __shfl_xor_sync(0xffffffffu, best, o);
-    best = w < best ? w : best;
+    const unsigned long long q = __shfl_xor_sync(0xffffffffu, best, o);
+    best = q < best ? q : best;
   }
-  __shared__ unsigned long long sm[32];
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = best;
+  __shared__ unsigned long long sm[kWarps];
+  __shared__ int sc[kWarps];
+  if (lane == 0) sm[w] = best;
+  __syncthreads();
+  best = sm[0];
+#pragma unroll
+  for (int q = 1; q < kWarps; ++q) best = sm[q] < best ? sm[q] : best;
+  int cnt = 0;
+#pragma unroll
+  for (int u = 0; u < kPer; ++u)
+    cnt += lo[j] + threadIdx.x + u * kSelThreads < hi[j] && v[u] == best ? 1 : 0;
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  if (lane == 0) sc[w] = cnt;
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) best = sm[w] < best ? sm[w] : best;
-    best = sm[0] < best ? sm[0] : best;
+    for (int q = 1; q < kWarps; ++q) cnt += sc[q];
     ch_min[j] = best;
+    ch_cnt[j] = cnt;
   }
 }
 
@@ -140,80 +159,60 @@ __device__ __forceinline__ double cluster_tmin(const unsigned long long* ch_min,
   return __longlong_as_double((long long)best);
 }
 
-// (also: an active cluster's block time must exceed the one it had at the
-// previous iteration of this launch, else the state has no valid steps, e.g.
-// dt = 0: NB_ST_STALLED, and the plan ends the loop)
-__global__ void b_sel_count(const int32_t* __restrict__ ch_cluster, const int64_t* __restrict__ lo,
-                            const int64_t* __restrict__ hi, const int32_t* __restrict__ cl_ch0,
-                            const unsigned long long* __restrict__ ch_min, const double* __restrict__ ti,
-                            const double* __restrict__ dt, double* __restrict__ tnext,
-                            int32_t* __restrict__ ch_cnt, const int64_t* __restrict__ ctrl,
-                            const BParams* __restrict__ prm, nb_dev_status* __restrict__ st) {
+// The cluster's block time from its chunks' minima, and the chunk's active rows
+// (those at it, ascending) behind those of the chunks before it; the first
+// chunk's CTA writes the cluster's block time and count.  An active cluster's
+// block time must exceed the one it had at the previous iteration of this
+// launch, else the state has no valid steps, e.g. dt = 0: NB_ST_STALLED, and
+// the plan ends the loop.
+__global__ void __launch_bounds__(kSelThreads) b_sel_write(
+    const int32_t* __restrict__ ch_cluster, const int64_t* __restrict__ lo, const int64_t* __restrict__ hi,
+    const int32_t* __restrict__ cl_ch0, const unsigned long long* __restrict__ ch_min,
+    const int32_t* __restrict__ ch_cnt, const int64_t* __restrict__ off, const double* __restrict__ ti,
+    const double* __restrict__ dt, double* __restrict__ tnext, const int64_t* __restrict__ ctrl,
+    const BParams* __restrict__ prm, int32_t* __restrict__ act, int32_t* __restrict__ nact,
+    nb_dev_status* __restrict__ st) {
   const int j = blockIdx.x;
   const int c = ch_cluster[j];
-  __shared__ double tn;
+  __shared__ unsigned long long s_tb;
+  __shared__ int base_s;
   if (threadIdx.x < 32) {
     const double t = cluster_tmin(ch_min, cl_ch0[c], cl_ch0[c + 1]);
+    const unsigned long long tb = (unsigned long long)__double_as_longlong(t);
+    int b = 0, tot = 0;  // counts of the cluster's chunks before this one, and in all
+    for (int q = cl_ch0[c] + (int)threadIdx.x; q < cl_ch0[c + 1]; q += 32) {
+      const int n = ch_min[q] == tb ? ch_cnt[q] : 0;
+      if (q < j) b += n;
+      tot += n;
+    }
+    b = __reduce_add_sync(0xffffffffu, b);
+    tot = __reduce_add_sync(0xffffffffu, tot);
     if (threadIdx.x == 0) {
-      tn = t;
+      s_tb = tb;
+      base_s = b;
       if (j == cl_ch0[c]) {
         if (ctrl[1] > 0 && t <= prm->t_end && !(t > tnext[c])) atomicOr(&st->flags, NB_ST_STALLED);
         tnext[c] = t;
+        nact[c] = t <= prm->t_end ? tot : 0;
       }
     }
   }
   __syncthreads();
-  int cnt = 0;
-  for (int64_t i = lo[j] + threadIdx.x; i < hi[j]; i += blockDim.x) cnt += (ti[i] + dt[i] == tn) ? 1 : 0;
-  for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-  __shared__ int sm[32];
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = cnt;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int s = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sm[w];
-    ch_cnt[j] = s;
-  }
-}
-
-__global__ void b_sel_write(const int32_t* __restrict__ ch_cluster, const int64_t* __restrict__ lo,
-                            const int64_t* __restrict__ hi, const int32_t* __restrict__ cl_ch0,
-                            const int32_t* __restrict__ ch_cnt, const int64_t* __restrict__ off,
-                            const double* __restrict__ ti, const double* __restrict__ dt,
-                            const double* __restrict__ tnext, const BParams* __restrict__ prm,
-                            int32_t* __restrict__ act, int32_t* __restrict__ nact) {
-  const int j = blockIdx.x;
-  const int c = ch_cluster[j];
-  const double tn = tnext[c];
-  __shared__ int base_s;
-  if (threadIdx.x < 32) {  // counts of the cluster's chunks before this one, and in all
-    int b = 0, tot = 0;
-    for (int q = cl_ch0[c] + (int)threadIdx.x; q < cl_ch0[c + 1]; q += 32) {
-      if (q < j) b += ch_cnt[q];
-      tot += ch_cnt[q];
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      b += __shfl_xor_sync(0xffffffffu, b, o);
-      tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    }
-    if (threadIdx.x == 0) {
-      base_s = b;
-      if (j == cl_ch0[c]) nact[c] = (tn <= prm->t_end) ? tot : 0;
-    }
-  }
-  __syncthreads();
+  const unsigned long long tb = s_tb;
+  if (ch_min[j] != tb) return;  // no row of this chunk
   int base = (int)off[c] + base_s;
-  __shared__ int wsum[32];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int64_t seg = lo[j]; seg < hi[j]; seg += blockDim.x) {
+  __shared__ int wsum[kSelThreads / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int64_t seg = lo[j]; seg < hi[j]; seg += kSelThreads) {
     const int64_t i = seg + threadIdx.x;
-    const bool f = (i < hi[j]) && (ti[i] + dt[i] == tn);
+    const bool f = (i < hi[j]) && (unsigned long long)__double_as_longlong(ti[i] + dt[i]) == tb;
     const unsigned bal = __ballot_sync(0xffffffffu, f);
     const int pre = __popc(bal & ((1u << lane) - 1u));
     if (lane == 0) wsum[wid] = __popc(bal);
     __syncthreads();
     int wpre = 0, tot = 0;
-    for (int w = 0; w < nw; ++w) {
+#pragma unroll
+    for (int w = 0; w < kSelThreads / 32; ++w) {
       const int cc = wsum[w];
       if (w < wid) wpre += cc;
       tot += cc;
@@ -242,33 +241,55 @@ __global__ void b_all_active(int32_t C, const int64_t* __restrict__ off, int64_t
 // The j-split length L is common to all clusters and chosen so that the whole
 // batch yields about 4 items per resident CTA.
 // ---------------------------------------------------------------------------
-__device__ int64_t block_excl_scan(int64_t v, int64_t* sh, int64_t* total) {
-  // Hillis-Steele over blockDim.x <= 1024 entries
-  const int t = threadIdx.x;
-  sh[t] = v;
-  __syncthreads();
-  for (int o = 1; o < (int)blockDim.x; o <<= 1) {
-    const int64_t add = t >= o ? sh[t - o] : 0;
-    __syncthreads();
-    sh[t] += add;
-    __syncthreads();
+constexpr int kPlanThreads = 1024;
+
+// exclusive sums over the CTA of K values a thread, and their totals: warp
+// scans by shuffles, then one warp over the 32 warps' totals (two barriers for
+// all K: the plan takes 5.7 us, 13.3 with Hillis-Steele scans in shared memory,
+// one value at a time)
+template <int K>
+__device__ __forceinline__ void block_excl_scan(int64_t (&v)[K], int64_t (&total)[K], int64_t (*sh)[K]) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int64_t in[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    in[k] = v[k];
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t u = __shfl_up_sync(0xffffffffu, in[k], o);
+      if (lane >= o) in[k] += u;
+    }
+    if (lane == 31) sh[w][k] = in[k];
   }
-  const int64_t incl = sh[t];
-  *total = sh[blockDim.x - 1];
   __syncthreads();
-  return incl - v;
+  if (w == 0) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      int64_t t = sh[lane][k];
+      for (int o = 1; o < 32; o <<= 1) {
+        const int64_t u = __shfl_up_sync(0xffffffffu, t, o);
+        if (lane >= o) t += u;
+      }
+      sh[lane][k] = t;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int64_t before = w > 0 ? sh[w - 1][k] : 0;
+    total[k] = sh[kPlanThreads / 32 - 1][k];
+    v[k] = before + in[k] - v[k];
+  }
+  __syncthreads();  // sh may be used again
 }
 
-__global__ void b_plan(int32_t C, const int64_t* __restrict__ off, const int32_t* __restrict__ nact,
-                       int per_cta, int jtile, int64_t target_items, int64_t part_cap,
-                       int32_t* __restrict__ itiles, int32_t* __restrict__ nsplit, int64_t* __restrict__ jps,
-                       int64_t* __restrict__ item_off, int64_t* __restrict__ part_off,
-                       int64_t* __restrict__ pstride, int64_t* __restrict__ ritem_off,
-                       int64_t* __restrict__ citem_off, unsigned long long* __restrict__ wq,
-                       int64_t* __restrict__ ctrl,
-                       const BParams* __restrict__ prm, nb_dev_status* __restrict__ st,
-                       cudaGraphConditionalHandle handle, int use_handle) {
-  __shared__ int64_t sh[1024];
+__global__ void __launch_bounds__(kPlanThreads) b_plan(
+    int32_t C, const int64_t* __restrict__ off, const int32_t* __restrict__ nact, int per_cta, int jtile,
+    int64_t target_items, int64_t part_cap, int32_t* __restrict__ itiles, int32_t* __restrict__ nsplit,
+    int64_t* __restrict__ jps, int64_t* __restrict__ item_off, int64_t* __restrict__ part_off,
+    int64_t* __restrict__ pstride, int64_t* __restrict__ ritem_off, int64_t* __restrict__ citem_off,
+    unsigned long long* __restrict__ wq, int64_t* __restrict__ ctrl, const BParams* __restrict__ prm,
+    nb_dev_status* __restrict__ st, cudaGraphConditionalHandle handle, int use_handle) {
+  __shared__ int64_t sh3[kPlanThreads / 32][3], sh4[kPlanThreads / 32][4];
   __shared__ int64_t s_L;
   __shared__ int s_retry;
   const int t = threadIdx.x;
@@ -282,10 +303,9 @@ __global__ void b_plan(int32_t C, const int64_t* __restrict__ off, const int32_t
     anyact += n > 0;
     inter += n * Nc;
   }
-  int64_t tot_w, tot_a, tot_i;
-  block_excl_scan(w, sh, &tot_w);
-  block_excl_scan(anyact, sh, &tot_a);
-  block_excl_scan(inter, sh, &tot_i);
+  int64_t v3[3] = {w, anyact, inter}, tot3[3];
+  block_excl_scan(v3, tot3, sh3);
+  const int64_t tot_w = tot3[0], tot_a = tot3[1], tot_i = tot3[2];
   if (t == 0) {
     int64_t L = tot_w / ((int64_t)per_cta * (target_items > 0 ? target_items : 1));
     L = ((L + jtile - 1) / jtile) * jtile;
@@ -315,28 +335,25 @@ __global__ void b_plan(int32_t C, const int64_t* __restrict__ off, const int32_t
         ps = ((n + 31) / 32) * 32;
         items = (int64_t)it * s;
         psz = s > 1 ? 7 * s * ps : 0;
-        ritems = s > 1 ? 7 * ((n + 31) / 32) : 0;
+        ritems = s > 1 ? (n + 31) / 32 : 0;
         citems = (n + kCorrItem - 1) / kCorrItem;
       }
-      int64_t tot_items, tot_part, tot_ritems, tot_citems;
-      const int64_t ex_items = block_excl_scan(items, sh, &tot_items);
-      const int64_t ex_part = block_excl_scan(psz, sh, &tot_part);
-      const int64_t ex_ritems = block_excl_scan(ritems, sh, &tot_ritems);
-      const int64_t ex_citems = block_excl_scan(citems, sh, &tot_citems);
+      int64_t ex[4] = {items, psz, ritems, citems}, tot[4];
+      block_excl_scan(ex, tot, sh4);
       if (c < C) {
         itiles[c] = it;
         nsplit[c] = ns;
         jps[c] = jp;
         pstride[c] = ps;
-        item_off[c] = item_carry + ex_items;
-        part_off[c] = part_carry + ex_part;
-        ritem_off[c] = ritem_carry + ex_ritems;
-        citem_off[c] = citem_carry + ex_citems;
+        item_off[c] = item_carry + ex[0];
+        part_off[c] = part_carry + ex[1];
+        ritem_off[c] = ritem_carry + ex[2];
+        citem_off[c] = citem_carry + ex[3];
       }
-      item_carry += tot_items;
-      part_carry += tot_part;
-      ritem_carry += tot_ritems;
-      citem_carry += tot_citems;
+      item_carry += tot[0];
+      part_carry += tot[1];
+      ritem_carry += tot[2];
+      citem_carry += tot[3];
     }
     if (t == 0) {
       item_off[C] = item_carry;
@@ -354,7 +371,7 @@ __global__ void b_plan(int32_t C, const int64_t* __restrict__ off, const int32_t
     ctrl[1] = iters;
     ctrl[2] += tot_i;
     int go = tot_a > 0;
-    if (go && (st->flags & NB_ST_STALLED)) go = 0;  // a block time did not advance (b_sel_count)
+    if (go && (st->flags & NB_ST_STALLED)) go = 0;  // a block time did not advance (b_sel_write)
     if (go && iters > prm->max_iters) {
       atomicOr(&st->flags, NB_ST_TIMEOUT);
       go = 0;
@@ -426,12 +443,19 @@ __global__ void __launch_bounds__(NB_BOX_TILE) b_predict_tiles(
 // ---------------------------------------------------------------------------
 // forces (Sec. 4.1 step 4): persistent CTAs over the flattened item list
 // ---------------------------------------------------------------------------
+// The cluster of an item: item_off[c] <= item < item_off[c + 1], by the whole
+// warp (every lane takes part with the same item): 32 probes and a ballot a
+// step, two steps up to 1024 clusters, where a binary search is a chain of ten
+// dependent loads at the head of every item.
 __device__ __forceinline__ int find_cluster(const int64_t* __restrict__ item_off, int C, int64_t item) {
+  const int lane = threadIdx.x & 31;
   int lo = 0, hi = C;  // item_off[lo] <= item < item_off[hi]
   while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (item_off[mid] <= item) lo = mid;
-    else hi = mid;
+    const int step = (hi - lo + 31) >> 5;
+    const int q = lo + lane * step;
+    const unsigned le = __ballot_sync(0xffffffffu, q < hi && item_off[q] <= item);  // lane 0's always holds
+    lo += (31 - __clz(le)) * step;
+    hi = min(hi, lo + step);
   }
   return lo;
 }
@@ -439,12 +463,14 @@ __device__ __forceinline__ int find_cluster(const int64_t* __restrict__ item_off
 // the next force item for this CTA from the step's work counter (reset by
 // b_plan): items go to whichever CTA is free first, so uneven items (near or
 // far tiles, big or small clusters) do not leave SMs idle at the end of a
-// step.  One atomic per item; no waiting.
-__device__ __forceinline__ int64_t next_item(unsigned long long* wq, int64_t* s_item) {
+// step.  One atomic per item; no waiting.  (Taken one item ahead, to hide the
+// atomic's round trip, it was 4% of a step slower: a register more, and items
+// held by busy CTAs while others were idle.)
+__device__ __forceinline__ int next_item(unsigned long long* wq, int* s_item) {
   __syncthreads();  // every thread has read the previous item
-  if (threadIdx.x == 0) *s_item = (int64_t)atomicAdd(wq, 1ULL);
+  if (threadIdx.x == 0) *s_item = (int)atomicAdd(wq, 1ULL);
   __syncthreads();
-  return *s_item;
+  return *s_item;  // (item numbers fit 32 bits: a few per active row and CTA at most)
 }
 
 // resident CTAs per SM asked of the register allocator: the host-launched
@@ -463,15 +489,14 @@ __global__ void __launch_bounds__(NT, mixed_min_ctas(NT)) b_force_mixed(
     int64_t fstride, double* __restrict__ part, const float4* __restrict__ tbox,
     const int64_t* __restrict__ tile_off, unsigned long long* __restrict__ wq) {
   __shared__ __align__(16) nbk::MixedSmem<JT> sm;
-  __shared__ int64_t s_item;
-  const int64_t total = item_off[C];
+  __shared__ int s_item;
+  const int total = (int)item_off[C];
   for (;;) {
-    const int64_t item = next_item(wq, &s_item);
+    const int item = next_item(wq, &s_item);
     if (item >= total) break;
     const int c = find_cluster(item_off, C, item);
-    const int64_t local = item - item_off[c];
-    const int it = itiles[c];
-    const int64_t itile = local % it, split = local / it;
+    const int local = item - (int)item_off[c], it = itiles[c];
+    const int64_t split = local / it, itile = local - split * it;
     const int64_t jlo = off[c] + split * jps[c];
     const int64_t jhi = min(jlo + jps[c], off[c + 1]);
     const bool fin = nsplit[c] == 1;
@@ -493,15 +518,14 @@ __global__ void __launch_bounds__(NT, 512 / NT) b_force_fp64(
     const int64_t* __restrict__ part_off, const int64_t* __restrict__ pstride, double* __restrict__ F,
     int64_t fstride, double* __restrict__ part, unsigned long long* __restrict__ wq) {
   __shared__ nbk::Fp64Smem<NT, JT> sm;
-  __shared__ int64_t s_item;
-  const int64_t total = item_off[C];
+  __shared__ int s_item;
+  const int total = (int)item_off[C];
   for (;;) {
-    const int64_t item = next_item(wq, &s_item);
+    const int item = next_item(wq, &s_item);
     if (item >= total) break;
     const int c = find_cluster(item_off, C, item);
-    const int64_t local = item - item_off[c];
-    const int it = itiles[c];
-    const int64_t itile = local % it, split = local / it;
+    const int local = item - (int)item_off[c], it = itiles[c];
+    const int64_t split = local / it, itile = local - split * it;
     const int64_t jlo = off[c] + split * jps[c];
     const int64_t jhi = min(jlo + jps[c], off[c + 1]);
     const bool fin = nsplit[c] == 1;
@@ -511,42 +535,42 @@ __global__ void __launch_bounds__(NT, 512 / NT) b_force_fp64(
   }
 }
 
-// split-j reduction of the active clusters: one item = one of the 7 result
-// rows of 32 consecutive positions of one cluster with splits (item list from
-// b_plan); block = 32 positions x kRedLanes split lanes; lane y sums splits
-// y, y + kRedLanes, ... in order and a fixed binary tree combines the lanes
-// (one summation order per split count).  Clusters with one split wrote their
-// results directly and have no items.
-#ifndef NB_ENS_RED_LANES
-#define NB_ENS_RED_LANES 8
-#endif
-constexpr int kRedLanes = NB_ENS_RED_LANES;
-__global__ void b_reduce(int32_t C, const int64_t* __restrict__ off, const int32_t* __restrict__ nact,
-                         const int32_t* __restrict__ nsplit, const int64_t* __restrict__ part_off,
-                         const int64_t* __restrict__ pstride, const int64_t* __restrict__ ritem_off,
-                         const double* __restrict__ part, double* __restrict__ F, int64_t fstride) {
-  __shared__ double sm[kRedLanes][33];
-  const int tx = threadIdx.x, ty = threadIdx.y;
+// split-j reduction of the active clusters: one item = 32 consecutive
+// positions of one cluster with splits (item list from b_plan), all 7 rows;
+// block = 32 positions x 7 rows x kRedLanes split lanes; lane z sums splits
+// z, z + kRedLanes, ... in order and lane 0 adds the lanes' sums in order (one
+// summation order per split count).  Bound by the latency of its few items a
+// CTA and by the L2 reads of the partials (20 MB a step at 240k rows in 96
+// clusters: 13 us, 16 with one row per item and a tree over 8 lanes): rows
+// side by side, the loads of four splits in flight.  Lanes: 2 are 1% of a step
+// faster than 4, 4 than 8, 16 are 7% slower.  Clusters with one split wrote
+// their results directly.
+constexpr int kRedLanes = 2;
+__global__ void __launch_bounds__(224 * kRedLanes) b_reduce(
+    int32_t C, const int64_t* __restrict__ off, const int32_t* __restrict__ nact, const int32_t* __restrict__ nsplit,
+    const int64_t* __restrict__ part_off, const int64_t* __restrict__ pstride, const int64_t* __restrict__ ritem_off,
+    const double* __restrict__ part, double* __restrict__ F, int64_t fstride) {
+  __shared__ double sm[kRedLanes][7][32];
+  const int tx = threadIdx.x, r = threadIdx.y, z = threadIdx.z;
   const int64_t total = ritem_off[C];
   for (int64_t item = blockIdx.x; item < total; item += gridDim.x) {
     const int c = find_cluster(ritem_off, C, item);
     const int S = nsplit[c];
-    const int64_t n = nact[c], o = off[c], ps = pstride[c];
-    const double* p = part + part_off[c];
-    const int64_t local = item - ritem_off[c];
-    const int r = (int)(local % 7);
-    const int64_t k = (local / 7) * 32 + tx;
+    const int64_t ps = pstride[c], k = (item - ritem_off[c]) * 32 + tx;
+    const bool in = k < nact[c];
+    const double* p = part + part_off[c] + r * ps + k;
     double acc = 0.0;
-    if (k < n)
-      for (int q = ty; q < S; q += kRedLanes) acc += p[((int64_t)q * 7 + r) * ps + k];
-    sm[ty][tx] = acc;
+    if (in)
+#pragma unroll 4
+      for (int q = z; q < S; q += kRedLanes) acc += p[(int64_t)q * 7 * ps];
+    sm[z][r][tx] = acc;
     __syncthreads();
+    if (z == 0 && in) {
 #pragma unroll
-    for (int h = kRedLanes / 2; h > 0; h >>= 1) {
-      if (ty < h) sm[ty][tx] += sm[ty + h][tx];
-      __syncthreads();
+      for (int q = 1; q < kRedLanes; ++q)
+        if (q < S) acc += sm[q][r][tx];
+      F[r * fstride + off[c] + k] = r == 6 ? -acc : acc;
     }
-    if (ty == 0 && k < n) F[r * fstride + o + k] = r == 6 ? -sm[0][tx] : sm[0][tx];
     __syncthreads();
   }
 }
@@ -614,19 +638,32 @@ __global__ void b_correct(int32_t C, int64_t n_pad, const int64_t* __restrict__ 
                           double* __restrict__ dt, const double* __restrict__ xp,
                           const double* __restrict__ vp, nb_dev_status* __restrict__ st) {
   const double eta = prm->eta, dt_min = prm->dt_min, dt_max = prm->dt_max;
-  // items of kCorrItem active particles of one cluster (planned by b_plan)
+  // items of kCorrItem active particles of one cluster (planned by b_plan),
+  // four lanes per particle: one thread's FP64 chain is the kernel's time
+  // when the blocks do not fill the SMs (a step of 16 small clusters: 47 us
+  // against 50 with one thread per particle), and level when they do
+  const int lane = threadIdx.x & 31, sub = lane & 3;
   const int64_t total = citem_off[C];
   for (int64_t item = blockIdx.x; item < total; item += gridDim.x) {
     const int c = find_cluster(citem_off, C, item);
-    const int64_t k = (item - citem_off[c]) * kCorrItem + threadIdx.x;
-    if (k >= nact[c]) continue;
+    const int64_t k = (item - citem_off[c]) * kCorrItem + (threadIdx.x >> 2);
+    const bool in = k < nact[c];
+    if (__all_sync(0xffffffffu, !in)) continue;
     const int64_t s = off[c] + k;
-    int64_t i = act[s];
+    int64_t i = in ? act[s] : 0;
     i = i < 0 ? 0 : (i >= n_pad ? n_pad - 1 : i);
-    double f[7];
-#pragma unroll
-    for (int r = 0; r < 7; ++r) f[r] = F[r * fstride + s];
-    nbh::correct_row(i, n_pad, tnext[c], f, eta, dt_min, dt_max, x, v, a, jk, pot, ti, dt, xp, vp, st);
+    nbh::CorrIn ci{};
+    double a1 = 0.0, j1 = 0.0, p1 = 0.0;
+    if (in) {
+      const int r = sub < 3 ? sub : 0;
+      const int64_t q = r * n_pad + i;
+      ci = nbh::CorrIn{ti[i], dt[i], a[q], jk[q], xp[q], vp[q]};
+      a1 = F[r * fstride + s];
+      j1 = F[(3 + r) * fstride + s];
+      p1 = F[6 * fstride + s];
+    }
+    nbh::correct_lanes4(i, n_pad, tnext[c], a1, j1, p1, ci, eta, dt_min, dt_max, x, v, a, jk, pot, ti, dt, st, sub,
+                        lane & ~3, in);
   }
 }
 
@@ -861,7 +898,7 @@ cudaError_t plan_only(nb_ctx* c, Batch* b) {
   const int per_cta = b->nt * (mixed ? kMixIPT : 1);
   const int jt = mixed ? kMixJT : kF64JT;
   const int grid = mixed ? b->grid_mixed : b->grid_fp64;
-  b_plan<<<1, 1024, 0, c->stream>>>(b->C, b->off, b->nact, per_cta, jt, b->waves * (int64_t)grid, c->part_elems,
+  b_plan<<<1, kPlanThreads, 0, c->stream>>>(b->C, b->off, b->nact, per_cta, jt, b->waves * (int64_t)grid, c->part_elems,
                                     b->itiles, b->nsplit, b->jps, b->item_off, b->part_off, b->pstride,
                                     b->ritem_off, b->citem_off, b->wq, b->ctrl,
                                     b->prm, c->status, 0, 0);
@@ -912,7 +949,7 @@ cudaError_t body_after_plan(nb_ctx* c, Batch* b, bool own_time) {
     launch_force<64>(c, b, mixed);
   else
     launch_force<128>(c, b, mixed);
-  b_reduce<<<c->sm_count * 8, dim3(32, kRedLanes), 0, c->stream>>>(
+  b_reduce<<<c->sm_count * std::max(1, 2048 / (224 * kRedLanes)), dim3(32, 7, kRedLanes), 0, c->stream>>>(
       b->C, b->off, b->nact, b->nsplit, b->part_off, b->pstride, b->ritem_off, c->part, c->F, c->n_pad);
   c->launches += 3;
   return cudaGetLastError();
@@ -924,22 +961,21 @@ cudaError_t capture_step(nb_ctx* c, Batch* b, cudaGraphConditionalHandle handle,
   const int per_cta = b->nt * (mixed ? kMixIPT : 1);
   const int jt = mixed ? kMixJT : kF64JT;
   const int grid = mixed ? b->grid_mixed : b->grid_fp64;
-  b_sel_min<<<b->nchunks, 256, 0, c->stream>>>(b->ch_lo, b->ch_hi, c->t, c->dt, b->ch_min);
-  b_sel_count<<<b->nchunks, 256, 0, c->stream>>>(b->ch_cluster, b->ch_lo, b->ch_hi, b->cl_ch0, b->ch_min, c->t,
-                                                 c->dt, b->tnext, b->ch_cnt, b->ctrl, b->prm, c->status);
-  b_sel_write<<<b->nchunks, 256, 0, c->stream>>>(b->ch_cluster, b->ch_lo, b->ch_hi, b->cl_ch0, b->ch_cnt, b->off,
-                                                 c->t, c->dt, b->tnext, b->prm, c->act, b->nact);
-  b_plan<<<1, 1024, 0, c->stream>>>(b->C, b->off, b->nact, per_cta, jt, b->waves * (int64_t)grid, c->part_elems,
+  b_sel_min<<<b->nchunks, kSelThreads, 0, c->stream>>>(b->ch_lo, b->ch_hi, c->t, c->dt, b->ch_min, b->ch_cnt);
+  b_sel_write<<<b->nchunks, kSelThreads, 0, c->stream>>>(b->ch_cluster, b->ch_lo, b->ch_hi, b->cl_ch0, b->ch_min,
+                                                         b->ch_cnt, b->off, c->t, c->dt, b->tnext, b->ctrl, b->prm,
+                                                         c->act, b->nact, c->status);
+  b_plan<<<1, kPlanThreads, 0, c->stream>>>(b->C, b->off, b->nact, per_cta, jt, b->waves * (int64_t)grid, c->part_elems,
                                     b->itiles, b->nsplit, b->jps, b->item_off, b->part_off, b->pstride,
                                     b->ritem_off, b->citem_off, b->wq, b->ctrl,
                                     b->prm, c->status, handle, use_handle);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if ((e = body_after_plan(c, b, false)) != cudaSuccess) return e;
-  b_correct<<<c->sm_count * 16, kCorrItem, 0, c->stream>>>(b->C, c->n_pad, b->citem_off, b->off, b->nact, b->tnext,
+  b_correct<<<c->sm_count * 16, 4 * kCorrItem, 0, c->stream>>>(b->C, c->n_pad, b->citem_off, b->off, b->nact, b->tnext,
                                                            c->act, c->F, c->n_pad, b->prm, c->x, c->v, c->a, c->jk,
                                                            c->pot, c->t, c->dt, c->xp, c->vp, c->status);
-  c->launches += 5;
+  c->launches += 4;
   return cudaGetLastError();
 }
 
@@ -1043,7 +1079,7 @@ int run_graph(nb_ctx* c, Batch* b, double t_end) {
     c->steps += steps;
     c->perm_age += (int)steps;
     c->interactions += (double)inter;
-    c->launches += iters * 8;
+    c->launches += iters * 7;
     total += iters;
     if (!more) break;
     if (total > cap) return NB_ETIMEOUT;  // cannot happen for valid block steps

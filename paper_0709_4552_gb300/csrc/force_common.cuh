@@ -494,7 +494,7 @@ __device__ __forceinline__ void mixed_item(SM& sm, const float4* __restrict__ jA
     acc_lo[k][c] += (a_ - (s_ - bb_)) + (b_ - bb_);             \
     acc_hi[k][c] = s_;                                          \
   } while (0)
-#define NB_ACC_GET(k, c) ((double)acc_hi[k][c] + (double)acc_lo[k][c])
+#define NB_ACC_GET(k, c) (nb_f64(acc_hi[k][c]) + nb_f64(acc_lo[k][c]))
 #define NB_ACC_DS(k, c) make_float2(acc_hi[k][c], acc_lo[k][c])
 #else
 #define NB_ACC_ZERO(k, c) (NB_ACC(k, c) = 0.0)
