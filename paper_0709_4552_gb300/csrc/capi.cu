@@ -488,7 +488,7 @@ int nb_create(nb_ctx** out, int64_t n_max, int precision, int device, void* cuda
   NB_ALLOC(c->sel_min, (size_t)c->sel_ctas + 1) NB_ALLOC(c->sel_cnt, (size_t)c->sel_ctas + 1)
   NB_ALLOC(c->red, NB_RED_DOUBLES) NB_ALLOC(c->status, 1)
   NB_ALLOC(c->perm, np) NB_ALLOC(c->iperm, np) NB_ALLOC(c->skey[0], np) NB_ALLOC(c->skey[1], np)
-  NB_ALLOC(c->sval[0], np) NB_ALLOC(c->sval[1], np) NB_ALLOC(c->shist, (np / 2048 + 1) * 256)
+  NB_ALLOC(c->sval[0], np) NB_ALLOC(c->sval[1], np) NB_ALLOC(c->shist, nb_sort_hist_ints(np))
   NB_ALLOC(c->tbox, 2 * (np / NB_BOX_TILE + 1))
 #undef NB_ALLOC
   if (e == cudaSuccess) e = cudaMallocHost(&c->hpin, kPinnedBytes);

@@ -268,13 +268,22 @@ __global__ void energy_partial_kernel(int64_t N, int64_t n_pad, const double* __
   }
 }
 
+// the partial energies summed by one warp: lane l takes partials l, l + 32, ...
+// and a butterfly adds the lanes (two FP64 sums a partial on one thread were 17
+// us at N = 32768, up to 60 for the largest states: an FP64 addition holds its
+// warp for 64 cycles)
 __global__ void energy_final_kernel(int nb, const double* __restrict__ red, double* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double k = 0.0, w = 0.0;
-    for (int b = 0; b < nb; ++b) {
-      k += red[2 * b];
-      w += red[2 * b + 1];
-    }
+  double k = 0.0, w = 0.0;
+#pragma unroll 4
+  for (int b = threadIdx.x; b < nb; b += 32) {
+    k += red[2 * b];
+    w += red[2 * b + 1];
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    k += __shfl_xor_sync(0xffffffffu, k, o);
+    w += __shfl_xor_sync(0xffffffffu, w, o);
+  }
+  if (threadIdx.x == 0) {
     out[0] = k;
     out[1] = w;
   }

@@ -35,8 +35,7 @@
 #define NB_JPAD 1024          // j-store padding granule (max j-tile)
 #define NB_PAD_POS 1.0e15     // position of padding particles (m = 0)
 #define NB_BOX_TILE 128       // j-tile of the spatial boxes (the mixed default j-tile)
-#define NB_RED_DOUBLES (8192 + 16)  // reduction scratch: partials, energies, bounding box
-#define NB_BBOX_OFFSET 8192         // 6 doubles of the particles' bounding box
+#define NB_RED_DOUBLES 8192         // reduction scratch: partials, energies, bounding boxes
 
 // device status word bits
 #define NB_ST_NUMERIC 1u
@@ -237,6 +236,7 @@ cudaError_t nb_forces(nb_ctx* c, const int32_t* d_list, int64_t n);
 
 // spatial.cu
 cudaError_t nb_spatial_sort(nb_ctx* c);       // new resident order from the current positions
+size_t nb_sort_hist_ints(int64_t n);  // ints of shist
 // new resident order: rows stably sorted by skey[0] (low `bits` bits), sval[0] = row numbers
 cudaError_t nb_order_rows_by_keys(nb_ctx* c, int bits);
 cudaError_t nb_unsort(nb_ctx* c);             // back to particle order (perm_valid = false)

@@ -12,164 +12,255 @@
 // the same pairs.
 //
 // nb_spatial_sort: bounding box -> 30-bit Morton keys on a 1024^3 grid ->
-// stable least-significant-digit radix sort (4 passes of 8 bits; per-block
-// digit histograms, one scan, stable scatter ranked with warp match) -> the
-// rows gathered into a scratch block and copied back, perm composed and
-// inverted.  Deterministic.
+// stable least-significant-digit radix sort (4 passes of 8 bits, ranked with
+// warp match) -> the rows gathered into a scratch block and copied back, with
+// perm composed and inverted on the way.  Deterministic.
+//
+// A block-step run sorts every 64 steps, so at 10^4 rows the sort is a chain of
+// small kernels, each the latency of its launch and a few dependent steps.
+// Hence few kernels (9 up to 131072 rows, 16 above; as bounding box, keys and
+// count / scan / scatter per pass it was 19 and a copy) and short chains.
+// Time: 12000 rows 139 -> 47 us, 32768 rows 155 -> 55 us; at 2^20 rows, where
+// one CTA's scan of all histograms was 4 x 205 us, 1125 -> 384 us.
 #include <float.h>
+
+#include <algorithm>
 
 #include "nb_internal.cuh"
 
 namespace {
 
 constexpr int kSortThreads = 256;
-constexpr int kSortItems = 8;                          // elements per thread per block
-constexpr int kSortChunk = kSortThreads * kSortItems;  // 2048 elements per block
 constexpr int kRadix = 256;
+static_assert(kSortThreads == kRadix, "thread = digit in the scatter");
+constexpr int kSortWarps = kSortThreads / 32;
+// elements per thread: short chunks while they still leave the chip mostly
+// idle, long ones (longer runs of equal digits to write) above
+constexpr int kItemsSmall = 2, kItemsLarge = 8;
+constexpr int64_t kSmallRows = 32768;
+// up to this many chunks a scatter CTA adds up the chunks' histograms itself
+// (64 coalesced rows, batched) and counts the next pass's digits as it writes:
+// one kernel a pass; above, a count and a prefix kernel before each scatter
+constexpr int kFusedChunks = 64;
 
-__global__ void bbox_partial(int64_t N, int64_t n_pad, const double* __restrict__ x, double* __restrict__ red) {
-  double lo[3] = {DBL_MAX, DBL_MAX, DBL_MAX}, hi[3] = {-DBL_MAX, -DBL_MAX, -DBL_MAX};
+// doubles as integers of the same order (min and max without the FP64 unit)
+__device__ __forceinline__ long long ord_of(double x) {
+  const long long b = __double_as_longlong(x);
+  return b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFLL);
+}
+__device__ __forceinline__ double of_ord(long long o) {
+  return __longlong_as_double(o ^ ((o >> 63) & 0x7FFFFFFFFFFFFFFFLL));
+}
+
+// minima b[0..2] and maxima b[3..5] over the CTA; valid on threads 0-5, the
+// value of component threadIdx.x
+__device__ __forceinline__ long long bbox_reduce(const long long (&in)[6], long long (*sm)[6]) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    long long v = in[c];
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long u = __shfl_xor_sync(0xffffffffu, v, o);
+      v = c < 3 ? min(u, v) : max(u, v);
+    }
+    if (lane == 0) sm[w][c] = v;
+  }
+  __syncthreads();
+  long long r = 0;
+  if (threadIdx.x < 6) {
+    r = sm[0][threadIdx.x];
+    for (int q = 1; q < kSortWarps; ++q)
+      r = threadIdx.x < 3 ? min(r, sm[q][threadIdx.x]) : max(r, sm[q][threadIdx.x]);
+  }
+  return r;
+}
+
+__device__ __forceinline__ void bbox_start(long long (&b)[6]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    b[c] = ord_of(DBL_MAX);
+    b[3 + c] = ord_of(-DBL_MAX);
+  }
+}
+
+__global__ void __launch_bounds__(kSortThreads) bbox_partial(int64_t N, int64_t n_pad, const double* __restrict__ x,
+                                                             long long* __restrict__ red) {
+  long long b[6];
+  bbox_start(b);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
+#pragma unroll
     for (int c = 0; c < 3; ++c) {
       const double v = x[c * n_pad + i];
-      lo[c] = fmin(lo[c], v);
-      hi[c] = fmax(hi[c], v);
+      if (isnan(v)) continue;
+      b[c] = min(b[c], ord_of(v));
+      b[3 + c] = max(b[3 + c], ord_of(v));
     }
-  __shared__ double s[6][kSortThreads];
-  for (int c = 0; c < 3; ++c) {
-    s[c][threadIdx.x] = lo[c];
-    s[3 + c][threadIdx.x] = hi[c];
-  }
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w)
-      for (int c = 0; c < 3; ++c) {
-        s[c][threadIdx.x] = fmin(s[c][threadIdx.x], s[c][threadIdx.x + w]);
-        s[3 + c][threadIdx.x] = fmax(s[3 + c][threadIdx.x], s[3 + c][threadIdx.x + w]);
-      }
-    __syncthreads();
-  }
-  if (threadIdx.x < 6) red[blockIdx.x * 6 + threadIdx.x] = s[threadIdx.x][0];
+  __shared__ long long sm[kSortWarps][6];
+  const long long r = bbox_reduce(b, sm);
+  if (threadIdx.x < 6) red[blockIdx.x * 6 + threadIdx.x] = r;
 }
 
-// one CTA of kSortThreads: strided partial minima/maxima, then a tree (min
-// and max are exact, so the order does not matter)
-__global__ void bbox_final(int nb, const double* __restrict__ red, double* __restrict__ out) {
-  double b[6] = {DBL_MAX, DBL_MAX, DBL_MAX, -DBL_MAX, -DBL_MAX, -DBL_MAX};
-  for (int k = threadIdx.x; k < nb; k += blockDim.x)
-    for (int c = 0; c < 3; ++c) {
-      b[c] = fmin(b[c], red[k * 6 + c]);
-      b[3 + c] = fmax(b[3 + c], red[k * 6 + 3 + c]);
+// keys on the grid of the box of the nb partial boxes, which every CTA reduces
+// for itself
+__global__ void __launch_bounds__(kSortThreads) morton_keys(int64_t N, int64_t n_pad, const double* __restrict__ x,
+                                                            int nb, const long long* __restrict__ red,
+                                                            uint32_t* __restrict__ key, int32_t* __restrict__ val) {
+  __shared__ long long sm[kSortWarps][6];
+  __shared__ double box[6], s_scale;
+  long long b[6];
+  bbox_start(b);
+  for (int k = threadIdx.x; k < nb; k += kSortThreads)
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      const long long v = red[k * 6 + c];
+      b[c] = c < 3 ? min(b[c], v) : max(b[c], v);
     }
-  __shared__ double s[6][kSortThreads];
-  for (int c = 0; c < 6; ++c) s[c][threadIdx.x] = b[c];
+  const long long r = bbox_reduce(b, sm);
+  if (threadIdx.x < 6) box[threadIdx.x] = of_ord(r);
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w)
-      for (int c = 0; c < 3; ++c) {
-        s[c][threadIdx.x] = fmin(s[c][threadIdx.x], s[c][threadIdx.x + w]);
-        s[3 + c][threadIdx.x] = fmax(s[3 + c][threadIdx.x], s[3 + c][threadIdx.x + w]);
-      }
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    const double w = fmax(box[3] - box[0], fmax(box[4] - box[1], box[5] - box[2]));
+    s_scale = w > 0.0 ? 1023.0 / w : 0.0;
   }
-  if (threadIdx.x < 6) out[threadIdx.x] = s[threadIdx.x][0];
-}
-
-__global__ void morton_keys(int64_t N, int64_t n_pad, const double* __restrict__ x, const double* __restrict__ box,
-                            uint32_t* __restrict__ key, int32_t* __restrict__ val) {
-  double scale = fmax(box[3] - box[0], fmax(box[4] - box[1], box[5] - box[2]));
-  scale = scale > 0.0 ? 1023.0 / scale : 0.0;
+  __syncthreads();
+  const double scale = s_scale;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
     uint32_t q[3];
-    for (int c = 0; c < 3; ++c) {
-      double f = (x[c * n_pad + i] - box[c]) * scale;
-      f = f < 0.0 ? 0.0 : (f > 1023.0 ? 1023.0 : f);
-      q[c] = (uint32_t)f;
-    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c)  // (the conversion saturates: below the grid, or NaN, is 0)
+      q[c] = min(__double2uint_rz((x[c * n_pad + i] - box[c]) * scale), 1023u);
     key[i] = nb_spread10(q[0]) | (nb_spread10(q[1]) << 1) | (nb_spread10(q[2]) << 2);
     val[i] = (int32_t)i;
   }
 }
 
-__global__ void radix_count(const uint32_t* __restrict__ key, int64_t N, int shift, int32_t* __restrict__ hist,
-                            int nblocks) {
+// hist[chunk][digit] of one pass; with zero: the histograms of `zero` more
+// passes cleared (they follow, gridDim.x chunks each)
+template <int K>
+__global__ void __launch_bounds__(kSortThreads) radix_count(const uint32_t* __restrict__ key, int64_t N, int shift,
+                                                            int32_t* __restrict__ hist, int zero) {
   __shared__ int cnt[kRadix];
-  for (int d = threadIdx.x; d < kRadix; d += blockDim.x) cnt[d] = 0;
+  cnt[threadIdx.x] = 0;
   __syncthreads();
-  const int64_t base = (int64_t)blockIdx.x * kSortChunk;
-  for (int it = 0; it < kSortItems; ++it) {
+  const int64_t base = (int64_t)blockIdx.x * (K * kSortThreads);
+#pragma unroll
+  for (int it = 0; it < K; ++it) {
     const int64_t e = base + it * kSortThreads + threadIdx.x;
     if (e < N) atomicAdd(&cnt[(key[e] >> shift) & 0xFFu], 1);
   }
   __syncthreads();
-  for (int d = threadIdx.x; d < kRadix; d += blockDim.x) hist[(int64_t)d * nblocks + blockIdx.x] = cnt[d];
+  const int64_t at = (int64_t)blockIdx.x * kRadix + threadIdx.x;
+  hist[at] = cnt[threadIdx.x];
+  for (int q = 1; q <= zero; ++q) hist[(int64_t)q * gridDim.x * kRadix + at] = 0;
 }
 
-// exclusive scan of n ints in one CTA of 1024 threads
-__global__ void scan_exclusive(int32_t* __restrict__ a, int64_t n) {
-  __shared__ int32_t s[1024];
-  __shared__ int32_t carry;
-  if (threadIdx.x == 0) carry = 0;
+// each digit's counts over the chunks -> exclusive prefixes in place, and the
+// digit's total; a CTA takes 8 digits (a 32-byte sector of a row), its threads
+// 128 runs of chunks
+constexpr int kPrefixRuns = 128;
+__global__ void __launch_bounds__(8 * kPrefixRuns) radix_prefix(int32_t* __restrict__ hist, int nblocks,
+                                                                int32_t* __restrict__ tot) {
+  __shared__ int32_t sm[kPrefixRuns][8];
+  const int d = threadIdx.x & 7, run = threadIdx.x >> 3;
+  const int per = (nblocks + kPrefixRuns - 1) / kPrefixRuns;
+  const int q0 = min(run * per, nblocks), q1 = min(q0 + per, nblocks);
+  int32_t* h = hist + blockIdx.x * 8 + d;
+  int32_t sum = 0;
+#pragma unroll 4
+  for (int q = q0; q < q1; ++q) sum += h[(int64_t)q * kRadix];
+  sm[run][d] = sum;
   __syncthreads();
-  for (int64_t b0 = 0; b0 < n; b0 += 1024) {
-    const int64_t i = b0 + threadIdx.x;
-    const int32_t v = i < n ? a[i] : 0;
-    s[threadIdx.x] = v;
+  for (int o = 1; o < kPrefixRuns; o <<= 1) {
+    const int32_t u = run >= o ? sm[run - o][d] : 0;
     __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-      const int32_t add = (int)threadIdx.x >= o ? s[threadIdx.x - o] : 0;
-      __syncthreads();
-      s[threadIdx.x] += add;
-      __syncthreads();
-    }
-    if (i < n) a[i] = carry + s[threadIdx.x] - v;
+    sm[run][d] += u;
     __syncthreads();
-    if (threadIdx.x == 1023) carry += s[1023];
-    __syncthreads();
+  }
+  int32_t at = sm[run][d] - sum;
+  if (run == kPrefixRuns - 1) tot[blockIdx.x * 8 + d] = sm[run][d];
+#pragma unroll 4
+  for (int q = q0; q < q1; ++q) {
+    const int32_t v = h[(int64_t)q * kRadix];
+    h[(int64_t)q * kRadix] = at;
+    at += v;
   }
 }
 
-// stable scatter: elements of a block keep their order among equal digits
-__global__ void radix_scatter(const uint32_t* __restrict__ kin, const int32_t* __restrict__ vin,
-                              uint32_t* __restrict__ kout, int32_t* __restrict__ vout, int64_t N, int shift,
-                              const int32_t* __restrict__ hist, int nblocks) {
-  constexpr int kWarps = kSortThreads / 32;
-  __shared__ int32_t base[kRadix];
-  __shared__ int32_t wcnt[kWarps][kRadix];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int d = threadIdx.x; d < kRadix; d += blockDim.x) base[d] = hist[(int64_t)d * nblocks + blockIdx.x];
-  const int64_t chunk = (int64_t)blockIdx.x * kSortChunk;
-  for (int it = 0; it < kSortItems; ++it) {
-    for (int q = threadIdx.x; q < kWarps * kRadix; q += blockDim.x) (&wcnt[0][0])[q] = 0;
-    __syncthreads();
-    const int64_t e = chunk + it * kSortThreads + threadIdx.x;
-    const bool valid = e < N;
-    const uint32_t k = valid ? kin[e] : 0u;
-    const int digit = valid ? (int)((k >> shift) & 0xFFu) : kRadix;  // kRadix: no element
+// Stable scatter of one chunk by one digit.  A warp owns 32 K consecutive
+// elements and ranks them 32 at a time against its own running counts, so the
+// CTA meets three times in all, whatever K.  FUSED: hist holds the chunks'
+// counts, which thread d adds up for digit d, and next (if any) receives the
+// next pass's; else hist holds exclusive prefixes and tot the digits' totals.
+template <int K, bool FUSED>
+__global__ void __launch_bounds__(kSortThreads) radix_scatter(
+    const uint32_t* __restrict__ kin, const int32_t* __restrict__ vin, uint32_t* __restrict__ kout,
+    int32_t* __restrict__ vout, int64_t N, int shift, const int32_t* __restrict__ hist,
+    const int32_t* __restrict__ tot, int32_t* __restrict__ next) {
+  constexpr int kChunk = K * kSortThreads;
+  __shared__ int32_t at[kSortWarps][kRadix];  // counts, then first places, by warp and digit
+  __shared__ int32_t wsum[kSortWarps];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int64_t first = (int64_t)blockIdx.x * kChunk + wid * (32 * K) + lane;
+  uint32_t k[K];
+  int32_t v[K];
+#pragma unroll
+  for (int it = 0; it < K; ++it) {
+    const int64_t e = first + it * 32;
+    k[it] = e < N ? kin[e] : 0u;
+    v[it] = e < N ? vin[e] : 0;
+  }
+  int32_t before = 0, total = 0;
+  if (FUSED) {
+#pragma unroll 8
+    for (int q = 0; q < (int)gridDim.x; ++q) {
+      const int32_t h = hist[q * kRadix + tid];
+      total += h;
+      before += q < (int)blockIdx.x ? h : 0;
+    }
+  } else {
+    before = hist[(int64_t)blockIdx.x * kRadix + tid];
+    total = tot[tid];
+  }
+  int32_t incl = total;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
+  }
+  if (lane == 31) wsum[wid] = incl;
+#pragma unroll
+  for (int w = 0; w < kSortWarps; ++w) at[w][tid] = 0;
+  __syncthreads();
+  int32_t place = incl - total + before;  // of the chunk's first element of digit tid
+  for (int w = 0; w < wid; ++w) place += wsum[w];
+  int rank[K];
+#pragma unroll
+  for (int it = 0; it < K; ++it) {
+    const bool valid = first + it * 32 < N;
+    const int digit = valid ? (int)((k[it] >> shift) & 0xFFu) : kRadix;  // kRadix: no element
     const unsigned peers = __match_any_sync(0xffffffffu, digit);
-    const int rank = __popc(peers & ((1u << lane) - 1u));
-    if (valid && rank == 0) wcnt[wid][digit] = __popc(peers);
-    __syncthreads();
-    if (valid) {
-      int off = 0;
-      for (int w = 0; w < wid; ++w) off += wcnt[w][digit];
-      const int64_t pos = (int64_t)base[digit] + off + rank;
-      kout[pos] = k;
-      vout[pos] = vin[e];
-    }
-    __syncthreads();
-    for (int d = threadIdx.x; d < kRadix; d += blockDim.x) {
-      int t = 0;
-      for (int w = 0; w < kWarps; ++w) t += wcnt[w][d];
-      base[d] += t;
-    }
-    __syncthreads();
+    const int lower = __popc(peers & ((1u << lane) - 1u));
+    const int c = valid ? at[wid][digit] : 0;
+    rank[it] = c + lower;
+    __syncwarp();
+    if (valid && lower == 0) at[wid][digit] = c + __popc(peers);
+    __syncwarp();
   }
-}
-
-__global__ void invert_perm(int64_t N, const int32_t* __restrict__ perm, int32_t* __restrict__ iperm) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x)
-    iperm[perm[k]] = (int32_t)k;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kSortWarps; ++w) {
+    const int32_t c = at[w][tid];
+    at[w][tid] = place;
+    place += c;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int it = 0; it < K; ++it)
+    if (first + it * 32 < N) {
+      const int32_t pos = at[wid][(k[it] >> shift) & 0xFFu] + rank[it];
+      kout[pos] = k[it];
+      vout[pos] = v[it];
+      if (FUSED && next) atomicAdd(&next[(pos / kChunk) * kRadix + ((k[it] >> (shift + 8)) & 0xFFu)], 1);
+    }
 }
 
 int grid_for(int64_t n, int threads, int cap) {
@@ -245,27 +336,32 @@ StateRows state_rows(nb_ctx* c) {
   return r;
 }
 
-// scratch[q][s] = row_q[src[s]] for s < N (a gather of every state row)
+// scratch[q][s] = row_q[src[s]] for s < N (a gather of every state row); with
+// order: order[s] = particle of the new row s (old row src[s] holds particle
+// perm[src[s]], or src[s] when perm is null), and its inverse
 __global__ void gather_state(int64_t N, int64_t n_pad, StateRows rows, const int32_t* __restrict__ src,
-                             double* __restrict__ scratch) {
+                             double* __restrict__ scratch, const int32_t* __restrict__ perm,
+                             int32_t* __restrict__ order, int32_t* __restrict__ inverse) {
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < N; s += (int64_t)gridDim.x * blockDim.x) {
     const int64_t from = src[s];
+    if (order) {
+      const int32_t particle = perm ? perm[from] : (int32_t)from;
+      order[s] = particle;
+      inverse[particle] = (int32_t)s;
+    }
 #pragma unroll
     for (int q = 0; q < kStateRows; ++q) scratch[q * n_pad + s] = rows.row[q][from];
   }
 }
 
-__global__ void copy_state_back(int64_t N, int64_t n_pad, StateRows rows, const double* __restrict__ scratch) {
-  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < N; s += (int64_t)gridDim.x * blockDim.x)
+// the gathered rows, and the order, to their places
+__global__ void copy_state_back(int64_t N, int64_t n_pad, StateRows rows, const double* __restrict__ scratch,
+                                const int32_t* __restrict__ order, int32_t* __restrict__ perm) {
+  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < N; s += (int64_t)gridDim.x * blockDim.x) {
+    if (order) perm[s] = order[s];
 #pragma unroll
     for (int q = 0; q < kStateRows; ++q) rows.row[q][s] = scratch[q * n_pad + s];
-}
-
-// out[s] = a[b[s]] (composition of two orders), or b[s] when a is null
-__global__ void compose(int64_t N, const int32_t* __restrict__ a, const int32_t* __restrict__ b,
-                        int32_t* __restrict__ out) {
-  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < N; s += (int64_t)gridDim.x * blockDim.x)
-    out[s] = a ? a[b[s]] : b[s];
+  }
 }
 
 // out[k] = map[in[k]] with in[k] clamped to [0, N) (in == out allowed)
@@ -301,8 +397,9 @@ __global__ void gather_rows(const double* __restrict__ src, int rows, int64_t n_
   }
 }
 
-// reorder every state row by src (new row s = old row src[s]) in place
-cudaError_t reorder_state(nb_ctx* c, const int32_t* src) {
+// reorder every state row by src (new row s = old row src[s]) in place; with
+// order (scratch of N): perm and iperm too
+cudaError_t reorder_state(nb_ctx* c, const int32_t* src, int32_t* order) {
   c->state_ver++;  // rows move: any row-keyed copy of the state (the j-memory) is stale
   if (!c->pscratch) {
     cudaError_t e = cudaMalloc(&c->pscratch, (size_t)kStateRows * c->n_pad * sizeof(double));
@@ -313,24 +410,40 @@ cudaError_t reorder_state(nb_ctx* c, const int32_t* src) {
   }
   const StateRows rows = state_rows(c);
   const int g = grid_for(c->n, 256, c->sm_count * 16);
-  gather_state<<<g, 256, 0, c->stream>>>(c->n, c->n_pad, rows, src, c->pscratch);
-  copy_state_back<<<g, 256, 0, c->stream>>>(c->n, c->n_pad, rows, c->pscratch);
+  gather_state<<<g, 256, 0, c->stream>>>(c->n, c->n_pad, rows, src, c->pscratch, c->perm_valid ? c->perm : nullptr,
+                                         order, c->iperm);
+  copy_state_back<<<g, 256, 0, c->stream>>>(c->n, c->n_pad, rows, c->pscratch, order, c->perm);
   c->launches += 2;
   return cudaGetLastError();
 }
 
 // stable LSD radix sort of (skey[0], sval[0])[0..n) on the low `bits` bits;
 // *cur = the buffer holding the result
+template <int K>
 cudaError_t sort_pairs(nb_ctx* c, int64_t n, int bits, int* cur) {
-  const int nblocks = (int)((n + kSortChunk - 1) / kSortChunk);
+  const int64_t chunk = K * kSortThreads;
+  const int nblocks = (int)((n + chunk - 1) / chunk), passes = (bits + 7) / 8;
+  const bool fused = nblocks <= kFusedChunks;
+  const int64_t histogram = (int64_t)nblocks * kRadix;
+  int32_t* tot = c->shist + histogram;  // (unfused: one histogram)
   int b = 0;
-  for (int shift = 0; shift < bits; shift += 8) {
-    radix_count<<<nblocks, kSortThreads, 0, c->stream>>>(c->skey[b], n, shift, c->shist, nblocks);
-    scan_exclusive<<<1, 1024, 0, c->stream>>>(c->shist, (int64_t)nblocks * kRadix);
-    radix_scatter<<<nblocks, kSortThreads, 0, c->stream>>>(c->skey[b], c->sval[b], c->skey[b ^ 1], c->sval[b ^ 1],
-                                                           n, shift, c->shist, nblocks);
-    b ^= 1;
-    c->launches += 3;
+  for (int p = 0; p < passes; ++p, b ^= 1) {
+    int32_t* hist = c->shist + (fused ? p * histogram : 0);
+    if (p == 0 || !fused) {
+      radix_count<K><<<nblocks, kSortThreads, 0, c->stream>>>(c->skey[b], n, 8 * p, hist, fused ? passes - 1 : 0);
+      c->launches += 1;
+    }
+    if (fused) {
+      radix_scatter<K, true><<<nblocks, kSortThreads, 0, c->stream>>>(
+          c->skey[b], c->sval[b], c->skey[b ^ 1], c->sval[b ^ 1], n, 8 * p, hist, nullptr,
+          p + 1 < passes ? hist + histogram : nullptr);
+    } else {
+      radix_prefix<<<kRadix / 8, 8 * kPrefixRuns, 0, c->stream>>>(hist, nblocks, tot);
+      radix_scatter<K, false><<<nblocks, kSortThreads, 0, c->stream>>>(
+          c->skey[b], c->sval[b], c->skey[b ^ 1], c->sval[b ^ 1], n, 8 * p, hist, tot, nullptr);
+      c->launches += 1;
+    }
+    c->launches += 1;
   }
   *cur = b;
   return cudaGetLastError();
@@ -338,37 +451,35 @@ cudaError_t sort_pairs(nb_ctx* c, int64_t n, int bits, int* cur) {
 
 }  // namespace
 
+// histogram scratch of a sort of up to n rows (and of the list order's counts)
+size_t nb_sort_hist_ints(int64_t n) {
+  const size_t chunks = std::max<size_t>((size_t)(n / (kItemsLarge * kSortThreads) + 1), 4 * kFusedChunks);
+  return (chunks + 1) * kRadix;
+}
+
 // stable sort of the rows by the keys in skey[0] (values = row numbers in
 // sval[0]) on the low `bits` bits, then the state reordered to that order
 cudaError_t nb_order_rows_by_keys(nb_ctx* c, int bits) {
   const int64_t N = c->n;
   int cur = 0;
-  cudaError_t e = sort_pairs(c, N, bits, &cur);
+  cudaError_t e =
+      N <= kSmallRows ? sort_pairs<kItemsSmall>(c, N, bits, &cur) : sort_pairs<kItemsLarge>(c, N, bits, &cur);
   if (e != cudaSuccess) return e;
   // sval[cur][s] = the current row that becomes row s
-  const int32_t* sigma = c->sval[cur];
-  e = reorder_state(c, sigma);
-  if (e != cudaSuccess) return e;
-  const int g = grid_for(N, 256, c->sm_count * 16);
-  int32_t* np = c->sval[cur ^ 1];
-  compose<<<g, 256, 0, c->stream>>>(N, c->perm_valid ? c->perm : nullptr, sigma, np);
-  e = cudaMemcpyAsync(c->perm, np, N * sizeof(int32_t), cudaMemcpyDeviceToDevice, c->stream);
-  if (e != cudaSuccess) return e;
-  invert_perm<<<g, 256, 0, c->stream>>>(N, c->perm, c->iperm);
-  c->launches += 2;
-  return cudaGetLastError();
+  return reorder_state(c, c->sval[cur], c->sval[cur ^ 1]);
 }
 
 cudaError_t nb_spatial_sort(nb_ctx* c) {
   const int64_t N = c->n;
   if (N <= 0) return cudaSuccess;
-  const int nbb = grid_for(N, kSortThreads, 1024);
-  double* box = c->red + NB_BBOX_OFFSET;
-  bbox_partial<<<nbb, kSortThreads, 0, c->stream>>>(N, c->n_pad, c->x, c->red);
-  bbox_final<<<1, kSortThreads, 0, c->stream>>>(nbb, c->red, box);
-  morton_keys<<<grid_for(N, 256, c->sm_count * 16), 256, 0, c->stream>>>(N, c->n_pad, c->x, box, c->skey[0],
-                                                                         c->sval[0]);
-  c->launches += 3;
+  // (the key kernel's CTAs read all partial boxes: two per SM are enough to
+  // stream the positions)
+  const int nbb = grid_for(N, kSortThreads, std::min(c->sm_count * 2, (int)(NB_RED_DOUBLES / 6)));
+  long long* red = reinterpret_cast<long long*>(c->red);
+  bbox_partial<<<nbb, kSortThreads, 0, c->stream>>>(N, c->n_pad, c->x, red);
+  morton_keys<<<grid_for(N, kSortThreads, c->sm_count * 8), kSortThreads, 0, c->stream>>>(
+      N, c->n_pad, c->x, nbb, red, c->skey[0], c->sval[0]);
+  c->launches += 2;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return nb_order_rows_by_keys(c, 30);
@@ -377,7 +488,7 @@ cudaError_t nb_spatial_sort(nb_ctx* c) {
 cudaError_t nb_unsort(nb_ctx* c) {
   if (!c->perm_valid) return cudaSuccess;
   // particle p = old row iperm[p]
-  cudaError_t e = reorder_state(c, c->iperm);
+  cudaError_t e = reorder_state(c, c->iperm, nullptr);
   if (e != cudaSuccess) return e;
   c->perm_valid = false;
   c->pred_valid = false;
