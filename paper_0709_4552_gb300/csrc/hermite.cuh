@@ -436,19 +436,6 @@ __device__ __forceinline__ double correct_lanes4(int64_t i, int64_t n_pad, doubl
   return t + dnew;
 }
 
-// correct_lanes4 with its inputs read from the state and the predicted rows
-__device__ __forceinline__ double correct_row_lanes4(int64_t i, int64_t n_pad, double t, double a1, double j1,
-                                                   double p1, double eta, double dt_min, double dt_max, double* __restrict__ x,
-                                                   double* __restrict__ v, double* __restrict__ a,
-                                                   double* __restrict__ jk, double* __restrict__ pot,
-                                                   double* __restrict__ ti, double* __restrict__ dt,
-                                                   const double* __restrict__ xp, const double* __restrict__ vp,
-                                                   nb_dev_status* __restrict__ st, int sub, int base, bool write) {
-  const int64_t q = (sub < 3 ? sub : 0) * n_pad + i;
-  const CorrIn in{ti[i], dt[i], a[q], jk[q], xp[q], vp[q]};
-  return correct_lanes4(i, n_pad, t, a1, j1, p1, in, eta, dt_min, dt_max, x, v, a, jk, pot, ti, dt, st, sub, base, write);
-}
-
 // j-memory record of row i (the on-the-fly j prediction's input, Sec. 4.4
 // step 4; layout in force_common.cuh): double-single position and velocity,
 // a/2 and jerk/6 in FP32, the mass, and the reach Rd >= |v_c| dt + |a_c| dt^2/2

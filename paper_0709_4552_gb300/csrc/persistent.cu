@@ -12,10 +12,10 @@
 //     its own offset in the active list; it writes its own active rows there
 //     (ascending), predicts its own rows to t (step 3) and, on the mixed path
 //     in spatial order, computes the boxes of its own tiles.    -> barrier B
-//   phase 2: force items (i-tile of 128 list positions x j-split) taken from
-//     a work counter, or by block index when every CTA has an SM of its own
-//     and the items fit (step 4, Eq. 3), the same items as the host-driven
-//     kernels, split partials as double-single pairs.            -> barrier C
+//   phase 2: force items (i-tile of 128 list positions x j-split; step 4,
+//     Eq. 3), the first by the CTA's place in an order that fills the SMs
+//     evenly, the others from a work counter; the same items as the
+//     host-driven kernels, split partials as double-single pairs. -> barrier C
 //   phase 3: every CTA sums the j-splits of its own list positions in a fixed
 //     order (double-single FP32), corrects them and picks their new steps
 //     (step 5; own rows' due times kept in shared memory), then publishes the
@@ -45,10 +45,13 @@ constexpr int kLWarps = kLT / 32;
 // resident CTAs per SM asked for.  Mixed: 4 (128 registers, a few spilled) where
 // the force phase is the longest part of a step, 2 (no spills) where its
 // latencies are (us a block step, 4 / 2: N = 512 19.1 / 17.9, N = 12000 34.3 /
-// 31.5, N = 32768 67.5 / 64.4, N = 40000 84.4 / 88.0, N = 65536 169 / 184).  FP64: 3 (168; with 4 the fixed-point pair spills: N =
-// 1024 32.4 against 31.8 us a block step, N = 32768 582 against 569)
+// 31.5, N = 32768 67.5 / 64.4, N = 40000 84.4 / 88.0, N = 65536 169 / 184; all
+// before the corrector's loads were batched and its rows read ahead, which took
+// N = 12000 from 30.3 to 28.0 and N = 32768 from 62.7 to 58.3).  FP64: 3 (168;
+// with 4 the fixed-point pair spills: N = 1024 32.4 against 31.8 us a block
+// step, N = 32768 582 against 569)
 constexpr int kLPerSmMixed = 4, kLPerSmMixedSmall = 2, kLPerSm64 = 3;
-constexpr int64_t kLMixedSmallHi = 32768;
+constexpr int64_t kLMixedSmallHi = 32768, kLMixedTwoLo = 2048;
 // j-tiles (the mixed one = the box tile).  FP64: an item's tile is its share of
 // a small system's force phase, so those take 32 and at least two CTAs per SM:
 // N = 1024 31.8 us a block step against 40.7 with 64 and one CTA (44.9 with 64
@@ -61,14 +64,18 @@ constexpr int64_t kLF64SmallLo = 2 * kLF64JT, kLF64SmallHi = 8192;
 constexpr long long kWaitNs = 4000000000LL;  // a barrier wait of the loop gives up after 4 s
 constexpr unsigned int kPollCap = 1u << 26;  // ... or after this many polls
 constexpr unsigned long long kInfBits = 0x7FF0000000000000ULL;  // +inf
-constexpr int kLItemWaves = 2;               // force items per step: about 2 per CTA ...
-constexpr int64_t kLMaxSplits = 256;         // ... with at most this many j-splits
+// force items per step: about this many per CTA.  Mixed, us a block step with 2,
+// 3, 4, 6: N = 24000 43.0, 42.5, 42.3, 42.5; N = 40000 81.2, 80.5, 81.0, 81.8.
+// FP64 with 2 and 4: N = 16384 176.7, 178.4; N = 32768 573, 559.
+constexpr int kLItemWavesMixed = 3, kLItemWaves64 = 2;
+constexpr int64_t kLMaxSplits = 256;         // ... in at most this many j-splits
 constexpr int kMaxSmid = 1024;               // SM ids counted by the CTA placement
+constexpr int kMaxRank = 32;                 // CTAs an SM can hold
 
 struct LoopCtl {
   unsigned long long bar;   // barrier arrivals in this launch
   unsigned long long wq;    // force-item counter of the current step
-  unsigned int nsm;         // SMs holding CTAs of this launch
+  unsigned int ranks[kMaxRank];   // CTAs of each rank on their SM
   unsigned int smrank[kMaxSmid];  // CTAs placed on each SM so far
   unsigned int abort;       // a CTA gave up waiting: every CTA leaves
   unsigned int more;        // the launch stopped after seg_steps steps
@@ -118,14 +125,20 @@ __device__ __forceinline__ long long globaltimer_ns() {
 // orders every thread's writes before thread 0's gpu-scope release add
 // (cumulative), and thread 0's acquire load before every thread's later
 // reads.  Returns false when this CTA must leave (another CTA gave up, or
-// this one waited longer than wait_ns).
-__device__ bool grid_barrier(LoopCtl* ctl, unsigned long long& epoch, unsigned int G, nb_dev_status* st,
-                             int* s_ok, long long wait_ns = kWaitNs) {
+// this one waited longer than wait_ns).  In two parts, for work that passes
+// between the arrival and the wait.
+__device__ __forceinline__ void grid_arrive(LoopCtl* ctl, unsigned long long& epoch) {
   __syncthreads();
   if (threadIdx.x == 0) {
     epoch += 1;
-    const unsigned long long target = epoch * (unsigned long long)G;
     red_release_add_u64(&ctl->bar, 1ULL);
+  }
+}
+
+__device__ bool grid_wait(LoopCtl* ctl, unsigned long long epoch, unsigned int G, nb_dev_status* st, int* s_ok,
+                          long long wait_ns = kWaitNs) {
+  if (threadIdx.x == 0) {
+    const unsigned long long target = epoch * (unsigned long long)G;
     int ok = 1;
     const long long t0 = globaltimer_ns();
     unsigned int polls = 0;
@@ -151,6 +164,12 @@ __device__ bool grid_barrier(LoopCtl* ctl, unsigned long long& epoch, unsigned i
   return *s_ok != 0;
 }
 
+__device__ __forceinline__ bool grid_barrier(LoopCtl* ctl, unsigned long long& epoch, unsigned int G,
+                                             nb_dev_status* st, int* s_ok, long long wait_ns = kWaitNs) {
+  grid_arrive(ctl, epoch);
+  return grid_wait(ctl, epoch, G, st, s_ok, wait_ns);
+}
+
 // (minimum, count at the minimum) combine
 __device__ __forceinline__ void min_count(unsigned long long& v, int& c, unsigned long long ov, int oc) {
   if (ov < v) {
@@ -162,13 +181,16 @@ __device__ __forceinline__ void min_count(unsigned long long& v, int& c, unsigne
 }
 
 constexpr int kLDue = 512;  // own rows whose due times a CTA keeps in shared memory
+constexpr int kOwn = 128;   // own active rows it keeps there
 
 struct LoopSmem {
   // own rows' next due time t_i + dt_i (bit pattern), kept by the corrector
   // when the CTA owns at most kLDue rows (else read from the state)
   unsigned long long due[kLDue];
+  int own[kOwn];           // own active rows (from the CTA's first), list order
   int rank;                // this CTA's rank among the CTAs on its SM
-  long long item;
+  int place;               // its place in the order of force items
+  int item;
   unsigned long long wv[kLWarps];
   int wc[kLWarps];
   long long ws[2][kLWarps];
@@ -290,7 +312,11 @@ __device__ void write_active(const LoopArgs& p, int64_t r0, int64_t r1, unsigned
       pre += w < warp ? s.wc[w] : 0;
       all += s.wc[w];
     }
-    if (on) p.act[base + pre + __popc(ball & ((1u << lane) - 1u))] = (int32_t)i;
+    if (on) {
+      const long long k = base + pre + __popc(ball & ((1u << lane) - 1u));
+      p.act[k] = (int32_t)i;
+      if (k - s.before < kOwn) s.own[k - s.before] = (int)(i - r0);
+    }
     base += all;
     __syncthreads();
   }
@@ -319,13 +345,14 @@ __device__ void predict_rows(const LoopArgs& p, int64_t r0, int64_t r1, double t
   }
 }
 
-// split-j factor of a step: about kLItemWaves force items per CTA (taken
+// split-j factor of a step: a few force items per CTA (taken
 // from a counter, so uneven items even out), at least one j-tile per split,
 // at most kLMaxSplits splits (their sums are the corrector phase's loads),
 // within the partial-sum scratch
+template <bool MIXED>
 __device__ __forceinline__ int64_t loop_splits(int64_t n, int64_t jtiles, unsigned int G, int64_t part_elems) {
   const int64_t nI = (n + kLT - 1) / kLT;
-  int64_t S = ((int64_t)kLItemWaves * G + nI - 1) / nI;
+  int64_t S = ((int64_t)(MIXED ? kLItemWavesMixed : kLItemWaves64) * G + nI - 1) / nI;
   if (S > jtiles) S = jtiles;
   if (S > kLMaxSplits) S = kLMaxSplits;
   const int64_t cap = part_elems / (7 * (((n + 31) / 32) * 32));
@@ -333,38 +360,68 @@ __device__ __forceinline__ int64_t loop_splits(int64_t n, int64_t jtiles, unsign
   return S < 1 ? 1 : S;
 }
 
-// phase 3 of a step: the j-split sums and the corrector (Sec. 4.1 step 5)
-// of this CTA's own list positions [before, before + mycnt).  The step's
-// values are read from shared memory here rather than kept in registers
-// across the force items.
-template <bool MIXED>
-__device__ void correct_own(const LoopArgs& p, LoopSmem& s, int64_t jtiles, unsigned int G, int64_t r0,
-                            int64_t r1) {
+// The own list positions are corrected up to round_of(mycnt) at a time: L =
+// kLT / P' threads per position (P' = the round's positions rounded up to a
+// power of two, at least 4), of which this thread is lane l of position q.
+// Up to 64 positions: 32 a round, which lanes 0-3 correct together (the
+// correction's FP64 chain is on the critical path of a step); more: one or two
+// threads each, as the FP64 unit is then busy anyway (N = 1024 in FP64, every
+// particle at every step: 33 us a step against 43 in rounds of 32).
+__device__ __forceinline__ int round_of(int mycnt) { return mycnt <= 64 ? 32 : kLT; }
+struct OwnRow {
+  int L, l, q;
+  bool have;       // position q exists in this round
+  int64_t i;       // its row (without a position: some own row, read only)
+  nbh::CorrIn in;  // L >= 4: what the correction reads of the row itself
+};
+
+__device__ __forceinline__ OwnRow own_row(const LoopArgs& p, const LoopSmem& s, int k0, int64_t r0) {
+  OwnRow o;
+  const int P = min(s.mycnt - k0, round_of(s.mycnt));
+  int Pp = 4;
+  while (Pp < P) Pp <<= 1;
+  o.L = kLT / Pp;
+  o.q = threadIdx.x / o.L;
+  o.l = threadIdx.x % o.L;
+  o.have = o.q < P;
+  o.i = r0;
+  o.in = nbh::CorrIn{};
+  if (P <= 0) return o;
+  const int k = k0 + (o.have ? o.q : 0);
+  o.i = k < kOwn ? r0 + s.own[k] : (int64_t)p.act[s.before + k];
+  if (o.L >= 4) {
+    const int64_t c = (o.l < 3 ? o.l : 0) * p.n_pad + o.i;
+    o.in = nbh::CorrIn{p.t[o.i], p.dt[o.i], p.a[c], p.jk[c], p.xp[c], p.vp[c]};
+  }
+  return o;
+}
+
+// phase 3 of a step: the j-split sums and the corrector (Sec. 4.1 step 5) of
+// this CTA's own list positions [before, before + mycnt): in each round the
+// lanes of a position sum its j-splits (lane l takes splits l, l + L, ... in
+// order; a butterfly over the L lanes) and correct it.  `first`: the first
+// round's rows, read before the forces were complete.  The active rows crowd in
+// the CTAs that own a system's core, so a step waits for one CTA's L2 round
+// trips: the loads of U splits are in flight per lane.
+template <bool MIXED, int U, bool FIRST>
+__device__ void correct_own(const LoopArgs& p, LoopSmem& s, const OwnRow& first, int64_t jtiles, unsigned int G,
+                            int64_t r0, int64_t r1) {
   const long long before = s.before;
   const int mycnt = s.mycnt;
   const double tn = __longlong_as_double((long long)s.tnb);
   const int64_t n = s.total;
-  const int64_t S = loop_splits(n, jtiles, G, p.part_elems);
+  const int64_t S = loop_splits<MIXED>(n, jtiles, G, p.part_elems);
   const int64_t pstride = ((n + 31) / 32) * 32;
   const bool fin = S == 1;
-  // own list positions, up to 128 per round: L = 128 / P' threads per
-  // position (P' = the round's positions rounded up to a power of two, at
-  // least 4) sum its j-splits (lane l takes splits l, l + L, ... in order;
-  // a butterfly over the L lanes), and the group corrects it (step 5): lanes
-  // 0-3 together when it has at least four (the correction's FP64 chain is
-  // the critical path of a small block's step), else lane 0 alone: one
-  // position per thread when the block is large, 32 lanes per position when
-  // it is small and the splits many
-  for (int k0 = 0; k0 < mycnt; k0 += kLT) {
-    const int P = min(mycnt - k0, kLT);
-    int Pp = 4;
-    while (Pp < P) Pp <<= 1;
-    const int L = kLT / Pp;
-    const int q = threadIdx.x / L, l = threadIdx.x % L;
-    const bool have = q < P;
-    const int64_t k = before + k0 + (have ? q : 0);
-    // the row's sums: final FP64 rows, double-single partials (the mixed item's
-    // split output, summed and exchanged in FP32), or FP64 partials
+  const bool cached = r1 - r0 <= kLDue;
+  const int round = round_of(mycnt);
+  for (int k0 = 0; k0 < mycnt; k0 += round) {
+    const OwnRow o = FIRST && k0 == 0 ? first : own_row(p, s, k0, r0);
+    const int L = o.L, l = o.l;
+    const bool have = o.have;
+    const int64_t k = before + k0 + (have ? o.q : 0);
+    // the row's sums: final FP64 rows, double-single partials (summed and
+    // exchanged in FP32), or FP64 partials
     float hi[7], lo[7];
     double f[7];
     if (fin) {
@@ -373,42 +430,55 @@ __device__ void correct_own(const LoopArgs& p, LoopSmem& s, int64_t jtiles, unsi
     } else if (MIXED) {
 #pragma unroll
       for (int r = 0; r < 7; ++r) hi[r] = lo[r] = 0.0f;
-      const float2* part2 = reinterpret_cast<const float2*>(p.part);
+      const float2* part2 = reinterpret_cast<const float2*>(p.part) + k;
       if (have)
-        for (int64_t sp = l; sp < S; sp += L)
+        for (int64_t sp = l; sp < S; sp += U * L) {
+          float2 v[U][7];  // (past the last split: zeros, which change nothing)
 #pragma unroll
-          for (int r = 0; r < 7; ++r) {
-            const float2 v = part2[(sp * 7 + r) * pstride + k];
-            nbk::ds_add(hi[r], lo[r], v.x, v.y);
-          }
-      for (int o = L / 2; o > 0; o >>= 1)
+          for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int r = 0; r < 7; ++r)
+              v[u][r] = sp + u * L < S ? part2[((sp + u * L) * 7 + r) * pstride] : make_float2(0.0f, 0.0f);
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int r = 0; r < 7; ++r) nbk::ds_add(hi[r], lo[r], v[u][r].x, v[u][r].y);
+        }
+      for (int w = L / 2; w > 0; w >>= 1)
 #pragma unroll
         for (int r = 0; r < 7; ++r) {
-          const float oh = __shfl_xor_sync(0xffffffffu, hi[r], o);
-          const float ol = __shfl_xor_sync(0xffffffffu, lo[r], o);
+          const float oh = __shfl_xor_sync(0xffffffffu, hi[r], w);
+          const float ol = __shfl_xor_sync(0xffffffffu, lo[r], w);
           nbk::ds_add(hi[r], lo[r], oh, ol);
         }
     } else {
 #pragma unroll
       for (int r = 0; r < 7; ++r) f[r] = 0.0;
       if (have)
-        for (int64_t sp = l; sp < S; sp += L)
+        for (int64_t sp = l; sp < S; sp += U * L) {
+          double v[U][7];
 #pragma unroll
-          for (int r = 0; r < 7; ++r) f[r] += p.part[(sp * 7 + r) * pstride + k];
-      for (int o = L / 2; o > 0; o >>= 1)
+          for (int u = 0; u < U; ++u)
 #pragma unroll
-        for (int r = 0; r < 7; ++r) f[r] += __shfl_xor_sync(0xffffffffu, f[r], o);
+            for (int r = 0; r < 7; ++r)
+              v[u][r] = sp + u * L < S ? p.part[((sp + u * L) * 7 + r) * pstride + k] : 0.0;
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (sp + u * L < S)
+#pragma unroll
+              for (int r = 0; r < 7; ++r) f[r] += v[u][r];
+        }
+      for (int w = L / 2; w > 0; w >>= 1)
+#pragma unroll
+        for (int r = 0; r < 7; ++r) f[r] += __shfl_xor_sync(0xffffffffu, f[r], w);
       f[6] = -f[6];
     }
-    const bool cached = r1 - r0 <= kLDue;
+    double nd = 0.0;
     if (L >= 4) {
       // every lane of the CTA takes this branch (L is uniform) and every
-      // shuffle inside; lanes without a row read a valid own row, write
-      // nothing.  Each lane forms the FP64 values of its own component only (an
-      // FP64 addition holds the warp for 64 cycles: 3 of them instead of 7, and
-      // none of the 14 conversions)
-      int64_t i = p.act[k];
-      i = i < r0 ? r0 : (i >= r1 ? r1 - 1 : i);  // own rows only
+      // shuffle inside; lanes without a row write nothing.  Each lane forms the
+      // FP64 values of its own component only (an FP64 addition holds the warp
+      // for 64 cycles: 3 of them instead of 7, and none of the 14 conversions)
       double a1, j1, p1;
       if (MIXED && !fin) {
         const float ah = l == 1 ? hi[1] : (l == 2 ? hi[2] : hi[0]), al = l == 1 ? lo[1] : (l == 2 ? lo[2] : lo[0]);
@@ -422,23 +492,27 @@ __device__ void correct_own(const LoopArgs& p, LoopSmem& s, int64_t jtiles, unsi
         p1 = f[6];
       }
       if (!(have && l < 4)) a1 = j1 = p1 = 0.0;
-      const double nd =
-          nbh::correct_row_lanes4(i, p.n_pad, tn, a1, j1, p1, p.eta, p.dt_min, p.dt_max, p.x, p.v, p.a, p.jk, p.pot,
-                                  p.t, p.dt, p.xp, p.vp, p.st, l, (int)(threadIdx.x & 31) - l, have);
-      if (have && l == 0 && cached) s.due[i - r0] = (unsigned long long)__double_as_longlong(nd);
+      nd = nbh::correct_lanes4(o.i, p.n_pad, tn, a1, j1, p1, o.in, p.eta, p.dt_min, p.dt_max, p.x, p.v, p.a, p.jk,
+                               p.pot, p.t, p.dt, p.st, l, (int)(threadIdx.x & 31) - l, have);
     } else if (have && l == 0) {
       if (MIXED && !fin) {
 #pragma unroll
         for (int r = 0; r < 7; ++r) f[r] = nb_f64(hi[r]) + nb_f64(lo[r]);
         f[6] = -f[6];
       }
-      int64_t i = p.act[k];
-      i = i < r0 ? r0 : (i >= r1 ? r1 - 1 : i);  // own rows only
-      const double nd = nbh::correct_row(i, p.n_pad, tn, f, p.eta, p.dt_min, p.dt_max, p.x, p.v, p.a, p.jk, p.pot,
-                                         p.t, p.dt, p.xp, p.vp, p.st);
-      if (cached) s.due[i - r0] = (unsigned long long)__double_as_longlong(nd);
+      nd = nbh::correct_row(o.i, p.n_pad, tn, f, p.eta, p.dt_min, p.dt_max, p.x, p.v, p.a, p.jk, p.pot, p.t, p.dt,
+                            p.xp, p.vp, p.st);
     }
+    if (have && l == 0 && cached) s.due[o.i - r0] = (unsigned long long)__double_as_longlong(nd);
   }
+}
+
+// the next force item off the step's counter, which counts from `first`
+__device__ __forceinline__ int next_item(const LoopArgs& p, LoopSmem& s, int first) {
+  __syncthreads();  // every thread has read the previous item
+  if (threadIdx.x == 0) s.item = first + (int)atomicAdd(&p.ctl->wq, 1ULL);
+  __syncthreads();
+  return s.item;
 }
 
 template <bool MIXED, int JT, int PER_SM>
@@ -446,6 +520,12 @@ __global__ void __launch_bounds__(kLT, PER_SM) loop_kernel(LoopArgs p) {
   using ForceSmem = typename std::conditional<MIXED, nbk::MixedSmem<JT>, nbk::Fp64Smem<kLT, JT>>::type;
   __shared__ __align__(16) ForceSmem fsm;
   __shared__ LoopSmem s;
+  // the variants for small systems, whose steps are a chain of latencies; in
+  // the others reading ahead costs the force items registers (N = 60000 mixed
+  // 143.4 us a block step against 140.0), and FP64 items placed ahead of time
+  // balance worse (N = 16384 179 against 176)
+  constexpr bool kShort = MIXED ? PER_SM == kLPerSmMixedSmall : JT == kLF64JTSmall;
+  constexpr bool kPlaced = MIXED || kShort;  // the first item by the CTA's place
   const unsigned int G = gridDim.x;
   const int64_t N = p.N;
   const int64_t T = (N + kLT - 1) / kLT;
@@ -457,15 +537,14 @@ __global__ void __launch_bounds__(kLT, PER_SM) loop_kernel(LoopArgs p) {
   long long steps = 0;
   double tn_prev = -INFINITY;  // the previous block time (they strictly increase)
 
-  // placement: this CTA's rank among the CTAs on its SM.  A step with few
-  // force items hands them to rank-0 CTAs first (one per SM), so that they
-  // do not share an SM's pipes while other SMs idle.
+  // placement: this CTA's rank among the CTAs on its SM, and its number among
+  // the CTAs of that rank.  The CTAs in this order take the force items of a
+  // step, so that a step with few items spreads them over the SMs.
   if (threadIdx.x == 0) {
     unsigned int smid;
     asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
-    const unsigned int r = atomicAdd(&p.ctl->smrank[smid % kMaxSmid], 1u);
-    if (r == 0) atomicAdd(&p.ctl->nsm, 1u);
-    s.rank = (int)r;
+    s.rank = (int)min(atomicAdd(&p.ctl->smrank[smid % kMaxSmid], 1u), (unsigned int)kMaxRank - 1);
+    s.place = (int)atomicAdd(&p.ctl->ranks[s.rank], 1u);
   }
   // rows between N and the end of the last tile are massless far-away
   // padding in the predicted j-store (they fill the last j-tile)
@@ -501,32 +580,25 @@ __global__ void __launch_bounds__(kLT, PER_SM) loop_kernel(LoopArgs p) {
       if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&p.st->flags, NB_ST_TIMEOUT);
       break;
     }
+    if (steps == 0 && threadIdx.x == 0)  // (every CTA has registered before its first barrier)
+      for (int r = 0; r < s.rank; ++r) s.place += (int)__ldcg(&p.ctl->ranks[r]);
     if (s.mine) write_active(p, r0, r1, tnb, s.before, s);
     predict_rows<MIXED>(p, r0, r1, tn, s);
     if (blockIdx.x == 0 && threadIdx.x == 0) p.ctl->wq = 0;  // nobody takes items before barrier B
     if (!grid_barrier(p.ctl, epoch, G, p.st, &s.ok)) return;  // B: list and j-store complete
 
-    // forces (Sec. 4.1 step 4): items i-tile x j-split from the step's
-    // counter, taken by the CTAs of rank < ceil(items / SMs).  When every CTA
-    // has an SM of its own and there are no more items than CTAs (every small
-    // block), CTA b takes item b: no counter round trips at all.
+    // forces (Sec. 4.1 step 4): items i-tile x j-split.  The first is the CTA's
+    // by its place (when there are no more items than CTAs, as in every small
+    // block, that is all, without counter round trips); the rest come from the
+    // step's counter.
     const int64_t nI = (n + kLT - 1) / kLT;
-    const int64_t S = loop_splits(n, jtiles, G, p.part_elems);
+    const int64_t S = loop_splits<MIXED>(n, jtiles, G, p.part_elems);
     const int64_t pstride = ((n + 31) / 32) * 32;
     const bool fin = S == 1;
     const int items = (int)(nI * S);
-    const unsigned int nsm = __ldcg(&p.ctl->nsm);
-    const bool fixed = nsm == G && items <= (int)G;
-    const bool takes = fixed ? (int)blockIdx.x < items : (int64_t)s.rank * nsm < items;
-    for (int round = 0;; ++round) {
-      if (!takes || (fixed && round > 0)) break;
-      if (!fixed) {
-        __syncthreads();  // every thread has read the previous item
-        if (threadIdx.x == 0) s.item = (long long)atomicAdd(&p.ctl->wq, 1ULL);
-        __syncthreads();
-      }
-      const int item = fixed ? (int)blockIdx.x : (int)min(s.item, (long long)items);
-      if (item >= items) break;
+    int item = s.place;
+    if (!kPlaced && item < items) item = next_item(p, s, 0);
+    for (; item < items;) {
       const int itile = item % (int)nI, split = item / (int)nI;
       const int64_t jlo = nbk::split_begin(split, S, jtiles) * JT;
       // mixed: the padding rows of the last j-tile are massless far-away
@@ -540,9 +612,14 @@ __global__ void __launch_bounds__(kLT, PER_SM) loop_kernel(LoopArgs p) {
       else
         nbk::fp64_item<kLT, JT>(fsm, p.xp, p.vp, p.m, p.n_pad, 1, jlo, jhi, p.n_pad, p.act, n, itile * kLT,
                                      p.eps2, out, ostride, fin);
+      if (kPlaced && items <= (int)G) break;
+      item = next_item(p, s, kPlaced ? (int)G : 0);
     }
-    if (!grid_barrier(p.ctl, epoch, G, p.st, &s.ok)) return;  // C: forces complete
-    correct_own<MIXED>(p, s, jtiles, G, r0, r1);
+    grid_arrive(p.ctl, epoch);
+    OwnRow first;
+    if (kShort) first = own_row(p, s, 0, r0);  // (its loads pass behind the wait)
+    if (!grid_wait(p.ctl, epoch, G, p.st, &s.ok)) return;  // C: forces complete
+    correct_own<MIXED, kShort ? 4 : 1, kShort>(p, s, first, jtiles, G, r0, r1);
     ++steps;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       p.ctl->steps = steps;
@@ -627,12 +704,14 @@ int nb_integrate_persistent(nb_ctx* c, double t_end) {
     return NB_ECUDA;
   }
   // as many CTAs as fit, but for a small system no more than twice its row
-  // tiles (at least 32; FP64: two CTAs per SM, whose force items are the step's
-  // longest part): the other CTAs would own no rows and take no force items of
-  // its small blocks, and each barrier waits for every CTA's arrival
+  // tiles, as each barrier waits for every CTA's arrival; at least 32, or two
+  // CTAs per SM where the force items are a good part of a step (FP64; mixed
+  // above the cluster loop's range: N = 4096 20.6 -> 19.5 us a block step, N =
+  // 12000 28.4 -> 28.0, but N = 512 17.4 -> 17.8)
   const int64_t row_tiles = (c->n + kLT - 1) / kLT;
+  const bool two = variant == 3 || (variant == 1 && c->n > kLMixedTwoLo);
   const int G = (int)std::min<int64_t>(std::min(c->sm_count * per_sm, kLMaxG),
-                                       std::max<int64_t>(variant == 3 ? 2 * c->sm_count : 32, 2 * row_tiles));
+                                       std::max<int64_t>(two ? 2 * c->sm_count : 32, 2 * row_tiles));
   if (G > L->gmax) {
     if (L->smin) cudaFree(L->smin);
     if (L->scnt) cudaFree(L->scnt);
