@@ -50,6 +50,7 @@ constexpr int kChunk = 128;    // j per FP32 partial sum before the double-singl
 constexpr int kMaxC = 16;      // CTAs per cluster at most
 constexpr int kCC = 256;       // own active particles whose corrector inputs stay in shared memory
 constexpr unsigned long long kInfBits = 0x7FF0000000000000ULL;
+constexpr int kRes = 256;      // rows per CTA whose FP64 state and j-memory records fit in shared memory too
 constexpr int kRB = 32;        // rows per ownership block (dealt round-robin to the CTAs)
 
 // row of own row index q of CTA me (blocks of kRB rows, block b owned by b % C)
@@ -62,7 +63,7 @@ __device__ __forceinline__ int own_index(int64_t row, int me, int C) {
   return (int)(b % C) == me ? (int)((b / C) * kRB + row % kRB) : -1;
 }
 // rows CTA me owns
-__device__ __forceinline__ int own_count(int64_t N, int me, int C) {
+__host__ __device__ __forceinline__ int own_count(int64_t N, int me, int C) {
   const int64_t nb = (N + kRB - 1) / kRB;  // blocks
   if (me >= nb) return 0;
   const int64_t mine = (nb - 1 - me) / C + 1;  // blocks me, me + C, ...
@@ -102,7 +103,7 @@ struct CSmem {
   // own rows predicted to the block time (double-single positions, FP32 v, m)
   float jxh[kCRows], jyh[kCRows], jzh[kCRows], jxl[kCRows], jyl[kCRows], jzl[kCRows];
   float jvx[kCRows], jvy[kCRows], jvz[kCRows], jms[kCRows];
-  int32_t irow[kCRows];
+  int32_t iq[kCRows];  // own active rows (own row indexes), list order
   // own rows' next due time t_i + dt_i (bit pattern), kept by the corrector
   unsigned long long due[kCRows];
   // this CTA's double-single partial sums on the group (read by the owners)
@@ -114,6 +115,10 @@ struct CSmem {
   double cT[kCC], cDT[kCC], cA0[3][kCC], cJ0[3][kCC], cXP[3][kCC], cVP[3][kCC];
   // every CTA's offset and count in the active list (read at barrier A)
   int cbefore[kMaxC], cmine[kMaxC];
+  // RES: the own rows' state and j-memory records (written through to global
+  // memory by the corrector), read by every step's predictions
+  double rx[3][kRes], rv[3][kRes], ra[3][kRes], rj[3][kRes], rt[kRes], rdt[kRes];
+  float4 rm[5][kRes];
   double tn;
   long long total;
   unsigned long long wmin[kCT / 32];
@@ -146,7 +151,7 @@ __device__ void publish(CSmem& s, cg::cluster_group& cl, int me, int C, int nr) 
   }
 }
 
-// own rows at the block time, ascending, into s.irow (each thread scans a
+// own rows at the block time, ascending, into s.iq (each thread scans a
 // contiguous run of rows; a block scan places the runs in order)
 __device__ void list_rows(CSmem& s, int me, int C, int nr, unsigned long long tnb) {
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -165,10 +170,45 @@ __device__ void list_rows(CSmem& s, int me, int C, int nr, unsigned long long tn
   for (int k = 0; k < w; ++k) base += s.wcnt[k];
   int at = base + inc - cnt;
   for (int q = q0; q < q1; ++q)
-    if (s.due[q] == tnb) s.irow[at++] = (int32_t)own_row(q, me, C);
+    if (s.due[q] == tnb) s.iq[at++] = q;
   __syncthreads();
 }
 
+static_assert(sizeof(CSmem) <= 227 * 1024, "shared memory of a CTA");
+
+// the corrector's copy of a row it writes
+struct KeepRow {
+  CSmem* s;
+  int q;
+  __device__ __forceinline__ void component(int c, double x1, double v1, double a1, double j1) const {
+    s->rx[c][q] = x1;
+    s->rv[c][q] = v1;
+    s->ra[c][q] = a1;
+    s->rj[c][q] = j1;
+  }
+  __device__ __forceinline__ void record(int c, float xh, float xl, float vh, float vl, float a2, float j6) const {
+    float* r = reinterpret_cast<float*>(&s->rm[0][q]);
+    r[c] = xh;
+    r[4 * kRes + c] = xl;
+    r[8 * kRes + c] = vh;
+    r[12 * kRes + c] = vl;
+    r[16 * kRes + c] = a2;
+    r[4 * kRes * (2 + c) + 3] = j6;
+  }
+  __device__ __forceinline__ void step(double t, double dt) const {
+    s->rt[q] = t;
+    s->rdt[q] = dt;
+  }
+};
+
+// RES: at most kRes rows per CTA, whose state and records stay in shared memory.
+// A step is a chain of latencies (N = 512 to 2048: one to four particles per
+// CTA and step), so what helps is to shorten it: with the state resident no
+// prediction waits for L2, each component of an active particle has a thread
+// of its own (6 FP64 instructions of 64 cycles instead of 18), the lanes' sums
+// cross in 9 exchanges instead of 35, and the new step comes from FP32 roots
+// (hermite.cuh).  Us a block step: N = 512 11.9 -> 9.7, N = 4096 35.5 -> 32.1.
+template <bool RES>
 __global__ void __launch_bounds__(kCT, 1) cluster_loop_kernel(ClusterArgs p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CSmem& s = *reinterpret_cast<CSmem*>(smem_raw);
@@ -184,6 +224,19 @@ __global__ void __launch_bounds__(kCT, 1) cluster_loop_kernel(ClusterArgs p) {
   for (int q = tid; q < nr; q += kCT) {
     const int64_t r = own_row(q, me, C);
     s.due[q] = (unsigned long long)__double_as_longlong(p.t[r] + p.dt[r]);
+    if (RES) {
+      s.rt[q] = p.t[r];
+      s.rdt[q] = p.dt[r];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        s.rx[d][q] = p.x[d * p.n_pad + r];
+        s.rv[d][q] = p.v[d * p.n_pad + r];
+        s.ra[d][q] = p.a[d * p.n_pad + r];
+        s.rj[d][q] = p.jk[d * p.n_pad + r];
+      }
+#pragma unroll
+      for (int k = 0; k < 5; ++k) s.rm[k][q] = p.jm[k * p.n_pad + r];
+    }
   }
   __syncthreads();
   cl.sync();  // every CTA of the cluster runs before any writes another's shared memory
@@ -234,61 +287,61 @@ __global__ void __launch_bounds__(kCT, 1) cluster_loop_kernel(ClusterArgs p) {
     const int mine = s.cmine[me], before = s.cbefore[me];
     const unsigned long long tnb = (unsigned long long)__double_as_longlong(tn);
     list_rows(s, me, C, nr, tnb);
-    // the first iw threads (whole warps) predict the own active particles,
-    // the others the own j rows: the two global round trips overlap
-    const int iw = min(kCT, (mine + 31) & ~31);
+    // the first iw threads (whole warps) predict the own active particles, a
+    // component each, the others the own j rows
+    const int iw = min(kCT, (4 * mine + 31) & ~31);
     // own active particles: FP64 prediction (step 3), double-single i data
     // for the forces, and the corrector's inputs
-    for (int k = tid; k < mine; k += kCT) {
-      const int64_t row = s.irow[k];
-      const double t0 = p.t[row], dt0 = p.dt[row];
-      double a0[3], j0[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        a0[d] = p.a[d * p.n_pad + row];
-        j0[d] = p.jk[d * p.n_pad + row];
+    for (int e = tid; e < 4 * mine; e += kCT) {
+      const int k = e >> 2, d = e & 3;
+      const int q = s.iq[k];
+      const int64_t row = own_row(q, me, C);
+      if (d == 3) {
+        s.iC[k].y = __int_as_float((int)row);
+        continue;
       }
-      double px[3], pv[3];
-      nbh::taylor(row, p.n_pad, tn - t0, p.x, p.v, p.a, p.jk, px, pv);
-      if (k < kCC) {
-        s.cT[k] = t0;
-        s.cDT[k] = dt0;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          s.cA0[d][k] = a0[d];
-          s.cJ0[d][k] = j0[d];
-          s.cXP[d][k] = px[d];
-          s.cVP[d][k] = pv[d];
+      const int64_t g = d * p.n_pad + row;
+      const double t0 = RES ? s.rt[q] : p.t[row], a0 = RES ? s.ra[d][q] : p.a[g], j0 = RES ? s.rj[d][q] : p.jk[g];
+      double px, pv;
+      nbh::taylor1(tn - t0, RES ? s.rx[d][q] : p.x[g], RES ? s.rv[d][q] : p.v[g], a0, j0, px, pv);
+      if (RES || k < kCC) {
+        if (d == 0) {
+          s.cT[k] = t0;
+          s.cDT[k] = RES ? s.rdt[q] : p.dt[row];
         }
+        s.cA0[d][k] = a0;
+        s.cJ0[d][k] = j0;
+        s.cXP[d][k] = px;
+        s.cVP[d][k] = pv;
       } else {
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          p.xp[d * p.n_pad + row] = px[d];
-          p.vp[d * p.n_pad + row] = pv[d];
-        }
+        p.xp[g] = px;
+        p.vp[g] = pv;
       }
-      float xh[3], xl[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) nb_split(px[d], xh[d], xl[d]);
-      s.iA[k] = make_float4(xh[0], xh[1], xh[2], nb_f32(pv[0]));
-      s.iB[k] = make_float4(xl[0], xl[1], xl[2], nb_f32(pv[1]));
-      s.iC[k] = make_float2(nb_f32(pv[2]), __int_as_float((int)row));
+      float xh, xl;
+      nb_split(px, xh, xl);
+      reinterpret_cast<float*>(&s.iA[k])[d] = xh;
+      reinterpret_cast<float*>(&s.iB[k])[d] = xl;
+      const float vf = nb_f32(pv);
+      if (d == 0) s.iA[k].w = vf;
+      if (d == 1) s.iB[k].w = vf;
+      if (d == 2) s.iC[k].x = vf;
     }
     // own j rows predicted on the fly from the j-memory (Sec. 4.4 step 4)
     for (int q = (tid - iw + kCT) % kCT; q < nr; q += kCT) {
       const int64_t row = own_row(q, me, C);
-      const float4 R0 = p.jm[row], R1 = p.jm[p.n_pad + row], R2 = p.jm[2 * p.n_pad + row],
-                   R3 = p.jm[3 * p.n_pad + row], R4 = p.jm[4 * p.n_pad + row];
-      const float h = nb_f32(tn - p.t[row]);
+      float4 R[5];
+#pragma unroll
+      for (int k = 0; k < 5; ++k) R[k] = RES ? s.rm[k][q] : p.jm[k * p.n_pad + row];
+      const float h = nb_f32(tn - (RES ? s.rt[q] : p.t[row]));
       const float h2 = 2.0f * h, h15 = 1.5f * h;
       float hi, lo, vv;
-      nbk::ds_predict(R0.x, R1.x, R2.x, R3.x, R4.x, R2.w, h, h2, h15, hi, lo, vv);
+      nbk::ds_predict(R[0].x, R[1].x, R[2].x, R[3].x, R[4].x, R[2].w, h, h2, h15, hi, lo, vv);
       s.jxh[q] = hi; s.jxl[q] = lo; s.jvx[q] = vv;
-      nbk::ds_predict(R0.y, R1.y, R2.y, R3.y, R4.y, R3.w, h, h2, h15, hi, lo, vv);
+      nbk::ds_predict(R[0].y, R[1].y, R[2].y, R[3].y, R[4].y, R[3].w, h, h2, h15, hi, lo, vv);
       s.jyh[q] = hi; s.jyl[q] = lo; s.jvy[q] = vv;
-      nbk::ds_predict(R0.z, R1.z, R2.z, R3.z, R4.z, R4.w, h, h2, h15, hi, lo, vv);
+      nbk::ds_predict(R[0].z, R[1].z, R[2].z, R[3].z, R[4].z, R[4].w, h, h2, h15, hi, lo, vv);
       s.jzh[q] = hi; s.jzl[q] = lo; s.jvz[q] = vv;
-      s.jms[q] = R0.w;
+      s.jms[q] = R[0].w;
     }
     if ((nr & 1) && tid == kCT - 1) {  // the pair loop's padding row: massless, far away
       s.jxh[nr] = s.jyh[nr] = s.jzh[nr] = nbk::kFarF;
@@ -396,16 +449,22 @@ __global__ void __launch_bounds__(kCT, 1) cluster_loop_kernel(ClusterArgs p) {
       }
       // the P parts of a particle, lanes of one warp: a double-single
       // butterfly in FP32 (every lane; the FP64 pipe is 1/64 of FP32 here)
-      for (int o = P / 2; o > 0; o >>= 1)
+      if (P >= 8) {
+        float h, l;
+        const int c = nbk::ds_sum_rows(hi7, lo7, P, h, l);
+        if (i < gn && c < 7 && part == nbk::ds_row_lane(c, P)) s.part[c][i] = make_float2(h, l);
+      } else {
+        for (int o = P / 2; o > 0; o >>= 1)
 #pragma unroll
-        for (int c = 0; c < 7; ++c) {
-          const float oh = __shfl_xor_sync(0xffffffffu, hi7[c], o);
-          const float ol = __shfl_xor_sync(0xffffffffu, lo7[c], o);
-          nbk::ds_add(hi7[c], lo7[c], oh, ol);
-        }
-      if (i < gn && part == 0)
+          for (int c = 0; c < 7; ++c) {
+            const float oh = __shfl_xor_sync(0xffffffffu, hi7[c], o);
+            const float ol = __shfl_xor_sync(0xffffffffu, lo7[c], o);
+            nbk::ds_add(hi7[c], lo7[c], oh, ol);
+          }
+        if (i < gn && part == 0)
 #pragma unroll
-        for (int c = 0; c < 7; ++c) s.part[c][i] = make_float2(hi7[c], lo7[c]);
+          for (int c = 0; c < 7; ++c) s.part[c][i] = make_float2(hi7[c], lo7[c]);
+      }
       __syncthreads();
       cl.sync();  // C: every CTA's partial sums on the group are ready
 
@@ -437,17 +496,23 @@ __global__ void __launch_bounds__(kCT, 1) cluster_loop_kernel(ClusterArgs p) {
         const double a1 = have ? s.fsum[cs][fk] : 0.0, j1 = have ? s.fsum[3 + cs][fk] : 0.0;
         const double p1 = have ? s.fsum[6][fk] : 0.0;
         const int kk = have ? pos - before : lo_pos - before;  // own active index
-        const int64_t row = s.irow[kk];
+        const int q = s.iq[kk];
+        const int64_t row = own_row(q, me, C);
         nbh::CorrIn in;
-        if (kk < kCC) {
+        if (RES || kk < kCC) {
           in = nbh::CorrIn{s.cT[kk], s.cDT[kk], s.cA0[cs][kk], s.cJ0[cs][kk], s.cXP[cs][kk], s.cVP[cs][kk]};
         } else {
-          const int64_t q = cs * p.n_pad + row;
-          in = nbh::CorrIn{p.t[row], p.dt[row], p.a[q], p.jk[q], p.xp[q], p.vp[q]};
+          const int64_t g = cs * p.n_pad + row;
+          in = nbh::CorrIn{p.t[row], p.dt[row], p.a[g], p.jk[g], p.xp[g], p.vp[g]};
         }
-        const double nd = nbh::correct_lanes4(row, p.n_pad, tn, a1, j1, p1, in, p.eta, p.dt_min, p.dt_max, p.x, p.v, p.a,
-                                              p.jk, p.pot, p.t, p.dt, p.st, sub, (tid & 31) - sub, have, p.jm);
-        if (have && sub == 0) s.due[own_index(row, me, C)] = (unsigned long long)__double_as_longlong(nd);
+        double nd;
+        if constexpr (RES)
+          nd = nbh::correct_lanes4(row, p.n_pad, tn, a1, j1, p1, in, p.eta, p.dt_min, p.dt_max, p.x, p.v, p.a, p.jk,
+                                   p.pot, p.t, p.dt, p.st, sub, (tid & 31) - sub, have, p.jm, KeepRow{&s, q});
+        else
+          nd = nbh::correct_lanes4(row, p.n_pad, tn, a1, j1, p1, in, p.eta, p.dt_min, p.dt_max, p.x, p.v, p.a, p.jk,
+                                   p.pot, p.t, p.dt, p.st, sub, (tid & 31) - sub, have, p.jm);
+        if (have && sub == 0) s.due[q] = (unsigned long long)__double_as_longlong(nd);
       }
       __syncthreads();
       if (g0 + kGI < n) cl.sync();  // D: the partials are read before the next group's are written
@@ -465,7 +530,7 @@ __global__ void __launch_bounds__(kCT, 1) cluster_loop_kernel(ClusterArgs p) {
 
 struct CLoop {
   ClusterCtl* ctl = nullptr;
-  int csize = 0;  // CTAs per cluster (0 = not yet chosen)
+  int csize = 0;  // CTAs per cluster (0 = not yet chosen; with the shared memory of either kernel)
 };
 
 }  // namespace
@@ -487,12 +552,12 @@ int nb_cluster_size(nb_ctx* c) {
   }
   if (L->csize) return L->csize;
   const size_t smem = sizeof(CSmem);
-  if (cudaFuncSetAttribute(cluster_loop_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(cluster_loop_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
+  for (const void* f : {(const void*)cluster_loop_kernel<false>, (const void*)cluster_loop_kernel<true>})
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
   for (int cs : {16, 8}) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
@@ -505,8 +570,9 @@ int nb_cluster_size(nb_ctx* c) {
     cfg.dynamicSmemBytes = smem;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, cluster_loop_kernel, &cfg) == cudaSuccess && nclusters >= 1) {
+    int n0 = 0, n1 = 0;
+    if (cudaOccupancyMaxActiveClusters(&n0, cluster_loop_kernel<false>, &cfg) == cudaSuccess && n0 >= 1 &&
+        cudaOccupancyMaxActiveClusters(&n1, cluster_loop_kernel<true>, &cfg) == cudaSuccess && n1 >= 1) {
       L->csize = cs;
       return cs;
     }
@@ -563,7 +629,8 @@ int nb_integrate_cluster(nb_ctx* c, double t_end) {
   cfg.stream = c->stream;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, cluster_loop_kernel, p) != cudaSuccess) {
+  const bool res = own_count(c->n, 0, C) <= kRes;  // (CTA 0 owns the most rows)
+  if (cudaLaunchKernelEx(&cfg, res ? cluster_loop_kernel<true> : cluster_loop_kernel<false>, p) != cudaSuccess) {
     cudaGetLastError();
     return NB_ECUDA;
   }

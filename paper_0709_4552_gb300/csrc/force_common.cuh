@@ -442,6 +442,48 @@ __device__ __forceinline__ void ds_add(float& hi, float& lo, float bh, float bl)
   hi = s;
 }
 
+// Sum of 7 double-single rows over the P lanes of a group (a power of two, 8 to
+// 32, lanes of one warp; every lane calls): the butterfly's sums, bit for bit,
+// but each lane exchanges and keeps only half of its rows in the first three
+// levels, so 9 or fewer pairs cross instead of 35 (7 log2 P).  Returns the row
+// this lane holds (7: none), its sum in (h, l).
+__device__ __forceinline__ int ds_sum_rows(const float (&hi)[7], const float (&lo)[7], int P, float& h, float& l) {
+  const int lane = threadIdx.x & 31;
+  const bool u1 = (lane & (P >> 1)) != 0, u2 = (lane & (P >> 2)) != 0, u3 = (lane & (P >> 3)) != 0;
+  float a[4], b[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const float h4 = r < 3 ? hi[4 + (r < 3 ? r : 0)] : 0.0f, l4 = r < 3 ? lo[4 + (r < 3 ? r : 0)] : 0.0f;
+    a[r] = u1 ? h4 : hi[r];
+    b[r] = u1 ? l4 : lo[r];
+    const float oh = __shfl_xor_sync(0xffffffffu, u1 ? hi[r] : h4, P >> 1);
+    const float ol = __shfl_xor_sync(0xffffffffu, u1 ? lo[r] : l4, P >> 1);
+    ds_add(a[r], b[r], oh, ol);
+  }
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const float oh = __shfl_xor_sync(0xffffffffu, u2 ? a[r] : a[2 + r], P >> 2);
+    const float ol = __shfl_xor_sync(0xffffffffu, u2 ? b[r] : b[2 + r], P >> 2);
+    a[r] = u2 ? a[2 + r] : a[r];
+    b[r] = u2 ? b[2 + r] : b[r];
+    ds_add(a[r], b[r], oh, ol);
+  }
+  const float oh = __shfl_xor_sync(0xffffffffu, u3 ? a[0] : a[1], P >> 3);
+  const float ol = __shfl_xor_sync(0xffffffffu, u3 ? b[0] : b[1], P >> 3);
+  h = u3 ? a[1] : a[0];
+  l = u3 ? b[1] : b[0];
+  ds_add(h, l, oh, ol);
+  for (int o = P >> 4; o > 0; o >>= 1) {
+    const float qh = __shfl_xor_sync(0xffffffffu, h, o), ql = __shfl_xor_sync(0xffffffffu, l, o);
+    ds_add(h, l, qh, ql);
+  }
+  return (u1 ? 4 : 0) + (u2 ? 2 : 0) + (u3 ? 1 : 0);
+}
+// the lane of a group of P that ds_sum_rows leaves row r on (the lowest one)
+__device__ __forceinline__ int ds_row_lane(int r, int P) {
+  return ((r & 4) ? P >> 1 : 0) + ((r & 2) ? P >> 2 : 0) + ((r & 1) ? P >> 3 : 0);
+}
+
 // an FP64 value as a double-single pair: hi = fl32(x), lo = fl32(x - hi)
 __device__ __forceinline__ float2 ds_split(double x) {
   const float hi = __double2float_rn(x);

@@ -172,34 +172,47 @@ __device__ __forceinline__ double new_step_fp64(double t, double dt_old, double 
   return (c >= two && two <= dt_max && qq == floor(qq)) ? two : dt_old;
 }
 
+// new_step_fp64's result from the exponent eq of q = fl(fl(eta num) / den), a
+// finite normal positive: the power-of-two floor of the correctly rounded
+// square root of q is 2^floor(eq / 2) (the square root never rounds up to a
+// power of two), and crit < dt_min = 2^m exactly when eq < 2m (under).  False
+// when a step bound or dt_old is not a power of two, or t is negative or
+// subnormal.
+__device__ __forceinline__ bool step_by_exponent(int eq, double t, double dt_old, double dt_min, double dt_max,
+                                                 double& dnew, bool& under) {
+  int emin, emax, eo;
+  if (!(is_pow2(dt_min, emin) && is_pow2(dt_max, emax) && is_pow2(dt_old, eo) && emin <= emax)) return false;
+  const int s = eo + 1;  // the doubled step 2^s
+  const int mt = eq >= -1022 && eq <= 1023 ? multiple_of_pow2(t, s) : -1;
+  if (mt < 0) return false;
+  under = eq < 2 * emin;
+  int ec = (eq - (eq & 1)) / 2;  // floor(eq / 2): exponent of the criterion's floor
+  if (ec > emax) ec = emax;
+  if (ec < emin) ec = emin;
+  dnew = ec < eo ? pow2i(ec) : ((ec >= s && s <= emax && mt == 1) ? pow2i(s) : dt_old);
+  return true;
+}
+
 // new_step_fp64's result from exponents.  For positive normal N = fl(eta num)
 // and D = den, fl(N / D) has exponent e_N - e_D, less one when N's
 // significand is below D's (a quotient of 53-bit significands never rounds up
-// to a power of two), and the power-of-two floor of the correctly rounded
-// square root of q = fl(N / D) is 2^floor(e_q / 2) (the square root never
-// rounds up to a power of two either); crit < dt_min = 2^m exactly when
-// e_q < 2m.  So no division or square root is needed; they are taken (the
-// FP64 expression) only when an operand is zero, subnormal or non-finite, a
-// step bound or dt_old is not a power of two, or t is negative or subnormal.
+// to a power of two).  So no division or square root is needed; they are taken
+// (the FP64 expression) only when an operand is zero, subnormal or non-finite
+// or step_by_exponent declines.
 __device__ __forceinline__ double new_step_nd(double t, double dt_old, double num, double den, double eta,
                                               double dt_min, double dt_max, nb_dev_status* st, bool& crit_nan) {
   crit_nan = false;
-  int emin, emax, eo;
-  if (den != 0.0 && is_pow2(dt_min, emin) && is_pow2(dt_max, emax) && is_pow2(dt_old, eo) && emin <= emax) {
+  if (den != 0.0) {
     const double nq = eta * num;
     const unsigned long long bN = dbits(nq), bD = dbits(den);
     const unsigned long long EN = bN >> 52, ED = bD >> 52;  // sign bits 0 for positive operands
     if (EN >= 1 && EN <= 2046 && ED >= 1 && ED <= 2046) {
       const int eq = (int)EN - (int)ED - ((bN & 0x000FFFFFFFFFFFFFULL) < (bD & 0x000FFFFFFFFFFFFFULL) ? 1 : 0);
-      const int s = eo + 1;  // the doubled step 2^s
-      const int mt = eq >= -1022 && eq <= 1023 ? multiple_of_pow2(t, s) : -1;
-      if (mt >= 0) {
-        if (eq < 2 * emin) atomicAdd(&st->dt_underflows, 1ULL);  // crit < dt_min
-        int ec = (eq - (eq & 1)) / 2;  // floor(eq / 2): exponent of the criterion's floor
-        if (ec > emax) ec = emax;
-        if (ec < emin) ec = emin;
-        if (ec < eo) return pow2i(ec);
-        return (ec >= s && s <= emax && mt == 1) ? pow2i(s) : dt_old;
+      double dnew;
+      bool under;
+      if (step_by_exponent(eq, t, dt_old, dt_min, dt_max, dnew, under)) {
+        if (under) atomicAdd(&st->dt_underflows, 1ULL);
+        return dnew;
       }
     }
   }
@@ -215,17 +228,69 @@ __device__ __forceinline__ double new_step(double t, double dt_old, double na, d
   return new_step_nd(t, dt_old, num, den, eta, dt_min, dt_max, st, crit_nan);
 }
 
+// The square root of a positive normal s as m 2^e, m in [1, 2), in FP32 to a few
+// 2^-24; e = kNoRoot for other s.
+constexpr int kNoRoot = 1 << 20;
+struct Root {
+  float m;
+  int e;
+};
+__device__ __forceinline__ Root root_of(double s) {
+  const unsigned long long b = dbits(s);
+  const int E = (int)(b >> 52);
+  Root r;
+  const int k = E - 1023;
+  const float f = __uint_as_float((0x3F800000u | ((unsigned int)(b >> 29) & 0x7FFFFFu)) + ((unsigned int)(k & 1) << 23));
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r.m) : "f"(f));  // f in [1, 4)
+  r.e = E >= 1 && E <= 2046 ? k >> 1 : kNoRoot;
+  return r;
+}
+
+// 2^-k for k >= 0, in FP32 (at least 2^-100)
+__device__ __forceinline__ float pow2neg(int k) { return __uint_as_float((unsigned int)(127 - min(k, 100)) << 23); }
+
+// The exponent of the criterion's square, floor(log2(eta (na n2 + nj^2) / (nj n3
+// + n2^2))), from the roots of the four squared norms in FP32.  Of the
+// criterion only this exponent reaches the new step (step_by_exponent), and
+// the FP64 expression rounds a few 2^-53: so where the FP32 value (truncated
+// operands, roots, products, sums of positive terms, one reciprocal: below
+// 1.5e-6 of it, 24 units of its last place) lies more than 64 units from a power
+// of two, the FP64 expression has the same exponent.  False otherwise (15 values
+// in 10^6), and where FP64 could leave its normal range: the caller then takes
+// the FP64 roots, 16 to 60 more FP64 instructions of 64 cycles each.
+__device__ __forceinline__ bool crit_exponent(const Root& na, const Root& nj, const Root& n2, const Root& n3,
+                                              double eta, int& eq) {
+  const unsigned long long be = dbits(eta);
+  const int Ee = (int)(be >> 52) - 1023;
+  const float fe = __uint_as_float(0x3F800000u | ((unsigned int)(be >> 29) & 0x7FFFFFu));
+  const int p1 = na.e + n2.e, p2 = 2 * nj.e, q1 = nj.e + n3.e, q2 = 2 * n2.e;
+  const int P = max(p1, p2), Q = max(q1, q2);
+  const float num = na.m * n2.m * pow2neg(P - p1) + nj.m * nj.m * pow2neg(P - p2);  // [1, 8)
+  const float den = nj.m * n3.m * pow2neg(Q - q1) + n2.m * n2.m * pow2neg(Q - q2);
+  float rden;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rden) : "f"(den));
+  const unsigned int r = __float_as_uint(fe * num * rden);  // 2^-3 .. 2^4
+  const unsigned int frac = r & 0x7FFFFFu;
+  eq = (int)(r >> 23) - 127 + Ee + P - Q;
+  // (a missing root makes its sums 2^20 or so and fails the range)
+  return frac >= 64u && frac <= 0x7FFFFFu - 64u && Ee >= -1000 && Ee <= 0 && P >= -900 && P <= 900 && Q >= -900 &&
+         Q <= 900 && eq >= -1022 && eq <= 1023;
+}
+
 // Predictor (Sec. 4.1 step 3) of row i over h = t - t_i, Horner form:
 //   xp = x + v h + a h^2/2 + jk h^3/6,   vp = v + a h + jk h^2/2
+__device__ __forceinline__ void taylor1(double h, double xv, double vv, double av, double jv, double& px,
+                                        double& pv) {
+  px = xv + h * (vv + h * (0.5 * av + h * (jv * (1.0 / 6.0))));
+  pv = vv + h * (av + h * (0.5 * jv));
+}
 __device__ __forceinline__ void taylor(int64_t i, int64_t n_pad, double h, const double* __restrict__ x,
                                        const double* __restrict__ v, const double* __restrict__ a,
                                        const double* __restrict__ jk, double (&px)[3], double (&pv)[3]) {
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const int64_t q = d * n_pad + i;
-    const double xv = x[q], vv = v[q], av = a[q], jv = jk[q];
-    px[d] = xv + h * (vv + h * (0.5 * av + h * (jv * (1.0 / 6.0))));
-    pv[d] = vv + h * (av + h * (0.5 * jv));
+    taylor1(h, x[q], v[q], a[q], jk[q], px[d], pv[d]);
   }
 }
 
@@ -307,9 +372,16 @@ __device__ __forceinline__ double correct_row(int64_t i, int64_t n_pad, double t
   }
   const double p1 = f[6];
   pot[i] = p1;
-  const double na = sqrt(na2), nj = sqrt(nj2), n2 = sqrt(n22), n3 = sqrt(n32);
-  bool crit_nan;
-  const double dnew = new_step(t, dt[i], na, nj, n2, n3, eta, dt_min, dt_max, st, crit_nan);
+  const double dt0 = dt[i];
+  bool crit_nan = false, under = false;
+  int eq;
+  double dnew;
+  if (crit_exponent(root_of(na2), root_of(nj2), root_of(n22), root_of(n32), eta, eq) &&
+      step_by_exponent(eq, t, dt0, dt_min, dt_max, dnew, under)) {
+    if (under) atomicAdd(&st->dt_underflows, 1ULL);
+  } else {
+    dnew = new_step(t, dt0, sqrt(na2), sqrt(nj2), sqrt(n22), sqrt(n32), eta, dt_min, dt_max, st, crit_nan);
+  }
   if (!finite || !isfinite(p1) || crit_nan) atomicOr(&st->flags, NB_ST_NUMERIC);
   ti[i] = t;
   dt[i] = dnew;
@@ -326,8 +398,8 @@ struct CorrIn {
 // The same correction spread over four lanes of a warp: lane `sub` < 3 of
 // the group takes component `sub` (the same FP64 operations in the same order
 // as correct_row), the squared norms are gathered by shuffles and summed in
-// component order on every lane, lanes 0-3 take one square root each, and
-// lane 0 applies the step rule.  The result is correct_row's, bit for bit;
+// component order, one on each of lanes 0-3, and lane 0 applies the step rule
+// to their roots.  The result is correct_row's, bit for bit;
 // the dependent FP64 chain is about a third as long, which matters where one
 // particle's correction is the critical path of a block step.
 //
@@ -341,15 +413,23 @@ struct CorrIn {
 // valid row and write nothing).  With jm the corrected row's j-memory record
 // is written as well (write_jm_record's values; its mass word is left as it
 // is): each lane its component, lane 0 the reach once the new step is known.
+// `keep` sees what is written, for a caller that holds the rows elsewhere too.
 // Returns, on the group's lane 0 of a real row, the row's next due time
 // t + dt_new (0 elsewhere).
+struct NoKeep {
+  __device__ __forceinline__ void component(int, double, double, double, double) const {}
+  __device__ __forceinline__ void record(int, float, float, float, float, float, float) const {}
+  __device__ __forceinline__ void step(double, double) const {}
+};
+template <class Keep = NoKeep>
 __device__ __forceinline__ double correct_lanes4(int64_t i, int64_t n_pad, double t, double a1, double j1,
                                                  double p1, const CorrIn& in, double eta, double dt_min, double dt_max,
                                                  double* __restrict__ x, double* __restrict__ v,
                                                  double* __restrict__ a, double* __restrict__ jk,
                                                  double* __restrict__ pot, double* __restrict__ ti,
                                                  double* __restrict__ dt, nb_dev_status* __restrict__ st, int sub,
-                                                 int base, bool write, float4* __restrict__ jm = nullptr) {
+                                                 int base, bool write, float4* __restrict__ jm = nullptr,
+                                                 const Keep keep = Keep()) {
   const double h = t - in.t0;
   const HPow hp = h_powers(h);
   double sq[4] = {0.0, 0.0, 0.0, 0.0};  // a1^2, j1^2, a2e^2, a3^2 of this lane's component
@@ -379,9 +459,12 @@ __device__ __forceinline__ double correct_lanes4(int64_t i, int64_t n_pad, doubl
         r[4 * n_pad + c] = xl;
         r[8 * n_pad + c] = vh;
         r[12 * n_pad + c] = vl;
-        r[16 * n_pad + c] = 0.5f * nb_f32(a1);
-        r[4 * n_pad * (2 + c) + 3] = nb_f32(j1 * (1.0 / 6.0));
+        const float a2f = 0.5f * nb_f32(a1), j6f = nb_f32(j1 * (1.0 / 6.0));
+        r[16 * n_pad + c] = a2f;
+        r[4 * n_pad * (2 + c) + 3] = j6f;
+        keep.record(c, xh, xl, vh, vl, a2f, j6f);
       }
+      keep.component(c, x1, v1, a1, j1);
     }
     sq[0] = a1 * a1;
     sq[1] = j1 * j1;
@@ -418,20 +501,37 @@ __device__ __forceinline__ double correct_lanes4(int64_t i, int64_t n_pad, doubl
   const int f0 = __shfl_sync(0xffffffffu, fin, base);
   const int f1 = __shfl_sync(0xffffffffu, fin, base + 1);
   const int f2 = __shfl_sync(0xffffffffu, fin, base + 2);
-  // one square root per lane, gathered on lane 0
-  const double root = sqrt(mine);
-  const double na = __shfl_sync(0xffffffffu, root, base);
-  const double nj = __shfl_sync(0xffffffffu, root, base + 1);
-  const double n2 = __shfl_sync(0xffffffffu, root, base + 2);
-  const double n3 = __shfl_sync(0xffffffffu, root, base + 3);
+  // one root per lane, all four on every lane
+  const Root root = root_of(mine);
+  Root rt[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    rt[k].m = __shfl_sync(0xffffffffu, root.m, base + k);
+    rt[k].e = __shfl_sync(0xffffffffu, root.e, base + k);
+  }
+  int eq;
+  double dnew = in.dt0;
+  bool under = false;
+  const bool quick = crit_exponent(rt[0], rt[1], rt[2], rt[3], eta, eq) &&
+                     step_by_exponent(eq, t, in.dt0, dt_min, dt_max, dnew, under);
+  double rn[4] = {0.0, 0.0, 0.0, 0.0};
+  if (__any_sync(0xffffffffu, write && !quick)) {  // (rare) the FP64 roots
+    const double r64 = sqrt(mine);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) rn[k] = __shfl_sync(0xffffffffu, r64, base + k);
+  }
   if (!write || sub != 0) return 0.0;
   pot[i] = p1;
-  bool crit_nan;
-  const double dnew = new_step(t, in.dt0, na, nj, n2, n3, eta, dt_min, dt_max, st, crit_nan);
+  bool crit_nan = false;
+  if (!quick)
+    dnew = new_step(t, in.dt0, rn[0], rn[1], rn[2], rn[3], eta, dt_min, dt_max, st, crit_nan);
+  else if (under)
+    atomicAdd(&st->dt_underflows, 1ULL);
   const bool finite = f0 && f1 && f2;
   if (!finite || !isfinite(p1) || crit_nan) atomicOr(&st->flags, NB_ST_NUMERIC);
   ti[i] = t;
   dt[i] = dnew;
+  keep.step(t, dnew);
   if (jm) reinterpret_cast<float*>(jm + n_pad + i)[3] = reach_of(sum_ab[0], sum_ab[1], sum_ab[2], dnew);
   return t + dnew;
 }

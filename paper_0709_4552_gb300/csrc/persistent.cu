@@ -444,13 +444,32 @@ __device__ void correct_own(const LoopArgs& p, LoopSmem& s, const OwnRow& first,
 #pragma unroll
             for (int r = 0; r < 7; ++r) nbk::ds_add(hi[r], lo[r], v[u][r].x, v[u][r].y);
         }
-      for (int w = L / 2; w > 0; w >>= 1)
+      if (L >= 8) {  // each lane ends with one row; lanes 0-3 take theirs from the lanes that hold them
+        float h, lw;
+        nbk::ds_sum_rows(hi, lo, L, h, lw);
+        const int base = (int)(threadIdx.x & 31) - l, c = l < 3 ? l : 0;
 #pragma unroll
-        for (int r = 0; r < 7; ++r) {
-          const float oh = __shfl_xor_sync(0xffffffffu, hi[r], w);
-          const float ol = __shfl_xor_sync(0xffffffffu, lo[r], w);
-          nbk::ds_add(hi[r], lo[r], oh, ol);
+        for (int r = 0; r < 7; r += 3) {  // component c of the acceleration and the jerk, and the potential
+          const int from = base + nbk::ds_row_lane(r < 6 ? r + c : 6, L);
+          hi[r] = __shfl_sync(0xffffffffu, h, from);
+          lo[r] = __shfl_sync(0xffffffffu, lw, from);
         }
+      } else {
+        for (int w = L / 2; w > 0; w >>= 1)
+#pragma unroll
+          for (int r = 0; r < 7; ++r) {
+            const float oh = __shfl_xor_sync(0xffffffffu, hi[r], w);
+            const float ol = __shfl_xor_sync(0xffffffffu, lo[r], w);
+            nbk::ds_add(hi[r], lo[r], oh, ol);
+          }
+        if (L >= 4) {
+#pragma unroll
+          for (int r = 0; r < 6; r += 3) {
+            hi[r] = l == 1 ? hi[r + 1] : (l == 2 ? hi[r + 2] : hi[r]);
+            lo[r] = l == 1 ? lo[r + 1] : (l == 2 ? lo[r + 2] : lo[r]);
+          }
+        }
+      }
     } else {
 #pragma unroll
       for (int r = 0; r < 7; ++r) f[r] = 0.0;
@@ -481,10 +500,8 @@ __device__ void correct_own(const LoopArgs& p, LoopSmem& s, const OwnRow& first,
       // for 64 cycles: 3 of them instead of 7, and none of the 14 conversions)
       double a1, j1, p1;
       if (MIXED && !fin) {
-        const float ah = l == 1 ? hi[1] : (l == 2 ? hi[2] : hi[0]), al = l == 1 ? lo[1] : (l == 2 ? lo[2] : lo[0]);
-        const float jh = l == 1 ? hi[4] : (l == 2 ? hi[5] : hi[3]), jl = l == 1 ? lo[4] : (l == 2 ? lo[5] : lo[3]);
-        a1 = nb_f64(ah) + nb_f64(al);
-        j1 = nb_f64(jh) + nb_f64(jl);
+        a1 = nb_f64(hi[0]) + nb_f64(lo[0]);
+        j1 = nb_f64(hi[3]) + nb_f64(lo[3]);
         p1 = -(nb_f64(hi[6]) + nb_f64(lo[6]));
       } else {
         a1 = l == 1 ? f[1] : (l == 2 ? f[2] : f[0]);

@@ -1,5 +1,5 @@
 // selftest.cu -- device self-check of the corrector's exponent forms
-// (hermite.cuh: h_powers, mul_pow2, new_step_nd) against their FP64
+// (hermite.cuh: h_powers, mul_pow2, new_step_nd, crit_exponent) against their FP64
 // expressions (h_powers_fp64, the product by 2^k, new_step_fp64) and of the
 // FP64 <-> FP32 conversions by bits (nb_internal.cuh: nb_f32, nb_split, nb_f64)
 // against the conversion instructions, on seeded random operands, bit for bit.
@@ -110,6 +110,26 @@ __global__ void selftest_kernel(int64_t samples, uint64_t seed, unsigned long lo
       const int64_t off = (int64_t)((r5 >> 2) % 3) - 1;
       const uint64_t frac = (uint64_t)((int64_t)(nb & 0x000FFFFFFFFFFFFFULL) + off) & 0x000FFFFFFFFFFFFFULL;
       den = from_bits((nbh::dbits(den) & 0xFFF0000000000000ULL) | frac);
+    }
+    // the criterion's exponent from FP32 roots, where it decides, against the
+    // FP64 roots' quotient: squared norms over a wide range, and num and den
+    // brought next to a power-of-two quotient through one of them
+    {
+      double sq[4];
+      const uint64_t rr[4] = {r1, r2, r3, r4};
+      for (int q = 0; q < 4; ++q)
+        sq[q] = (rr[q] & 255) == 0 ? random_norm(rr[q] >> 8, r5) : make_pos(1023 - 60 + (int)((rr[q] >> 8) % 120), mix64(rr[q]));
+      if ((r0 & 3) == 0) {  // na n2 >> nj^2 and n2^2 >> nj n3: quotient eta na / n2, na from eta and n2
+        sq[1] = sq[3] = 0x1p-400;
+        const double w = sqrt(sq[2]) / eta * nbh::pow2i((int)(r5 % 40) - 20);
+        sq[0] = w * w * (1.0 + (double)((int64_t)(r5 >> 40) % 4096 - 2048) * 0x1p-30);
+      }
+      int eq;
+      if (nbh::crit_exponent(nbh::root_of(sq[0]), nbh::root_of(sq[1]), nbh::root_of(sq[2]), nbh::root_of(sq[3]), eta, eq)) {
+        const double na = sqrt(sq[0]), nj = sqrt(sq[1]), n2 = sqrt(sq[2]), n3 = sqrt(sq[3]);
+        const double q = eta * (na * n2 + nj * nj) / (nj * n3 + n2 * n2);
+        if (!(q > 0.0) || isinf(q) || (int)(nbh::dbits(q) >> 52) - 1023 != eq) atomicAdd(bad, 1ULL);
+      }
     }
     bool nan_a, nan_b;
     const double da = nbh::new_step_nd(t, dt_old, num, den, eta, dt_min, dt_max, st_fast, nan_a);
