@@ -668,9 +668,9 @@ int nb_compute_forces(nb_ctx* c, const int32_t* i_idx, int64_t n, double* acc, d
   if (r) return r;
   set_device_outputs(c, acc, jerk, pot, ptr_kind);
   const DeviceOutputsScope fo_scope{c};
-  NB_CUDA(c, cudaEventRecord(c->ev[4], c->stream));
+  if (ptr_kind == NB_PTR_HOST) NB_CUDA(c, cudaEventRecord(c->ev[4], c->stream));  // (timed only where the call waits)
   NB_CUDA(c, nb_forces(c, d_list, n));
-  NB_CUDA(c, cudaEventRecord(c->ev[5], c->stream));
+  if (ptr_kind == NB_PTR_HOST) NB_CUDA(c, cudaEventRecord(c->ev[5], c->stream));
   c->f_n = n;
   c->f_valid = true;
   c->f_list = d_list;
@@ -695,7 +695,7 @@ int nb_compute_forces_at(nb_ctx* c, double t, const int32_t* i_idx, int64_t n, d
   if ((r = caller_list(c, i_idx, n, ptr_kind, &d_list))) return r;
   set_device_outputs(c, acc, jerk, pot, ptr_kind);
   const DeviceOutputsScope fo_scope{c};
-  NB_CUDA(c, cudaEventRecord(c->ev[4], c->stream));
+  if (ptr_kind == NB_PTR_HOST) NB_CUDA(c, cudaEventRecord(c->ev[4], c->stream));  // (timed only where the call waits)
   if (c->precision == NB_MIXED) {
     if ((r = nb_jm_ensure(c))) return fail(c, r);
     const float4* boxes = nullptr;
@@ -708,7 +708,7 @@ int nb_compute_forces_at(nb_ctx* c, double t, const int32_t* i_idx, int64_t n, d
     NB_CUDA(c, nb_launch_predict(c, t, false));
     NB_CUDA(c, nb_forces(c, d_list, n));
   }
-  NB_CUDA(c, cudaEventRecord(c->ev[5], c->stream));
+  if (ptr_kind == NB_PTR_HOST) NB_CUDA(c, cudaEventRecord(c->ev[5], c->stream));
   // the listed rows now hold their prediction at t, the others an older one
   c->pred_valid = c->precision == NB_FP64;
   c->t_pred = t;
