@@ -376,18 +376,19 @@ __device__ __forceinline__ void mixed_tile_pass(const float4* __restrict__ sA, c
 // issue slots of the FP32 work.  ni* hold the NEGATED i coordinates and
 // velocity in both lanes, so x_j + (-x_i) is the scalar x_j - x_i bit for
 // bit.  The two lanes of p sum the even and the odd j of the tile.
-template <int IPT, int JT, int MODE>
+template <int IPT, int JC, int MODE, int JT>
 __device__ __forceinline__ void mixed_pair_pass(const PairTile<JT>& t, const float2 (&nxh)[IPT][3],
                                                 const float2 (&nxl)[IPT][3], const float2 (&nv)[IPT][3],
-                                                const int (&rel)[IPT], float2 eps2, float2 (&p)[IPT][7]) {
-  const float4* __restrict__ P0 = (const float4*)t.p0;
-  const float4* __restrict__ P1 = (const float4*)t.p1;
-  const float4* __restrict__ P2 = (const float4*)t.p2;
-  const float4* __restrict__ P3 = (const float4*)t.p3;
-  const float4* __restrict__ P4 = (const float4*)t.p4;
+                                                const int (&rel)[IPT], float2 eps2, float2 (&p)[IPT][7],
+                                                int j0 = 0) {
+  const float4* __restrict__ P0 = (const float4*)t.p0 + j0 / 2;
+  const float4* __restrict__ P1 = (const float4*)t.p1 + j0 / 2;
+  const float4* __restrict__ P2 = (const float4*)t.p2 + j0 / 2;
+  const float4* __restrict__ P3 = (const float4*)t.p3 + j0 / 2;
+  const float4* __restrict__ P4 = (const float4*)t.p4 + j0 / 2;
   const float2 m3 = make_float2(-3.0f, -3.0f);
   NB_PRAGMA_UNROLL(NB_MIXED_UNROLL)
-  for (int u = 0; u < JT / 2; ++u) {
+  for (int u = 0; u < JC / 2; ++u) {
     const float4 a = P0[u], b = P1[u], c = P2[u], d = P3[u];
     float4 e;
     if (MODE != kFar) e = P4[u];
@@ -490,12 +491,40 @@ __device__ __forceinline__ float2 ds_split(double x) {
   return make_float2(hi, __double2float_rn(x - (double)hi));
 }
 
+// Groups of threads that share the j of a tile (mixed_item's JG: 1, 2, 4 or 8,
+// i-tiles of 128 / JG) for n i-particles on `tiles` j-tiles with room for R
+// CTAs of 128 threads: the fewest thread slots, a slot costing 1, 1.08, 1.18 or
+// 1.45 with the groups (the shorter the runs of j, the more of a tile's time is
+// staging and folding: n = 2000 at N = 2^20 2018, 2165, 2363, 2884 us; n = 16
+// 159, 101, 70, 55; n = 48 164, 104, 121, 109; n = 160 291, 243, 224, 265); then
+// more while the items still fit one wave, as each is then only latency (n = 512
+// on 2048 16.5 -> 14.5 us, 16 on 30000 25 -> 21).
+__host__ __device__ __forceinline__ int j_groups(int64_t n, int64_t tiles, int64_t R) {
+  constexpr int kCost[4] = {100, 108, 118, 145};
+  int best = 0;
+  int64_t work = 0;
+  for (int k = 0; k < 4; ++k) {
+    const int64_t w = ((n + (128 >> k) - 1) >> (7 - k)) * (128 >> k) * kCost[k];
+    if (k == 0 || w < work) {
+      best = k;
+      work = w;
+    }
+  }
+  while (best < 3 && ((n + (64 >> best) - 1) >> (6 - best)) * tiles <= R) ++best;
+  return 1 << best;
+}
+
 // Mixed-precision item: i-tile starting at list position ibase (n entries in
 // list, entries clamped to [0, idx_hi)), j-range [jlo, jhi).  Writes 7 rows
 // out[c * ostride + pos] (final: acc, jerk, pot with its sign) or raw sums.
 // With FusedSmem the j-tiles come from the j-memory (fa) and are predicted
 // to fa.T as they are staged; the i-particles always come from jA/jB/jC.
-template <int NT, int IPT, int JT, typename SM>
+//
+// JG > 1 (few i-particles): the CTA takes NT / JG of them, and JG groups of
+// threads share the j of each tile, JT / JG each, so that a block of a few
+// particles does not leave most threads to recompute its last one; the groups'
+// double-single sums are added in group order at the end.
+template <int NT, int IPT, int JT, int JG = 1, typename SM>
 __device__ __forceinline__ void mixed_item(SM& sm, const float4* __restrict__ jA,
                                            const float4* __restrict__ jB, const float2* __restrict__ jC,
                                            int64_t jlo, int64_t jhi, int64_t idx_hi,
@@ -511,7 +540,10 @@ __device__ __forceinline__ void mixed_item(SM& sm, const float4* __restrict__ jA
   // order); results always go to the list positions.  tbox (optional):
   // boxes of every NB_BOX_TILE slots from slot box_origin on (j-ranges start
   // at box_origin plus a multiple of JT), which allow the far-tile pass.
-  const int tid = threadIdx.x;
+  constexpr int NI = NT / JG, JC = JT / JG;  // i-particles of the CTA (IPT = 1) and j of a group and tile
+  static_assert(JG == 1 || (IPT == 1 && NB_MIXED_DS_FOLD && NB_MIXED_PACKED), "groups: one i per thread, packed loop");
+  static_assert(sizeof(SM) >= (JG - 1) * 7 * NI * sizeof(float2), "room for the groups' sums");
+  const int tid = threadIdx.x, il = JG == 1 ? tid : tid % NI, jg = JG == 1 ? 0 : tid / NI;
   float xh[IPT][3], xl[IPT][3], vi[IPT][3];
   int64_t self[IPT];
 #if NB_MIXED_DS_FOLD
@@ -546,7 +578,7 @@ __device__ __forceinline__ void mixed_item(SM& sm, const float4* __restrict__ jA
 #endif
 #pragma unroll
   for (int k = 0; k < IPT; ++k) {
-    int64_t pos = ibase + k * NT + tid;
+    int64_t pos = ibase + k * NI + il;
     if (pos >= n) pos = n - 1;
     if (ord) pos = ord[pos];
     int64_t p = list[pos];
@@ -653,8 +685,8 @@ __device__ __forceinline__ void mixed_item(SM& sm, const float4* __restrict__ jA
     bool hit = false;
 #pragma unroll
     for (int k = 0; k < IPT; ++k) {
-      const int64_t d = self[k] - jt;
-      rel[k] = (d >= 0 && d < JT) ? (int)d : -1;
+      const int64_t d = self[k] - (jt + jg * JC);
+      rel[k] = (d >= 0 && d < JC) ? (int)d : -1;
       hit = hit || rel[k] >= 0;
     }
     float p[IPT][7];
@@ -692,11 +724,11 @@ __device__ __forceinline__ void mixed_item(SM& sm, const float4* __restrict__ jA
 #pragma unroll
         for (int c = 0; c < 7; ++c) p2[k][c] = make_float2(0.0f, 0.0f);
       if (__any_sync(0xffffffffu, hit))
-        mixed_pair_pass<IPT, JT, kSelf>(pt, nxh, nxl, nv, rel, e2, p2);
+        mixed_pair_pass<IPT, JC, kSelf>(pt, nxh, nxl, nv, rel, e2, p2, jg * JC);
       else if (__all_sync(0xffffffffu, far))
-        mixed_pair_pass<IPT, JT, kFar>(pt, nxh, nxl, nv, rel, e2, p2);
+        mixed_pair_pass<IPT, JC, kFar>(pt, nxh, nxl, nv, rel, e2, p2, jg * JC);
       else
-        mixed_pair_pass<IPT, JT, kNear>(pt, nxh, nxl, nv, rel, e2, p2);
+        mixed_pair_pass<IPT, JC, kNear>(pt, nxh, nxl, nv, rel, e2, p2, jg * JC);
 #pragma unroll
       for (int k = 0; k < IPT; ++k)
 #pragma unroll
@@ -718,6 +750,26 @@ __device__ __forceinline__ void mixed_item(SM& sm, const float4* __restrict__ jA
   }
   cp_async_wait<0>();
 
+#if NB_MIXED_DS_FOLD
+  if constexpr (JG > 1) {
+    float2* red = reinterpret_cast<float2*>(&sm);
+    __syncthreads();  // no copy into the tiles is in flight
+    if (jg > 0)
+#pragma unroll
+      for (int c = 0; c < 7; ++c) red[((jg - 1) * 7 + c) * NI + il] = NB_ACC_DS(0, c);
+    __syncthreads();
+    if (jg == 0)
+#pragma unroll
+      for (int q = 0; q < JG - 1; ++q)
+#pragma unroll
+        for (int c = 0; c < 7; ++c) {
+          const float2 v = red[(q * 7 + c) * NI + il];
+          ds_add(acc_hi[0][c], acc_lo[0][c], v.x, v.y);
+        }
+    __syncthreads();  // (another item may load its tiles)
+  }
+#endif
+
   // final results (one split): FP64 with the potential's sign; partial sums
   // of a split: FP64, or with ds_out the double-single pair (hi, lo) in the
   // same 8-byte slot (no FP64 instruction: the FP64 pipe issues a warp
@@ -726,8 +778,8 @@ __device__ __forceinline__ void mixed_item(SM& sm, const float4* __restrict__ jA
   float2* out2 = reinterpret_cast<float2*>(out);
 #pragma unroll
   for (int k = 0; k < IPT; ++k) {
-    int64_t pos = ibase + k * NT + tid;
-    if (pos >= n) continue;
+    int64_t pos = ibase + k * NI + il;
+    if (pos >= n || jg > 0) continue;
     if (ord) pos = ord[pos];
     if (ds_out && !finalize) {
 #pragma unroll

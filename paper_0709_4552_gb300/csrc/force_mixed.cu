@@ -6,6 +6,8 @@
 // partials [split][7][n] (an FP32 pair per 8-byte slot) that the split-j
 // reduction sums in FP32, in a fixed order (deterministic for a given launch
 // configuration), and converts to FP64 once per result.
+#include <algorithm>
+
 #include "force_common.cuh"
 
 namespace {
@@ -21,7 +23,7 @@ namespace {
 #define NB_MIXED_BOUNDS(NT, IPT) __launch_bounds__(NT)
 #endif
 
-template <int NT, int IPT, int JT>
+template <int NT, int IPT, int JT, int JG = 1>
 __global__ void NB_MIXED_BOUNDS(NT, IPT) force_mixed_kernel(
     const float4* __restrict__ jA, const float4* __restrict__ jB, const float2* __restrict__ jC,
     int64_t n_j, const int32_t* __restrict__ list, int64_t n, int64_t tiles, float eps2,
@@ -32,13 +34,13 @@ __global__ void NB_MIXED_BOUNDS(NT, IPT) force_mixed_kernel(
   const int64_t jlo = nbk::split_begin(split, gridDim.y, tiles) * JT;
   const int64_t jhi = min(nbk::split_begin(split + 1, gridDim.y, tiles) * JT, n_j);
   double* o = finalize ? out : out + (int64_t)split * 7 * ostride;
-  nbk::mixed_item<NT, IPT, JT>(sm, jA, jB, jC, jlo, jhi, n_j, list, n, (int64_t)blockIdx.x * (NT * IPT),
+  nbk::mixed_item<NT, IPT, JT, JG>(sm, jA, jB, jC, jlo, jhi, n_j, list, n, (int64_t)blockIdx.x * (NT / JG * IPT),
                                eps2, o, ostride, finalize != 0, tbox, ord, 0, nbk::FusedArgs(), is, true);
 }
 
 // the same item with on-the-fly prediction of the j-tiles from the j-memory
 // (Sec. 4.4 step 4); the i-particles' predicted rows are in jA/jB/jC
-template <int NT, int JT>
+template <int NT, int JT, int JG>
 __global__ void __launch_bounds__(NT) force_mixed_fused_kernel(
     const float4* __restrict__ jA, const float4* __restrict__ jB, const float2* __restrict__ jC,
     int64_t n_j, const int32_t* __restrict__ list, int64_t n, int64_t tiles, float eps2,
@@ -55,29 +57,55 @@ __global__ void __launch_bounds__(NT) force_mixed_fused_kernel(
   fa.stride = jm_stride;
   fa.tj = tj;
   fa.T = T;
-  nbk::mixed_item<NT, 1, JT>(sm, jA, jB, jC, jlo, jhi, n_j, list, n, (int64_t)blockIdx.x * NT, eps2, o, ostride,
+  nbk::mixed_item<NT, 1, JT, JG>(sm, jA, jB, jC, jlo, jhi, n_j, list, n, (int64_t)blockIdx.x * (NT / JG), eps2, o, ostride,
                              finalize != 0, tbox, ord, 0, fa, nbk::ISrc(), true);
 }
 
-// resident CTAs per SM of an instantiation (0 when the query fails)
+// resident CTAs per SM of a kernel (0 when the query fails); `kept`: the
+// caller's place for the answer, which is the same for every call
+int resident(const void* kernel, int threads, int& kept) {
+  if (kept == 0 && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&kept, kernel, threads, 0) != cudaSuccess) {
+    cudaGetLastError();
+    kept = 0;
+  }
+  return kept;
+}
+
 template <int NT, int IPT, int JT>
 int per_sm_of() {
   static int per_sm = 0;
-  if (per_sm == 0 &&
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, force_mixed_kernel<NT, IPT, JT>, NT, 0) != cudaSuccess) {
-    cudaGetLastError();
-    per_sm = 0;
-  }
-  return per_sm;
+  return resident((const void*)force_mixed_kernel<NT, IPT, JT>, NT, per_sm);
+}
+
+// the j-splits of a launch of shape cfg (an explicit count, or as many items as
+// fill the GPU; of a single i-tile one wave: its items are short, and a second
+// wave would start them all over)
+int splits_for(const nb_ctx* c, int64_t n, const nb_tuning& cfg, int per_sm) {
+  if (cfg.nsplit > 0) return cfg.nsplit;
+  const int s = nb_auto_split(c, n, cfg, per_sm);
+  return n <= (int64_t)cfg.threads * cfg.ipt ? std::min(s, std::max(1, per_sm) * c->sm_count) : s;
 }
 
 template <int NT, int IPT, int JT>
 cudaError_t launch(nb_ctx* c, const int32_t* d_list, int64_t n, const nb_tuning& cfg, float eps2,
                    const int32_t* ord, const nbk::ISrc& is) {
-  const int per_sm = per_sm_of<NT, IPT, JT>();
+  auto kernel = force_mixed_kernel<NT, IPT, JT>;
+  int per_sm = per_sm_of<NT, IPT, JT>();
+  nb_tuning shape = cfg;
+  if constexpr (NT == 128 && IPT == 1 && JT == 128) {
+    static int kept[3] = {0, 0, 0};
+    const int jg = nbk::j_groups(n, (c->n + JT - 1) / JT, per_sm * (int64_t)c->sm_count);
+    if (jg > 1) {
+      kernel = jg == 8   ? force_mixed_kernel<NT, IPT, JT, 8>
+               : jg == 4 ? force_mixed_kernel<NT, IPT, JT, 4>
+                         : force_mixed_kernel<NT, IPT, JT, 2>;
+      per_sm = resident((const void*)kernel, NT, kept[jg == 8 ? 2 : jg / 4]);
+      shape.threads = NT / jg;
+    }
+  }
   if (per_sm == 0) return cudaErrorInvalidValue;
-  int nsplit = cfg.nsplit > 0 ? cfg.nsplit : nb_auto_split(c, n, cfg, per_sm);
-  const int64_t per_cta = (int64_t)NT * IPT;
+  int nsplit = splits_for(c, n, shape, per_sm);
+  const int64_t per_cta = (int64_t)shape.threads * IPT;
   const int64_t itiles = (n + per_cta - 1) / per_cta;
   const int64_t n_j = ((c->n + JT - 1) / JT) * JT;  // padding particles (m = 0) fill the last tile
   const int64_t tiles = n_j / JT;
@@ -92,8 +120,8 @@ cudaError_t launch(nb_ctx* c, const int32_t* d_list, int64_t n, const nb_tuning&
   // resident spatial order: far-tile boxes when the tiles match (unless the
   // context asks for double-single differences on every tile)
   const float4* tbox = (c->perm_valid && c->far_tiles) ? c->tbox : nullptr;
-  force_mixed_kernel<NT, IPT, JT><<<grid, NT, 0, c->stream>>>(c->jA, c->jB, c->jC, n_j, d_list, n, tiles,
-                                                              eps2, out, ostride, fin ? 1 : 0, tbox, ord, is);
+  kernel<<<grid, NT, 0, c->stream>>>(c->jA, c->jB, c->jC, n_j, d_list, n, tiles, eps2, out, ostride, fin ? 1 : 0,
+                                     tbox, ord, is);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || fin) return e;
   return nb_launch_split_reduce_ds(c, n, nsplit, ostride);
@@ -108,15 +136,20 @@ cudaError_t nb_forces_mixed_fused(nb_ctx* c, const int32_t* d_list, int64_t n, c
                                   const int32_t* ord, double T, const float4* boxes) {
   constexpr int NT = 128, JT = 128;
   if (n <= 0) return cudaSuccess;
-  static int per_sm = 0;
-  if (per_sm == 0 &&
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, force_mixed_fused_kernel<NT, JT>, NT, 0) != cudaSuccess)
-    return cudaGetLastError();
-  const nb_tuning shape{1, NT, JT, cfg.nsplit};
-  int nsplit = cfg.nsplit > 0 ? cfg.nsplit : nb_auto_split(c, n, shape, per_sm);
-  const int64_t itiles = (n + NT - 1) / NT;
+  static int kept[4] = {0, 0, 0, 0};
   const int64_t n_j = ((c->n + JT - 1) / JT) * JT;
   const int64_t tiles = n_j / JT;
+  const int per_sm1 = resident((const void*)force_mixed_fused_kernel<NT, JT, 1>, NT, kept[0]);
+  const int jg = nbk::j_groups(n, tiles, per_sm1 * (int64_t)c->sm_count);
+  auto kernel = jg == 8   ? force_mixed_fused_kernel<NT, JT, 8>
+                : jg == 4 ? force_mixed_fused_kernel<NT, JT, 4>
+                : jg == 2 ? force_mixed_fused_kernel<NT, JT, 2>
+                          : force_mixed_fused_kernel<NT, JT, 1>;
+  const int per_sm = resident((const void*)kernel, NT, kept[jg == 8 ? 3 : jg / 2]);
+  if (per_sm == 0) return cudaErrorInvalidValue;
+  const nb_tuning shape{1, NT / jg, JT, cfg.nsplit};
+  int nsplit = splits_for(c, n, shape, per_sm);
+  const int64_t itiles = (n + shape.threads - 1) / shape.threads;
   if (nsplit > tiles) nsplit = (int)tiles;
   if (nsplit < 1) nsplit = 1;
   const bool fin = nsplit == 1;
@@ -125,7 +158,7 @@ cudaError_t nb_forces_mixed_fused(nb_ctx* c, const int32_t* d_list, int64_t n, c
   if (!fin && (int64_t)nsplit * 7 * ostride > c->part_elems) return cudaErrorInvalidValue;
   c->launches += fin ? 1 : 2;
   const float eps2 = (float)(c->eps * c->eps);
-  force_mixed_fused_kernel<NT, JT><<<dim3((unsigned)itiles, (unsigned)nsplit), NT, 0, c->stream>>>(
+  kernel<<<dim3((unsigned)itiles, (unsigned)nsplit), NT, 0, c->stream>>>(
       c->jA, c->jB, c->jC, n_j, d_list, n, tiles, eps2, out, ostride, fin ? 1 : 0, boxes, ord, c->jm, c->n_pad,
       c->t, T);
   cudaError_t e = cudaGetLastError();

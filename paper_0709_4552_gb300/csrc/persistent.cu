@@ -12,7 +12,8 @@
 //     its own offset in the active list; it writes its own active rows there
 //     (ascending), predicts its own rows to t (step 3) and, on the mixed path
 //     in spatial order, computes the boxes of its own tiles.    -> barrier B
-//   phase 2: force items (i-tile of 128 list positions x j-split; step 4,
+//   phase 2: force items (i-tile of 128 list positions, fewer on the mixed
+//     path when groups of threads share a tile's j, x j-split; step 4,
 //     Eq. 3), the first by the CTA's place in an order that fills the SMs
 //     evenly, the others from a work counter; the same items as the
 //     host-driven kernels, split partials as double-single pairs. -> barrier C
@@ -345,13 +346,24 @@ __device__ void predict_rows(const LoopArgs& p, int64_t r0, int64_t r1, double t
   }
 }
 
+// groups of threads that share the j of an item's tile (a step's i-tile is kLT
+// divided by them), and the i-tiles
+template <bool MIXED>
+__device__ __forceinline__ int loop_groups(int64_t n, int64_t jtiles, unsigned int G) {
+  return MIXED ? nbk::j_groups(n, jtiles, G) : 1;
+}
+__device__ __forceinline__ int64_t loop_itiles(int64_t n, int groups) {
+  const int ni = kLT / groups;
+  return (n + ni - 1) / ni;
+}
+
 // split-j factor of a step: a few force items per CTA (taken
 // from a counter, so uneven items even out), at least one j-tile per split,
 // at most kLMaxSplits splits (their sums are the corrector phase's loads),
 // within the partial-sum scratch
 template <bool MIXED>
-__device__ __forceinline__ int64_t loop_splits(int64_t n, int64_t jtiles, unsigned int G, int64_t part_elems) {
-  const int64_t nI = (n + kLT - 1) / kLT;
+__device__ __forceinline__ int64_t loop_splits(int64_t n, int64_t nI, int64_t jtiles, unsigned int G,
+                                               int64_t part_elems) {
   int64_t S = ((int64_t)(MIXED ? kLItemWavesMixed : kLItemWaves64) * G + nI - 1) / nI;
   if (S > jtiles) S = jtiles;
   if (S > kLMaxSplits) S = kLMaxSplits;
@@ -410,7 +422,7 @@ __device__ void correct_own(const LoopArgs& p, LoopSmem& s, const OwnRow& first,
   const int mycnt = s.mycnt;
   const double tn = __longlong_as_double((long long)s.tnb);
   const int64_t n = s.total;
-  const int64_t S = loop_splits<MIXED>(n, jtiles, G, p.part_elems);
+  const int64_t S = loop_splits<MIXED>(n, loop_itiles(n, loop_groups<MIXED>(n, jtiles, G)), jtiles, G, p.part_elems);
   const int64_t pstride = ((n + 31) / 32) * 32;
   const bool fin = S == 1;
   const bool cached = r1 - r0 <= kLDue;
@@ -608,8 +620,9 @@ __global__ void __launch_bounds__(kLT, PER_SM) loop_kernel(LoopArgs p) {
     // by its place (when there are no more items than CTAs, as in every small
     // block, that is all, without counter round trips); the rest come from the
     // step's counter.
-    const int64_t nI = (n + kLT - 1) / kLT;
-    const int64_t S = loop_splits<MIXED>(n, jtiles, G, p.part_elems);
+    const int groups = loop_groups<MIXED>(n, jtiles, G);
+    const int64_t nI = loop_itiles(n, groups);
+    const int64_t S = loop_splits<MIXED>(n, nI, jtiles, G, p.part_elems);
     const int64_t pstride = ((n + 31) / 32) * 32;
     const bool fin = S == 1;
     const int items = (int)(nI * S);
@@ -623,9 +636,21 @@ __global__ void __launch_bounds__(kLT, PER_SM) loop_kernel(LoopArgs p) {
       const int64_t jhi = min(nbk::split_begin(split + 1, S, jtiles) * JT, MIXED ? n_j : N);
       double* out = fin ? p.F : p.part + split * 7 * pstride;
       const int64_t ostride = fin ? p.n_pad : pstride;
-      if constexpr (MIXED)
-        nbk::mixed_item<kLT, 1, JT>(fsm, p.jA, p.jB, p.jC, jlo, jhi, n_j, p.act, n, itile * kLT, p.eps2f,
-                                         out, ostride, fin, p.tbox, nullptr, 0, nbk::FusedArgs(), nbk::ISrc(), true);
+      if constexpr (MIXED) {
+        const int64_t ibase = (int64_t)itile * (kLT / groups);
+#define NB_LOOP_ITEM(JG)                                                                                              \
+  nbk::mixed_item<kLT, 1, JT, JG>(fsm, p.jA, p.jB, p.jC, jlo, jhi, n_j, p.act, n, ibase, p.eps2f, out, ostride, fin, \
+                                  p.tbox, nullptr, 0, nbk::FusedArgs(), nbk::ISrc(), true)
+        if (groups == 8)
+          NB_LOOP_ITEM(8);
+        else if (groups == 4)
+          NB_LOOP_ITEM(4);
+        else if (groups == 2)
+          NB_LOOP_ITEM(2);
+        else
+          NB_LOOP_ITEM(1);
+#undef NB_LOOP_ITEM
+      }
       else
         nbk::fp64_item<kLT, JT>(fsm, p.xp, p.vp, p.m, p.n_pad, 1, jlo, jhi, p.n_pad, p.act, n, itile * kLT,
                                      p.eps2, out, ostride, fin);
