@@ -514,6 +514,22 @@ __host__ __device__ __forceinline__ int j_groups(int64_t n, int64_t tiles, int64
   return 1 << best;
 }
 
+// The same for the FP64 item: groups are whole warps, so 1, 2 or 4 of them and
+// i-tiles of 128, 64 or 32; without groups the warps past n compute nothing, so
+// a partial i-tile counts its warps, at least three (N = 200000, n = 16 193, 154,
+// 131 us; n = 64 257, 216, 240; n = 96 320, 353, 331; n = 160 600, 518, 507; n =
+// 320 979, 876, 927; n = 1000 2679, 2705, 2848).  More groups only while the
+// items leave SMs empty (N = 1500, n = 16 39, 27, 23; n = 448 39, 33, 37; the
+// staging of a tile is the same work for fewer pairs).
+__host__ __device__ __forceinline__ int j_groups64(int64_t n, int64_t tiles, int64_t sms) {
+  const int64_t part = n & 127;
+  const int64_t w0 = (n - part + (part == 0 ? 0 : (part <= 96 ? 96 : 128))) * 100;
+  const int64_t w1 = ((n + 63) >> 6) * 64 * 103, w2 = ((n + 31) >> 5) * 32 * 110;
+  int k = w0 <= w1 && w0 <= w2 ? 0 : (w1 <= w2 ? 1 : 2);
+  while (k < 2 && ((n + (64 >> k) - 1) >> (6 - k)) * tiles <= sms) ++k;
+  return 1 << k;
+}
+
 // Mixed-precision item: i-tile starting at list position ibase (n entries in
 // list, entries clamped to [0, idx_hi)), j-range [jlo, jhi).  Writes 7 rows
 // out[c * ostride + pos] (final: acc, jerk, pot with its sign) or raw sums.
@@ -943,7 +959,10 @@ __device__ __forceinline__ uint32_t fx64_chunk(const Fp64Smem<NT, JT>& sm, int q
 // integers, are folded into FP64 every kFold pairs and not per tile.  It
 // depends on the j-range alone and on nothing the other i of the CTA hold, so
 // a particle's result does not depend on which particles share its item.
-template <int NT, int JT>
+//
+// JG > 1: groups of NT / JG threads (whole warps) share the j of each tile, as in
+// mixed_item; their 96-bit sums are on one grid and add exactly.
+template <int NT, int JT, int JG = 1>
 __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __restrict__ xp,
                                           const double* __restrict__ vp, const double* __restrict__ m, int64_t cs,
                                           int64_t js, int64_t jlo, int64_t jhi, int64_t idx_hi,
@@ -951,9 +970,11 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
                                           double* __restrict__ out, int64_t ostride, bool finalize,
                                           const ISrc is = ISrc()) {
   static_assert(JT % 32 == 0 && NT % 32 == 0, "tiles of whole warps");
+  constexpr int NI = NT / JG, JC = JT / JG;  // i-particles of the CTA, j of a group and tile
+  static_assert(NI % 32 == 0, "a group is whole warps");
   constexpr int kPer = (JT + NT - 1) / NT;  // j-particles a thread stages
-  const int tid = threadIdx.x;
-  const int64_t pos0 = ibase + tid;
+  const int tid = threadIdx.x, il = JG == 1 ? tid : tid % NI, jg = JG == 1 ? 0 : tid / NI;
+  const int64_t pos0 = ibase + il;
   const int64_t pos = pos0 < n ? pos0 : n - 1;
   int64_t self = list[pos];
   const double *xi, *vi;  // this i's position and velocity, read again when its grid changes
@@ -986,7 +1007,7 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
   fi.wmin = wmin;
   // a warp whose list positions all lie past n computes nothing (its
   // results are not written); it still loads its share of every j-tile
-  const bool wact = ibase + (int64_t)(tid & ~31) < n;
+  const bool wact = ibase + (int64_t)(il & ~31) < n;
 
   for (int64_t jt = jlo; jt < jhi; jt += JT) {
     double jx[kPer][3], jv[kPer][3], jm[kPer];
@@ -1090,9 +1111,10 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
     const int64_t d = self - jt;
     const int rel = d >= 0 && d < qn ? (int)d : -1;
     const bool shifted = __any_sync(0xffffffffu, (fi.kx | fi.kv) != 0);
+    const int qe = JG == 1 ? qn : min(qn, (jg + 1) * JC);
 #pragma unroll 1
-    for (int q0 = 0; q0 < qn; q0 += 32, ++chunk) {
-      const int count = min(32, qn - q0);
+    for (int q0 = jg * JC; q0 < qe; q0 += 32, ++chunk) {
+      const int count = min(32, qe - q0);
       uint32_t left = 0xffffffffu >> (32 - count);
       // an i that left most pairs of a chunk to FP64 (a system far from the
       // origin against its size, say) leaves all of them for the next ones,
@@ -1110,9 +1132,44 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
                    eps2, state);
     }
   }
-  if (filled > 0) fp64_fold(sm, a, in_range, (state & kHighUsed) == 0, g, gv, EM);
+  if constexpr (JG > 1) {
+    // the groups' sums to group 0: what they hold in FP64 (early folds, pairs
+    // left to FP64; rare), then, through the same slots, the 96-bit sums, which
+    // are on one grid for all groups of an i and add exactly
+    if (__syncthreads_or(jg > 0 && state != 0)) {
+      if (jg == 0)
+#pragma unroll 1
+        for (int q = 1; q < JG; ++q)
+#pragma unroll
+          for (int c = 0; c < 7; ++c) {
+            sum_add(sm.hi[c][il], sm.lo[c][il], sm.hi[c][q * NI + il]);
+            sm.lo[c][il] += sm.lo[c][q * NI + il];
+          }
+      state |= kHighUsed;
+      __syncthreads();
+    }
+    if (jg > 0)
+#pragma unroll
+      for (int c = 0; c < 7; ++c) {
+        sm.hi[c][tid] = __longlong_as_double((long long)(((uint64_t)a[c].w1 << 32) | a[c].w0));
+        sm.lo[c][tid] = __longlong_as_double((long long)a[c].w2);
+      }
+    __syncthreads();
+    if (jg == 0)
+#pragma unroll
+      for (int q = 1; q < JG; ++q)
+#pragma unroll
+        for (int c = 0; c < 7; ++c) {
+          const uint64_t b = (uint64_t)__double_as_longlong(sm.hi[c][q * NI + il]);
+          const uint64_t l = (((uint64_t)a[c].w1 << 32) | a[c].w0) + b;
+          a[c].w2 += (uint32_t)__double_as_longlong(sm.lo[c][q * NI + il]) + (l < b ? 1u : 0u);
+          a[c].w1 = (uint32_t)(l >> 32);
+          a[c].w0 = (uint32_t)l;
+        }
+  }
+  if (filled > 0 && jg == 0) fp64_fold(sm, a, in_range, (state & kHighUsed) == 0, g, gv, EM);
   __syncthreads();  // the caller may reuse shared memory for its next item
-  if (pos0 >= n) return;
+  if (pos0 >= n || jg > 0) return;
 #pragma unroll
   for (int c = 0; c < 6; ++c) out[c * ostride + pos0] = sm.hi[c][tid] + sm.lo[c][tid];
   const double w = sm.hi[6][tid] + sm.lo[6][tid];

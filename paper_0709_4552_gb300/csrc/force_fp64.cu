@@ -8,7 +8,7 @@
 
 namespace {
 
-template <int NT, int JT>
+template <int NT, int JT, int JG = 1>
 // 16 warps per SM (128 registers): measured best of 12, 16 and 20
 __global__ void __launch_bounds__(NT, 512 / NT) force_fp64_kernel(
     const double* __restrict__ xp, const double* __restrict__ vp, const double* __restrict__ m,
@@ -21,18 +21,31 @@ __global__ void __launch_bounds__(NT, 512 / NT) force_fp64_kernel(
   const int64_t jlo = nbk::split_begin(split, gridDim.y, tiles) * JT;
   const int64_t jhi = min(nbk::split_begin(split + 1, gridDim.y, tiles) * JT, N);
   double* o = finalize ? out : out + (int64_t)split * 7 * ostride;
-  nbk::fp64_item<NT, JT>(sm, xp, vp, m, n_pad, 1, jlo, jhi, n_pad, list, n, (int64_t)blockIdx.x * NT, eps2, o,
-                         ostride, finalize != 0, is);
+  nbk::fp64_item<NT, JT, JG>(sm, xp, vp, m, n_pad, 1, jlo, jhi, n_pad, list, n, (int64_t)blockIdx.x * (NT / JG), eps2,
+                             o, ostride, finalize != 0, is);
 }
 
 template <int NT, int JT>
 cudaError_t launch(nb_ctx* c, const int32_t* d_list, int64_t n, const nb_tuning& cfg, const nbk::ISrc& is) {
-  static int per_sm = 0;  // resident CTAs per SM of this instantiation
+  static int per_sm = 0;  // resident CTAs per SM of this instantiation (with groups too: same bounds)
   if (per_sm == 0 && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, force_fp64_kernel<NT, JT>, NT, 0) !=
                          cudaSuccess)
     return cudaGetLastError();
-  int nsplit = cfg.nsplit > 0 ? cfg.nsplit : nb_auto_split(c, n, cfg, per_sm);
-  const int64_t itiles = (n + NT - 1) / NT;
+  auto kernel = force_fp64_kernel<NT, JT>;
+  nb_tuning shape = cfg;
+  if constexpr (NT == 128 && JT == 64) {
+    // (an explicit split count asks for exactly that launch, whose results depend
+    // on nothing but the j-range; the automatic one depends on n anyway)
+    const int jg =
+        cfg.nsplit > 0 ? 1 : nbk::j_groups64(n, (c->n + JT - 1) / JT, c->sm_count);
+    if (jg > 1) kernel = jg == 4 ? force_fp64_kernel<NT, JT, 4> : force_fp64_kernel<NT, JT, 2>;
+    shape.threads = NT / jg;
+  }
+  int nsplit = cfg.nsplit > 0 ? cfg.nsplit : nb_auto_split(c, n, shape, per_sm);
+  // a single i-tile of fewer than NT in one wave (N = 200000, n = 16 145 -> 131 us, n = 64 228 -> 216; but n =
+  // 96 320 -> 337, n = 128 385 -> 396)
+  if (cfg.nsplit <= 0 && shape.threads < NT && n <= shape.threads) nsplit = std::min(nsplit, per_sm * c->sm_count);
+  const int64_t itiles = (n + shape.threads - 1) / shape.threads;
   const int64_t n_j = ((c->n + JT - 1) / JT) * JT;
   const int64_t tiles = n_j / JT;
   if (nsplit > tiles) nsplit = (int)tiles;
@@ -43,8 +56,8 @@ cudaError_t launch(nb_ctx* c, const int32_t* d_list, int64_t n, const nb_tuning&
   if (!fin && (int64_t)nsplit * 7 * ostride > c->part_elems) return cudaErrorInvalidValue;
   dim3 grid((unsigned)itiles, (unsigned)nsplit);
   c->launches += fin ? 1 : 2;
-  force_fp64_kernel<NT, JT><<<grid, NT, 0, c->stream>>>(c->xp, c->vp, c->m, c->n_pad, c->n, d_list, n,
-                                                        tiles, c->eps * c->eps, out, ostride, fin ? 1 : 0, is);
+  kernel<<<grid, NT, 0, c->stream>>>(c->xp, c->vp, c->m, c->n_pad, c->n, d_list, n, tiles, c->eps * c->eps, out,
+                                     ostride, fin ? 1 : 0, is);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || fin) return e;
   return nb_launch_split_reduce(c, n, nsplit, ostride);

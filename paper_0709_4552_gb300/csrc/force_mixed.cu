@@ -94,7 +94,8 @@ cudaError_t launch(nb_ctx* c, const int32_t* d_list, int64_t n, const nb_tuning&
   nb_tuning shape = cfg;
   if constexpr (NT == 128 && IPT == 1 && JT == 128) {
     static int kept[3] = {0, 0, 0};
-    const int jg = nbk::j_groups(n, (c->n + JT - 1) / JT, per_sm * (int64_t)c->sm_count);
+    // (an explicit split count asks for exactly that launch)
+    const int jg = cfg.nsplit > 0 ? 1 : nbk::j_groups(n, (c->n + JT - 1) / JT, per_sm * (int64_t)c->sm_count);
     if (jg > 1) {
       kernel = jg == 8   ? force_mixed_kernel<NT, IPT, JT, 8>
                : jg == 4 ? force_mixed_kernel<NT, IPT, JT, 4>
@@ -140,7 +141,7 @@ cudaError_t nb_forces_mixed_fused(nb_ctx* c, const int32_t* d_list, int64_t n, c
   const int64_t n_j = ((c->n + JT - 1) / JT) * JT;
   const int64_t tiles = n_j / JT;
   const int per_sm1 = resident((const void*)force_mixed_fused_kernel<NT, JT, 1>, NT, kept[0]);
-  const int jg = nbk::j_groups(n, tiles, per_sm1 * (int64_t)c->sm_count);
+  const int jg = cfg.nsplit > 0 ? 1 : nbk::j_groups(n, tiles, per_sm1 * (int64_t)c->sm_count);
   auto kernel = jg == 8   ? force_mixed_fused_kernel<NT, JT, 8>
                 : jg == 4 ? force_mixed_fused_kernel<NT, JT, 4>
                 : jg == 2 ? force_mixed_fused_kernel<NT, JT, 2>

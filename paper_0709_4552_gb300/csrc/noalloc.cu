@@ -30,6 +30,7 @@ namespace {
 
 constexpr int kNT = 128;  // i-particles per CTA (one per thread)
 constexpr int kJT = 64;   // j-particles per shared-memory tile
+constexpr int kPerSm = 512 / kNT;  // resident CTAs per SM
 constexpr int kMaxDevices = 64;
 
 __device__ __align__(256) double g_scratch[NB_NOALLOC_SCRATCH_DOUBLES];
@@ -69,7 +70,8 @@ unsigned long long current_context_id() {
 // The library's FP64 force item (Sec. 4.1 step 4, Eq. 3) on row-major [N][3]
 // caller arrays: CTA (x, y) = (i-tile, j-split); partial sums of split y go
 // to part[y][7][pstride].  The self pair (j == i) is excluded by index.
-__global__ void __launch_bounds__(kNT, 512 / kNT) noalloc_force_kernel(int64_t N, const double* __restrict__ m,
+template <int JG>
+__global__ void __launch_bounds__(kNT, kPerSm) noalloc_force_kernel(int64_t N, const double* __restrict__ m,
                                                             const double* __restrict__ x,
                                                             const double* __restrict__ v, double eps2,
                                                             const int32_t* __restrict__ list, int64_t n,
@@ -77,8 +79,8 @@ __global__ void __launch_bounds__(kNT, 512 / kNT) noalloc_force_kernel(int64_t N
                                                             int64_t pstride) {
   __shared__ nbk::Fp64Smem<kNT, kJT> sm;
   const int64_t jlo = (int64_t)blockIdx.y * j_per_split;
-  nbk::fp64_item<kNT, kJT>(sm, x, v, m, 1, 3, jlo, min(jlo + j_per_split, N), N, list, n, (int64_t)blockIdx.x * kNT,
-                           eps2, part + (int64_t)blockIdx.y * 7 * pstride, pstride, false);
+  nbk::fp64_item<kNT, kJT, JG>(sm, x, v, m, 1, 3, jlo, min(jlo + j_per_split, N), N, list, n,
+                               (int64_t)blockIdx.x * (kNT / JG), eps2, part + (int64_t)blockIdx.y * 7 * pstride, pstride, false);
 }
 
 // device address of the scratch array for the current device (set up once)
@@ -117,11 +119,13 @@ extern "C" int nb_forces_fp64_noalloc(int64_t N, const double* m, const double* 
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
     return NB_ECUDA;
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  const int64_t itiles = (n + kNT - 1) / kNT;
   const int64_t pstride = ((n + 31) / 32) * 32;
   const int64_t tiles = (N + kJT - 1) / kJT;
-  // enough CTAs for about four waves, at least one j-tile per split, within the scratch
-  int64_t nsplit = (16 * (int64_t)sms + itiles - 1) / itiles;
+  const int jg = nbk::j_groups64(n, tiles, sms), ni = kNT / jg;
+  const int64_t itiles = (n + ni - 1) / ni;
+  // enough CTAs for about four waves (one for a single i-tile of fewer than
+  // kNT), at least one j-tile per split, within the scratch
+  int64_t nsplit = ((itiles > 1 || jg == 1 ? 4 : 1) * kPerSm * (int64_t)sms + itiles - 1) / itiles;
   const int64_t cap = NB_NOALLOC_SCRATCH_DOUBLES / (7 * pstride);
   if (nsplit > cap) nsplit = cap;
   if (nsplit > tiles) nsplit = tiles;
@@ -129,8 +133,9 @@ extern "C" int nb_forces_fp64_noalloc(int64_t N, const double* m, const double* 
   if (nsplit < 1) nsplit = 1;
   const int64_t tps = (tiles + nsplit - 1) / nsplit;
   nsplit = (tiles + tps - 1) / tps;
-  noalloc_force_kernel<<<dim3((unsigned)itiles, (unsigned)nsplit), kNT, 0, s>>>(N, m, x, v, eps * eps, i_idx, n,
-                                                                                tps * kJT, scratch, pstride);
+  auto kernel = jg == 4 ? noalloc_force_kernel<4> : (jg == 2 ? noalloc_force_kernel<2> : noalloc_force_kernel<1>);
+  kernel<<<dim3((unsigned)itiles, (unsigned)nsplit), kNT, 0, s>>>(N, m, x, v, eps * eps, i_idx, n, tps * kJT, scratch,
+                                                                  pstride);
   if (cudaGetLastError() != cudaSuccess) return NB_ECUDA;
   if (nbk::launch_split_reduce((const double*)scratch, pstride, (int)nsplit, n, (double*)nullptr, 0, acc, jerk, pot,
                                sms, s) != cudaSuccess)

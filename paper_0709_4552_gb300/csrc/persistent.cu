@@ -347,7 +347,9 @@ __device__ void predict_rows(const LoopArgs& p, int64_t r0, int64_t r1, double t
 }
 
 // groups of threads that share the j of an item's tile (a step's i-tile is kLT
-// divided by them), and the i-tiles
+// divided by them), and the i-tiles.  (FP64: none, as the item's two more forms
+// cost the loop registers: N = 1024 with one shared step 48.7 -> 49.9 us, N =
+// 4096 45.3 -> 46.7, and 31.0 -> 31.1 for the small blocks of N = 1024.)
 template <bool MIXED>
 __device__ __forceinline__ int loop_groups(int64_t n, int64_t jtiles, unsigned int G) {
   return MIXED ? nbk::j_groups(n, jtiles, G) : 1;
@@ -636,8 +638,8 @@ __global__ void __launch_bounds__(kLT, PER_SM) loop_kernel(LoopArgs p) {
       const int64_t jhi = min(nbk::split_begin(split + 1, S, jtiles) * JT, MIXED ? n_j : N);
       double* out = fin ? p.F : p.part + split * 7 * pstride;
       const int64_t ostride = fin ? p.n_pad : pstride;
+      const int64_t ibase = (int64_t)itile * (kLT / groups);
       if constexpr (MIXED) {
-        const int64_t ibase = (int64_t)itile * (kLT / groups);
 #define NB_LOOP_ITEM(JG)                                                                                              \
   nbk::mixed_item<kLT, 1, JT, JG>(fsm, p.jA, p.jB, p.jC, jlo, jhi, n_j, p.act, n, ibase, p.eps2f, out, ostride, fin, \
                                   p.tbox, nullptr, 0, nbk::FusedArgs(), nbk::ISrc(), true)
@@ -650,10 +652,10 @@ __global__ void __launch_bounds__(kLT, PER_SM) loop_kernel(LoopArgs p) {
         else
           NB_LOOP_ITEM(1);
 #undef NB_LOOP_ITEM
+      } else {
+        nbk::fp64_item<kLT, JT>(fsm, p.xp, p.vp, p.m, p.n_pad, 1, jlo, jhi, p.n_pad, p.act, n, ibase, p.eps2, out,
+                                ostride, fin);
       }
-      else
-        nbk::fp64_item<kLT, JT>(fsm, p.xp, p.vp, p.m, p.n_pad, 1, jlo, jhi, p.n_pad, p.act, n, itile * kLT,
-                                     p.eps2, out, ostride, fin);
       if (kPlaced && items <= (int)G) break;
       item = next_item(p, s, kPlaced ? (int)G : 0);
     }
