@@ -930,8 +930,7 @@ void launch_force(nb_ctx* c, Batch* b, bool mixed) {
         b->item_off, b->part_off, b->pstride, c->F, c->n_pad, c->part, b->wq);
 }
 
-cudaError_t body_after_plan(nb_ctx* c, Batch* b, bool own_time) {
-  const bool mixed = c->precision == NB_MIXED;
+cudaError_t launch_predict(nb_ctx* c, Batch* b, bool own_time) {
   if (single_boxes(c, b) || cluster_boxes(c, b)) {
     const bool cl = cluster_boxes(c, b);
     const int64_t tiles = cl ? b->ntiles : (b->N + NB_BOX_TILE - 1) / NB_BOX_TILE;
@@ -941,8 +940,14 @@ cudaError_t body_after_plan(nb_ctx* c, Batch* b, bool own_time) {
   } else {
     b_predict<<<grid_for(b->N, 256, c->sm_count * 16), 256, 0, c->stream>>>(
         b->N, c->n_pad, b->cid, b->nact, b->tnext, own_time ? 1 : 0, c->m, c->x, c->v, c->a, c->jk, c->t, c->xp, c->vp,
-        c->jA, c->jB, c->jC, 1, mixed ? 1 : 0);
+        c->jA, c->jB, c->jC, 1, c->precision == NB_MIXED ? 1 : 0);
   }
+  c->launches += 1;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_forces(nb_ctx* c, Batch* b) {
+  const bool mixed = c->precision == NB_MIXED;
   if (b->nt == 32)
     launch_force<32>(c, b, mixed);
   else if (b->nt == 64)
@@ -951,12 +956,31 @@ cudaError_t body_after_plan(nb_ctx* c, Batch* b, bool own_time) {
     launch_force<128>(c, b, mixed);
   b_reduce<<<c->sm_count * std::max(1, 2048 / (224 * kRedLanes)), dim3(32, 7, kRedLanes), 0, c->stream>>>(
       b->C, b->off, b->nact, b->nsplit, b->part_off, b->pstride, b->ritem_off, c->part, c->F, c->n_pad);
-  c->launches += 3;
+  c->launches += 2;
   return cudaGetLastError();
 }
 
-// one block step of every active cluster, all on the device
-cudaError_t capture_step(nb_ctx* c, Batch* b, cudaGraphConditionalHandle handle, int use_handle) {
+// a second stream of a capture and the events that fork to it and join it
+struct Fork {
+  cudaStream_t stream = nullptr;
+  cudaEvent_t out = nullptr, back = nullptr;
+  cudaError_t create() {
+    cudaError_t e = cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&out, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&back, cudaEventDisableTiming);
+    return e;
+  }
+  ~Fork() {
+    if (out) cudaEventDestroy(out);
+    if (back) cudaEventDestroy(back);
+    if (stream) cudaStreamDestroy(stream);
+  }
+};
+
+// one block step of every active cluster, all on the device.  The plan (one
+// CTA) needs the selection, the prediction too, and the forces both: the plan
+// takes a branch of its own beside the prediction (NB_T_FORK).
+cudaError_t capture_step(nb_ctx* c, Batch* b, cudaGraphConditionalHandle handle, int use_handle, const Fork& fork) {
   const bool mixed = c->precision == NB_MIXED;
   const int per_cta = b->nt * (mixed ? kMixIPT : 1);
   const int jt = mixed ? kMixJT : kF64JT;
@@ -965,13 +989,21 @@ cudaError_t capture_step(nb_ctx* c, Batch* b, cudaGraphConditionalHandle handle,
   b_sel_write<<<b->nchunks, kSelThreads, 0, c->stream>>>(b->ch_cluster, b->ch_lo, b->ch_hi, b->cl_ch0, b->ch_min,
                                                          b->ch_cnt, b->off, c->t, c->dt, b->tnext, b->ctrl, b->prm,
                                                          c->act, b->nact, c->status);
-  b_plan<<<1, kPlanThreads, 0, c->stream>>>(b->C, b->off, b->nact, per_cta, jt, b->waves * (int64_t)grid, c->part_elems,
-                                    b->itiles, b->nsplit, b->jps, b->item_off, b->part_off, b->pstride,
-                                    b->ritem_off, b->citem_off, b->wq, b->ctrl,
-                                    b->prm, c->status, handle, use_handle);
   cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaEventRecord(fork.out, c->stream);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(fork.stream, fork.out, 0);
   if (e != cudaSuccess) return e;
-  if ((e = body_after_plan(c, b, false)) != cudaSuccess) return e;
+  b_plan<<<1, kPlanThreads, 0, fork.stream>>>(b->C, b->off, b->nact, per_cta, jt, b->waves * (int64_t)grid,
+                                              c->part_elems, b->itiles, b->nsplit, b->jps, b->item_off, b->part_off,
+                                              b->pstride, b->ritem_off, b->citem_off, b->wq, b->ctrl, b->prm,
+                                              c->status, handle, use_handle);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaEventRecord(fork.back, fork.stream);
+  const cudaError_t ep = launch_predict(c, b, false);
+  if (e == cudaSuccess) e = ep;
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, fork.back, 0);
+  if (e == cudaSuccess) e = launch_forces(c, b);
+  if (e != cudaSuccess) return e;
   b_correct<<<c->sm_count * 16, 4 * kCorrItem, 0, c->stream>>>(b->C, c->n_pad, b->citem_off, b->off, b->nact, b->tnext,
                                                            c->act, c->F, c->n_pad, b->prm, c->x, c->v, c->a, c->jk,
                                                            c->pot, c->t, c->dt, c->xp, c->vp, c->status);
@@ -1008,6 +1040,8 @@ cudaError_t build_graph(nb_ctx* c, Batch* b, bool pick = true) {
   // default stream, which cannot be captured); the graph runs on c->stream
   cudaStream_t cap = nullptr;
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
+  Fork fork;
+  if (e == cudaSuccess) e = fork.create();
   if (e == cudaSuccess) {
     cudaGraph_t body = np.conditional.phGraph_out[0];
     e = cudaStreamBeginCaptureToGraph(cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
@@ -1015,7 +1049,7 @@ cudaError_t build_graph(nb_ctx* c, Batch* b, bool pick = true) {
       const int64_t launches = c->launches;
       cudaStream_t own = c->stream;
       c->stream = cap;
-      cudaError_t ec = capture_step(c, b, h, 1);
+      cudaError_t ec = capture_step(c, b, h, 1, fork);
       c->stream = own;
       c->launches = launches;
       cudaGraph_t got = nullptr;
@@ -1097,7 +1131,8 @@ cudaError_t all_forces(nb_ctx* c, Batch* b) {
   cudaError_t e = plan_only(c, b);
   if (e != cudaSuccess) return e;
   c->launches += 2;
-  return body_after_plan(c, b, true);
+  e = launch_predict(c, b, true);
+  return e == cudaSuccess ? launch_forces(c, b) : e;
 }
 
 // copy rows [src + o, src + o + n) of every SoA array between contexts
