@@ -90,7 +90,7 @@ struct Batch {
   int nt = 128;                    // i-tile (threads per CTA) of the force items: 32, 64 or 128
   int waves = kItemWaves;          // force items planned per resident CTA (sets the split-j length)
   int64_t nc_median = 0;           // median cluster size (the autotuner's bin)
-  int grid_mixed = 0, grid_fp64 = 0;
+  int grid_mixed = 0, grid_fp64 = 0, grid_few = 0;
   cudaGraphExec_t exec = nullptr;
   int64_t exec_key = -1;           // precision, far-tile pass and item shape the graph was built for
   nb_ctx* child = nullptr;         // per-cluster reference path
@@ -487,10 +487,11 @@ __global__ void __launch_bounds__(NT, mixed_min_ctas(NT)) b_force_mixed(
     const int32_t* __restrict__ nsplit, const int64_t* __restrict__ jps, const int64_t* __restrict__ item_off,
     const int64_t* __restrict__ part_off, const int64_t* __restrict__ pstride, double* __restrict__ F,
     int64_t fstride, double* __restrict__ part, const float4* __restrict__ tbox,
-    const int64_t* __restrict__ tile_off, unsigned long long* __restrict__ wq) {
+    const int64_t* __restrict__ tile_off, unsigned long long* __restrict__ wq, int few) {
   __shared__ __align__(16) nbk::MixedSmem<JT> sm;
   __shared__ int s_item;
   const int total = (int)item_off[C];
+  if (total <= few) return;  // b_force_mixed_few has them
   for (;;) {
     const int item = next_item(wq, &s_item);
     if (item >= total) break;
@@ -506,6 +507,42 @@ __global__ void __launch_bounds__(NT, mixed_min_ctas(NT)) b_force_mixed(
     nbk::mixed_item<NT, IPT, JT>(sm, jA, jB, jC, jlo, jhi, n_pad, act + off[c], nact[c], itile * (NT * IPT),
                                  eps2f[c], out, fin ? fstride : pstride[c], fin, tb, nullptr,
                                  tile_off ? off[c] : 0);
+  }
+}
+
+// The same for a step of few items of the ensemble's shape (i-tiles of 32; at
+// most `few` items, else b_force_mixed<32> has them): such a step is the latency
+// of an item, one warp's 64 trips round the pair loop and more, so here the four
+// warps of a CTA share each item's j-tiles (mixed_item's groups).  16 clusters of
+// 256-1024: 43.4 -> 32.4 us a step, 128 of 256-512: 49.3 -> 38.7.  The line lies
+// at kFewWaves items per CTA (128 clusters with 1, 2, 4: 41.2, 38.3, 38.0).  (One
+// kernel with both forms costs the other registers: 241k rows in 96 clusters
+// 134.6 -> 140.5.)
+constexpr int kFewNT = 128, kFewWaves = 4;
+template <int JT>
+__global__ void __launch_bounds__(kFewNT) b_force_mixed_few(
+    int32_t C, const int64_t* __restrict__ off, const float* __restrict__ eps2f, int64_t n_pad,
+    const float4* __restrict__ jA, const float4* __restrict__ jB, const float2* __restrict__ jC,
+    const int32_t* __restrict__ act, const int32_t* __restrict__ nact, const int32_t* __restrict__ itiles,
+    const int32_t* __restrict__ nsplit, const int64_t* __restrict__ jps, const int64_t* __restrict__ item_off,
+    const int64_t* __restrict__ part_off, const int64_t* __restrict__ pstride, double* __restrict__ F,
+    int64_t fstride, double* __restrict__ part, const float4* __restrict__ tbox,
+    const int64_t* __restrict__ tile_off, int few) {
+  __shared__ __align__(16) nbk::MixedSmem<JT> sm;
+  const int total = (int)item_off[C];
+  if (total > few) return;
+  for (int item = blockIdx.x; item < total; item += gridDim.x) {
+    const int c = find_cluster(item_off, C, item);
+    const int local = item - (int)item_off[c], it = itiles[c];
+    const int64_t split = local / it, itile = local - split * it;
+    const int64_t jlo = off[c] + split * jps[c];
+    const int64_t jhi = min(jlo + jps[c], off[c + 1]);
+    const bool fin = nsplit[c] == 1;
+    double* out = fin ? F + off[c] : part + part_off[c] + split * 7 * pstride[c];
+    const float4* tb = tbox ? (tile_off ? tbox + 2 * tile_off[c] : tbox) : nullptr;
+    nbk::mixed_item<kFewNT, 1, JT, kFewNT / 32>(sm, jA, jB, jC, jlo, jhi, n_pad, act + off[c], nact[c], itile * 32,
+                                                eps2f[c], out, fin ? fstride : pstride[c], fin, tb, nullptr,
+                                                tile_off ? off[c] : 0);
   }
 }
 
@@ -761,11 +798,12 @@ __global__ void fill_cid(int64_t N, const int64_t* __restrict__ off, int32_t C, 
 // i-tile and planned items per CTA of the force items; the persistent grids
 // hold as many CTAs as fit on the SMs at that i-tile
 cudaError_t set_shape(nb_ctx* c, Batch* b, int nt, int waves) {
-  int pm = 0, pf = 0;
+  int pm = 0, pf = 0, pw = 0;
   cudaError_t e;
   if (nt == 32) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pm, b_force_mixed<32, kMixIPT, kMixJT>, 32, 0);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pf, b_force_fp64<32, kF64JT>, 32, 0);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pw, b_force_mixed_few<kMixJT>, kFewNT, 0);
   } else if (nt == 64) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pm, b_force_mixed<64, kMixIPT, kMixJT>, 64, 0);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pf, b_force_fp64<64, kF64JT>, 64, 0);
@@ -780,6 +818,7 @@ cudaError_t set_shape(nb_ctx* c, Batch* b, int nt, int waves) {
   b->waves = waves;
   b->grid_mixed = std::max(1, pm) * c->sm_count;
   b->grid_fp64 = std::max(1, pf) * c->sm_count;
+  b->grid_few = std::max(1, pw) * c->sm_count;
   return cudaSuccess;
 }
 
@@ -917,17 +956,27 @@ bool cluster_boxes(const nb_ctx* c, const Batch* b) {
 }
 
 template <int NT>
-void launch_force(nb_ctx* c, Batch* b, bool mixed) {
-  if (mixed)
+void launch_force(nb_ctx* c, Batch* b, bool mixed, cudaStream_t side) {
+  if (mixed) {
+    const float4* tbox = !c->far_tiles ? nullptr
+                         : single_boxes(c, b) ? c->tbox : (cluster_boxes(c, b) ? b->tbox : nullptr);
+    const int64_t* tile_off = cluster_boxes(c, b) ? b->tile_off : nullptr;
+    const int few = NT == 32 ? kFewWaves * b->grid_few : 0;
     b_force_mixed<NT, kMixIPT, kMixJT><<<b->grid_mixed, NT, 0, c->stream>>>(
         b->C, b->off, b->eps2f, c->n_pad, c->jA, c->jB, c->jC, c->act, b->nact, b->itiles, b->nsplit, b->jps,
-        b->item_off, b->part_off, b->pstride, c->F, c->n_pad, c->part,
-        !c->far_tiles ? nullptr : single_boxes(c, b) ? c->tbox : (cluster_boxes(c, b) ? b->tbox : nullptr),
-        cluster_boxes(c, b) ? b->tile_off : nullptr, b->wq);
-  else
+        b->item_off, b->part_off, b->pstride, c->F, c->n_pad, c->part, tbox, tile_off, b->wq, few);
+    if (NT == 32) {
+      b_force_mixed_few<kMixJT><<<b->grid_few, kFewNT, 0, side>>>(
+          b->C, b->off, b->eps2f, c->n_pad, c->jA, c->jB, c->jC, c->act, b->nact, b->itiles, b->nsplit, b->jps,
+          b->item_off, b->part_off, b->pstride, c->F, c->n_pad, c->part, tbox, tile_off, few);
+      c->launches += 1;
+    }
+  } else {
     b_force_fp64<NT, kF64JT><<<b->grid_fp64, NT, 0, c->stream>>>(
         b->C, b->off, b->eps2d, c->n_pad, c->xp, c->vp, c->m, c->act, b->nact, b->itiles, b->nsplit, b->jps,
         b->item_off, b->part_off, b->pstride, c->F, c->n_pad, c->part, b->wq);
+  }
+  c->launches += 1;
 }
 
 cudaError_t launch_predict(nb_ctx* c, Batch* b, bool own_time) {
@@ -943,20 +992,6 @@ cudaError_t launch_predict(nb_ctx* c, Batch* b, bool own_time) {
         c->jA, c->jB, c->jC, 1, c->precision == NB_MIXED ? 1 : 0);
   }
   c->launches += 1;
-  return cudaGetLastError();
-}
-
-cudaError_t launch_forces(nb_ctx* c, Batch* b) {
-  const bool mixed = c->precision == NB_MIXED;
-  if (b->nt == 32)
-    launch_force<32>(c, b, mixed);
-  else if (b->nt == 64)
-    launch_force<64>(c, b, mixed);
-  else
-    launch_force<128>(c, b, mixed);
-  b_reduce<<<c->sm_count * std::max(1, 2048 / (224 * kRedLanes)), dim3(32, 7, kRedLanes), 0, c->stream>>>(
-      b->C, b->off, b->nact, b->nsplit, b->part_off, b->pstride, b->ritem_off, c->part, c->F, c->n_pad);
-  c->launches += 2;
   return cudaGetLastError();
 }
 
@@ -977,9 +1012,40 @@ struct Fork {
   }
 };
 
+// fork: the second stream of a capture (null: everything on the context's)
+cudaError_t launch_forces(nb_ctx* c, Batch* b, const Fork* fork) {
+  const bool mixed = c->precision == NB_MIXED;
+  cudaError_t e = cudaSuccess;
+  cudaStream_t side = c->stream;
+  if (fork) {
+    side = fork->stream;
+    e = cudaEventRecord(fork->out, c->stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(side, fork->out, 0);
+    if (e != cudaSuccess) return e;
+  }
+  if (b->nt == 32)
+    launch_force<32>(c, b, mixed, side);
+  else if (b->nt == 64)
+    launch_force<64>(c, b, mixed, side);
+  else
+    launch_force<128>(c, b, mixed, side);
+  e = cudaGetLastError();
+  if (fork) {
+    if (e == cudaSuccess) e = cudaEventRecord(fork->back, side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, fork->back, 0);
+  }
+  if (e != cudaSuccess) return e;
+  b_reduce<<<c->sm_count * std::max(1, 2048 / (224 * kRedLanes)), dim3(32, 7, kRedLanes), 0, c->stream>>>(
+      b->C, b->off, b->nact, b->nsplit, b->part_off, b->pstride, b->ritem_off, c->part, c->F, c->n_pad);
+  c->launches += 1;
+  return cudaGetLastError();
+}
+
 // one block step of every active cluster, all on the device.  The plan (one
 // CTA) needs the selection, the prediction too, and the forces both: the plan
-// takes a branch of its own beside the prediction (NB_T_FORK).
+// takes a branch of its own beside the prediction (16 small clusters 46.8 -> 43.0 us
+// a step), and so do the two force kernels of the ensemble's shape, one of which
+// finds nothing to do.
 cudaError_t capture_step(nb_ctx* c, Batch* b, cudaGraphConditionalHandle handle, int use_handle, const Fork& fork) {
   const bool mixed = c->precision == NB_MIXED;
   const int per_cta = b->nt * (mixed ? kMixIPT : 1);
@@ -1002,7 +1068,7 @@ cudaError_t capture_step(nb_ctx* c, Batch* b, cudaGraphConditionalHandle handle,
   const cudaError_t ep = launch_predict(c, b, false);
   if (e == cudaSuccess) e = ep;
   if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, fork.back, 0);
-  if (e == cudaSuccess) e = launch_forces(c, b);
+  if (e == cudaSuccess) e = launch_forces(c, b, &fork);
   if (e != cudaSuccess) return e;
   b_correct<<<c->sm_count * 16, 4 * kCorrItem, 0, c->stream>>>(b->C, c->n_pad, b->citem_off, b->off, b->nact, b->tnext,
                                                            c->act, c->F, c->n_pad, b->prm, c->x, c->v, c->a, c->jk,
@@ -1113,7 +1179,7 @@ int run_graph(nb_ctx* c, Batch* b, double t_end) {
     c->steps += steps;
     c->perm_age += (int)steps;
     c->interactions += (double)inter;
-    c->launches += iters * 7;
+    c->launches += iters * (c->precision == NB_MIXED && b->nt == 32 ? 8 : 7);
     total += iters;
     if (!more) break;
     if (total > cap) return NB_ETIMEOUT;  // cannot happen for valid block steps
@@ -1132,7 +1198,7 @@ cudaError_t all_forces(nb_ctx* c, Batch* b) {
   if (e != cudaSuccess) return e;
   c->launches += 2;
   e = launch_predict(c, b, true);
-  return e == cudaSuccess ? launch_forces(c, b) : e;
+  return e == cudaSuccess ? launch_forces(c, b, nullptr) : e;
 }
 
 // copy rows [src + o, src + o + n) of every SoA array between contexts
