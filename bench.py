@@ -827,10 +827,12 @@ def main():
         fp64_rate = float(k) * N / (e0.elapsed_time(e1) / 1e3)
         s.set_precision(prec)
         pk = s.measure_peaks()
-        # the FP64 item issues 32 FP64-pipe instructions per interaction (source count)
+        # the FP64 item's pair runs in 64-bit fixed point on the integer units; in FP64 arithmetic
+        # it would be 32 FP64-pipe instructions per interaction (source count)
         extra["fp64_gpu_path"] = {"value": fp64_rate, "unit": UNIT,
                                   "sample": f"{k} active x N={N}", "vs_mixed": fp64_rate / value * ws,
-                                  "fp64_pipe_frac": fp64_rate * 32 / (pk["fp64_tflops"] * 1e12 / 2)}
+                                  "arithmetic": "64-bit fixed point",
+                                  "vs_fp64_pipe_bound": fp64_rate * 32 / (pk["fp64_tflops"] * 1e12 / 2)}
         # how the FP64 unit issues (cycles per FMA for one warp, dependent chain with 32 or 1
         # lanes, four chains; SM cycles per warp instruction with 16 warps)
         pk["fp64_issue_cycles"] = s.measure_fp64_issue()

@@ -49,9 +49,11 @@ extern "C" {
 #define NB_ESTATE    -7   /* call out of order (e.g. forces before predict) */
 
 /* ---- force-path precision ---------------------------------------------- */
-#define NB_FP64   0  /* IEEE FP64 pairwise arithmetic; 1/s from an FP32 seed
-                        refined in FP64 (any s^2 > 0; s^2 = 0 only for the
-                        self pair, which is excluded by index)                 */
+#define NB_FP64   0  /* FP64 inputs, sums and results; the pair arithmetic in
+                        64-bit fixed point, at least as accurate as FP64
+                        arithmetic (any s^2 > 0; s^2 = 0 only for the self
+                        pair, which is excluded by index); pairs that the
+                        fixed-point formats do not hold are taken in FP64      */
 #define NB_MIXED  1  /* FP32 pairwise arithmetic on double-single position
                         differences; the FP32 sum over each j-tile is folded
                         into a double-single (FP32 hi + lo, TwoSum)
@@ -328,8 +330,7 @@ int nb_step(nb_ctx* ctx, double* t_out, int64_t* n_active_out);
  *                       for the context's precision and N: the cluster loop
  *                       for mixed systems of N <= 2048 (where the GPU
  *                       co-schedules the cluster), the persistent loop up to
- *                       N = 131072 (mixed) or 2048 (FP64, whose force phase
- *                       outweighs the step overhead sooner), the host loop
+ *                       N = 131072 (mixed) or 2048 (FP64), the host loop
  *                       beyond.
  * All of them take the same block steps with the same per-particle arithmetic;
  * sums over j-splits may group differently.  The mixed path renews its
@@ -429,8 +430,9 @@ int nb_get_far_tiles(nb_ctx* ctx, int* enabled);
 /*
  * nb_selftest_corrector -- device self-check of the corrector's exact
  * shortcuts (Sec. 4.1 step 5): the powers of a power-of-two step and the
- * power-of-two step rule taken from exponent bits instead of FP64 products,
- * division and square root.  On `samples` seeded random operand sets (steps,
+ * power-of-two step rule taken from exponent bits and FP32 roots instead of
+ * FP64 products, division and square roots, and FP64 <-> FP32 conversions by
+ * bits.  On `samples` seeded random operand sets (steps,
  * norms, times, step bounds; boundary, zero, subnormal, infinite and NaN
  * cases included) each shortcut is compared bit for bit with its FP64
  * expression on `device`; *mismatches receives the number of differences

@@ -790,7 +790,7 @@ __device__ __forceinline__ void mixed_item(SM& sm, const float4* __restrict__ jA
   // of a split: FP64, or with ds_out the double-single pair (hi, lo) in the
   // same 8-byte slot (no FP64 instruction: the FP64 pipe issues a warp
   // instruction every 64 cycles per warp on this GPU), which the split
-  // reduction sums in FP32 (split_reduce_ds)
+  // reduction sums in FP32
   float2* out2 = reinterpret_cast<float2*>(out);
 #pragma unroll
   for (int k = 0; k < IPT; ++k) {

@@ -1,7 +1,8 @@
 // force_mixed.cu -- host-driven launch of the mixed-precision force item
 // (force_common.cuh; Sec. 4.1 step 4, Eq. 3) for sm_103a.
 //
-// Grid: (i-tiles of NT*IPT active particles) x (j-range splits).  With one
+// Grid: (i-tiles of NT*IPT active particles, fewer in small blocks whose
+// threads share the j of a tile) x (j-range splits).  With one
 // split the item writes final results into F; otherwise double-single
 // partials [split][7][n] (an FP32 pair per 8-byte slot) that the split-j
 // reduction sums in FP32, in a fixed order (deterministic for a given launch
@@ -57,8 +58,8 @@ __global__ void __launch_bounds__(NT) force_mixed_fused_kernel(
   fa.stride = jm_stride;
   fa.tj = tj;
   fa.T = T;
-  nbk::mixed_item<NT, 1, JT, JG>(sm, jA, jB, jC, jlo, jhi, n_j, list, n, (int64_t)blockIdx.x * (NT / JG), eps2, o, ostride,
-                             finalize != 0, tbox, ord, 0, fa, nbk::ISrc(), true);
+  nbk::mixed_item<NT, 1, JT, JG>(sm, jA, jB, jC, jlo, jhi, n_j, list, n, (int64_t)blockIdx.x * (NT / JG), eps2, o,
+                                 ostride, finalize != 0, tbox, ord, 0, fa, nbk::ISrc(), true);
 }
 
 // resident CTAs per SM of a kernel (0 when the query fails); `kept`: the

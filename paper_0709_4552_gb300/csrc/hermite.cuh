@@ -240,7 +240,8 @@ __device__ __forceinline__ Root root_of(double s) {
   const int E = (int)(b >> 52);
   Root r;
   const int k = E - 1023;
-  const float f = __uint_as_float((0x3F800000u | ((unsigned int)(b >> 29) & 0x7FFFFFu)) + ((unsigned int)(k & 1) << 23));
+  const unsigned int m = 0x3F800000u | ((unsigned int)(b >> 29) & 0x7FFFFFu);
+  const float f = __uint_as_float(m + ((unsigned int)(k & 1) << 23));
   asm("sqrt.approx.f32 %0, %1;" : "=f"(r.m) : "f"(f));  // f in [1, 4)
   r.e = E >= 1 && E <= 2046 ? k >> 1 : kNoRoot;
   return r;

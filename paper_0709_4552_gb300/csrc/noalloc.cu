@@ -80,7 +80,8 @@ __global__ void __launch_bounds__(kNT, kPerSm) noalloc_force_kernel(int64_t N, c
   __shared__ nbk::Fp64Smem<kNT, kJT> sm;
   const int64_t jlo = (int64_t)blockIdx.y * j_per_split;
   nbk::fp64_item<kNT, kJT, JG>(sm, x, v, m, 1, 3, jlo, min(jlo + j_per_split, N), N, list, n,
-                               (int64_t)blockIdx.x * (kNT / JG), eps2, part + (int64_t)blockIdx.y * 7 * pstride, pstride, false);
+                               (int64_t)blockIdx.x * (kNT / JG), eps2, part + (int64_t)blockIdx.y * 7 * pstride,
+                               pstride, false);
 }
 
 // device address of the scratch array for the current device (set up once)

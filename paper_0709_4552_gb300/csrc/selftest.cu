@@ -118,14 +118,16 @@ __global__ void selftest_kernel(int64_t samples, uint64_t seed, unsigned long lo
       double sq[4];
       const uint64_t rr[4] = {r1, r2, r3, r4};
       for (int q = 0; q < 4; ++q)
-        sq[q] = (rr[q] & 255) == 0 ? random_norm(rr[q] >> 8, r5) : make_pos(1023 - 60 + (int)((rr[q] >> 8) % 120), mix64(rr[q]));
+        sq[q] = (rr[q] & 255) == 0 ? random_norm(rr[q] >> 8, r5)
+                                   : make_pos(1023 - 60 + (int)((rr[q] >> 8) % 120), mix64(rr[q]));
       if ((r0 & 3) == 0) {  // na n2 >> nj^2 and n2^2 >> nj n3: quotient eta na / n2, na from eta and n2
         sq[1] = sq[3] = 0x1p-400;
         const double w = sqrt(sq[2]) / eta * nbh::pow2i((int)(r5 % 40) - 20);
         sq[0] = w * w * (1.0 + (double)((int64_t)(r5 >> 40) % 4096 - 2048) * 0x1p-30);
       }
       int eq;
-      if (nbh::crit_exponent(nbh::root_of(sq[0]), nbh::root_of(sq[1]), nbh::root_of(sq[2]), nbh::root_of(sq[3]), eta, eq)) {
+      if (nbh::crit_exponent(nbh::root_of(sq[0]), nbh::root_of(sq[1]), nbh::root_of(sq[2]), nbh::root_of(sq[3]), eta,
+                             eq)) {
         const double na = sqrt(sq[0]), nj = sqrt(sq[1]), n2 = sqrt(sq[2]), n3 = sqrt(sq[3]);
         const double q = eta * (na * n2 + nj * nj) / (nj * n3 + n2 * n2);
         if (!(q > 0.0) || isinf(q) || (int)(nbh::dbits(q) >> 52) - 1023 != eq) atomicAdd(bad, 1ULL);
