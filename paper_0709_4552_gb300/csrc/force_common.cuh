@@ -514,20 +514,31 @@ __host__ __device__ __forceinline__ int j_groups(int64_t n, int64_t tiles, int64
   return 1 << best;
 }
 
-// The same for the FP64 item: groups are whole warps, so 1, 2 or 4 of them and
-// i-tiles of 128, 64 or 32; without groups the warps past n compute nothing, so
-// a partial i-tile counts its warps, at least three (N = 200000, n = 16 193, 154,
-// 131 us; n = 64 257, 216, 240; n = 96 320, 353, 331; n = 160 600, 518, 507; n =
-// 320 979, 876, 927; n = 1000 2679, 2705, 2848).  More groups only while the
-// items leave SMs empty (N = 1500, n = 16 39, 27, 23; n = 448 39, 33, 37; the
-// staging of a tile is the same work for fewer pairs).
+// The same for the FP64 item, 1, 2, 4 or 8 groups and i-tiles of 128, 64, 32 or
+// 16, a slot costing 1, 1.02, 1.04 or 1.17; without groups the warps past n
+// compute nothing, so a partial i-tile counts 96 slots (120 behind whole tiles
+// with three warps).  N = 200000, with 1, 2, 4, 8 groups, us: n = 16 202, 136, 124,
+// 81; n = 48 255, 215, 224, 203; n = 80 319, 351, 311, 288; n = 128 385, 398, 393, 418;
+// n = 160 596, 518, 475, 513; n = 320 977, 882, 891, 982; n = 1000 2677, 2725, 2765,
+// 3075.  Two groups also while the items fit about one wave, four while they fit
+// half of one (N = 20000, n = 96 70, 58, 53; N = 1500, n = 320 39, 31, 29; but N = n =
+// 1024 98, 98, 105: the staging of a tile is the same work for fewer pairs).
 __host__ __device__ __forceinline__ int j_groups64(int64_t n, int64_t tiles, int64_t sms) {
+  constexpr int kCost[4] = {100, 102, 104, 117};
   const int64_t part = n & 127;
-  const int64_t w0 = (n - part + (part == 0 ? 0 : (part <= 96 ? 96 : 128))) * 100;
-  const int64_t w1 = ((n + 63) >> 6) * 64 * 103, w2 = ((n + 31) >> 5) * 32 * 110;
-  int k = w0 <= w1 && w0 <= w2 ? 0 : (w1 <= w2 ? 1 : 2);
-  while (k < 2 && ((n + (64 >> k) - 1) >> (6 - k)) * tiles <= sms) ++k;
-  return 1 << k;
+  int best = 0;
+  int64_t work = 0;
+  for (int k = 0; k < 4; ++k) {
+    int64_t slots = ((n + (128 >> k) - 1) >> (7 - k)) * (128 >> k);
+    if (k == 0 && part > 0 && part <= 96) slots += (part > 64 && n > 128 ? 120 : 96) - 128;
+    if (k == 0 || slots * kCost[k] < work) {
+      best = k;
+      work = slots * kCost[k];
+    }
+  }
+  for (int k = best + 1; k <= 2; ++k)
+    if (((n + (128 >> k) - 1) >> (7 - k)) * tiles <= (k == 1 ? 5 : 2) * sms) best = k;
+  return 1 << best;
 }
 
 // Mixed-precision item: i-tile starting at list position ibase (n entries in
@@ -960,7 +971,7 @@ __device__ __forceinline__ uint32_t fx64_chunk(const Fp64Smem<NT, JT>& sm, int q
 // depends on the j-range alone and on nothing the other i of the CTA hold, so
 // a particle's result does not depend on which particles share its item.
 //
-// JG > 1: groups of NT / JG threads (whole warps) share the j of each tile, as in
+// JG > 1: groups of NT / JG threads (whole or half warps) share the j of each tile, as in
 // mixed_item; their 96-bit sums are on one grid and add exactly.
 template <int NT, int JT, int JG = 1>
 __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __restrict__ xp,
@@ -971,7 +982,7 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
                                           const ISrc is = ISrc()) {
   static_assert(JT % 32 == 0 && NT % 32 == 0, "tiles of whole warps");
   constexpr int NI = NT / JG, JC = JT / JG;  // i-particles of the CTA, j of a group and tile
-  static_assert(NI % 32 == 0, "a group is whole warps");
+  static_assert(NI % 16 == 0 && (JG == 1 || JC <= 32), "groups of whole or half warps, a chunk of a tile each");
   constexpr int kPer = (JT + NT - 1) / NT;  // j-particles a thread stages
   const int tid = threadIdx.x, il = JG == 1 ? tid : tid % NI, jg = JG == 1 ? 0 : tid / NI;
   const int64_t pos0 = ibase + il;
@@ -1111,11 +1122,13 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
     const int64_t d = self - jt;
     const int rel = d >= 0 && d < qn ? (int)d : -1;
     const bool shifted = __any_sync(0xffffffffu, (fi.kx | fi.kv) != 0);
-    const int qe = JG == 1 ? qn : min(qn, (jg + 1) * JC);
+    // (with groups every group takes one trip, of no pairs past a ragged tile's
+    // end: half-warps of one warp vote together below)
+    const int qe = JG == 1 ? qn : (jg + 1) * JC;
 #pragma unroll 1
     for (int q0 = jg * JC; q0 < qe; q0 += 32, ++chunk) {
-      const int count = min(32, qe - q0);
-      uint32_t left = 0xffffffffu >> (32 - count);
+      const int count = JG == 1 ? min(32, qe - q0) : max(0, min(JC, qn - q0));
+      uint32_t left = JG > 1 && count == 0 ? 0u : 0xffffffffu >> (32 - count);
       // an i that left most pairs of a chunk to FP64 (a system far from the
       // origin against its size, say) leaves all of them for the next ones,
       // and a warp of such i skips the fixed-point pass; tried again every
@@ -1124,7 +1137,7 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
       if (tile_ok && __any_sync(0xffffffffu, fi.wmin != nbx::kNoPairs)) {
         left = shifted ? fx64_chunk<true>(sm, q0, count, rel, fi, a)
                        : fx64_chunk<false>(sm, q0, count, rel, fi, a);
-        if (4 * __popc(left) >= 3 * count) fi.wmin = nbx::kNoPairs;
+        if (4 * __popc(left) >= 3 * count && (JG == 1 || count > 0)) fi.wmin = nbx::kNoPairs;
       }
       if (rel >= q0 && rel < q0 + 32) left &= ~(1u << (rel - q0));
       if (left)
@@ -1137,14 +1150,18 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
     // left to FP64; rare), then, through the same slots, the 96-bit sums, which
     // are on one grid for all groups of an i and add exactly
     if (__syncthreads_or(jg > 0 && state != 0)) {
-      if (jg == 0)
+      // (a row of an i per thread: eight FP64 instructions a group)
+      for (int t = tid; t < 7 * NI; t += NT) {
+        const int c = t / NI, i = t % NI;
+        double hi = sm.hi[c][i], lo = sm.lo[c][i];
 #pragma unroll 1
-        for (int q = 1; q < JG; ++q)
-#pragma unroll
-          for (int c = 0; c < 7; ++c) {
-            sum_add(sm.hi[c][il], sm.lo[c][il], sm.hi[c][q * NI + il]);
-            sm.lo[c][il] += sm.lo[c][q * NI + il];
-          }
+        for (int q = 1; q < JG; ++q) {
+          sum_add(hi, lo, sm.hi[c][q * NI + i]);
+          lo += sm.lo[c][q * NI + i];
+        }
+        sm.hi[c][i] = hi;
+        sm.lo[c][i] = lo;
+      }
       state |= kHighUsed;
       __syncthreads();
     }

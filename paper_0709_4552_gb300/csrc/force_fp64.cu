@@ -38,7 +38,10 @@ cudaError_t launch(nb_ctx* c, const int32_t* d_list, int64_t n, const nb_tuning&
     // on nothing but the j-range; the automatic one depends on n anyway)
     const int jg =
         cfg.nsplit > 0 ? 1 : nbk::j_groups64(n, (c->n + JT - 1) / JT, c->sm_count);
-    if (jg > 1) kernel = jg == 4 ? force_fp64_kernel<NT, JT, 4> : force_fp64_kernel<NT, JT, 2>;
+    if (jg > 1)
+      kernel = jg == 8   ? force_fp64_kernel<NT, JT, 8>
+               : jg == 4 ? force_fp64_kernel<NT, JT, 4>
+                         : force_fp64_kernel<NT, JT, 2>;
     shape.threads = NT / jg;
   }
   int nsplit = cfg.nsplit > 0 ? cfg.nsplit : nb_auto_split(c, n, shape, per_sm);

@@ -134,7 +134,10 @@ extern "C" int nb_forces_fp64_noalloc(int64_t N, const double* m, const double* 
   if (nsplit < 1) nsplit = 1;
   const int64_t tps = (tiles + nsplit - 1) / nsplit;
   nsplit = (tiles + tps - 1) / tps;
-  auto kernel = jg == 4 ? noalloc_force_kernel<4> : (jg == 2 ? noalloc_force_kernel<2> : noalloc_force_kernel<1>);
+  auto kernel = jg == 8   ? noalloc_force_kernel<8>
+                : jg == 4 ? noalloc_force_kernel<4>
+                : jg == 2 ? noalloc_force_kernel<2>
+                          : noalloc_force_kernel<1>;
   kernel<<<dim3((unsigned)itiles, (unsigned)nsplit), kNT, 0, s>>>(N, m, x, v, eps * eps, i_idx, n, tps * kJT, scratch,
                                                                   pstride);
   if (cudaGetLastError() != cudaSuccess) return NB_ECUDA;

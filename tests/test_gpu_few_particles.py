@@ -35,8 +35,8 @@ def test_small_block_parity(nbl, N, n, at):
         assert np.median(e) <= 1e-6 and e.max() <= 1e-5  # the mixed path's bounds
 
 
-@pytest.mark.parametrize("N", [130, 300, 20000])
-@pytest.mark.parametrize("n", [1, 31, 32, 33, 64, 65, 96, 97, 129, 160, 161])
+@pytest.mark.parametrize("N", [130, 299, 300, 20000])
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 31, 32, 33, 64, 65, 96, 97, 129, 160, 161])
 @pytest.mark.parametrize("noalloc", [False, True])
 def test_small_fp64_block_parity(nbl, N, n, noalloc):
     # FP64: every pair is at least as accurate as in FP64 arithmetic, so the sum
