@@ -328,7 +328,7 @@ int nb_step(nb_ctx* ctx, double* t_out, int64_t* n_active_out);
  *                       NB_CLUSTER_MAX_N (8192 on an 8-CTA cluster).
  *   NB_LOOP_AUTO        the driver measured fastest per block step on a GB300
  *                       for the context's precision and N: the cluster loop
- *                       for mixed systems of N <= 2048 (where the GPU
+ *                       for mixed systems of N <= 1792 (where the GPU
  *                       co-schedules the cluster), the persistent loop up to
  *                       N = 131072 (mixed) or 2048 (FP64), the host loop
  *                       beyond.

@@ -18,8 +18,10 @@ constexpr double kDefaultDtMin = 1.0 / 4194304.0;  // Sec. 2: 2^-22
 constexpr double kDefaultDtMax = 0.125;            // Sec. 2: 2^-3
 // NB_LOOP_AUTO's crossovers (block-step loops timed per N on a GB300; the
 // persistent mixed loop: 1.25x the host loop at N = 65536, 1.02x at 131072,
-// 0.96x at 196608)
-constexpr int64_t kAutoClusterMaxN = 2048;
+// 0.96x at 196608; the cluster loop against the persistent one, us a block step
+// over four systems: N = 1024 11.3 / 15.5, 1700 14.7 / 16.2, 1792 16.2 / 16.4, 1800
+// 17.1 / 16.4, 2000 17.1 / 16.3, 2048 17.4 / 16.6)
+constexpr int64_t kAutoClusterMaxN = 1792;
 constexpr int64_t kAutoPersistentMaxNMixed = 131072;
 constexpr int64_t kAutoPersistentMaxNFp64 = 2048;
 constexpr size_t kPinnedBytes = 1 << 16;

@@ -52,7 +52,7 @@ constexpr int kLWarps = kLT / 32;
 // with 4 the fixed-point pair spills: N = 1024 32.4 against 31.8 us a block
 // step, N = 32768 582 against 569)
 constexpr int kLPerSmMixed = 4, kLPerSmMixedSmall = 2, kLPerSm64 = 3;
-constexpr int64_t kLMixedSmallHi = 32768, kLMixedTwoLo = 2048;
+constexpr int64_t kLMixedSmallHi = 32768, kLMixedTwoLo = 1024;
 // j-tiles (the mixed one = the box tile).  FP64: an item's tile is its share of
 // a small system's force phase, so those take 32 and at least two CTAs per SM:
 // N = 1024 31.8 us a block step against 40.7 with 64 and one CTA (44.9 with 64
@@ -749,9 +749,9 @@ int nb_integrate_persistent(nb_ctx* c, double t_end) {
   }
   // as many CTAs as fit, but for a small system no more than twice its row
   // tiles, as each barrier waits for every CTA's arrival; at least 32, or two
-  // CTAs per SM where the force items are a good part of a step (FP64; mixed
-  // above the cluster loop's range: N = 4096 20.6 -> 19.5 us a block step, N =
-  // 12000 28.4 -> 28.0, but N = 512 17.4 -> 17.8)
+  // CTAs per SM where the force items are a good part of a step (FP64; mixed, us
+  // a block step with 32 and with two per SM: N = 300 16.2 / 16.3, N = 1024 15.5 /
+  // 15.5, N = 1300 16.8 / 16.0, N = 2048 19.0 / 17.1, N = 4096 20.6 / 19.5)
   const int64_t row_tiles = (c->n + kLT - 1) / kLT;
   const bool two = variant == 3 || (variant == 1 && c->n > kLMixedTwoLo);
   const int G = (int)std::min<int64_t>(std::min(c->sm_count * per_sm, kLMaxG),
