@@ -838,6 +838,8 @@ struct Fp64Smem {
 };
 constexpr int kOdd = 64;
 
+__device__ __forceinline__ int64_t words(uint32_t lo, uint32_t hi) { return (int64_t)(((uint64_t)hi << 32) | lo); }
+
 // exponent e of the largest magnitude among values whose high words (sign
 // cleared) have maximum w: |x| < 2^e (NaN, Inf: 1025)
 __device__ __forceinline__ int exp_above(int w) { return (w >> 20) - 1022; }
@@ -920,29 +922,29 @@ __device__ __noinline__ int fp64_pairs(Fp64Smem<NT, JT>& sm, const double* __res
   return state | kHighUsed;
 }
 
-// the 96-bit sums into the thread's FP64 sums (in_range: they hold its
+// the integer sums into the thread's FP64 sums (in_range: they hold its
 // pairs, else nothing of worth; first: those sums are still zero); cleared
 template <int NT, int JT>
-__device__ __forceinline__ void fp64_fold(Fp64Smem<NT, JT>& sm, nbx::Sum96 (&a)[7], bool in_range, bool first, int g,
+__device__ __forceinline__ void fp64_fold(Fp64Smem<NT, JT>& sm, nbx::Sums& a, bool in_range, bool first, int g,
                                           int gv, int em) {
 #pragma unroll
   for (int c = 0; c < 7; ++c) {
     const int e = c < 3 ? em - 2 * g + nbx::kAccScale
                         : (c < 6 ? em - 3 * g + gv + nbx::kJerkScale : em - g + nbx::kPotScale);
     if (in_range) {
-      const double p = nbx::to_double(a[c], e);
+      const double p = c < 6 ? nbx::to_double(a.f[c % 6], e) : nbx::to_double(a.p, e);
       if (first)
         sm.hi[c][threadIdx.x] = p;
       else
         sum_add(sm.hi[c][threadIdx.x], sm.lo[c][threadIdx.x], p);
     }
-    a[c].w0 = a[c].w1 = a[c].w2 = 0u;
   }
+  a = nbx::Sums{};
 }
 
 template <bool SH, int NT, int JT>
 __device__ __forceinline__ uint32_t fx64_chunk(const Fp64Smem<NT, JT>& sm, int q0, int count, int rel,
-                                               const nbx::IFix& fi, nbx::Sum96 (&a)[7]) {
+                                               const nbx::IFix& fi, nbx::Sums& a) {
   uint32_t left = 0u;
 #pragma unroll 1
   for (int q = 0; q < count; ++q) {
@@ -966,13 +968,13 @@ __device__ __forceinline__ uint32_t fx64_chunk(const Fp64Smem<NT, JT>& sm, int q
 // Per tile the CTA puts JT j-particles on a common grid, 2^G above the tile's
 // largest coordinate (and eps), 2^GV above its largest velocity component, EM
 // the exponent of its largest mass.  The grid is kept while it stays within a
-// factor 2 (mass: 8) of the tile's own, so that the sums, exact 96-bit
+// factor 2 (mass: 8) of the tile's own, so that the sums, exact
 // integers, are folded into FP64 every kFold pairs and not per tile.  It
 // depends on the j-range alone and on nothing the other i of the CTA hold, so
 // a particle's result does not depend on which particles share its item.
 //
 // JG > 1: groups of NT / JG threads (whole or half warps) share the j of each tile, as in
-// mixed_item; their 96-bit sums are on one grid and add exactly.
+// mixed_item; their integer sums are on one grid and add exactly.
 template <int NT, int JT, int JG = 1>
 __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __restrict__ xp,
                                           const double* __restrict__ vp, const double* __restrict__ m, int64_t cs,
@@ -1007,9 +1009,7 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
   const int eeps = (exp_above(abs_hi(eps2)) + 1) >> 1;
 #pragma unroll
   for (int c = 0; c < 7; ++c) sm.hi[c][tid] = sm.lo[c][tid] = 0.0;
-  nbx::Sum96 a[7];
-#pragma unroll
-  for (int c = 0; c < 7; ++c) a[c].w0 = a[c].w1 = a[c].w2 = 0u;
+  nbx::Sums a = {};
   nbx::IFix fi = {};
   int G = 0, GV = 0, EM = 0, g = 0, gv = 0, filled = 0;  // grid of the tiles so far, this i's grid, pairs in a
   bool have = false, in_range = false;
@@ -1147,7 +1147,7 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
   }
   if constexpr (JG > 1) {
     // the groups' sums to group 0: what they hold in FP64 (early folds, pairs
-    // left to FP64; rare), then, through the same slots, the 96-bit sums, which
+    // left to FP64; rare), then, through the same slots, the integer sums, which
     // are on one grid for all groups of an i and add exactly
     if (__syncthreads_or(jg > 0 && state != 0)) {
       // (a row of an i per thread: eight FP64 instructions a group)
@@ -1168,8 +1168,10 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
     if (jg > 0)
 #pragma unroll
       for (int c = 0; c < 7; ++c) {
-        sm.hi[c][tid] = __longlong_as_double((long long)(((uint64_t)a[c].w1 << 32) | a[c].w0));
-        sm.lo[c][tid] = __longlong_as_double((long long)a[c].w2);
+        const uint32_t w[4] = {c < 6 ? a.f[c % 6].w0 : a.p.w0, c < 6 ? a.f[c % 6].w1 : a.p.w1,
+                               c < 6 ? a.f[c % 6].w2 : a.p.w2, c < 6 ? a.f[c % 6].w3 : 0u};
+        sm.hi[c][tid] = __longlong_as_double(words(w[0], w[1]));
+        sm.lo[c][tid] = __longlong_as_double(words(w[2], w[3]));
       }
     __syncthreads();
     if (jg == 0)
@@ -1178,10 +1180,11 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
 #pragma unroll
         for (int c = 0; c < 7; ++c) {
           const uint64_t b = (uint64_t)__double_as_longlong(sm.hi[c][q * NI + il]);
-          const uint64_t l = (((uint64_t)a[c].w1 << 32) | a[c].w0) + b;
-          a[c].w2 += (uint32_t)__double_as_longlong(sm.lo[c][q * NI + il]) + (l < b ? 1u : 0u);
-          a[c].w1 = (uint32_t)(l >> 32);
-          a[c].w0 = (uint32_t)l;
+          const uint64_t d = (uint64_t)__double_as_longlong(sm.lo[c][q * NI + il]);
+          if (c < 6)
+            nbx::add4(a.f[c % 6], (uint32_t)b, (uint32_t)(b >> 32), (uint32_t)d, (uint32_t)(d >> 32));
+          else
+            nbx::add3(a.p.w0, a.p.w1, a.p.w2, (uint32_t)b, (uint32_t)(b >> 32), (uint32_t)d);
         }
   }
   if (filled > 0 && jg == 0) fp64_fold(sm, a, in_range, (state & kHighUsed) == 0, g, gv, EM);

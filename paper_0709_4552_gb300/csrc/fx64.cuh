@@ -7,22 +7,16 @@
 // IMAD.HI 32, IMAD, shifts and logic 63, adds 128), so a pair is computed here
 // with mantissas of 58 to 63 bits held in two 32-bit words: the upper 64 bits
 // of a product of two of them are one IMAD.WIDE and two IMAD.HI.  29 and 32 of
-// those and about 220 cheaper instructions make a pair, 135 cycles per warp
-// and SM (7.4e10 pairs/s at N = 65536, n = 4096); the half of the FMA pipe that
-// multiplies integers is busy for three quarters of them.  Measured on the way
+// those and the cheaper instructions make a pair; the half of the FMA pipe that
+// multiplies integers is the busiest.  Measured on the way
 // there, on the same case: cross terms by IMAD.WIDE with a rounded sum 144
 // cycles; C++ carries instead of add.cc chains 156; 3 or 5 CTAs of 128 threads
 // per SM instead of 4, or two pairs interleaved, level to 4% slower; the cross
 // terms of D.W rounded down one by one 6% faster, and the jerk's error twice
 // as large, so not kept.
 //
-// No step holds fewer than the 53 bits of an FP64 number: each rounds at 2^-56
-// of its own result or finer, and the sums over j are exact.  Measured against
-// long double sums (Plummer spheres of 513 to 60000, equal and Salpeter masses,
-// and sets with outliers, close pairs, wide mass ratios), the rms errors are
-// 0.5 to 1.0 (acceleration), 0.35 to 1.0 (jerk) and 0.4 to 1.0 (potential)
-// times those of the FP64 evaluation (1.0, 1.13 and 1.15 for 33 particles, one
-// 2^30 away, whose pairs are nearly all left to FP64).
+// No term holds fewer bits than FP64 arithmetic gives it: each rounds at 2^-54
+// of its length or finer, and the sums over j are exact.
 //
 // Formats.  2^g bounds the coordinates of the pair and eps, 2^gv the
 // velocities, em is the exponent of the largest mass near by:
@@ -34,7 +28,9 @@
 //   MY = M Y 2^-64, G = MY Z 2^-64, U = W - 3 (D.W) D / (D.D + eps^2),
 // and the three kinds of terms are MY (potential), G D 2^-64 (acceleration)
 // and G U 2^-64 (jerk), to be scaled by 2^(s-k), 2^(2s-k) and 2^(3s-k).  They
-// are added up as 96-bit integers at one scale for all pairs.
+// are added up at one scale for all pairs, as integers of 96 bits (potential)
+// and of 96 bits with 32 fraction bits, from which k may take up to 15: a light
+// particle's terms keep their bits, as they are all there is on the heaviest one.
 // 1/sigma: the hardware's FP32 rsqrt gives y0 to 2^-18 or better; e = 1 - R y0^2
 // is formed to 2^-57 and y0 (1 + e/2 + 3 e^2 / 8) keeps that.
 //
@@ -49,16 +45,23 @@
 namespace nbx {
 
 constexpr int kKMax = 15;       // largest mass exponent below the tile's
-constexpr int kFold = 512;      // pairs a 96-bit sum takes (its headroom: 2^9 terms)
+constexpr int kFold = 512;      // pairs a sum takes (its headroom: 2^9 terms)
 constexpr int kExpLo = -300, kExpHi = 300;  // exponents the formats take
-// scales of the sums: potential 2^(em-g-78), acceleration 2^(em-2g-68),
-// jerk 2^(em-3g+gv-59) times the integer
-constexpr int kPotScale = -78, kAccScale = -68, kJerkScale = -59;
+// scales of the sums: potential 2^(em-g-78), acceleration 2^(em-2g-91),
+// jerk 2^(em-3g+gv-91) times the integer
+constexpr int kPotScale = -78, kAccScale = -91, kJerkScale = -91;
 constexpr int32_t kWMin = 1 << 20;      // high word of the smallest velocity difference taken, 2^(gv-8) ...
 constexpr int32_t kNoPairs = 0x7FFFFFFF;  // ... and the value that no pair reaches
 
 struct Sum96 {
   uint32_t w0, w1, w2;
+};
+struct Sum128 {
+  uint32_t w0, w1, w2, w3;
+};
+struct Sums {
+  Sum128 f[6];  // acceleration, jerk
+  Sum96 p;      // potential
 };
 
 // one j-particle on the tile's grid
@@ -97,6 +100,22 @@ __device__ __forceinline__ int32_t min_u32(int32_t a, int32_t b) {
   return d;
 }
 
+__device__ __forceinline__ uint32_t sar(uint32_t a, int n) {  // n = 32 gives the sign
+  uint32_t d;
+  asm("shr.s32 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(n));
+  return d;
+}
+
+__device__ __forceinline__ void add3(uint32_t& a0, uint32_t& a1, uint32_t& a2, uint32_t b0, uint32_t b1, uint32_t b2) {
+  asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+      : "+&r"(a0), "+&r"(a1), "+&r"(a2)
+      : "r"(b0), "r"(b1), "r"(b2));
+}
+__device__ __forceinline__ void add4(Sum128& s, uint32_t b0, uint32_t b1, uint32_t b2, uint32_t b3) {
+  asm("add.cc.u32 %0, %0, %4;\n\taddc.cc.u32 %1, %1, %5;\n\taddc.cc.u32 %2, %2, %6;\n\taddc.u32 %3, %3, %7;"
+      : "+&r"(s.w0), "+&r"(s.w1), "+&r"(s.w2), "+&r"(s.w3)
+      : "r"(b0), "r"(b1), "r"(b2), "r"(b3));
+}
 // a b 2^-64 for a, b in signed digits, to a unit: the cross terms are rounded
 // down and the mean of that, one unit, is put back (one = min_u32(ah, 1)), the
 // low digits' product is left out.  Without bias, odd in a and b (a force and
@@ -119,40 +138,42 @@ __device__ __forceinline__ uint64_t umul_fl(uint64_t a, uint64_t b) {
 // sum += t 2^L (0 <= L < 32)
 __device__ __forceinline__ void add_shifted(Sum96& s, int64_t t, int L) {
   const uint32_t t0 = (uint32_t)t, t1 = (uint32_t)((uint64_t)t >> 32);
-  uint32_t a2;
-  asm("shr.s32 %0, %1, %2;" : "=r"(a2) : "r"(t1), "r"(32 - L));  // (a shift by 32 gives the sign)
-  asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
-      : "+&r"(s.w0), "+&r"(s.w1), "+&r"(s.w2)
-      : "r"(__funnelshift_l(0u, t0, L)), "r"(__funnelshift_l(t0, t1, L)), "r"(a2));
+  add3(s.w0, s.w1, s.w2, __funnelshift_l(0u, t0, L), __funnelshift_l(t0, t1, L), sar(t1, 32 - L));
+}
+
+// sum += floor(t 2^(32-k)) 2^L (0 <= k, L < 32)
+__device__ __forceinline__ void add_shifted(Sum128& s, int64_t t, int k, int L) {
+  uint32_t t0, t1 = (uint32_t)t, t2 = (uint32_t)((uint64_t)t >> 32);
+  t0 = __funnelshift_r(0u, t1, k);
+  t1 = __funnelshift_r(t1, t2, k);
+  t2 = sar(t2, k);
+  add4(s, __funnelshift_l(0u, t0, L), __funnelshift_l(t0, t1, L), __funnelshift_l(t1, t2, L), sar(t2, 32 - L));
 }
 
 // s 2^e, rounded once to nearest: a normal FP64 number built from the sum's
-// bits.  About 40 integer instructions; by FP64 conversions, products and a
+// bits.  About 50 integer instructions; by FP64 conversions, products and a
 // TwoSum it was eleven FP64 ones, which a warp issues 64 cycles apart, 7 sums
 // 2.4 us at the end of every item of a small system.
-__device__ __forceinline__ double to_double(Sum96 s, int e) {
-  const uint32_t neg = (uint32_t)((int32_t)s.w2 >> 31);
-  uint32_t a0 = s.w0 ^ neg, a1 = s.w1 ^ neg, a2 = s.w2 ^ neg;
-  asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, 0;\n\taddc.u32 %2, %2, 0;"
-      : "+&r"(a0), "+&r"(a1), "+&r"(a2)
-      : "r"(neg & 1u));
-  // the leading bit to bit 95: whole words, then the rest
+__device__ __forceinline__ double to_double(Sum128 s, int e) {
+  const uint32_t neg = sar(s.w3, 31);
+  Sum128 a = {s.w0 ^ neg, s.w1 ^ neg, s.w2 ^ neg, s.w3 ^ neg};
+  add4(a, neg & 1u, 0u, 0u, 0u);
+  // the leading bit to bit 127: whole words, then the rest
   int n = 0;
-  if (a2 == 0u) {
-    n = 32;
-    a2 = a1;
-    a1 = a0;
-    a0 = 0u;
-    if (a2 == 0u) {
-      n = 64;
-      a2 = a1;
-      a1 = 0u;
+#pragma unroll
+  for (int w = 0; w < 3; ++w)
+    if (a.w3 == 0u) {
+      n += 32;
+      a.w3 = a.w2;
+      a.w2 = a.w1;
+      a.w1 = a.w0;
+      a.w0 = 0u;
     }
-  }
-  if (a2 == 0u) return 0.0;
-  const int z = __clz((int)a2);
-  const uint32_t m1 = __funnelshift_l(a1, a2, z), m0 = __funnelshift_l(a0, a1, z), rest = __funnelshift_l(0u, a0, z);
-  const int E = 95 - n - z + e + 1023;
+  if (a.w3 == 0u) return 0.0;
+  const int z = __clz((int)a.w3);
+  const uint32_t m1 = __funnelshift_l(a.w2, a.w3, z), m0 = __funnelshift_l(a.w1, a.w2, z);
+  const uint32_t rest = __funnelshift_l(a.w0, a.w1, z) | a.w0;
+  const int E = 127 - n - z + e + 1023;
   const uint64_t m = ((uint64_t)m1 << 32) | m0;
   const uint32_t r = m0 & 0x7FFu;
   const uint32_t up = (r > 0x400u || (r == 0x400u && (rest != 0u || (m0 & 0x800u) != 0u))) ? 1u : 0u;
@@ -162,6 +183,17 @@ __device__ __forceinline__ double to_double(Sum96 s, int e) {
   const double d = scalbn((double)f, E - 1075);
   return neg ? -d : d;
 }
+__device__ __forceinline__ double to_double(Sum96 s, int e) {
+  return to_double(Sum128{s.w0, s.w1, s.w2, sar(s.w2, 31)}, e);
+}
+
+// j's value on i's coarser grid: (x2 x1 . x0) >>= k (0 to 63)
+__device__ __forceinline__ void coarser(uint32_t& x0, uint32_t& x1, uint32_t& x2, int k) {
+  const int64_t q = (int64_t)(((uint64_t)x2 << 32) | x1) >> k;
+  x0 = k < 32 ? __funnelshift_r(x0, x1, k) : __funnelshift_r(x1, x2, k);
+  x1 = (uint32_t)q;
+  x2 = (uint32_t)((uint64_t)q >> 32);
+}
 
 // The pair (i, j): its seven terms added to a (acc, jerk, pot).  Returns
 // false, and adds nothing, when skip is set or the pair is not one of those
@@ -169,7 +201,7 @@ __device__ __forceinline__ double to_double(Sum96 s, int e) {
 // (Every shift by a computed amount is a funnel shift, whose amount is taken
 // modulo 32: a pair that is left computes with meaningless shifts.)
 template <bool SH>
-__device__ __forceinline__ bool pair(const JFix& j, const IFix& i, bool skip, Sum96 (&a)[7]) {
+__device__ __forceinline__ bool pair(const JFix& j, const IFix& i, bool skip, Sums& a) {
   int64_t D[3], W[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -216,17 +248,7 @@ __device__ __forceinline__ bool pair(const JFix& j, const IFix& i, bool skip, Su
   const uint32_t yh = (uint32_t)(Y >> 32), yl = (uint32_t)Y;
   const uint64_t Z = (uint64_t)yh * yh + (__umulhi(yh, yl) << 1);
   const uint64_t MY = umul_fl(ok ? j.M : 0ull, Y);
-  const uint64_t Gn = umul_fl(MY, Z);
-
-  // shifts of the terms: potential 15 + s - k, acceleration 9 + 2s - k, jerk
-  // 3s - k; where the last is negative (light j far away) G is shifted instead.
-  // (max as an instruction: written in C++, the compiler dropped it.)
-  const int k = j.k, d3 = 3 * s - k;
-  int Lj;
-  asm("max.s32 %0, %1, 0;" : "=r"(Lj) : "r"(d3));
-  const int rho = Lj - d3;  // at most kKMax
-  const uint32_t g1 = (uint32_t)(Gn >> 32);
-  const uint64_t G = ((uint64_t)__funnelshift_r(g1, 0u, rho) << 32) | __funnelshift_r((uint32_t)Gn, g1, rho);
+  const uint64_t G = umul_fl(MY, Z);
 
   // D.W 2^-64, then T = 8 (-6 D.W) Z 2^-64: A = 16 T D 2^-64 is the jerk's
   // -3 (r.v) r / s^2.  The sum's cross terms are rounded once: their error
@@ -247,14 +269,15 @@ __device__ __forceinline__ bool pair(const JFix& j, const IFix& i, bool skip, Su
   digits((int64_t)G, gh, gl);
 
   const int32_t one_t = min_u32(th, 1), one_g = min_u32(gh, 1);
-  add_shifted(a[6], (int64_t)MY, 15 + s - k);
+  const int k = j.k;
+  add_shifted(a.p, (int64_t)MY, 15 + s - k);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const int64_t U = W[c] + (int64_t)((uint64_t)mul_odd(th, tl, one_t, dh[c], dl[c]) << 4);
     int32_t uh, ul;
     digits(U, uh, ul);
-    add_shifted(a[c], mul_odd(gh, gl, one_g, dh[c], dl[c]), Lj + 9 - s);
-    add_shifted(a[3 + c], mul_odd(gh, gl, one_g, uh, ul), Lj);
+    add_shifted(a.f[c], mul_odd(gh, gl, one_g, dh[c], dl[c]), k, 2 * s);
+    add_shifted(a.f[3 + c], mul_odd(gh, gl, one_g, uh, ul), k, 3 * s);
   }
   return ok;
 }
