@@ -830,13 +830,17 @@ __device__ __forceinline__ void mixed_item(SM& sm, const float4* __restrict__ jA
 // the same formulas and 5 times as fast on this GPU.
 template <int NT, int JT>
 struct Fp64Smem {
-  // a j-particle of the tile: (X0, X1), (X2, V0), (V1, V2), (M, k); k = kOdd:
-  // not for the fixed-point pair (negative, subnormal or very small mass)
-  longlong2 j[JT][4];
+  // a j-particle of the tile: (X0, X1), (X2, V0), (V1, V2), (M + k, fractions of
+  // X0 and X1), (of X2 and V0, of V1 and V2).  M is a multiple of 1024; k =
+  // kOdd: not for the fixed-point pair (negative, subnormal or very small mass)
+  longlong2 j[JT][5];
   double hi[7][NT], lo[7][NT];  // the thread's sums (TwoSum)
-  int red[NT / 32][3];
+  int4 red[JT / 32][4];         // a warp's bounds: X and V, minima and maxima (keys), the mass; its slow j
+  int4 box[3];                  // the tile's, high words on its grid
 };
 constexpr int kOdd = 64;
+// a tile's pairs as an i sees them (fp64_view)
+constexpr int kPlain = 0, kFine = 1, kNone = 2;
 
 __device__ __forceinline__ int64_t words(uint32_t lo, uint32_t hi) { return (int64_t)(((uint64_t)hi << 32) | lo); }
 
@@ -846,16 +850,29 @@ __device__ __forceinline__ int exp_above(int w) { return (w >> 20) - 1022; }
 __device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7FFFFFFF; }
 __device__ __forceinline__ double pow2d(int e) { return __hiloint2double((e + 1023) << 20, 0); }  // e in [-1022, 1023]
 
-// x 2^sh rounded to the nearest integer (|x| 2^sh <= 2^60), from x's bits:
-// a shift of the significand costs a tenth of the two FP64 instructions
-__device__ __forceinline__ int64_t to_fixed(double x, int sh) {
+// the key that orders double high words, and the magnitude's word from it
+__device__ __forceinline__ int hi_key(double x) {
+  const int h = __double2hiint(x);
+  return h ^ ((h >> 31) & 0x7FFFFFFF);
+}
+__device__ __forceinline__ int abs_key(int k) { return k ^ (k >> 31); }
+__device__ __forceinline__ double of_hi_key(int k) { return __hiloint2double(k ^ ((k >> 31) & 0x7FFFFFFF), 0); }
+
+// x 2^sh (|x| 2^sh <= 2^60) as an integer and 32 fraction bits, from x's bits:
+// a shift of the significand costs a tenth of the FP64 instructions
+__device__ __forceinline__ int64_t to_fixed(double x, int sh, uint32_t& frac) {
   const uint64_t b = (uint64_t)__double_as_longlong(x);
   const int E = (int)(b >> 52) & 0x7FF;
-  const uint64_t f = (b & 0x000FFFFFFFFFFFFFull) | (E ? 0x0010000000000000ull : 0ull);
-  const int n = min((E ? E : 1) - 1075 + sh, 8);
-  const int r = max(min(-n, 63), 1);
-  const uint64_t mag = n >= 0 ? f << n : (f + (1ull << (r - 1))) >> r;
-  return (int64_t)b < 0 ? -(int64_t)mag : (int64_t)mag;
+  const uint64_t f = ((b & 0x000FFFFFFFFFFFFFull) | (E ? 0x0010000000000000ull : 0ull)) << 11;
+  const int r = max(3, min(1086 - (E ? E : 1) - sh, 95));
+  const uint64_t hi = r < 64 ? f >> (r & 63) : 0ull;
+  const uint32_t lo = r < 32 ? (uint32_t)(f << ((32 - r) & 63)) : (uint32_t)(f >> ((r - 32) & 63));
+  if ((int64_t)b >= 0) {
+    frac = lo;
+    return (int64_t)hi;
+  }
+  frac = 0u - lo;
+  return -(int64_t)hi - (lo != 0u ? 1 : 0);
 }
 
 // (hi, lo) += p: TwoSum (Knuth), hi + p = s + e exactly
@@ -942,22 +959,76 @@ __device__ __forceinline__ void fp64_fold(Fp64Smem<NT, JT>& sm, nbx::Sums& a, bo
   a = nbx::Sums{};
 }
 
-template <bool SH, int NT, int JT>
+template <bool SH, bool FINE, int NT, int JT>
 __device__ __forceinline__ uint32_t fx64_chunk(const Fp64Smem<NT, JT>& sm, int q0, int count, int rel,
                                                const nbx::IFix& fi, nbx::Sums& a) {
   uint32_t left = 0u;
 #pragma unroll 1
   for (int q = 0; q < count; ++q) {
-    const longlong2 A = sm.j[q0 + q][0], B = sm.j[q0 + q][1], C = sm.j[q0 + q][2], K = sm.j[q0 + q][3];
+    const longlong2* row = sm.j[q0 + q];
+    const longlong2 A = row[0], B = row[1], C = row[2], K = row[3];
     nbx::JFix fj;
     fj.X[0] = A.x; fj.X[1] = A.y; fj.X[2] = B.x;
     fj.V[0] = B.y; fj.V[1] = C.x; fj.V[2] = C.y;
-    fj.M = (uint64_t)K.x;
-    fj.k = (int)K.y;
-    const bool ok = nbx::pair<SH>(fj, fi, (q0 + q == rel) | (fj.k == kOdd), a);
+    fj.k = (int)K.x & 1023;
+    fj.M = (uint64_t)K.x & ~1023ull;
+    fj.xl[0] = (uint32_t)K.y;
+    fj.xl[1] = (uint32_t)((uint64_t)K.y >> 32);
+    if (FINE) {
+      const longlong2 L = row[4];
+      fj.xl[2] = (uint32_t)L.x;
+      fj.vl[0] = (uint32_t)((uint64_t)L.x >> 32);
+      fj.vl[1] = (uint32_t)L.y;
+      fj.vl[2] = (uint32_t)((uint64_t)L.y >> 32);
+    } else {
+      fj.xl[2] = *reinterpret_cast<const uint32_t*>(&row[4]);
+    }
+    const bool ok = nbx::pair<SH, FINE>(fj, fi, (q0 + q == rel) | (fj.k == kOdd), a);
     left |= ok ? 0u : 1u << q;
   }
   return left;
+}
+
+// How i sees the tile.  The fixed point holds the components of a difference,
+// and of the products with it, to a fraction of what the largest one needs, so
+// a tile that is flat from i (every tile of a disc) would have its small ones in
+// too few bits: from 2^-kFlat of the largest extent on the pair keeps the
+// products' last bits (kFine), and from 2^-kThin on it goes to FP64 (kNone), as
+// does a tile none of whose pairs the grid resolves.  kFine too where most
+// velocity differences are small against the grid's unit of speed, as for
+// a common velocity or most of a tile's j moving at less than 2^-kSlow of the
+// fastest (a hard binary among them).  An axis on which every coordinate is zero,
+// and i's, has no differences: it is judged by its velocities, the other part of
+// the jerk, if there are any.  The extents are lower bounds, from the box of the
+// high words.
+constexpr int kFlat = 6, kThin = 16, kSlow = 4;
+template <int NT, int JT>
+__device__ __forceinline__ int fp64_view(const Fp64Smem<NT, JT>& sm, const nbx::IFix& fi, int zero, int qn) {
+  const int4 p = sm.box[0], q = sm.box[1], r = sm.box[2];
+  const int lo[6] = {p.x, p.y, p.z, p.w, q.x, q.y}, hi[6] = {q.z, q.w, r.x, r.y, r.z, r.w};
+  int e[6], most[2] = {0, 0};
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const int k = min(c < 3 ? fi.kx : fi.kv, 31);
+    const int64_t own = c < 3 ? fi.X[c % 3] : fi.V[c % 3];
+    const uint32_t frac = c < 3 ? fi.xl[c % 3] : fi.vl[c % 3];
+    const int l = lo[c] >> k, h = hi[c] >> k, x = (int)(own >> 32);
+    if (own != 0 || frac != 0u) zero &= ~(1 << c);
+    e[c] = max(max(h - x, x - l) - (max(abs(l), abs(h)) >> 20) - 2, 0);  // (a high word: to 2^-20 of itself)
+    most[c / 3] = max(most[c / 3], e[c]);
+  }
+  int slow = 0;
+#pragma unroll
+  for (int w = 0; w < (NT < JT ? NT : JT) / 32; ++w) slow += sm.red[w][3].y;
+  bool fine = most[1] < 3 << 24 || 2 * slow >= qn;
+  bool none = most[0] < 1 << 20;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const bool zx = (zero >> c) & 1, zv = (zero >> (3 + c)) & 1;
+    fine = fine || (!zx && e[c] < most[0] >> kFlat) || (!zv && e[3 + c] < most[1] >> kFlat);
+    none = none || (zx ? !zv && e[3 + c] < most[1] >> kThin : e[c] < most[0] >> kThin);
+  }
+  return none ? kNone : (fine ? kFine : kPlain);
 }
 
 // FP64 item: one i per thread (i-tile of NT), j-range [jlo, jhi).  Component c
@@ -1022,7 +1093,13 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
 
   for (int64_t jt = jlo; jt < jhi; jt += JT) {
     double jx[kPer][3], jv[kPer][3], jm[kPer];
-    int wx = 0, wv = 0, wm = 0;
+    int b[13];  // keys: minima of X and V, maxima of X and V; the mass
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      b[c] = 0x7FFFFFFF;
+      b[6 + c] = ~0x7FFFFFFF;
+    }
+    b[12] = 0;
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
       const int q = tid + u * NT;
@@ -1032,27 +1109,45 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
       for (int c = 0; c < 3; ++c) {
         jx[u][c] = in ? xp[c * cs + j * js] : 0.0;
         jv[u][c] = in ? vp[c * cs + j * js] : 0.0;
-        wx = max(wx, abs_hi(jx[u][c]));
-        wv = max(wv, abs_hi(jv[u][c]));
+        const int kx = hi_key(jx[u][c]), kv = hi_key(jv[u][c]);
+        b[c] = min(b[c], in ? kx : 0x7FFFFFFF);
+        b[3 + c] = min(b[3 + c], in ? kv : 0x7FFFFFFF);
+        b[6 + c] = max(b[6 + c], in ? kx : ~0x7FFFFFFF);
+        b[9 + c] = max(b[9 + c], in ? kv : ~0x7FFFFFFF);
       }
       jm[u] = in ? m[j] : 0.0;
-      wm = max(wm, abs_hi(jm[u]));
+      b[12] = max(b[12], abs_hi(jm[u]));
     }
-    wx = __reduce_max_sync(0xffffffffu, wx);
-    wv = __reduce_max_sync(0xffffffffu, wv);
-    wm = __reduce_max_sync(0xffffffffu, wm);
-    if ((tid & 31) == 0) {
-      sm.red[tid >> 5][0] = wx;
-      sm.red[tid >> 5][1] = wv;
-      sm.red[tid >> 5][2] = wm;
-    }
-    __syncthreads();  // the previous tile is done with, the maxima are there
+    if (tid < JT) {  // (whole warps)
 #pragma unroll
-    for (int w = 0; w < NT / 32; ++w) {
-      wx = max(wx, sm.red[w][0]);
-      wv = max(wv, sm.red[w][1]);
-      wm = max(wm, sm.red[w][2]);
+      for (int c = 0; c < 13; ++c)
+        b[c] = c < 6 ? __reduce_min_sync(0xffffffffu, b[c]) : __reduce_max_sync(0xffffffffu, b[c]);
+      if ((tid & 31) == 0) {
+        sm.red[tid >> 5][0] = make_int4(b[0], b[1], b[2], b[3]);
+        sm.red[tid >> 5][1] = make_int4(b[4], b[5], b[6], b[7]);
+        sm.red[tid >> 5][2] = make_int4(b[8], b[9], b[10], b[11]);
+        sm.red[tid >> 5][3].x = b[12];
+      }
     }
+    __syncthreads();  // the previous tile is done with, the bounds are there
+#pragma unroll
+    for (int w = 0; w < (NT < JT ? NT : JT) / 32; ++w) {
+      const int4 r0 = sm.red[w][0], r1 = sm.red[w][1], r2 = sm.red[w][2];
+      const int r[13] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w, r2.x, r2.y, r2.z, r2.w, sm.red[w][3].x};
+#pragma unroll
+      for (int c = 0; c < 13; ++c) b[c] = w == 0 ? r[c] : (c < 6 ? min(b[c], r[c]) : max(b[c], r[c]));
+    }
+    int wx = 0, wv = 0, zero = 0;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      const int w = max(abs_key(b[c]), abs_key(b[6 + c]));
+      if (c < 3)
+        wx = max(wx, w);
+      else
+        wv = max(wv, w);
+      zero |= w == 0 ? 1 << c : 0;
+    }
+    const int wm = b[12];
     const int gx = max(max(exp_above(wx), eeps), nbx::kExpLo), gw = max(exp_above(wv), nbx::kExpLo),
               gm = max(exp_above(wm), nbx::kExpLo);
     const bool tile_ok = gx <= nbx::kExpHi && gw <= nbx::kExpHi && gm <= nbx::kExpHi;
@@ -1077,8 +1172,8 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
         if (in_range) {
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
-            fi.X[c] = to_fixed(xi[c * ics], 60 - g);
-            fi.V[c] = to_fixed(vi[c * ics], 60 - gv);
+            fi.X[c] = to_fixed(xi[c * ics], 60 - g, fi.xl[c]);
+            fi.V[c] = to_fixed(vi[c * ics], 60 - gv, fi.vl[c]);
           }
           const double e2 = eps2 * pow2d(56 - 2 * g);
           const uint64_t e2h = (uint64_t)e2;
@@ -1092,27 +1187,43 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
       }
     }
     if (tile_ok) {
+      if (tid < 12) {
+        uint32_t f;
+        int key = b[0];
+#pragma unroll
+        for (int c = 1; c < 12; ++c) key = tid == c ? b[c] : key;
+        reinterpret_cast<int*>(sm.box)[tid] = (int)(to_fixed(of_hi_key(key), tid % 6 < 3 ? 60 - G : 60 - GV, f) >> 32);
+      }
+      int slow = 0;  // j of less than 2^-kSlow of the grid's speed
 #pragma unroll
       for (int u = 0; u < kPer; ++u) {
         const int q = tid + u * NT;
         if (q < JT) {
+          slow += jt + q < jhi &&
+                  exp_above(max(abs_hi(jv[u][0]), max(abs_hi(jv[u][1]), abs_hi(jv[u][2])))) <= GV - kSlow;
           int64_t X[3], V[3];
+          uint32_t xl[3], vl[3];
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
-            X[c] = to_fixed(jx[u][c], 60 - G);
-            V[c] = to_fixed(jv[u][c], 60 - GV);
+            X[c] = to_fixed(jx[u][c], 60 - G, xl[c]);
+            V[c] = to_fixed(jv[u][c], 60 - GV, vl[c]);
           }
           const uint64_t mb = (uint64_t)__double_as_longlong(jm[u]);
           const int E = (int)(mb >> 52);  // with the sign: negative masses are odd
           const int k = EM - (E - 1022);
-          const bool zero = mb << 1 == 0;
-          const bool odd = !zero && (E < 1 || E > 2046 || k > nbx::kKMax);
-          const uint64_t M = zero || odd ? 0ull : ((mb & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << 10;
+          const bool none = mb << 1 == 0;
+          const bool odd = !none && (E < 1 || E > 2046 || k > nbx::kKMax);
+          const uint64_t M = none || odd ? 0ull : ((mb & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << 10;
           sm.j[q][0] = make_longlong2(X[0], X[1]);
           sm.j[q][1] = make_longlong2(X[2], V[0]);
           sm.j[q][2] = make_longlong2(V[1], V[2]);
-          sm.j[q][3] = make_longlong2((int64_t)M, zero ? 0 : (odd ? kOdd : k));
+          sm.j[q][3] = make_longlong2((int64_t)(M | (uint64_t)(none ? 0 : (odd ? kOdd : k))), words(xl[0], xl[1]));
+          sm.j[q][4] = make_longlong2(words(xl[2], vl[0]), words(vl[1], vl[2]));
         }
+      }
+      if (tid < JT) {
+        slow = __reduce_add_sync(0xffffffffu, slow);
+        if ((tid & 31) == 0) sm.red[tid >> 5][3].y = slow;
       }
       filled += JT;
     }
@@ -1122,8 +1233,8 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
     const int64_t d = self - jt;
     const int rel = d >= 0 && d < qn ? (int)d : -1;
     const bool shifted = __any_sync(0xffffffffu, (fi.kx | fi.kv) != 0);
-    // (with groups every group takes one trip, of no pairs past a ragged tile's
-    // end: half-warps of one warp vote together below)
+    const int view = tile_ok && in_range ? fp64_view(sm, fi, zero, qn) : kNone;
+    // (with groups every group takes one trip, of no pairs past a ragged tile's end)
     const int qe = JG == 1 ? qn : (jg + 1) * JC;
 #pragma unroll 1
     for (int q0 = jg * JC; q0 < qe; q0 += 32, ++chunk) {
@@ -1134,9 +1245,13 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
       // and a warp of such i skips the fixed-point pass; tried again every
       // 8th chunk.  Each i decides for itself, from the j-range alone.
       if ((chunk & 7) == 0) fi.wmin = wmin;
-      if (tile_ok && __any_sync(0xffffffffu, fi.wmin != nbx::kNoPairs)) {
-        left = shifted ? fx64_chunk<true>(sm, q0, count, rel, fi, a)
-                       : fx64_chunk<false>(sm, q0, count, rel, fi, a);
+      if (view != kNone && fi.wmin != nbx::kNoPairs) {
+        if (view == kPlain)
+          left = shifted ? fx64_chunk<true, false>(sm, q0, count, rel, fi, a)
+                         : fx64_chunk<false, false>(sm, q0, count, rel, fi, a);
+        else
+          left = shifted ? fx64_chunk<true, true>(sm, q0, count, rel, fi, a)
+                         : fx64_chunk<false, true>(sm, q0, count, rel, fi, a);
         if (4 * __popc(left) >= 3 * count && (JG == 1 || count > 0)) fi.wmin = nbx::kNoPairs;
       }
       if (rel >= q0 && rel < q0 + 32) left &= ~(1u << (rel - q0));

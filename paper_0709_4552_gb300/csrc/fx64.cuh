@@ -5,22 +5,30 @@
 // cycles; measured 1.6e10 pairs/s, 89% of that).  The 32-bit integer units are
 // 15 to 75 times faster (measured, lanes per clock and SM: IMAD.WIDE 25,
 // IMAD.HI 32, IMAD, shifts and logic 63, adds 128), so a pair is computed here
-// with mantissas of 58 to 63 bits held in two 32-bit words: the upper 64 bits
-// of a product of two of them are one IMAD.WIDE and two IMAD.HI.  29 and 32 of
-// those and the cheaper instructions make a pair; the half of the FMA pipe that
-// multiplies integers is the busiest.  Measured on the way
-// there, on the same case: cross terms by IMAD.WIDE with a rounded sum 144
-// cycles; C++ carries instead of add.cc chains 156; 3 or 5 CTAs of 128 threads
-// per SM instead of 4, or two pairs interleaved, level to 4% slower; the cross
-// terms of D.W rounded down one by one 6% faster, and the jerk's error twice
-// as large, so not kept.
+// with mantissas of 58 to 63 bits held in two 32-bit words.  40 IMAD.WIDE, 20
+// IMAD.HI and about 275 cheaper instructions make a pair, 150 cycles per warp
+// and SM (6.7e10 pairs/s at N = 65536, n = 4096); no pipe is busy for more than
+// two thirds of them.  Measured, on another case (N = 40000, n = 4864): this
+// form 2.92 ms; the products with their last bits and the velocities' fractions
+// in every pair (FINE) 3.43; the upper 64 bits of each product only (an
+// IMAD.WIDE and two IMAD.HI) with 96-bit sums 2.55, but the small components of
+// a flat system and the forces of light particles then hold too few bits; 3
+// CTAs of 128 threads per SM instead of 4 level.
 //
-// No term holds fewer bits than FP64 arithmetic gives it: each rounds at 2^-54
-// of its length or finer, and the sums over j are exact.
+// No result holds fewer bits than FP64 arithmetic gives it, component by
+// component: the sums over j are exact and hold 32 bits below the unit of a
+// product, and a tile that would need more is left to FP64 (fp64_view in
+// force_common.cuh).  Against 113-bit sums, each component in units of the sum of
+// its terms' sizes, the rms errors are 0.14 to 0.93 of those of FP64 arithmetic
+// in Plummer spheres of 33 to 4000 (equal and Salpeter masses) and at most 0.98
+// of them in discs of thickness 0.3 to 1e-4, needles, sheets, cold velocities,
+// discs far from the origin or with a halo, a star's companions of 2^-4 to 2^-15
+// of its mass and pairs of clusters; where nearly all pairs are left to FP64
+// (flatter ones, far from the origin) they are FP64's.
 //
 // Formats.  2^g bounds the coordinates of the pair and eps, 2^gv the
 // velocities, em is the exponent of the largest mass near by:
-//   X = x 2^(60-g), V = v 2^(60-gv)         integers, rounded to nearest
+//   X = x 2^(60-g), V = v 2^(60-gv)         integers and 32 fraction bits
 //   M in [2^62, 2^63), m = M 2^(em-k-63)    exact (k: this mass's own exponent)
 // The pair is normalised by the even power 4^s that brings R = (r^2 + eps^2)
 // into [2^58, 2^60) (units 2^(2(g-60)+64)); with sigma = sqrt(R 2^-60):
@@ -35,9 +43,8 @@
 // is formed to 2^-57 and y0 (1 + e/2 + 3 e^2 / 8) keeps that.
 //
 // Pairs this does not cover are left to FP64 arithmetic by the caller: those
-// whose difference of position (velocity) is below 2^(g-8) (2^(gv-8)), so that
-// the grid would round it to fewer than 52 bits, and j whose mass is below
-// 2^-kKMax of the largest, or negative.
+// whose difference of position (velocity) is below 2^(g-8) (2^(gv-8)), and j
+// whose mass is below 2^-kKMax of the largest, or negative.
 #pragma once
 
 #include <stdint.h>
@@ -64,9 +71,10 @@ struct Sums {
   Sum96 p;      // potential
 };
 
-// one j-particle on the tile's grid
+// one j-particle on the tile's grid; xl, vl: 32 fraction bits below the unit
 struct JFix {
   int64_t X[3], V[3];
+  uint32_t xl[3], vl[3];
   uint64_t M;
   int k;
 };
@@ -75,6 +83,7 @@ struct JFix {
 // 32.32 bits above a 32-bit fraction and in FP32
 struct IFix {
   int64_t X[3], V[3];
+  uint32_t xl[3], vl[3];
   uint32_t e2[3];
   float e2f;
   float rmin;    // square of the smallest distance taken (high words): 2^(g-8), or eps / 16
@@ -106,6 +115,9 @@ __device__ __forceinline__ uint32_t sar(uint32_t a, int n) {  // n = 32 gives th
   return d;
 }
 
+__device__ __forceinline__ void add2(uint32_t& a0, uint32_t& a1, uint32_t b0) {
+  asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+&r"(a0), "+&r"(a1) : "r"(b0));
+}
 __device__ __forceinline__ void add3(uint32_t& a0, uint32_t& a1, uint32_t& a2, uint32_t b0, uint32_t b1, uint32_t b2) {
   asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
       : "+&r"(a0), "+&r"(a1), "+&r"(a2)
@@ -116,22 +128,45 @@ __device__ __forceinline__ void add4(Sum128& s, uint32_t b0, uint32_t b1, uint32
       : "+&r"(s.w0), "+&r"(s.w1), "+&r"(s.w2), "+&r"(s.w3)
       : "r"(b0), "r"(b1), "r"(b2), "r"(b3));
 }
+__device__ __forceinline__ void sub3(uint32_t& a0, uint32_t& a1, uint32_t& a2, uint32_t b0, uint32_t b1, uint32_t b2) {
+  asm("sub.cc.u32 %0, %0, %3;\n\tsubc.cc.u32 %1, %1, %4;\n\tsubc.u32 %2, %2, %5;"
+      : "+&r"(a0), "+&r"(a1), "+&r"(a2)
+      : "r"(b0), "r"(b1), "r"(b2));
+}
+
 // a b 2^-64 for a, b in signed digits, to a unit: the cross terms are rounded
 // down and the mean of that, one unit, is put back (one = min_u32(ah, 1)), the
-// low digits' product is left out.  Without bias, odd in a and b (a force and
-// its reaction stay opposite), zero where one of them is.
+// low digits' product is left out.  Without bias, odd in a and b, zero where
+// one of them is.
 __device__ __forceinline__ int64_t mul_odd(int32_t ah, int32_t al, int32_t one, int32_t bh, int32_t bl) {
   return (int64_t)ah * bh + mad_hi(al, bh, mad_hi(ah, bl, min_u32(bh, one)));
 }
 
-// the same for positive numbers below 2^63, without the unit put back
+// a b 2^-64 with 32 fraction bits.  Without FINE the low digits' product is
+// left out, up to a quarter of a unit; with it all but a few units of the last
+// bit are there, those of the fractions af and bf of a and b too.  Odd in a and
+// b, but for what is left out, so a force and its reaction stay opposite.  The
+// cross terms' sum must fit 63 bits.
+template <bool FINE>
+__device__ __forceinline__ int64_t mul(int32_t ah, int32_t al, uint32_t af, int32_t bh, int32_t bl, uint32_t bf,
+                                       uint32_t& frac) {
+  int64_t t = (int64_t)ah * bl;
+  if (FINE) {
+    t += (int64_t)__mulhi(al, bl);
+    t += 2 * (int64_t)__mulhi(ah, (int32_t)(bf >> 1));
+    t += 2 * (int64_t)__mulhi(bh, (int32_t)(af >> 1));
+  }
+  t = (int64_t)al * bh + t;
+  frac = (uint32_t)t;
+  return (int64_t)ah * bh + (int64_t)(int32_t)(t >> 32);
+}
+
+// a b 2^-64 for positive numbers below 2^63, rounded down to a unit
 __device__ __forceinline__ uint64_t umul_fl(uint64_t a, uint64_t b) {
   const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
   const uint64_t t = (uint64_t)ah * bh;
   uint32_t lo = (uint32_t)t, hi = (uint32_t)(t >> 32);
-  asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, 0;"
-      : "+&r"(lo), "+&r"(hi)
-      : "r"(__umulhi(ah, bl) + __umulhi(al, bh)));
+  add2(lo, hi, __umulhi(ah, bl) + __umulhi(al, bh));
   return ((uint64_t)hi << 32) | lo;
 }
 
@@ -141,10 +176,10 @@ __device__ __forceinline__ void add_shifted(Sum96& s, int64_t t, int L) {
   add3(s.w0, s.w1, s.w2, __funnelshift_l(0u, t0, L), __funnelshift_l(t0, t1, L), sar(t1, 32 - L));
 }
 
-// sum += floor(t 2^(32-k)) 2^L (0 <= k, L < 32)
-__device__ __forceinline__ void add_shifted(Sum128& s, int64_t t, int k, int L) {
-  uint32_t t0, t1 = (uint32_t)t, t2 = (uint32_t)((uint64_t)t >> 32);
-  t0 = __funnelshift_r(0u, t1, k);
+// sum += floor(t 2^-k) 2^L, t with 32 fraction bits f (0 <= k, L < 32)
+__device__ __forceinline__ void add_shifted(Sum128& s, int64_t t, uint32_t f, int k, int L) {
+  uint32_t t0 = f, t1 = (uint32_t)t, t2 = (uint32_t)((uint64_t)t >> 32);
+  t0 = __funnelshift_r(t0, t1, k);
   t1 = __funnelshift_r(t1, t2, k);
   t2 = sar(t2, k);
   add4(s, __funnelshift_l(0u, t0, L), __funnelshift_l(t0, t1, L), __funnelshift_l(t1, t2, L), sar(t2, 32 - L));
@@ -195,18 +230,32 @@ __device__ __forceinline__ void coarser(uint32_t& x0, uint32_t& x1, uint32_t& x2
   x2 = (uint32_t)((uint64_t)q >> 32);
 }
 
-// The pair (i, j): its seven terms added to a (acc, jerk, pot).  Returns
-// false, and adds nothing, when skip is set or the pair is not one of those
-// described above.  SH: some lane of the warp has kx or kv > 0.
+// The pair (i, j): its seven terms added to a.  Returns false, and adds
+// nothing, when skip is set or the pair is not one of those described above.
+// SH: some lane of the warp has kx or kv > 0.  FINE: see mul.
 // (Every shift by a computed amount is a funnel shift, whose amount is taken
 // modulo 32: a pair that is left computes with meaningless shifts.)
-template <bool SH>
+template <bool SH, bool FINE>
 __device__ __forceinline__ bool pair(const JFix& j, const IFix& i, bool skip, Sums& a) {
   int64_t D[3], W[3];
+  uint32_t df[3], wf[3];  // fractions
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    D[c] = (SH ? j.X[c] >> i.kx : j.X[c]) - i.X[c];
-    W[c] = (SH ? j.V[c] >> i.kv : j.V[c]) - i.V[c];
+    uint32_t x0 = j.xl[c], x1 = (uint32_t)j.X[c], x2 = (uint32_t)((uint64_t)j.X[c] >> 32);
+    if (SH) coarser(x0, x1, x2, i.kx);
+    sub3(x0, x1, x2, i.xl[c], (uint32_t)i.X[c], (uint32_t)((uint64_t)i.X[c] >> 32));
+    df[c] = x0;
+    D[c] = (int64_t)(((uint64_t)x2 << 32) | x1);
+    wf[c] = 0u;
+    if (FINE) {
+      x0 = j.vl[c], x1 = (uint32_t)j.V[c], x2 = (uint32_t)((uint64_t)j.V[c] >> 32);
+      if (SH) coarser(x0, x1, x2, i.kv);
+      sub3(x0, x1, x2, i.vl[c], (uint32_t)i.V[c], (uint32_t)((uint64_t)i.V[c] >> 32));
+      wf[c] = x0;
+      W[c] = (int64_t)(((uint64_t)x2 << 32) | x1);
+    } else {
+      W[c] = (SH ? j.V[c] >> i.kv : j.V[c]) - i.V[c];
+    }
   }
   int32_t wh[3], wl[3];
 #pragma unroll
@@ -223,7 +272,8 @@ __device__ __forceinline__ bool pair(const JFix& j, const IFix& i, bool skip, Su
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const uint32_t lo = (uint32_t)D[c], hi = (uint32_t)((uint64_t)D[c] >> 32);
-    digits((int64_t)(((uint64_t)__funnelshift_l(lo, hi, s) << 32) | __funnelshift_l(0u, lo, s)), dh[c], dl[c]);
+    digits((int64_t)(((uint64_t)__funnelshift_l(lo, hi, s) << 32) | __funnelshift_l(df[c], lo, s)), dh[c], dl[c]);
+    df[c] = __funnelshift_l(0u, df[c], s);
   }
 
   // R = D.D 2^-64 + eps^2
@@ -250,34 +300,51 @@ __device__ __forceinline__ bool pair(const JFix& j, const IFix& i, bool skip, Su
   const uint64_t MY = umul_fl(ok ? j.M : 0ull, Y);
   const uint64_t G = umul_fl(MY, Z);
 
-  // D.W 2^-64, then T = 8 (-6 D.W) Z 2^-64: A = 16 T D 2^-64 is the jerk's
-  // -3 (r.v) r / s^2.  The sum's cross terms are rounded once: their error
-  // grows by up to 24 on the way to A, the largest of all.
-  int64_t cw = (int64_t)dh[0] * wl[0] + 0x80000000ll;
-  cw = (int64_t)dl[0] * wh[0] + cw;
-  cw = (int64_t)dh[1] * wl[1] + cw;
-  cw = (int64_t)dl[1] * wh[1] + cw;
-  cw = (int64_t)dh[2] * wl[2] + cw;
-  cw = (int64_t)dl[2] * wh[2] + cw;
-  int64_t RW = (int64_t)dh[0] * wh[0] + (int64_t)(int32_t)(cw >> 32);
+  // 6 D.W 2^-64, then T = 8 (6 D.W) Z 2^-64: A = 16 T D 2^-64 is the jerk's
+  // 3 (r.v) r / s^2
+  int32_t qh, ql, zh, zl, th, tl, gh, gl;
+  uint32_t tf = 0u;
+  digits((int64_t)Z, zh, zl);
+  digits((int64_t)G, gh, gl);
+  int64_t RW = (int64_t)dh[0] * wh[0];
   RW = (int64_t)dh[1] * wh[1] + RW;
   RW = (int64_t)dh[2] * wh[2] + RW;
-  int32_t qh, ql, zh, zl, th, tl, gh, gl;
-  digits(RW * -6, qh, ql);
-  digits((int64_t)Z, zh, zl);
-  digits((int64_t)((uint64_t)mul_odd(zh, zl, 1, qh, ql) << 3), th, tl);
-  digits((int64_t)G, gh, gl);
+  if (FINE) {
+    int64_t t = 0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      t = (int64_t)dh[c] * wl[c] + t;
+      t = (int64_t)dl[c] * wh[c] + t;
+      t += (int64_t)__mulhi(dl[c], wl[c]);
+      t += 2 * ((int64_t)__mulhi(dh[c], (int32_t)(wf[c] >> 1)) + (int64_t)__mulhi(wh[c], (int32_t)(df[c] >> 1)));
+    }
+    const uint64_t low = 6 * (uint64_t)(uint32_t)t;
+    digits((RW + (t >> 32)) * 6 + (int64_t)(low >> 32), qh, ql);
+    const uint64_t T = (uint64_t)mul<true>(zh, zl, 0u, qh, ql, (uint32_t)low, tf);
+    digits((int64_t)((T << 3) | (tf >> 29)), th, tl);
+    tf <<= 3;
+  } else {
+    int32_t cw = 3;  // (the mean of what the six lose)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) cw = mad_hi(dl[c], wh[c], mad_hi(dh[c], wl[c], cw));
+    digits((RW + cw) * 6, qh, ql);
+    digits((int64_t)((uint64_t)mul_odd(zh, zl, 1, qh, ql) << 3), th, tl);
+  }
 
-  const int32_t one_t = min_u32(th, 1), one_g = min_u32(gh, 1);
   const int k = j.k;
   add_shifted(a.p, (int64_t)MY, 15 + s - k);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const int64_t U = W[c] + (int64_t)((uint64_t)mul_odd(th, tl, one_t, dh[c], dl[c]) << 4);
+    uint32_t f;
+    const uint64_t A = (uint64_t)mul<FINE>(th, tl, tf, dh[c], dl[c], df[c], f);
+    uint32_t u0 = wf[c], u1 = (uint32_t)W[c], u2 = (uint32_t)((uint64_t)W[c] >> 32);
+    sub3(u0, u1, u2, f << 4, __funnelshift_l(f, (uint32_t)A, 4), __funnelshift_l((uint32_t)A, (uint32_t)(A >> 32), 4));
     int32_t uh, ul;
-    digits(U, uh, ul);
-    add_shifted(a.f[c], mul_odd(gh, gl, one_g, dh[c], dl[c]), k, 2 * s);
-    add_shifted(a.f[3 + c], mul_odd(gh, gl, one_g, uh, ul), k, 3 * s);
+    digits((int64_t)(((uint64_t)u2 << 32) | u1), uh, ul);
+    int64_t t = mul<FINE>(gh, gl, 0u, dh[c], dl[c], df[c], f);
+    add_shifted(a.f[c], t, f, k, 2 * s);
+    t = mul<FINE>(gh, gl, 0u, uh, ul, u0, f);
+    add_shifted(a.f[3 + c], t, f, k, 3 * s);
   }
   return ok;
 }

@@ -1,7 +1,8 @@
 """The FP64 path's results component by component, on systems whose components or
 masses differ so much that the fixed-point pair's integers could run out of bits:
-a star among light companions; through the kernels of every group count and the
-allocation-free call.
+a star among light companions, thin discs (one far from the origin too), needles,
+cold velocities; through the kernels of every group count and the allocation-free
+call.
 
 Bound.  With u = 2^-53, an FP64 evaluation of a component's term is good to about
 16 u of its size: the differences 1 each, s^2 6, 1/s and its powers 10 at most,
@@ -30,6 +31,27 @@ def _set(kind):
         m, x, v = np.full(61, 2.0 ** -t), x[:61], v[:61]
         x *= (np.linspace(0.6, 1.0, 61) / np.linalg.norm(x, axis=1))[:, None]
         m[7], x[7], v[7] = 1.0, 0.0, 0.0
+    elif what in ("disc", "away"):
+        x[:, 2] *= t
+        v[:, 2] *= t
+        if what == "away":
+            x += [3.0, 4.0, 5.0]
+    elif what == "needle":
+        x[:, :2] *= t
+        v[:, :2] *= t
+    elif what == "cold":
+        v[:, 2] *= t
+    elif what == "sheet":  # no extent along z, little motion
+        x[:, 2] = 0.0
+        v[:, 2] *= t
+    elif what == "moving":
+        v[:, 0] += t
+    elif what == "slow":  # but for a few of each tile
+        v[np.arange(N) % 50 > 0] *= t
+    elif what == "halo":  # a disc and a few particles far above it
+        x[:, 2] *= t
+        v[:, 2] *= t
+        x[::50, 2] /= t
     return m, x, v, 1.0 / 1024
 
 
@@ -63,7 +85,10 @@ def _noalloc(nbl, m, x, v, eps, idx):
     return [q.cpu().numpy() for q in out]
 
 
-@pytest.mark.parametrize("kind", ["plain", "star 6", "star 10", "star 14"])
+@pytest.mark.parametrize("kind", ["plain", "star 6", "star 10", "star 14", "disc 0.3", "disc 0.05", "disc 0.01",
+                                  "disc 1e-3", "disc 1e-4", "disc 1e-5", "disc 1e-6", "disc 1e-9", "away 0.1", "away 1e-3",
+                                  "away 1e-6", "needle 1e-3", "cold 1e-3", "sheet 0", "sheet 1e-3", "halo 1e-3", "moving 7", "moving 30",
+                                  "slow 0.02"])
 def test_every_component(nbl, kind):
     m, x, v, eps = _set(kind)
     idx = np.unique(np.append(np.arange(0, len(m), max(1, len(m) // 161))[:160], 7)).astype(np.int32)  # (with the star)
