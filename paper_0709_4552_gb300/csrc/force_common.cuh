@@ -884,22 +884,22 @@ __device__ __forceinline__ void sum_add(double& hi, double& lo, double p) {
 }
 
 // the pairs of one i with the j-particles of the bits in mask (jt + bit), in
-// FP64: the few that the fixed-point pair leaves (closer than its grid
-// resolves, odd masses, values outside its exponent range).  state: the calls
-// so far, kHighUsed once the high sums have been written; returns the new one.
+// FP64: those that the fixed-point pair leaves, a few (closer than its grid
+// resolves, odd masses) or all of a tile (fp64_view).  state: calls with a few,
+// kHighUsed once the high sums have been written; returns the new one.
 constexpr int kHighUsed = 1 << 30;
 template <int NT, int JT>
 __device__ __noinline__ int fp64_pairs(Fp64Smem<NT, JT>& sm, const double* __restrict__ xp,
                                         const double* __restrict__ vp, const double* __restrict__ m, int64_t cs,
-                                        int64_t js, int64_t jt, uint32_t mask, double x0, double x1, double x2,
+                                        int64_t js, int64_t jt, uint64_t mask, double x0, double x1, double x2,
                                         double v0, double v1, double v2, double eps2, int state) {
-  const uint32_t mask0 = mask;
+  const int count = __popcll(mask);
   double p[7];
 #pragma unroll
   for (int c = 0; c < 7; ++c) p[c] = 0.0;
   while (mask) {
-    const int64_t j = jt + (__ffs((int)mask) - 1);
-    mask &= mask - 1u;
+    const int64_t j = jt + (__ffsll((long long)mask) - 1);
+    mask &= mask - 1ull;
     const double* xj = xp + j * js;
     const double* vj = vp + j * js;
     const double dx = xj[0] - x0, dy = xj[cs] - x1, dz = xj[2 * cs] - x2;
@@ -919,42 +919,49 @@ __device__ __noinline__ int fp64_pairs(Fp64Smem<NT, JT>& sm, const double* __res
     p[4] = fma(mr3, fma(a3, dy, wy), p[4]);
     p[5] = fma(mr3, fma(a3, dz, wz), p[5]);
   }
-  // a few pairs: into the low sum alone (each FP64 instruction holds the warp
-  // for 64 cycles, and a TwoSum is six); many, and every eighth time, both
-  // into the high sum without error
-  state += 1;
-  if (__popc(mask0) <= 4 && (state & 7) != 0) {
+  // Each FP64 instruction holds the warp for 64 cycles.  A few pairs: into the
+  // low sum alone, and every eighth time that into the high one without error;
+  // many: a TwoSum into the high sum, none for the first
+  if (count <= 4) {
+    state += 1;
+    if ((state & 7) != 0) {
 #pragma unroll
-    for (int c = 0; c < 7; ++c) sm.lo[c][threadIdx.x] += p[c];
-    return state;
+      for (int c = 0; c < 7; ++c) sm.lo[c][threadIdx.x] += p[c];
+      return state;
+    }
   }
 #pragma unroll
   for (int c = 0; c < 7; ++c) {
-    double hi = sm.hi[c][threadIdx.x], lo = 0.0;
-    sum_add(hi, lo, sm.lo[c][threadIdx.x]);
-    sum_add(hi, lo, p[c]);
+    double hi = p[c], lo = 0.0;
+    if (state != 0) {
+      hi = sm.hi[c][threadIdx.x];
+      lo = sm.lo[c][threadIdx.x];
+      if (count <= 4) {
+        const double q = lo;
+        lo = 0.0;
+        sum_add(hi, lo, q);
+      }
+      sum_add(hi, lo, p[c]);
+    }
     sm.hi[c][threadIdx.x] = hi;
     sm.lo[c][threadIdx.x] = lo;
   }
   return state | kHighUsed;
 }
 
-// the integer sums into the thread's FP64 sums (in_range: they hold its
-// pairs, else nothing of worth; first: those sums are still zero); cleared
+// the integer sums into the thread's FP64 sums (first: those are still zero);
+// cleared
 template <int NT, int JT>
-__device__ __forceinline__ void fp64_fold(Fp64Smem<NT, JT>& sm, nbx::Sums& a, bool in_range, bool first, int g,
-                                          int gv, int em) {
+__device__ __forceinline__ void fp64_fold(Fp64Smem<NT, JT>& sm, nbx::Sums& a, bool first, int g, int gv, int em) {
 #pragma unroll
   for (int c = 0; c < 7; ++c) {
     const int e = c < 3 ? em - 2 * g + nbx::kAccScale
                         : (c < 6 ? em - 3 * g + gv + nbx::kJerkScale : em - g + nbx::kPotScale);
-    if (in_range) {
-      const double p = c < 6 ? nbx::to_double(a.f[c % 6], e) : nbx::to_double(a.p, e);
-      if (first)
-        sm.hi[c][threadIdx.x] = p;
-      else
-        sum_add(sm.hi[c][threadIdx.x], sm.lo[c][threadIdx.x], p);
-    }
+    const double p = c < 6 ? nbx::to_double(a.f[c % 6], e) : nbx::to_double(a.p, e);
+    if (first)
+      sm.hi[c][threadIdx.x] = p;
+    else
+      sum_add(sm.hi[c][threadIdx.x], sm.lo[c][threadIdx.x], p);
   }
   a = nbx::Sums{};
 }
@@ -994,7 +1001,8 @@ __device__ __forceinline__ uint32_t fx64_chunk(const Fp64Smem<NT, JT>& sm, int q
 // a tile that is flat from i (every tile of a disc) would have its small ones in
 // too few bits: from 2^-kFlat of the largest extent on the pair keeps the
 // products' last bits (kFine), and from 2^-kThin on it goes to FP64 (kNone), as
-// does a tile none of whose pairs the grid resolves.  kFine too where most
+// does a tile of which the grid resolves few pairs (a system far from the origin,
+// a common velocity: those cost a pass of their own).  kFine too where most
 // velocity differences are small against the grid's unit of speed, as for
 // a common velocity or most of a tile's j moving at less than 2^-kSlow of the
 // fastest (a hard binary among them).  An axis on which every coordinate is zero,
@@ -1017,11 +1025,12 @@ __device__ __forceinline__ int fp64_view(const Fp64Smem<NT, JT>& sm, const nbx::
     e[c] = max(max(h - x, x - l) - (max(abs(l), abs(h)) >> 20) - 2, 0);  // (a high word: to 2^-20 of itself)
     most[c / 3] = max(most[c / 3], e[c]);
   }
+  const float ext = (float)most[0];
   int slow = 0;
 #pragma unroll
   for (int w = 0; w < (NT < JT ? NT : JT) / 32; ++w) slow += sm.red[w][3].y;
   bool fine = most[1] < 3 << 24 || 2 * slow >= qn;
-  bool none = most[0] < 1 << 20;
+  bool none = ext * ext < 16.0f * fi.rmin || (fi.wmin != 0 && most[1] < 4 * nbx::kWMin);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const bool zx = (zero >> c) & 1, zv = (zero >> (3 + c)) & 1;
@@ -1083,10 +1092,10 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
   nbx::Sums a = {};
   nbx::IFix fi = {};
   int G = 0, GV = 0, EM = 0, g = 0, gv = 0, filled = 0;  // grid of the tiles so far, this i's grid, pairs in a
-  bool have = false, in_range = false;
-  int32_t wmin = nbx::kNoPairs;
-  int chunk = 0, state = 0;
-  fi.wmin = wmin;
+  bool have = false, in_range = false, used = false;  // used: a may hold pairs
+  int tile = 0, state = 0;
+  bool skip = false;
+  uint64_t left64 = 0ull;
   // a warp whose list positions all lie past n computes nothing (its
   // results are not written); it still loads its share of every j-tile
   const bool wact = ibase + (int64_t)(il & ~31) < n;
@@ -1153,9 +1162,10 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
     const bool tile_ok = gx <= nbx::kExpHi && gw <= nbx::kExpHi && gm <= nbx::kExpHi;
     const bool moved = !have || gx > G || gx < G - 1 || gw > GV || gw < GV - 1 || gm > EM || gm < EM - 3;
     if (tile_ok && (moved || filled + JT > nbx::kFold)) {
-      if (filled > 0) {
-        fp64_fold(sm, a, in_range, (state & kHighUsed) == 0, g, gv, EM);
+      if (used) {
+        fp64_fold(sm, a, (state & kHighUsed) == 0, g, gv, EM);
         state |= kHighUsed;
+        used = false;
       }
       filled = 0;
       if (moved) {
@@ -1165,8 +1175,7 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
         g = max(G, exi);
         gv = max(GV, evi);
         in_range = g <= nbx::kExpHi && gv <= nbx::kExpHi;
-        wmin = !in_range ? nbx::kNoPairs : (GV == nbx::kExpLo && evi == -1022 ? 0 : nbx::kWMin);
-        fi.wmin = wmin;
+        fi.wmin = GV == nbx::kExpLo && evi == -1022 ? 0 : nbx::kWMin;
         fi.kx = min(g - G, 63);
         fi.kv = min(gv - GV, 63);
         if (in_range) {
@@ -1233,32 +1242,37 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
     const int64_t d = self - jt;
     const int rel = d >= 0 && d < qn ? (int)d : -1;
     const bool shifted = __any_sync(0xffffffffu, (fi.kx | fi.kv) != 0);
-    const int view = tile_ok && in_range ? fp64_view(sm, fi, zero, qn) : kNone;
+    // An i that left most pairs of a tile to FP64 (one of a small core in a tile
+    // with a far particle, say) leaves all of the next ones, and a warp of such i
+    // skips the fixed-point pass; tried again every 256 j.  Each i decides for
+    // itself, from the j-range alone.
+    if (tile++ % (256 / JT) == 0) skip = false;
+    const int view = tile_ok && in_range && !skip ? fp64_view(sm, fi, zero, qn) : kNone;
+    used = used || view != kNone;
     // (with groups every group takes one trip, of no pairs past a ragged tile's end)
     const int qe = JG == 1 ? qn : (jg + 1) * JC;
+    int left_count = 0;
 #pragma unroll 1
-    for (int q0 = jg * JC; q0 < qe; q0 += 32, ++chunk) {
+    for (int q0 = jg * JC; q0 < qe; q0 += 32) {
       const int count = JG == 1 ? min(32, qe - q0) : max(0, min(JC, qn - q0));
       uint32_t left = JG > 1 && count == 0 ? 0u : 0xffffffffu >> (32 - count);
-      // an i that left most pairs of a chunk to FP64 (a system far from the
-      // origin against its size, say) leaves all of them for the next ones,
-      // and a warp of such i skips the fixed-point pass; tried again every
-      // 8th chunk.  Each i decides for itself, from the j-range alone.
-      if ((chunk & 7) == 0) fi.wmin = wmin;
-      if (view != kNone && fi.wmin != nbx::kNoPairs) {
-        if (view == kPlain)
-          left = shifted ? fx64_chunk<true, false>(sm, q0, count, rel, fi, a)
-                         : fx64_chunk<false, false>(sm, q0, count, rel, fi, a);
-        else
-          left = shifted ? fx64_chunk<true, true>(sm, q0, count, rel, fi, a)
-                         : fx64_chunk<false, true>(sm, q0, count, rel, fi, a);
-        if (4 * __popc(left) >= 3 * count && (JG == 1 || count > 0)) fi.wmin = nbx::kNoPairs;
-      }
+      if (view == kPlain)
+        left = shifted ? fx64_chunk<true, false>(sm, q0, count, rel, fi, a)
+                       : fx64_chunk<false, false>(sm, q0, count, rel, fi, a);
+      else if (view == kFine)
+        left = shifted ? fx64_chunk<true, true>(sm, q0, count, rel, fi, a)
+                       : fx64_chunk<false, true>(sm, q0, count, rel, fi, a);
       if (rel >= q0 && rel < q0 + 32) left &= ~(1u << (rel - q0));
-      if (left)
-        state = fp64_pairs(sm, xp, vp, m, cs, js, jt + q0, left, xi[0], xi[ics], xi[2 * ics], vi[0], vi[ics], vi[2 * ics],
-                   eps2, state);
+      left_count += __popc(left);
+      // up to 64 pairs a call
+      left64 |= (uint64_t)left << (JG == 1 ? q0 & 32 : 0);
+      if (left64 && (JG > 1 || (q0 & 32) || q0 + 32 >= qe)) {
+        state = fp64_pairs(sm, xp, vp, m, cs, js, jt + (JG == 1 ? q0 & ~32 : q0), left64, xi[0], xi[ics], xi[2 * ics],
+                           vi[0], vi[ics], vi[2 * ics], eps2, state);
+        left64 = 0ull;
+      }
     }
+    skip = skip || (view != kNone && 4 * left_count >= 3 * (JG == 1 ? qn : JC));
   }
   if constexpr (JG > 1) {
     // the groups' sums to group 0: what they hold in FP64 (early folds, pairs
@@ -1302,7 +1316,7 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
             nbx::add3(a.p.w0, a.p.w1, a.p.w2, (uint32_t)b, (uint32_t)(b >> 32), (uint32_t)d);
         }
   }
-  if (filled > 0 && jg == 0) fp64_fold(sm, a, in_range, (state & kHighUsed) == 0, g, gv, EM);
+  if (used && jg == 0) fp64_fold(sm, a, (state & kHighUsed) == 0, g, gv, EM);
   __syncthreads();  // the caller may reuse shared memory for its next item
   if (pos0 >= n || jg > 0) return;
 #pragma unroll

@@ -57,8 +57,7 @@ constexpr int kExpLo = -300, kExpHi = 300;  // exponents the formats take
 // scales of the sums: potential 2^(em-g-78), acceleration 2^(em-2g-91),
 // jerk 2^(em-3g+gv-91) times the integer
 constexpr int kPotScale = -78, kAccScale = -91, kJerkScale = -91;
-constexpr int32_t kWMin = 1 << 20;      // high word of the smallest velocity difference taken, 2^(gv-8) ...
-constexpr int32_t kNoPairs = 0x7FFFFFFF;  // ... and the value that no pair reaches
+constexpr int32_t kWMin = 1 << 20;      // high word of the smallest velocity difference taken, 2^(gv-8)
 
 struct Sum96 {
   uint32_t w0, w1, w2;
@@ -88,7 +87,7 @@ struct IFix {
   float e2f;
   float rmin;    // square of the smallest distance taken (high words): 2^(g-8), or eps / 16
   int kx, kv;    // the i-particle lies 2^kx (2^kv) outside the tile's grid: its own grid is that much coarser
-  int32_t wmin;  // kWMin; 0 where every velocity is zero; kNoPairs: take no pair
+  int32_t wmin;  // kWMin; 0 where every velocity is zero
 };
 
 // a = h 2^32 + l with both digits signed

@@ -121,3 +121,32 @@ def test_groups_on_the_fixed_points_hard_cases(nbl, kind):
             for got, ref, size in ((a, ar[idx], A), (j, jr[idx], J), (p[:, None], pr[idx, None], P)):
                 off = np.linalg.norm(got - ref, axis=1)
                 assert (off <= 2.0 ** -48 * size).all(), (kind, n, (off / np.maximum(size, 1e-300)).max())
+
+
+@pytest.mark.parametrize("kind", ["away", "moving"])
+def test_systems_the_grid_does_not_resolve_cost_what_fp64_arithmetic_does(nbl, kind):
+    # far from the origin, or with a common velocity, no pair is for the fixed point: the time is then
+    # that of the 34 FP64 instructions a pair takes, 1.2 times what the unit's measured rate allows (the
+    # start and end of a launch), not that of the attempts as well (1.34)
+    import torch
+    n_all, n = 20000, 2000
+    m, x, v = inputs.plummer(n_all, 3, "salpeter")
+    (x if kind == "away" else v)[:] += 1000.0
+    stream = torch.cuda.current_stream()
+    with nbl.NBody(n_all, nbl.NB_FP64, 0, stream=stream) as s:
+        s.set_params(1.0 / 1024, 0.01, 2.0 ** -22, 2.0 ** -5)
+        s.set_j_particles(0, m, x, v)
+        s.predict(0.0)
+        idx = torch.as_tensor(inputs.sample_indices(n_all, n, 5), device="cuda", dtype=torch.int32)
+        out = [torch.empty(n, 3, device="cuda", dtype=torch.float64) for _ in range(2)]
+        out.append(torch.empty(n, device="cuda", dtype=torch.float64))
+        ms = []
+        for _ in range(9):
+            a, b = torch.cuda.Event(True), torch.cuda.Event(True)
+            a.record(stream)
+            s.compute_forces(idx, *out)
+            b.record(stream)
+            torch.cuda.synchronize()
+            ms.append(a.elapsed_time(b))
+        rate = s.measure_peaks()["fp64_tflops"] * 1e12 / 2
+    assert min(ms) * 1e-3 <= 1.27 * 34 * n_all * n / rate, (min(ms), 34e3 * n_all * n / rate)
