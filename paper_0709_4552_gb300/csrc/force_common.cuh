@@ -1054,14 +1054,16 @@ __device__ __forceinline__ int fp64_view(const Fp64Smem<NT, JT>& sm, const nbx::
 // a particle's result does not depend on which particles share its item.
 //
 // JG > 1: groups of NT / JG threads (whole or half warps) share the j of each tile, as in
-// mixed_item; their integer sums are on one grid and add exactly.
+// mixed_item; their integer sums are on one grid and add exactly.  The pairs left
+// to FP64 are added up group by group, unless in_order (items of a single tile),
+// which gives the bits of JG = 1.
 template <int NT, int JT, int JG = 1>
 __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __restrict__ xp,
                                           const double* __restrict__ vp, const double* __restrict__ m, int64_t cs,
                                           int64_t js, int64_t jlo, int64_t jhi, int64_t idx_hi,
                                           const int32_t* __restrict__ list, int64_t n, int64_t ibase, double eps2,
                                           double* __restrict__ out, int64_t ostride, bool finalize,
-                                          const ISrc is = ISrc()) {
+                                          const ISrc is = ISrc(), bool in_order = false) {
   static_assert(JT % 32 == 0 && NT % 32 == 0, "tiles of whole warps");
   constexpr int NI = NT / JG, JC = JT / JG;  // i-particles of the CTA, j of a group and tile
   static_assert(NI % 16 == 0 && (JG == 1 || JC <= 32), "groups of whole or half warps, a chunk of a tile each");
@@ -1266,7 +1268,7 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
       left_count += __popc(left);
       // up to 64 pairs a call
       left64 |= (uint64_t)left << (JG == 1 ? q0 & 32 : 0);
-      if (left64 && (JG > 1 || (q0 & 32) || q0 + 32 >= qe)) {
+      if (left64 && (JG > 1 ? !in_order : (q0 & 32) || q0 + 32 >= qe)) {
         state = fp64_pairs(sm, xp, vp, m, cs, js, jt + (JG == 1 ? q0 & ~32 : q0), left64, xi[0], xi[ics], xi[2 * ics],
                            vi[0], vi[ics], vi[2 * ics], eps2, state);
         left64 = 0ull;
@@ -1275,6 +1277,20 @@ __device__ __forceinline__ void fp64_item(Fp64Smem<NT, JT>& sm, const double* __
     skip = skip || (view != kNone && 4 * left_count >= 3 * (JG == 1 ? qn : JC));
   }
   if constexpr (JG > 1) {
+    if (in_order) {  // all of an i's left pairs in one call, as without groups
+      __syncthreads();  // the tile is done with
+      uint64_t* left = reinterpret_cast<uint64_t*>(sm.j);
+      left[tid] = left64 << (jg * JC);
+      __syncthreads();
+      if (jg == 0) {
+        uint64_t all = 0ull;
+#pragma unroll
+        for (int q = 0; q < JG; ++q) all |= left[q * NI + il];
+        if (all)
+          state = fp64_pairs(sm, xp, vp, m, cs, js, jlo, all, xi[0], xi[ics], xi[2 * ics], vi[0], vi[ics],
+                             vi[2 * ics], eps2, state);
+      }
+    }
     // the groups' sums to group 0: what they hold in FP64 (early folds, pairs
     // left to FP64; rare), then, through the same slots, the integer sums, which
     // are on one grid for all groups of an i and add exactly

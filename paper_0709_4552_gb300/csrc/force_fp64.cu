@@ -13,7 +13,7 @@ template <int NT, int JT, int JG = 1>
 __global__ void __launch_bounds__(NT, 512 / NT) force_fp64_kernel(
     const double* __restrict__ xp, const double* __restrict__ vp, const double* __restrict__ m,
     int64_t n_pad, int64_t N, const int32_t* __restrict__ list, int64_t n, int64_t tiles,
-    double eps2, double* __restrict__ out, int64_t ostride, int finalize, const nbk::ISrc is) {
+    double eps2, double* __restrict__ out, int64_t ostride, int finalize, const nbk::ISrc is, int in_order) {
   __shared__ nbk::Fp64Smem<NT, JT> sm;
   const int split = blockIdx.y;
   // j-range of this split, cut at N: the item fills the rest of the last
@@ -22,7 +22,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) force_fp64_kernel(
   const int64_t jhi = min(nbk::split_begin(split + 1, gridDim.y, tiles) * JT, N);
   double* o = finalize ? out : out + (int64_t)split * 7 * ostride;
   nbk::fp64_item<NT, JT, JG>(sm, xp, vp, m, n_pad, 1, jlo, jhi, n_pad, list, n, (int64_t)blockIdx.x * (NT / JG), eps2,
-                             o, ostride, finalize != 0, is);
+                             o, ostride, finalize != 0, is, in_order != 0);
 }
 
 template <int NT, int JT>
@@ -53,6 +53,9 @@ cudaError_t launch(nb_ctx* c, const int32_t* d_list, int64_t n, const nb_tuning&
   const int64_t tiles = n_j / JT;
   if (nsplit > tiles) nsplit = (int)tiles;
   if (nsplit < 1) nsplit = 1;
+  // the systems whose sums every loop driver splits alike (one tile a split):
+  // the same bits from each
+  const bool in_order = tiles <= 2 && nsplit == tiles;
   const bool fin = nsplit == 1;
   const int64_t ostride = fin ? c->n_pad : ((n + 31) / 32) * 32;
   double* out = fin ? c->F : c->part;
@@ -60,7 +63,7 @@ cudaError_t launch(nb_ctx* c, const int32_t* d_list, int64_t n, const nb_tuning&
   dim3 grid((unsigned)itiles, (unsigned)nsplit);
   c->launches += fin ? 1 : 2;
   kernel<<<grid, NT, 0, c->stream>>>(c->xp, c->vp, c->m, c->n_pad, c->n, d_list, n, tiles, c->eps * c->eps, out,
-                                     ostride, fin ? 1 : 0, is);
+                                     ostride, fin ? 1 : 0, is, in_order ? 1 : 0);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || fin) return e;
   return nb_launch_split_reduce(c, n, nsplit, ostride);

@@ -150,3 +150,25 @@ def test_systems_the_grid_does_not_resolve_cost_what_fp64_arithmetic_does(nbl, k
             ms.append(a.elapsed_time(b))
         rate = s.measure_peaks()["fp64_tflops"] * 1e12 / 2
     assert min(ms) * 1e-3 <= 1.27 * 34 * n_all * n / rate, (min(ms), 34e3 * n_all * n / rate)
+
+
+@pytest.mark.parametrize("n", [2, 33, 64, 100, 128])
+def test_loops_agree_to_the_bit_with_close_pairs(nbl, n):
+    # systems of at most two j-tiles, binaries that the fixed point leaves to FP64 arithmetic among
+    # them: the host loop's groups, the persistent loop and the graph add up the same (the graph with
+    # one tile: it may split two otherwise)
+    m, x, v = inputs.plummer(n, 950 + n, "salpeter")
+    k = n // 2
+    rng = np.random.default_rng(n)
+    x[k:2 * k] = x[:k] + 2.0 ** rng.uniform(-14, -8, (k, 1)) * rng.normal(size=(k, 3))
+    runs = []
+    for loop in [nbl.NB_LOOP_HOST, nbl.NB_LOOP_PERSISTENT] + ([nbl.NB_LOOP_GRAPH] if n <= 64 else []):
+        with nbl.NBody(n, nbl.NB_FP64, 0) as s:
+            s.set_params(2.0 ** -9, 0.01, 2.0 ** -22, 2.0 ** -6)
+            s.set_j_particles(0, m, x, v)
+            s.initial_forces_and_dt()
+            s.integrate(2.0 ** -6, loop=loop)
+            runs.append(s.get_particles(0, n))
+    for r in runs[1:]:
+        for key in ("x", "v", "a", "jerk", "pot", "t", "dt"):
+            assert np.array_equal(runs[0][key], r[key]), key
