@@ -34,6 +34,7 @@ namespace {
 constexpr int kItemWaves = NB_ENS_ITEM_WAVES;  // force items planned per resident CTA
 constexpr int kCorrItem = 32;     // active particles per corrector item (four threads of its CTA each)
 constexpr int kSelChunk = 512;    // particles per selection chunk (chunks never straddle clusters)
+constexpr int kRedWide = 64;      // splits above which a reduction item is a single row (b_reduce)
 constexpr int kSelThreads = 256;
 // batched item shapes: i-tile = threads per CTA, one i per thread.  An
 // ensemble of small clusters has small active blocks (n = 0.20 N^0.81 is 18
@@ -335,7 +336,7 @@ __global__ void __launch_bounds__(kPlanThreads) b_plan(
         ps = ((n + 31) / 32) * 32;
         items = (int64_t)it * s;
         psz = s > 1 ? 7 * s * ps : 0;
-        ritems = s > 1 ? (n + 31) / 32 : 0;
+        ritems = s > 1 ? (s > kRedWide ? 7 : 1) * ((n + 31) / 32) : 0;
         citems = (n + kCorrItem - 1) / kCorrItem;
       }
       int64_t ex[4] = {items, psz, ritems, citems}, tot[4];
@@ -582,30 +583,39 @@ __global__ void __launch_bounds__(NT, 512 / NT) b_force_fp64(
 // side by side, the loads of four splits in flight.  Lanes: 2 are 1% of a step
 // faster than 4, 4 than 8, 16 are 7% slower.  Clusters with one split wrote
 // their results directly.
-constexpr int kRedLanes = 2;
-__global__ void __launch_bounds__(224 * kRedLanes) b_reduce(
+//
+// Above kRedWide splits (a cluster of more j-tiles than that with a small block)
+// the additions are what counts, 7 S a position and all on one SM's FP64 unit:
+// 50 steps of one system of N = 131072 took 104 us each here.  Such an item is
+// one row, its splits over all the block's warps: 21 us (30 with 8 lanes and a
+// row an item); at 64 splits the seven rows' additions take 4 us.
+constexpr int kRedLanes = 2, kRedWarps = 7 * kRedLanes;
+__global__ void __launch_bounds__(32 * kRedWarps) b_reduce(
     int32_t C, const int64_t* __restrict__ off, const int32_t* __restrict__ nact, const int32_t* __restrict__ nsplit,
     const int64_t* __restrict__ part_off, const int64_t* __restrict__ pstride, const int64_t* __restrict__ ritem_off,
     const double* __restrict__ part, double* __restrict__ F, int64_t fstride) {
-  __shared__ double sm[kRedLanes][7][32];
-  const int tx = threadIdx.x, r = threadIdx.y, z = threadIdx.z;
+  __shared__ double sm[kRedWarps][32];
+  const int tx = threadIdx.x, w = threadIdx.y + 7 * threadIdx.z;
   const int64_t total = ritem_off[C];
   for (int64_t item = blockIdx.x; item < total; item += gridDim.x) {
     const int c = find_cluster(ritem_off, C, item);
     const int S = nsplit[c];
-    const int64_t ps = pstride[c], k = (item - ritem_off[c]) * 32 + tx;
+    const bool wide = S > kRedWide;
+    const int64_t local = item - ritem_off[c];
+    const int r = wide ? (int)(local % 7) : threadIdx.y;  // row
+    const int lanes = wide ? kRedWarps : kRedLanes, z = wide ? w : threadIdx.z;
+    const int64_t ps = pstride[c], k = (wide ? local / 7 : local) * 32 + tx;
     const bool in = k < nact[c];
     const double* p = part + part_off[c] + r * ps + k;
     double acc = 0.0;
     if (in)
 #pragma unroll 4
-      for (int q = z; q < S; q += kRedLanes) acc += p[(int64_t)q * 7 * ps];
-    sm[z][r][tx] = acc;
+      for (int q = z; q < S; q += lanes) acc += p[(int64_t)q * 7 * ps];
+    sm[w][tx] = acc;
     __syncthreads();
     if (z == 0 && in) {
-#pragma unroll
-      for (int q = 1; q < kRedLanes; ++q)
-        if (q < S) acc += sm[q][r][tx];
+      for (int q = 1; q < lanes; ++q)
+        if (q < S) acc += sm[wide ? q : w + 7 * q][tx];
       F[r * fstride + off[c] + k] = r == 6 ? -acc : acc;
     }
     __syncthreads();
@@ -1035,7 +1045,7 @@ cudaError_t launch_forces(nb_ctx* c, Batch* b, const Fork* fork) {
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, fork->back, 0);
   }
   if (e != cudaSuccess) return e;
-  b_reduce<<<c->sm_count * std::max(1, 2048 / (224 * kRedLanes)), dim3(32, 7, kRedLanes), 0, c->stream>>>(
+  b_reduce<<<c->sm_count * std::max(1, 2048 / (32 * kRedWarps)), dim3(32, 7, kRedLanes), 0, c->stream>>>(
       b->C, b->off, b->nact, b->nsplit, b->part_off, b->pstride, b->ritem_off, c->part, c->F, c->n_pad);
   c->launches += 1;
   return cudaGetLastError();
