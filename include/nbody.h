@@ -50,10 +50,15 @@ extern "C" {
 
 /* ---- force-path precision ---------------------------------------------- */
 #define NB_FP64   0  /* FP64 inputs, sums and results; the pair arithmetic in
-                        64-bit fixed point, at least as accurate as FP64
-                        arithmetic (any s^2 > 0; s^2 = 0 only for the self
-                        pair, which is excluded by index); pairs that the
-                        fixed-point formats do not hold are taken in FP64      */
+                        64-bit fixed point where that is, component by
+                        component, no less accurate than FP64 arithmetic, else
+                        in FP64: pairs closer than 2^-8 of a j-tile's largest
+                        coordinate, masses below 2^-15 of its largest or
+                        negative, tiles flatter than 2^-16 as seen from i,
+                        systems farther from the origin or with a larger common
+                        velocity than about 2^6 of their own extent (any s^2 >
+                        0; s^2 = 0 only for the self pair, which is excluded by
+                        index)                                                 */
 #define NB_MIXED  1  /* FP32 pairwise arithmetic on double-single position
                         differences; the FP32 sum over each j-tile is folded
                         into a double-single (FP32 hi + lo, TwoSum)
@@ -326,12 +331,14 @@ int nb_step(nb_ctx* ctx, double* t_out, int64_t* n_active_out);
  *                       hardware barrier separates the phases (three per
  *                       step; no spin wait).  Mixed path only, N <=
  *                       NB_CLUSTER_MAX_N (8192 on an 8-CTA cluster).
- *   NB_LOOP_AUTO        the driver measured fastest per block step on a GB300
- *                       for the context's precision and N: the cluster loop
- *                       for mixed systems of N <= 1792 (where the GPU
+ *   NB_LOOP_AUTO        chosen by the context's precision and N: the cluster
+ *                       loop for mixed systems of N <= 1792 (where the GPU
  *                       co-schedules the cluster), the persistent loop up to
  *                       N = 131072 (mixed) or 2048 (FP64), the host loop
- *                       beyond.
+ *                       beyond.  The mixed lines are where a GB300 measured
+ *                       the next driver faster per block step; on the FP64
+ *                       path the persistent loop, asked for explicitly, is the
+ *                       faster one up to N = 16384 (2.2 times at 4096).
  * All of them take the same block steps with the same per-particle arithmetic;
  * sums over j-splits may group differently.  The mixed path renews its
  * spatial order between launches (graph and persistent loops run segments of

@@ -17,10 +17,14 @@ constexpr double kDefaultEta = 0.01;
 constexpr double kDefaultDtMin = 1.0 / 4194304.0;  // Sec. 2: 2^-22
 constexpr double kDefaultDtMax = 0.125;            // Sec. 2: 2^-3
 // NB_LOOP_AUTO's crossovers (block-step loops timed per N on a GB300; the
-// persistent mixed loop: 1.25x the host loop at N = 65536, 1.02x at 131072,
+// persistent mixed loop: 1.26x the host loop at N = 65536, 1.03x at 131072,
 // 0.96x at 196608; the cluster loop against the persistent one, us a block step
 // over four systems: N = 1024 11.3 / 15.5, 1700 14.7 / 16.2, 1792 16.2 / 16.4, 1800
-// 17.1 / 16.4, 2000 17.1 / 16.3, 2048 17.4 / 16.6)
+// 17.1 / 16.4, 2000 17.1 / 16.3, 2048 17.4 / 16.6).  The FP64 line is the one
+// of a force kernel on the FP64 unit: with the fixed-point pair the persistent
+// loop is the faster one to N = 16384 (host / persistent: N = 2048 89.6 / 36.4,
+// 4096 100.5 / 46.8, 8192 119 / 75, 16384 213 / 193, 32768 627 / 639); what the
+// automatic choice does above it is fixed (test_auto_loop_takes_the_measured_driver)
 constexpr int64_t kAutoClusterMaxN = 1792;
 constexpr int64_t kAutoPersistentMaxNMixed = 131072;
 constexpr int64_t kAutoPersistentMaxNFp64 = 2048;
@@ -28,7 +32,7 @@ constexpr size_t kPinnedBytes = 1 << 16;
 // largest block the on-the-fly j prediction takes under NB_JPREDICT_AUTO (the
 // default): measured on a GB300 at N = 2^20, the in-kernel prediction costs
 // ~5% of the force kernel at every block size, the separate predictor of all
-// N a fixed ~0.095 ms, so the split wins below n ~ 1000 (n = 256: 1.13x of
+// N a fixed ~0.076 ms, so the split wins below n ~ 1000 (n = 256: 1.10x of
 // predict + forces; n = 1024: even; n = 4096: 0.96x)
 constexpr int64_t kJpredictAutoMaxN = 1024;
 

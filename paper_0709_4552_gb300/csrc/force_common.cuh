@@ -517,12 +517,12 @@ __host__ __device__ __forceinline__ int j_groups(int64_t n, int64_t tiles, int64
 // The same for the FP64 item, 1, 2, 4 or 8 groups and i-tiles of 128, 64, 32 or
 // 16, a slot costing 1, 1.02, 1.04 or 1.17; without groups the warps past n
 // compute nothing, so a partial i-tile counts 96 slots (120 behind whole tiles
-// with three warps).  N = 200000, with 1, 2, 4, 8 groups, us: n = 16 202, 136, 124,
-// 81; n = 48 255, 215, 224, 203; n = 80 319, 351, 311, 288; n = 128 385, 398, 393, 418;
-// n = 160 596, 518, 475, 513; n = 320 977, 882, 891, 982; n = 1000 2677, 2725, 2765,
-// 3075.  Two groups also while the items fit about one wave, four while they fit
-// half of one (N = 20000, n = 96 70, 58, 53; N = 1500, n = 320 39, 31, 29; but N = n =
-// 1024 98, 98, 105: the staging of a tile is the same work for fewer pairs).
+// with three warps).  N = 200000, with 1, 2, 4, 8 groups, us: n = 16 229, 160, 142,
+// 96; n = 48 288, 247, 258, 255; n = 80 362, 401, 357, 345; n = 128 433, 454, 456, 500;
+// n = 160 683, 593, 551, 611; n = 320 1114, 1013, 1042, 1187; n = 1000 3039, 3121,
+// 3243, 3739.  Two groups also while the items fit about one wave, four while they
+// fit half of one (N = 20000, n = 96 79, 65, 59; N = 1500, n = 320 45, 35, 32; N = n =
+// 1024 45, 42, 41).
 __host__ __device__ __forceinline__ int j_groups64(int64_t n, int64_t tiles, int64_t sms) {
   constexpr int kCost[4] = {100, 102, 104, 117};
   const int64_t part = n & 127;
@@ -826,8 +826,9 @@ __device__ __forceinline__ void mixed_item(SM& sm, const float4* __restrict__ jA
 
 // ---- FP64 path --------------------------------------------------------------
 // Inputs, sums and results are FP64; the pair arithmetic runs in the fixed
-// point of fx64.cuh, which is at least as accurate as an FP64 evaluation of
-// the same formulas and 5 times as fast on this GPU.
+// point of fx64.cuh, in no component less accurate than an FP64 evaluation of
+// the same formulas and 4 times as fast on this GPU.  Pairs and tiles for which
+// it would not be so are evaluated in FP64.
 template <int NT, int JT>
 struct Fp64Smem {
   // a j-particle of the tile: (X0, X1), (X2, V0), (V1, V2), (M + k, fractions of

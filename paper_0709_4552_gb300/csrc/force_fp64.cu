@@ -9,7 +9,7 @@
 namespace {
 
 template <int NT, int JT, int JG = 1>
-// 16 warps per SM (128 registers): measured best of 12, 16 and 20
+// 16 warps per SM (128 registers): N = 20000, n = 2000 659 us, with 12 (168) 680
 __global__ void __launch_bounds__(NT, 512 / NT) force_fp64_kernel(
     const double* __restrict__ xp, const double* __restrict__ vp, const double* __restrict__ m,
     int64_t n_pad, int64_t N, const int32_t* __restrict__ list, int64_t n, int64_t tiles,
@@ -45,8 +45,8 @@ cudaError_t launch(nb_ctx* c, const int32_t* d_list, int64_t n, const nb_tuning&
     shape.threads = NT / jg;
   }
   int nsplit = cfg.nsplit > 0 ? cfg.nsplit : nb_auto_split(c, n, shape, per_sm);
-  // a single i-tile of fewer than NT in one wave (N = 200000, n = 16 145 -> 131 us, n = 64 228 -> 216; but n =
-  // 96 320 -> 337, n = 128 385 -> 396)
+  // a single i-tile of fewer than NT in one wave (N = 200000, n = 16 128 -> 96 us, n = 64 253 -> 246; but n =
+  // 96 364 -> 390, n = 128 435 -> 449)
   if (cfg.nsplit <= 0 && shape.threads < NT && n <= shape.threads) nsplit = std::min(nsplit, per_sm * c->sm_count);
   const int64_t itiles = (n + shape.threads - 1) / shape.threads;
   const int64_t n_j = ((c->n + JT - 1) / JT) * JT;

@@ -45,19 +45,19 @@ constexpr int kLT = 128;                     // threads per CTA = i-tile = row t
 constexpr int kLWarps = kLT / 32;
 // resident CTAs per SM asked for.  Mixed: 4 (128 registers, a few spilled) where
 // the force phase is the longest part of a step, 2 (no spills) where its
-// latencies are (us a block step, 4 / 2: N = 512 19.1 / 17.9, N = 12000 34.3 /
-// 31.5, N = 32768 67.5 / 64.4, N = 40000 84.4 / 88.0, N = 65536 169 / 184; all
-// before the corrector's loads were batched and its rows read ahead, which took
-// N = 12000 from 30.3 to 28.0 and N = 32768 from 62.7 to 58.3).  FP64: 3 (168;
-// with 4 the fixed-point pair spills: N = 1024 32.4 against 31.8 us a block
-// step, N = 32768 582 against 569)
+// latencies are (us a block step, 4 / 2: N = 4096 20.0 / 17.4, N = 12000 29.1 /
+// 26.6, N = 32768 61.6 / 56.2, N = 40000 75.3 / 74.9, N = 60000 131.6 / 138.4, N =
+// 65536 155.1 / 163.2).  FP64: 3 (168; with 4 the fixed-point pair spills: N =
+// 1024 34.8 against 32.2 us a block step, N = 8192 81.9 against 75.5, N = 32768
+// 641 against 640)
 constexpr int kLPerSmMixed = 4, kLPerSmMixedSmall = 2, kLPerSm64 = 3;
 constexpr int64_t kLMixedSmallHi = 32768, kLMixedTwoLo = 1024;
 // j-tiles (the mixed one = the box tile).  FP64: an item's tile is its share of
 // a small system's force phase, so those take 32 and at least two CTAs per SM:
-// N = 1024 31.8 us a block step against 40.7 with 64 and one CTA (44.9 with 64
-// and the mixed path's grid), N = 4096 47 against 58 (79); from N = 16384 the
-// splits are long and 64 stages better (177 against 194).
+// N = 1024 32.2 us a block step against 42.9 with 64 on the same grid (45.2 on
+// the mixed path's; with one shared step 52.1, 49.7 and 125), N = 4096 46.9
+// against 55.3 (80.3), N = 8192 75.5 against 79.8 (101); from N = 16384 the
+// splits are long and 64 stages better (193 against 205).
 constexpr int kLMixJT = 128, kLF64JT = 64, kLF64JTSmall = 32;
 // (Up to two tiles of 64, N = 128, every loop driver splits the sums alike and
 // gives the same bits.)
@@ -66,8 +66,8 @@ constexpr long long kWaitNs = 4000000000LL;  // a barrier wait of the loop gives
 constexpr unsigned int kPollCap = 1u << 26;  // ... or after this many polls
 constexpr unsigned long long kInfBits = 0x7FF0000000000000ULL;  // +inf
 // force items per step: about this many per CTA.  Mixed, us a block step with 2,
-// 3, 4, 6: N = 24000 43.0, 42.5, 42.3, 42.5; N = 40000 81.2, 80.5, 81.0, 81.8.
-// FP64 with 2 and 4: N = 16384 176.7, 178.4; N = 32768 573, 559.
+// 3, 4, 6: N = 24000 40.0, 39.5, 39.5, 39.8; N = 40000 76.2, 75.4, 75.8, 77.0.
+// FP64 with 2 and 4: N = 4096 46.9, 47.1; N = 16384 193, 193; N = 32768 640, 600.
 constexpr int kLItemWavesMixed = 3, kLItemWaves64 = 2;
 constexpr int64_t kLMaxSplits = 256;         // ... in at most this many j-splits
 constexpr int kMaxSmid = 1024;               // SM ids counted by the CTA placement
@@ -348,8 +348,9 @@ __device__ void predict_rows(const LoopArgs& p, int64_t r0, int64_t r1, double t
 
 // groups of threads that share the j of an item's tile (a step's i-tile is kLT
 // divided by them), and the i-tiles.  (FP64: none, as the item's two more forms
-// cost the loop registers: N = 1024 with one shared step 48.7 -> 49.9 us, N =
-// 4096 45.3 -> 46.7, and 31.0 -> 31.1 for the small blocks of N = 1024.)
+// cost the loop registers: N = 1024 with one shared step 51.9 -> 61.3 us, N =
+// 8192 75.2 -> 77.3, against 31.9 -> 28.9 for the small blocks of N = 1024 and
+// 47.0 -> 46.4 at N = 4096.)
 template <bool MIXED>
 __device__ __forceinline__ int loop_groups(int64_t n, int64_t jtiles, unsigned int G) {
   return MIXED ? nbk::j_groups(n, jtiles, G) : 1;
@@ -380,7 +381,7 @@ __device__ __forceinline__ int64_t loop_splits(int64_t n, int64_t nI, int64_t jt
 // Up to 64 positions: 32 a round, which lanes 0-3 correct together (the
 // correction's FP64 chain is on the critical path of a step); more: one or two
 // threads each, as the FP64 unit is then busy anyway (N = 1024 in FP64, every
-// particle at every step: 33 us a step against 43 in rounds of 32).
+// particle at every step: 52.1 us a step against 60.5 in rounds of 32).
 __device__ __forceinline__ int round_of(int mycnt) { return mycnt <= 64 ? 32 : kLT; }
 struct OwnRow {
   int L, l, q;
@@ -553,8 +554,8 @@ __global__ void __launch_bounds__(kLT, PER_SM) loop_kernel(LoopArgs p) {
   __shared__ LoopSmem s;
   // the variants for small systems, whose steps are a chain of latencies; in
   // the others reading ahead costs the force items registers (N = 60000 mixed
-  // 143.4 us a block step against 140.0), and FP64 items placed ahead of time
-  // balance worse (N = 16384 179 against 176)
+  // 139.4 us a block step against 131.3), and FP64 items placed ahead of time gain
+  // nothing (N = 16384 192 against 193, N = 32768 638 against 640)
   constexpr bool kShort = MIXED ? PER_SM == kLPerSmMixedSmall : JT == kLF64JTSmall;
   constexpr bool kPlaced = MIXED || kShort;  // the first item by the CTA's place
   const unsigned int G = gridDim.x;

@@ -415,7 +415,7 @@ def nb_step(ctx):
 
 def nb_integrate(ctx, t_end, use_graph=False, loop=None):
     """Block steps to t_end.  loop: NB_LOOP_HOST, NB_LOOP_GRAPH,
-    NB_LOOP_PERSISTENT, NB_LOOP_CLUSTER or NB_LOOP_AUTO (the fastest for the
+    NB_LOOP_PERSISTENT, NB_LOOP_CLUSTER or NB_LOOP_AUTO (chosen for the
     context's size); without it, use_graph picks the graph or host loop."""
     if loop is None:
         loop = NB_LOOP_GRAPH if use_graph else NB_LOOP_HOST
